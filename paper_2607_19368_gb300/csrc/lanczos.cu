@@ -555,7 +555,7 @@ int lanczos_plan(int64_t nmax, int D, int r, int nprob, int* groups, int* ctas_p
     *groups = (int)gr;
     *ctas_per_group = (int)g;
   }
-  // rows per CTA must fit the shared-memory staging of u
+  // at most 8192 rows per CTA (one prompt of 1.2 million tokens)
   const int64_t rows = (nmax + *ctas_per_group - 1) / *ctas_per_group;
   if (rows > 8192) return SLS_ERR_UNSUPPORTED;
   (void)D;
@@ -574,57 +574,41 @@ int launch_lanczos(const LanczosBatch& bt, void* scratch, size_t scratch_bytes, 
   // barrier words and group sums of every group start at zero (one strided memset)
   SLS_CUDA_TRY(cudaMemset2DAsync((char*)scratch + L.bar, L.total, 0, L.zero_end - L.bar, groups,
                                  stream));
-  const int C4 = bt.D / 4;
-  const int P = (C4 >= LZ_CT) ? 1 : (LZ_CT / C4);
-  const int gpt = gpt_of(bt.D);
-  if (gpt == 0) return SLS_ERR_UNSUPPORTED;
-  const int teams = lz_teams(gpt, P);
-  // z' of the strip, rounded up to an even count so the arrays after it stay
-  // 16-byte aligned
-  const int rows_cap = (int)(((bt.nmax + g - 1) / g + 2) & ~(int64_t)1);
-  const size_t limit = 227 * 1024 - 1024;  // leave room for static shared memory
+  if (bt.D > SLS_MAX_D) return SLS_ERR_UNSUPPORTED;
   if (bt.phi_bf16 && (bt.D % 8)) return SLS_ERR_UNSUPPORTED;  // 16-byte rows for the copies
-  const int esz = bt.phi_bf16 ? 2 : 4;
-  // the stage count and the mbarriers that go with it: take the largest S
-  // whose ring and other shared memory fit
-  RingShape R = ring_shape(bt.D, q_ld(bt.r), 0, esz, teams);
+  const LzShape shp = lz_shape(bt.D);
+  const size_t limit = 227 * 1024 - 1024;  // leave room for static shared memory
+  const size_t stage = lz_stage_bytes(bt.D, q_ld(bt.r), bt.phi_bf16 ? 2 : 4, shp.R);
+  const int teams = LZ_NCW / shp.wpr;
+  // the deepest rings that fit; at least 2 stages each: a team of several
+  // warps refills a slot once the exchange of its next batch shows that every
+  // warp is done with it, so a ring of one stage would wait for its own refill
+  // (and the pass ends use two stages of room)
   int stages = 0;
-  for (int s = RING_MAX_STAGES; s >= 1; --s) {
-    if ((size_t)s * R.stage + lz_smem_other(bt.D, bt.r, rows_cap, teams, s) <= limit) {
+  for (int s = LZ_MAX_STAGES; s >= 2; --s) {
+    if ((size_t)teams * s * stage + lz_smem_other(bt.r, shp, s) <= limit) {
       stages = s;
       break;
     }
   }
-  // Room for the pass ends' scratch in the ring, and at least 2 teams + 2
-  // stages: a team refills the slots of its previous pair after the first
-  // barrier of its current pair, so chunk c is issued after the first barrier
-  // of the pair `teams` pairs after the one holding chunk c - S; with fewer
-  // stages (or 2 teams + 1) a team would wait for a chunk that only its own
-  // later refill issues.
-  if (stages < 2 * teams + 2) return SLS_ERR_UNSUPPORTED;
-  if ((size_t)stages * R.stage < lz_pass_end_bytes(gpt, bt.r, teams)) return SLS_ERR_UNSUPPORTED;
-  const size_t smem = (size_t)stages * R.stage + lz_smem_other(bt.D, bt.r, rows_cap, teams, stages);
-  const int kt = (bt.r <= 32) ? 1 : (bt.r <= 64) ? 2 : 4;  // 32-wide tiles of k < r
-#define SLS_LZ_CALL(fn) \
-  fn(bt, scratch, L.total, groups, g, rows_cap, stages, status, smem, stream, kt, teams)
-  if (bt.phi_bf16) {
-    switch (gpt) {
-      case 1: return SLS_LZ_CALL(launch_lanczos_bf16_gpt1);
-      case 2: return SLS_LZ_CALL(launch_lanczos_bf16_gpt2);
-      case 4: return SLS_LZ_CALL(launch_lanczos_bf16_gpt4);
-      case 8: return SLS_LZ_CALL(launch_lanczos_bf16_gpt8);
-      default: break;
-    }
-  } else {
-    switch (gpt) {
-      case 1: return SLS_LZ_CALL(launch_lanczos_gpt1);
-      case 2: return SLS_LZ_CALL(launch_lanczos_gpt2);
-      case 4: return SLS_LZ_CALL(launch_lanczos_gpt4);
-      case 8: return SLS_LZ_CALL(launch_lanczos_gpt8);
-      default: break;
-    }
-  }
-#undef SLS_LZ_CALL
+  if (stages < 2) return SLS_ERR_UNSUPPORTED;
+  const size_t smem = (size_t)teams * stages * stage + lz_smem_other(bt.r, shp, stages);
+#define SLS_LZ_CASE(NV, WPR)                                                               \
+  if (shp.nv == NV && shp.wpr == WPR)                                                      \
+    return bt.phi_bf16 ? launch_lanczos_bf16_##NV##_##WPR(bt, scratch, L.total, groups, g, \
+                                                          stages, status, smem, stream)    \
+                       : launch_lanczos_f32_##NV##_##WPR(bt, scratch, L.total, groups, g,  \
+                                                         stages, status, smem, stream)
+  SLS_LZ_CASE(2, 1);
+  SLS_LZ_CASE(3, 1);
+  SLS_LZ_CASE(4, 1);
+  SLS_LZ_CASE(6, 1);
+  SLS_LZ_CASE(8, 1);
+  SLS_LZ_CASE(6, 2);
+  SLS_LZ_CASE(8, 2);
+  SLS_LZ_CASE(8, 4);
+  SLS_LZ_CASE(8, 8);
+#undef SLS_LZ_CASE
   return SLS_ERR_UNSUPPORTED;
 }
 

@@ -1,0 +1,11 @@
+// Lanczos kernel instantiations for 3 float4 column groups of Phi per lane and
+// 1 warp per row (D <= 384), bfloat16 Phi, for every basis tile count KT.
+#include "lanczos_kernel.cuh"
+
+namespace sls {
+
+int launch_lanczos_bf16_3_1(SLS_LZ_LAUNCH_ARGS) {
+  return launch_lanczos_kt<3, 1, uint16_t>(SLS_LZ_PASS_ARGS);
+}
+
+}  // namespace sls
