@@ -388,9 +388,9 @@ int sls_compress_tokens(const sls_config_t* cfg, const void* table, int x_dtype,
  * that sls_lanczos_topr takes.  Arguments and results are those of
  * sls_lanczos_topr (the caller still passes Phi, q1 and the output arrays).
  *
- * Scratch lives in one statically sized device array of
- * SLS_NOALLOC_MAX_BYTES inside the library; every GPU that loads the library
- * holds it until the process exits.  No cudaMalloc, cudaFree or allocating
+ * Scratch lives in one statically sized device array inside the library
+ * (SLS_NOALLOC_MAX_BYTES and 24 MiB for the kernel's exchange slots); every
+ * GPU that loads the library holds it until the process exits.  No cudaMalloc, cudaFree or allocating
  * library routine is called.  The first call on a device (with that device
  * current) looks up the array's device address once; make that first call
  * before any stream capture.  All calls share the array and it keeps the
@@ -403,8 +403,8 @@ int sls_compress_tokens(const sls_config_t* cfg, const void* table, int x_dtype,
  * process.  *r_eff is set to -1 when the call is enqueued and stays -1 if a
  * device-side wait gave up.  Errors: those of sls_lanczos_topr (arguments are
  * checked before anything is enqueued), and SLS_ERR_WORKSPACE, with nothing
- * enqueued, when sls_lanczos_workspace_size(N, D, r) exceeds
- * SLS_NOALLOC_MAX_BYTES.
+ * enqueued, when sls_lanczos_workspace_size(N, D, r) without those slots
+ * exceeds SLS_NOALLOC_MAX_BYTES.
  */
 #define SLS_NOALLOC_MAX_BYTES (32u << 20)
 int sls_lanczos_topr_noalloc(const float* Phi, int64_t N, int D, int r,

@@ -87,6 +87,10 @@ struct LanczosBatch {
 };
 
 size_t lanczos_scratch_bytes(int64_t nmax, int D, int r, int groups, int ctas_per_group);
+// Scratch of one problem's exchange slots beyond one g x D set of column
+// partials, one D-wide total and the scalars' sums (what
+// SLS_NOALLOC_MAX_BYTES counts).
+size_t lanczos_exchange_extra(int64_t N, int D, int r);
 int lanczos_plan(int64_t nmax, int D, int r, int nprob, int* groups, int* ctas_per_group);
 int launch_lanczos(const LanczosBatch& bt, void* scratch, size_t scratch_bytes, int* status,
                    int groups, int ctas_per_group, cudaStream_t stream);

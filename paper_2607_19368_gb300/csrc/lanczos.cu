@@ -567,32 +567,42 @@ size_t lanczos_scratch_bytes(int64_t nmax, int D, int r, int groups, int g) {
   return (size_t)groups * lz_layout(nmax, D, r, g).total;
 }
 
+size_t lanczos_exchange_extra(int64_t N, int D, int r) {
+  int groups = 0, g = 0;
+  if (lanczos_plan(N, D, r, 1, &groups, &g) != SLS_OK) return 0;
+  const LzLayout L = lz_layout(N, D, r, g);
+  return L.ones_end - (256 + lz_al((size_t)2 * (r + 4) * 8) + lz_al((size_t)g * D * 8) +
+                       lz_al((size_t)D * 8));
+}
+
 int launch_lanczos(const LanczosBatch& bt, void* scratch, size_t scratch_bytes, int* status,
                    int groups, int g, cudaStream_t stream) {
   const LzLayout L = lz_layout(bt.nmax, bt.D, bt.r, g);
   if ((size_t)groups * L.total > scratch_bytes) return SLS_ERR_WORKSPACE;
-  // barrier words and group sums of every group start at zero (one strided memset)
-  SLS_CUDA_TRY(cudaMemset2DAsync((char*)scratch + L.bar, L.total, 0, L.zero_end - L.bar, groups,
-                                 stream));
+  // the exchange slots of every group start empty (one strided memset)
+  SLS_CUDA_TRY(cudaMemset2DAsync((char*)scratch + L.bar, L.total, 0xff, L.ones_end - L.bar,
+                                 groups, stream));
   if (bt.D > SLS_MAX_D) return SLS_ERR_UNSUPPORTED;
   if (bt.phi_bf16 && (bt.D % 8)) return SLS_ERR_UNSUPPORTED;  // 16-byte rows for the copies
   const LzShape shp = lz_shape(bt.D);
   const size_t limit = 227 * 1024 - 1024;  // leave room for static shared memory
   const size_t stage = lz_stage_bytes(bt.D, q_ld(bt.r), bt.phi_bf16 ? 2 : 4, shp.R);
   const int teams = LZ_NCW / shp.wpr;
+  const LzOwn own = lz_own(bt.D, bt.r, g);
+  const int red = lz_red_rows(own) * own.WB;
   // the deepest rings that fit; at least 2 stages each: a team of several
   // warps refills a slot once the exchange of its next batch shows that every
   // warp is done with it, so a ring of one stage would wait for its own refill
   // (and the pass ends use two stages of room)
   int stages = 0;
   for (int s = LZ_MAX_STAGES; s >= 2; --s) {
-    if ((size_t)teams * s * stage + lz_smem_other(bt.r, shp, s) <= limit) {
+    if ((size_t)teams * s * stage + lz_smem_other(bt.D, bt.r, shp, red, s) <= limit) {
       stages = s;
       break;
     }
   }
   if (stages < 2) return SLS_ERR_UNSUPPORTED;
-  const size_t smem = (size_t)teams * stages * stage + lz_smem_other(bt.r, shp, stages);
+  const size_t smem = (size_t)teams * stages * stage + lz_smem_other(bt.D, bt.r, shp, red, stages);
 #define SLS_LZ_CASE(NV, WPR)                                                               \
   if (shp.nv == NV && shp.wpr == WPR)                                                      \
     return bt.phi_bf16 ? launch_lanczos_bf16_##NV##_##WPR(bt, scratch, L.total, groups, g, \
@@ -602,11 +612,11 @@ int launch_lanczos(const LanczosBatch& bt, void* scratch, size_t scratch_bytes, 
   SLS_LZ_CASE(2, 1);
   SLS_LZ_CASE(3, 1);
   SLS_LZ_CASE(4, 1);
-  SLS_LZ_CASE(6, 1);
-  SLS_LZ_CASE(8, 1);
-  SLS_LZ_CASE(6, 2);
-  SLS_LZ_CASE(8, 2);
-  SLS_LZ_CASE(8, 4);
+  SLS_LZ_CASE(3, 2);
+  SLS_LZ_CASE(4, 2);
+  SLS_LZ_CASE(3, 4);
+  SLS_LZ_CASE(4, 4);
+  SLS_LZ_CASE(4, 8);
   SLS_LZ_CASE(8, 8);
 #undef SLS_LZ_CASE
   return SLS_ERR_UNSUPPORTED;

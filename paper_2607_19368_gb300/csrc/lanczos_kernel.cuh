@@ -4,8 +4,8 @@
 // groups of CTAs; a group owns one problem at a time (one prompt, or one
 // adaptive window) and every CTA owns a contiguous strip of the problem's rows
 // of the feature matrix Phi (N x D, float32 or bfloat16) and of the basis Q.
-// The eight warps of a CTA form teams of WPR warps (WPR = 1 up to D = 1024, 2
-// up to 2048, 4, 8): a team takes whole rows of the strip, R at a time, and
+// The eight warps of a CTA form teams of WPR warps (WPR = 1 up to D = 512, 2 up
+// to 1024, 4 up to 2048, then 8): a team takes whole rows of the strip, R at a time, and
 // every lane keeps its columns of w_j and of the column sums in registers.  A
 // team streams its rows through its own shared-memory ring with
 // one-dimensional bulk copies (cp.async.bulk + mbarrier): a stage holds R rows
@@ -17,13 +17,14 @@
 // j of Q), the CTA partials of Phi^T z' and the group sums of c = Q^T z' and
 // of |z'|^2:
 //
-//   [barrier 1]
-//   slice phase   c from the group sums; each CTA finishes a slice of the D
-//                 columns of Phi^T z1 = Phi^T z' - sum_k c_k w_k with
-//                 z1 = z' - Q c and w_k = Phi^T q_k kept from earlier steps.
-//   [barrier 2]
+//   exchange 1    every CTA publishes its partials of Phi^T z', c and |z'|^2;
+//                 the owner of a coefficient or column adds the CTAs' partials.
+//   exchange 2    the owners publish c and |z'|^2; column owners subtract
+//                 sum_k c_k w_k: Phi^T z1 with z1 = z' - Q c and w_k =
+//                 Phi^T q_k kept from earlier steps.
+//   exchange 3    the owners publish Phi^T z1; every CTA forms
 //                 beta_{j-1} = |z1| = sqrt(|z'|^2 - |c|^2), the break test,
-//                 w_j = Phi^T q_j, alpha_j = |w_j|^2.
+//                 w_j = Phi^T q_j = Phi^T z1 / beta and alpha_j = |w_j|^2.
 //   fused pass    per R rows of a team: the implicit matvec rows s = Phi w_j
 //                 (Eq. implicit_matvec); z1 = z' - Q c and q_j = z1 / beta;
 //                 the three-term recurrence z' = s - alpha_j q_j -
@@ -39,11 +40,30 @@
 // would change z1 only in the second order of the rounding unit.  Passes
 // alternate direction so each starts on the rows the previous one left in
 // L2.  Vectors are double-float (two float32) and every sum over N or D is
-// compensated.  The column sums of Phi^T z' are added over the CTAs in a fixed
-// order; the group sums of the scalars (c, |z'|^2, |Phi^T z1|^2) are float64
-// atomic additions, one per CTA, whose order may vary in the last float64 bit.
-// Barriers and waits poll without sleeping and give up after about a second
-// of clock cycles, reporting SLS_ERR_TIMEOUT through the status word.
+// compensated; every sum over the CTAs runs in a fixed order (c and |z'|^2 in
+// float64).  Waits poll without sleeping and give up after about a second of
+// clock cycles, reporting SLS_ERR_TIMEOUT through the status word.
+//
+// The exchanges.  The CTAs of a group hold no barrier: a value is published as
+// one 64-bit store into a slot that holds the all-ones pattern until then (a
+// NaN the arithmetic cannot produce), and a reader polls the value itself, so
+// an exchange costs one store and one load through L2.  Readers put the
+// pattern back: the partials' slots (two buffers, by exchange parity) by the
+// one CTA that reads them, as it reads them; the totals' slots (three buffers)
+// by their owner, one exchange later, when the partials of every CTA show that
+// all have read them.  A slot is written again only after its writer has seen
+// a later value from the CTA that put the pattern back, with one GPU-scope
+// fence per thread and step (before a pass's partials are published) between
+// the two on either side.
+//
+// A one-way trip through L2 takes 525 cycles within a die and 850 across (ping-
+// pong of two CTAs).  Two barriers of the group with the sums in between
+// (float64 atomics for the scalars, each phase behind its own round trips) took
+// 22000 cycles per step at N = 8180, D = 1024 on 152 CTAs, more than the pass
+// over Phi; the exchanges take 16000.  What is left is mostly their own
+// instructions: they run once per step, cold after the row loop.  A slot block
+// is contiguous per owner: polling partials spread by source (a sector per
+// value) saturated L2 and was slower than the barriers.
 //
 // Why whole rows per team: a row's scalars (q_j, z', its products with the
 // basis) are a serial chain of double-float operations.  When all eight warps
@@ -52,11 +72,12 @@
 // Here 32 / R lanes share a row's chain, R rows at a time, and the teams run
 // independently (with WPR = 1 a pass holds no barrier at all), so one team's
 // chain is hidden behind the sweeps of the others, and inside a warp behind the
-// row dots of the next R rows.  Measured against the CTA-wide form (whole
-// sls_lanczos_topr calls, both built and timed alternately): 64 windows of 2048
-// rows at D = 1024, r = 32 5.91 -> 4.32 ms; N = 32756, D = 2048, r = 64 4.57 ->
-// 4.01 ms; N = 8180, D = 1024, r = 32 0.750 -> 0.731 ms; windows of 1024 rows at
-// D = 256 2.95 -> 1.07 ms; N = 12000, D = 1536, r = 48 2.10 -> 1.34 ms.
+// row dots of the next R rows.  Measured against the CTA-wide form with two
+// group barriers per step (whole sls_lanczos_topr calls, both built and timed
+// alternately): 64 windows of 2048 rows at D = 1024, r = 32 5.91 -> 3.87 ms;
+// N = 32756, D = 2048, r = 64 4.57 -> 3.82 ms; N = 8180, D = 1024, r = 32 0.750 ->
+// 0.600 ms; windows of 1024 rows at D = 256 2.95 -> 1.01 ms; N = 12000, D = 1536,
+// r = 48 2.10 -> 1.46 ms; N = 488, D = 256, r = 16 0.308 -> 0.223 ms.
 //
 // The kernel is a template over NV (float4 column groups of Phi per lane), WPR,
 // KT (32-wide tiles of the basis index k < r), FULLD (D = 128 NV WPR, no ragged
@@ -79,31 +100,95 @@ constexpr int LZ_NT = LZ_NCW * 32;        // threads per CTA
 constexpr unsigned BAR_ALL = 1;           // named barrier: every warp
 constexpr unsigned BAR_TEAM = 2;          // named barriers 2 .. 5: the warps of a team
 
+// Who owns what in the exchanges of a group of g CTAs: CTA i the columns
+// [i cw, (i + 1) cw) and, counted from the last CTA, the coefficients
+// [i' kw, (i' + 1) kw) of the r + 1 (c_0 .. c_{r-1}, |z'|^2), i' = g - 1 - i.
+// WB: slots of a block (one CTA's partials for one owner): kw coefficients,
+// then cw columns.  The form of the owner's sums (mode):
+//   0  blocks of at most 16 slots (large groups), padded to a power of two: the
+//      threads split over (source, slot pair), then a warp per sum
+//   1  at most 256 slots, padded likewise: the same, then a thread per sum
+//   2  wider (a few CTAs): a thread per column pair adds the sources
+struct LzOwn {
+  int cw, kw, WB, mode;
+};
+
+__host__ __device__ inline LzOwn lz_own(int D, int r, int g) {
+  LzOwn o;
+  o.cw = (D + g - 1) / g;
+  o.kw = (r + 1 + g - 1) / g;
+  o.WB = 2;
+  while (o.WB < o.cw + o.kw) o.WB *= 2;
+  o.mode = o.WB <= 16 ? 0 : o.WB <= 256 ? 1 : 2;
+  if (o.mode == 2) {
+    o.cw = (o.cw + 1) & ~1;
+    o.kw = (o.kw + 1) & ~1;
+    o.WB = o.cw + o.kw;
+  }
+  return o;
+}
+
+// Rows of WB sums that the warps leave in shared memory (modes 0 and 1): one
+// per warp, or per set of warps that spans the WB / 2 slot pairs.
+__host__ __device__ inline int lz_red_rows(LzOwn o) {
+  return o.mode == 2 ? 0 : o.WB <= 64 ? LZ_NCW : 2 * LZ_NT / o.WB;
+}
+
 // Per-group scratch layout (byte offsets), identical on host and device.
-//   acc:   2 x (r + 4) float64 group sums by step parity: c_k (k <= r), |z'|^2
-//          at r + 1, |Phi^T z1|^2 at r + 2 (float64 atomic additions)
-//   wpart: g x D double-float CTA partials of Phi^T z'
-//   wred:  D double-float: Phi^T z1, finished slice by slice
-//   Wm:    r x D double-float: w_k = Phi^T q_k (each CTA writes its slice)
+//   bar:  word 0: all ones, 0 once a CTA of the group has given up
+//   part: 2 x g owners x g sources x WB values: the sources' partials of
+//         c, |z'|^2 and the columns of Phi^T z', double-float
+//   tot:  3 x E values: Phi^T z1 (D), c (r) and |z'|^2, double-float
+//   Wm:   r x D double-float: w_k = Phi^T q_k (each CTA its columns; by column
+//         in mode 0, else by k)
+// [bar, ones_end) is set to all ones before the launch.
 struct LzLayout {
-  size_t bar, acc, zero_end, wpart, wred, Wm, total;
+  size_t bar, part, tot, ones_end, Wm, total;
 };
 
 __host__ __device__ inline size_t lz_al(size_t x) { return (x + 255) & ~(size_t)255; }
-__host__ __device__ inline int lz_acc_stride(int r) { return r + 4; }
+__host__ __device__ inline int lz_exch_len(int D, int r) { return (D + r + 2) & ~1; }
 
 __host__ __device__ inline LzLayout lz_layout(int64_t nmax, int D, int r, int g) {
   (void)nmax;
   LzLayout L;
+  const size_t E = (size_t)lz_exch_len(D, r);
   size_t o = 0;
   L.bar = o;    o += 256;
-  L.acc = o;    o += lz_al((size_t)2 * lz_acc_stride(r) * sizeof(double));
-  L.zero_end = o;  // [bar, zero_end) starts at zero before the launch
-  L.wpart = o;  o += lz_al((size_t)g * D * sizeof(float2));
-  L.wred = o;   o += lz_al((size_t)D * sizeof(float2));
+  L.part = o;   o += lz_al(2 * (size_t)g * g * lz_own(D, r, g).WB * 8);
+  L.tot = o;    o += lz_al(3 * E * 8);
+  L.ones_end = o;
   L.Wm = o;     o += lz_al((size_t)D * r * sizeof(float2));
   L.total = o;
   return L;
+}
+
+// ---- exchange slots ---------------------------------------------------------
+
+constexpr unsigned long long LZ_EMPTY = ~0ull;
+
+SLS_DEV unsigned long long x_ld(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+SLS_DEV void x_ld2(const unsigned long long* p, unsigned long long& a, unsigned long long& b) {
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+SLS_DEV void x_st(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+SLS_DEV void x_st2(unsigned long long* p, unsigned long long a, unsigned long long b) {
+  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
+}
+// A double-float as a slot's value, never the empty pattern.
+SLS_DEV unsigned long long x_pack(dfloat v) {
+  const unsigned long long u =
+      ((unsigned long long)__float_as_uint(v.lo) << 32) | (unsigned long long)__float_as_uint(v.hi);
+  return u == LZ_EMPTY ? 0x7fffffff7fffffffull : u;
+}
+SLS_DEV dfloat x_unpack(unsigned long long u) {
+  return df_make(__uint_as_float((unsigned)u), __uint_as_float((unsigned)(u >> 32)));
 }
 
 SLS_DEV dfloat shfl_xor_df(dfloat v, int m) {
@@ -112,32 +197,31 @@ SLS_DEV dfloat shfl_xor_df(dfloat v, int m) {
   return v;
 }
 
-// float64 atomic addition whose result is not used (a reduction operation)
-SLS_DEV void red_add_f64(double* p, double v) { atomicAdd(p, v); }
-
 // The split of a row over a team: NV float4 column groups per lane, WPR warps
-// (NV * 32 * 4 * WPR >= D), R rows at a time.  NV <= 8: a lane keeps w_j, the
-// column sums and their offset sums (10 float32 per column pair and group) in
-// registers, 160 of 255 at NV = 8.  The narrowest split that holds the row is
-// taken: lanes past the row's end would do their share of the arithmetic on
-// nothing.  R = 4 up to D = 512, where a row's sweeps are shorter than its row
-// work; 2 above, where 3 stages of 2 rows per team fill the shared memory.
+// (NV * 32 * 4 * WPR >= D), R rows at a time.  A lane keeps w_j, the column sums
+// and their offset sums (10 float32 per column pair and group) in registers:
+// at NV = 4 with R = 4 the row loop runs without spills.  Measured at D = 1024 /
+// 2048 (N = 8180 / 32756; 64 windows of 2048 rows): NV = 8 with half the warps
+// and R = 2, whose 160 registers of state spill, 690 / 3937 / 4300 us; NV = 4
+// 630 / 3825 / 3863; NV = 2 with twice the warps and R = 8 668 / 4217 / 4283.
+// The narrowest split that holds the row is taken: lanes past the row's end
+// would do their share of the arithmetic on nothing.
 struct LzShape {
   int nv, wpr, R;
 };
 
-__host__ __device__ constexpr int lz_rows(int nv) { return nv >= 6 ? 2 : 4; }
+__host__ __device__ constexpr int lz_rows(int nv) { return nv >= 8 ? 2 : 4; }
 
 __host__ __device__ inline LzShape lz_shape(int D) {
   LzShape s{8, 8, lz_rows(8)};
   if (D <= 256) s = LzShape{2, 1, lz_rows(2)};
   else if (D <= 384) s = LzShape{3, 1, lz_rows(3)};
   else if (D <= 512) s = LzShape{4, 1, lz_rows(4)};
-  else if (D <= 768) s = LzShape{6, 1, lz_rows(6)};
-  else if (D <= 1024) s = LzShape{8, 1, lz_rows(8)};
-  else if (D <= 1536) s = LzShape{6, 2, lz_rows(6)};
-  else if (D <= 2048) s = LzShape{8, 2, lz_rows(8)};
-  else if (D <= 4096) s = LzShape{8, 4, lz_rows(8)};
+  else if (D <= 768) s = LzShape{3, 2, lz_rows(3)};
+  else if (D <= 1024) s = LzShape{4, 2, lz_rows(4)};
+  else if (D <= 1536) s = LzShape{3, 4, lz_rows(3)};
+  else if (D <= 2048) s = LzShape{4, 4, lz_rows(4)};
+  else if (D <= 4096) s = LzShape{4, 8, lz_rows(4)};
   return s;
 }
 
@@ -149,11 +233,43 @@ __host__ __device__ inline unsigned lz_stage_bytes(int D, int ldq, int esz, int 
   return (unsigned)R * ((unsigned)D * (unsigned)esz + (unsigned)ldq * 8u);
 }
 
+// w_j passes through shared memory when several teams need each column.
+__host__ __device__ constexpr bool lz_stage_w(int wpr) { return wpr <= 2; }
+
+// What the exchanges of a CTA share, at the start of its shared memory: they
+// are functions of their own (not inlined), so that the compiler gives the row
+// loops of the kernel all registers.
+struct LzXch {
+  unsigned long long *part, *tot;
+  float2* Wm;
+  unsigned* poison;
+  int* status;
+  double *alpha_out, *beta_out;  // of the problem (rank 0)
+  LzOwn own;
+  int g, rank, D, r, E;
+  int cbeg, cend, kbeg, kend;   // this CTA's columns and coefficients
+  unsigned cw_magic;            // c / cw = umulhi(c, cw_magic)
+  unsigned rings, ring_bytes;   // offsets: the teams' rings (column sums, coefficients),
+  unsigned whs, wls, red, cs;   // w_j, sums of a block, c
+  float2 tol, scale;            // of the break test
+  float2 invb, beta, alpha;     // of the step
+  float2 tmpw[LZ_NCW];
+  int brk;
+  volatile int err;             // a wait of this CTA gave up
+};
+
+constexpr unsigned LZ_RING0 = (sizeof(LzXch) + 127) / 128 * 128;  // offset of the first ring
+
 // Shared memory besides the rings (bytes), in the order the kernel carves it:
-// the row sums the warps of a team exchange, c, then the mbarriers.
-__host__ __device__ inline size_t lz_smem_other(int r, LzShape s, int stages) {
+// the exchanges' state (before the rings); w_j (high parts, low parts), the
+// warps' sums of an exchange block (red slots), the row sums the warps of a
+// team exchange, c, then the mbarriers.
+__host__ __device__ inline size_t lz_smem_other(int D, int r, LzShape s, int red, int stages) {
   const int teams = LZ_NCW / s.wpr;
-  size_t b = sizeof(float4) * (size_t)(teams * 2 * s.R * s.wpr);
+  size_t b = LZ_RING0;
+  b += lz_stage_w(s.wpr) ? 2 * sizeof(float) * (size_t)D : 0;
+  b += sizeof(float2) * (size_t)red;
+  b += sizeof(float4) * (size_t)(teams * 2 * s.R * s.wpr);
   b += sizeof(float2) * (size_t)(r + 1);
   b = (b + 15) & ~(size_t)15;
   b += (size_t)teams * stages * 8;
@@ -219,6 +335,31 @@ SLS_DEV void last_row_phase(float2* __restrict__ Qs, int ldq, int nrows, int j,
   }
 }
 
+// 1 / sqrt(x), x > 0: the float32 reciprocal square root y and the correction
+// y (h / 2 + 3 h^2 / 8) with h = 1 - x y^2 formed to double-float precision;
+// |h| < 2^-21, so the series ends below 2^-62 and the rounding of the
+// correction stays near 2^-46 of the result.
+SLS_DEV dfloat df_rsqrt(dfloat x) {
+  // x in the float32 range; a power of four keeps x y^2 clear of its ends
+  float sc = 1.f, scy = 1.f;
+  if (x.hi < 0x1p-90f) {
+    sc = 0x1p60f;
+    scy = 0x1p30f;
+  }
+  x = df_make(x.hi * sc, x.lo * sc);
+  const float y = rsqrtf(x.hi);
+  float p, e;
+  two_prod(y, y, p, e);
+  const dfloat t = df_mul(x, df_make(p, e));
+  const float h = __fsub_rn(__fsub_rn(1.f, t.hi), t.lo);
+  const float corr = y * (h * __fmaf_rn(0.375f, h, 0.5f));
+  const dfloat r = df_norm(y, corr);
+  return df_make(r.hi * scy, r.lo * scy);
+}
+
+// a < b (false if either is NaN)
+SLS_DEV bool df_less(dfloat a, dfloat b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
+
 // A wait of this CTA gave up: report it and leave at the next group barrier.
 SLS_DEV void lz_fail(int* status, volatile int* err) {
   atomicExch(status, SLS_ERR_TIMEOUT);
@@ -231,104 +372,442 @@ SLS_DEV int nprob_of(const LanczosBatch& bt) {
   return nprob;
 }
 
-// Slice phase of step j for the CTA's columns [cbeg, cend): the sum of the g
-// CTA partials of Phi^T z' minus sum_{k < j} c_k w_k, into wred, and the
-// CTA's part of |Phi^T z1|^2 (each thread returns its own columns' share).
-// A column is summed by a segment of G lanes of one warp (G a power of two,
-// as many as the compute threads allow), each lane over every G-th partial
-// and every G-th basis index, then a butterfly within the segment.  The loads
-// of the first column batch are issued before the named barrier after which
-// c is ready (warp 0 fills it meanwhile); `synced` records that barrier.
-// True when the last warp of the CTA sums no column in the slice phase (the
-// column split of slice_columns below): it is free then for beta.
-template <int NCW>
-SLS_DEV bool slice_last_warp_idle(int ncol) {
-  constexpr int NCT = NCW * 32;
-  int G = 1;
-  while (G < 32 && G * 2 * ncol <= NCT) G *= 2;
-  return (NCW - 1) * (32 / G) >= ncol;
-}
+// Polls of exchange slots by a warp, bounded: `more` is called by every lane
+// for each repetition and returns false once this CTA or another of the group
+// has given up.
+struct XWait {
+  unsigned* poison;   // word of the group: all ones until a CTA gives up
+  int* status;
+  volatile int* err;  // this CTA's flag
+  long long t0;
+  unsigned it;
 
-// c itself (cs[k] = the group sum accj[k], k < j) is loaded by warp cwarp:
-// after it has issued its first batch when it sums columns, so that both
-// round trips to L2 overlap, else before it reaches the named barrier.
-template <int NCW>
-SLS_DEV void load_c(float2* __restrict__ cs, const double* __restrict__ accj, int j) {
-  const int lane = threadIdx.x & 31;
-  for (int k = lane; k < j; k += 32) cs[k] = f2(df_from_double(accj[k]));
-}
-
-template <int NCW>
-SLS_DEV dfloat slice_columns(const float2* __restrict__ wpart, const float2* __restrict__ Wm,
-                             float2* __restrict__ wred, float2* __restrict__ cs,
-                             const double* __restrict__ accj, int cwarp, int g, int D, int j,
-                             int cbeg, int cend, bool& synced) {
-  constexpr int NCT = NCW * 32;
-  constexpr int BATCH = 8;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ncol = cend - cbeg;
-  int G = 1;
-  while (G < 32 && G * 2 * ncol <= NCT) G *= 2;
-  const int cpw = 32 / G;
-  const int sub = lane & (G - 1), slot = lane / G;
-  dfloat sq = df_make(0.f, 0.f);
-  for (int cb = warp * cpw; cb < ncol; cb += NCW * cpw) {
-    const int cl = cb + slot;
-    const bool valid = cl < ncol;
-    const int c = cbeg + (valid ? cl : 0);
-    // partials of Phi^T z' and basis columns: the first batches in flight together
-    float2 pv[BATCH], wv[BATCH];
-#pragma unroll
-    for (int u = 0; u < BATCH; ++u) {
-      const int b = sub + G * u;
-      pv[u] = (valid && b < g) ? wpart[(size_t)b * D + c] : make_float2(0.f, 0.f);
-      wv[u] = (valid && b < j) ? Wm[(size_t)b * D + c] : make_float2(0.f, 0.f);
+  __device__ __noinline__ bool more() {
+    bool bad = false;
+    if ((++it & 31u) == 0u) {
+      if (it == 32u) t0 = clock64();
+      if (*err) {
+        bad = true;
+      } else if (ld_relaxed_gpu(poison) != ~0u) {
+        *err = 1;
+        bad = true;
+      } else if (clock64() - t0 > SLS_WAIT_CYCLES) {
+        lz_fail(status, err);
+        atomicExch(poison, 0u);
+        bad = true;
+      }
     }
-    if (!synced && warp == cwarp) load_c<NCW>(cs, accj, j);
+    return !__any_sync(0xffffffffu, bad);
+  }
+};
+
+// One slot per lane (where `need`), polled until full.
+SLS_DEV unsigned long long x_poll(const unsigned long long* p, bool need, XWait& w) {
+  unsigned long long v = need ? x_ld(p) : 0ull;
+  w.it = 0u;
+  while (__any_sync(0xffffffffu, v == LZ_EMPTY) && w.more())
+    if (v == LZ_EMPTY) v = x_ld(p);
+  return v;
+}
+
+// B pairs of slots p + u * step (those with need bit u) per lane; wa, wb: which
+// slots of a pair are ever written.
+template <int B>
+SLS_DEV void x_poll2(const unsigned long long* p, size_t step, unsigned need, bool wa, bool wb,
+                     unsigned long long (&a)[B], unsigned long long (&b)[B], XWait& w) {
+#pragma unroll
+  for (int u = 0; u < B; ++u) {
+    a[u] = b[u] = 0ull;
+    if (need >> u & 1u) x_ld2(p + u * step, a[u], b[u]);
+  }
+  w.it = 0u;
+  for (;;) {
+    bool miss = false;
+#pragma unroll
+    for (int u = 0; u < B; ++u) miss |= (wa && a[u] == LZ_EMPTY) || (wb && b[u] == LZ_EMPTY);
+    if (!__any_sync(0xffffffffu, miss) || !w.more()) break;
+#pragma unroll
+    for (int u = 0; u < B; ++u)
+      if ((need >> u & 1u) && ((wa && a[u] == LZ_EMPTY) || (wb && b[u] == LZ_EMPTY)))
+        x_ld2(p + u * step, a[u], b[u]);
+  }
+}
+
+SLS_DEV bool named_sync_any(unsigned id, unsigned nthreads, bool pred) {
+  unsigned r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n"
+      " bar.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((unsigned)pred), "r"(id), "r"(nthreads)
+      : "memory");
+  return r != 0;
+}
+
+// The kernel's dynamic shared memory.  Functions that are not inlined address
+// it from here by offsets: a pointer handed to them would lose its address
+// space.
+SLS_DEV unsigned char* lz_smem() {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  return smem_raw;
+}
+
+SLS_DEV LzXch& lz_xch() { return *reinterpret_cast<LzXch*>(lz_smem()); }
+
+// After a pass: the column sums and coefficient partials (k < K) the teams left
+// in their rings are added and published as exchange xpar; false when a wait of
+// this CTA has given up (nothing is published then).
+template <int TEAMS>
+__device__ __noinline__ bool lz_publish(int K, unsigned xpar) {
+  constexpr int NCT = LZ_NT;
+  LzXch& X = lz_xch();
+  const int tid = threadIdx.x;
+  if (named_sync_any(BAR_ALL, NCT, X.err != 0)) {
+    if (tid == 0) atomicExch(X.poison, 0u);
+    return false;
+  }
+  const LzOwn own = X.own;
+  const int g = X.g, rank = X.rank, D = X.D, r = X.r;
+  unsigned long long* part = X.part;
+  const unsigned cw_magic = X.cw_magic;
+  auto tcol = [&](int t) {
+    return reinterpret_cast<float2*>(lz_smem() + X.rings + (size_t)t * X.ring_bytes);
+  };
+  auto tco = [&](int t) { return tcol(t) + D; };
+  // slot i of this CTA's block for owner d
+  auto slot = [&](unsigned d, unsigned i) {
+    return part + (((size_t)xpar * g + d) * g + rank) * own.WB + i;
+  };
+  // coefficient e (|z'|^2 at r): the TEAMS partials summed by two lanes
+#pragma unroll 1
+  for (int e0 = 0; e0 <= r; e0 += NCT / 2) {
+    const int e = e0 + tid / 2, h = tid & 1;
     dfloat s = df_make(0.f, 0.f);
+    if (e < K || e == r)
+      for (int t = h; t < TEAMS; t += 2) s = df_add(s, dfv(tco(t)[e]));
+    s = df_add_fast(s, shfl_xor_df(s, 1));
+    if (h == 0 && e <= r) x_st(slot(g - 1 - e / own.kw, e % own.kw), x_pack(s));
+  }
+#pragma unroll 1
+  for (int c = 2 * tid; c < D; c += 2 * NCT) {
+    float4 v[TEAMS];
 #pragma unroll
-    for (int u = 0; u < BATCH; ++u) s = df_add_fast(s, dfv(pv[u]));
-    for (int b0 = sub + G * BATCH; b0 < g; b0 += G * BATCH) {
+    for (int t = 0; t < TEAMS; ++t) v[t] = reinterpret_cast<const float4*>(tcol(t) + c)[0];
 #pragma unroll
-      for (int u = 0; u < BATCH; ++u) {
-        const int b = b0 + G * u;
-        pv[u] = (valid && b < g) ? wpart[(size_t)b * D + c] : make_float2(0.f, 0.f);
+    for (int w = 1; w < TEAMS; w *= 2)
+#pragma unroll
+      for (int t = 0; t + w < TEAMS; t += 2 * w) {
+        const dfloat a = df_add_fast(df_make(v[t].x, v[t].y), df_make(v[t + w].x, v[t + w].y));
+        const dfloat b = df_add_fast(df_make(v[t].z, v[t].w), df_make(v[t + w].z, v[t + w].w));
+        v[t] = make_float4(a.hi, a.lo, b.hi, b.lo);
       }
-#pragma unroll
-      for (int u = 0; u < BATCH; ++u) s = df_add_fast(s, dfv(pv[u]));
-    }
-    if (!synced) {
-      named_sync(BAR_ALL, NCT);  // c is in shared memory
-      synced = true;
-    }
-    // sum_k c_k w_k (Dot2), subtracted from the lane's part of the column sum
-    float ch = 0.f, cl2 = 0.f;
-#pragma unroll
-    for (int u = 0; u < BATCH; ++u) {
-      const int k = sub + G * u;
-      if (k < j) dot2_acc_df(ch, cl2, dfv(wv[u]), dfv(cs[k]));
-    }
-    for (int k0 = sub + G * BATCH; k0 < j; k0 += G * BATCH) {
-#pragma unroll
-      for (int u = 0; u < BATCH; ++u) {
-        const int k = k0 + G * u;
-        wv[u] = (valid && k < j) ? Wm[(size_t)k * D + c] : make_float2(0.f, 0.f);
-      }
-#pragma unroll
-      for (int u = 0; u < BATCH; ++u) {
-        const int k = k0 + G * u;
-        if (k < j) dot2_acc_df(ch, cl2, dfv(wv[u]), dfv(cs[k]));
-      }
-    }
-    s = df_sub(s, df_norm(ch, cl2));
-    for (int o = 1; o < G; o <<= 1) s = df_add_fast(s, shfl_xor_df(s, o));
-    if (sub == 0 && valid) {
-      wred[c] = f2(s);
-      dot2_acc_df(sq.hi, sq.lo, s, s);
+    const unsigned long long v0 = x_pack(df_make(v[0].x, v[0].y));
+    const unsigned long long v1 = x_pack(df_make(v[0].z, v[0].w));
+    const unsigned d0 = own.cw == 1 ? (unsigned)c : __umulhi((unsigned)c, cw_magic);
+    const unsigned i0 = (unsigned)c - d0 * own.cw;
+    if (own.mode == 2) {  // cw and kw are even: the pair has one owner
+      x_st2(slot(d0, own.kw + i0), v0, v1);
+    } else {
+      x_st(slot(d0, own.kw + i0), v0);
+      if (i0 + 1 < (unsigned)own.cw) x_st(slot(d0, own.kw + i0 + 1), v1);
+      else x_st(slot(d0 + 1, own.kw), v1);
     }
   }
-  if (!synced && warp == cwarp) load_c<NCW>(cs, accj, j);  // a warp without columns
-  return sq;
+  named_sync(BAR_ALL, NCT);  // the rings are free
+  return true;
+}
+
+// c (into shared memory) and beta_{j-1} = |z1|, by one warp: |z1|^2 = |z'|^2 -
+// |c|^2 (Q orthonormal; |c|^2 is below the rounding of |z'|^2 until a
+// breakdown, so its sum over the lanes is plain).  The whole group waits for
+// this chain: double-float (float64 has a long dependent latency on this part)
+// and as few instructions as it takes, since they run cold after each pass.
+SLS_DEV void lz_beta(LzXch& X, int j, const unsigned long long* now, XWait& xw) {
+  const int lane = threadIdx.x & 31;
+  const int D = X.D, r = X.r;
+  float2* cs = reinterpret_cast<float2*>(lz_smem() + X.cs);
+  dfloat cn = df_make(0.f, 0.f);
+  unsigned long long n0 = x_ld(now + D + r);
+#pragma unroll 1
+  for (int k0 = 0; k0 < r; k0 += 32) {  // (0 from k = j on)
+    const int k = k0 + lane;
+    const dfloat c = x_unpack(x_poll(now + D + k, k < r, xw));
+    if (k < r) cs[k] = f2(c);
+    dot2_acc_df(cn.hi, cn.lo, c, c);
+  }
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) {
+    cn.hi += __shfl_xor_sync(0xffffffffu, cn.hi, o);
+    cn.lo += __shfl_xor_sync(0xffffffffu, cn.lo, o);
+  }
+  if (__any_sync(0xffffffffu, n0 == LZ_EMPTY)) n0 = x_poll(now + D + r, true, xw);
+  const dfloat nrm2 = df_sub(x_unpack(n0), df_norm(cn.hi, cn.lo));  // |z1|^2
+  const bool pos = nrm2.hi > 0.f;
+  const dfloat inv = pos ? df_rsqrt(nrm2) : df_make(0.f, 0.f);  // 1 / beta
+  const dfloat bnew = pos ? df_mul(nrm2, inv) : df_make(0.f, 0.f);
+  if (lane == 0) {
+    X.invb = f2(inv);
+    X.beta = f2(bnew);
+  }
+  (void)j;
+}
+
+// The break test of step j, by the warp that formed beta, while the columns of
+// exchange 3 travel.
+SLS_DEV void lz_break_test(LzXch& X, int j) {
+  const dfloat bnew = dfv(X.beta);
+  dfloat scale = dfv(X.scale);
+  bool brk = !(bnew.hi > 0.f);
+  if (j > 0) {
+    const dfloat a = dfv(X.alpha);  // of step j - 1
+    const dfloat sc = df_add(a.hi < 0.f ? df_neg(a) : a, bnew);
+    if (df_less(scale, sc)) scale = sc;
+    brk = !df_less(df_mul(dfv(X.tol), scale), bnew);
+  }
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) {
+    X.scale = f2(scale);
+    X.brk = brk;
+    if (X.rank == 0 && j > 0 && !brk) X.beta_out[j - 1] = df_to_double(bnew);
+  }
+}
+
+// Exchanges 1 and 2 of step j: this CTA's coefficients and columns of
+// Phi^T z1 are published, c and beta_{j-1} formed.
+__device__ __noinline__ void lz_exchange12(int j, unsigned xpar, unsigned x3) {
+  constexpr int NCW = LZ_NCW, NCT = LZ_NT;
+  LzXch& X = lz_xch();
+  const LzOwn own = X.own;
+  const int g = X.g, D = X.D, r = X.r;
+  const int cbeg = X.cbeg, ncol = X.cend - X.cbeg, kbeg = X.kbeg, ncoef = X.kend - X.kbeg;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int red_rows = lz_red_rows(own);
+  float2* red = reinterpret_cast<float2*>(lz_smem() + X.red);
+  const float2* cs = reinterpret_cast<const float2*>(lz_smem() + X.cs);
+  const float2* Wm = X.Wm;
+  XWait xw{X.poison, X.status, &X.err, 0ll, 0u};
+  unsigned long long* src = X.part + ((size_t)xpar * g + X.rank) * g * own.WB;  // my block
+  unsigned long long* now = X.tot + (size_t)x3 * X.E;
+  unsigned long long* old = X.tot + (size_t)(x3 == 0u ? 2u : x3 - 1u) * X.E;
+  // the g partials of this CTA's coefficients and columns; the columns less
+  // sum_{k < j} c_k w_k.  Slots are emptied as they are read.
+  if (own.mode < 2) {
+    // thread t: the slot pair t % P of the sources t / P, t / P + NCT / P, ...;
+    // the lanes and then (through red) the warps that share a pair are added
+    const int P = own.WB >> 1, SP = NCT / P;
+    const int pr = tid & (P - 1), s0 = tid / P, i0 = 2 * pr;
+    const bool wa = i0 < own.kw ? i0 < ncoef : i0 - own.kw < ncol;
+    const bool wb = i0 + 1 < own.kw ? i0 + 1 < ncoef : i0 + 1 - own.kw < ncol;
+    dfloat a = df_make(0.f, 0.f), b = a;
+    constexpr int B = 5;
+#pragma unroll 1
+    for (int b0 = 0; b0 < g; b0 += B * SP) {
+      unsigned need = 0u;
+#pragma unroll
+      for (int u = 0; u < B; ++u)
+        if (b0 + s0 + u * SP < g) need |= 1u << u;
+      unsigned long long va[B], vb[B];
+      unsigned long long* p0 = src + (size_t)(b0 + s0) * own.WB + i0;
+      const size_t step = (size_t)SP * own.WB;
+      x_poll2<B>(p0, step, need, wa, wb, va, vb, xw);
+#pragma unroll
+      for (int u = 0; u < B; ++u)
+        if (need >> u & 1u) {
+          x_st2(p0 + u * step, LZ_EMPTY, LZ_EMPTY);
+          if (wa) a = df_add_fast(a, x_unpack(va[u]));
+          if (wb) b = df_add_fast(b, x_unpack(vb[u]));
+        }
+    }
+#pragma unroll 1
+    for (int o = P; o < 32; o <<= 1) {
+      a = df_add_fast(a, shfl_xor_df(a, o));
+      b = df_add_fast(b, shfl_xor_df(b, o));
+    }
+    if (lane < P) {
+      float2* rp = red + (P <= 32 ? warp : warp / (P / 32)) * own.WB + i0;
+      rp[0] = f2(a);
+      rp[1] = f2(b);
+    }
+    named_sync(BAR_ALL, NCT);
+  }
+  if (own.mode == 0) {
+    // sum i of the block by warp i % NCW: coefficients first
+#pragma unroll 1
+    for (int i = warp; i < own.kw + ncol; i += NCW) {
+      dfloat v = (lane < red_rows) ? dfv(red[lane * own.WB + i]) : df_make(0.f, 0.f);
+      size_t at;
+      if (i < own.kw) {
+        if (i >= ncoef) continue;
+        at = D + kbeg + i;
+      } else {
+        at = cbeg + i - own.kw;
+        float ch = 0.f, cl = 0.f;
+#pragma unroll 1
+        for (int k0 = 0; k0 < j; k0 += 32) {
+          const int k = k0 + lane;
+          const float2 w = k < j ? Wm[at * r + k] : make_float2(0.f, 0.f);
+          dot2_acc_df(ch, cl, dfv(w), x_unpack(x_poll(now + D + k, k < j, xw)));
+        }
+        v = df_sub(v, df_norm(ch, cl));
+      }
+#pragma unroll 1
+      for (int o = 16; o > 0; o >>= 1) v = df_add_fast(v, shfl_xor_df(v, o));
+      if (lane == 0) {
+        x_st(now + at, x_pack(v));
+        x_st(old + at, LZ_EMPTY);
+      }
+    }
+    if (warp == NCW - 1) lz_beta(X, j, now, xw);
+  } else {
+    dfloat a = df_make(0.f, 0.f), b = a;
+    if (own.mode == 1) {
+      // a thread per sum
+      if (tid < own.WB)
+#pragma unroll 1
+        for (int w = 0; w < red_rows; ++w) a = df_add(a, dfv(red[w * own.WB + tid]));
+      if (tid < ncoef) {
+        x_st(now + D + kbeg + tid, x_pack(a));
+        x_st(old + D + kbeg + tid, LZ_EMPTY);
+      }
+    } else if (warp == NCW - 1) {
+      // coefficients by the last warp
+#pragma unroll 1
+      for (int i = lane; i - lane < ncoef; i += 32) {
+        dfloat v = df_make(0.f, 0.f);
+#pragma unroll 1
+        for (int sI = 0; sI < g; ++sI) {
+          unsigned long long* p0 = src + (size_t)sI * own.WB + i;
+          v = df_add(v, x_unpack(x_poll(p0, i < ncoef, xw)));
+          if (i < ncoef) x_st(p0, LZ_EMPTY);
+        }
+        if (i < ncoef) {
+          x_st(now + D + kbeg + i, x_pack(v));
+          x_st(old + D + kbeg + i, LZ_EMPTY);
+        }
+      }
+    }
+    if (warp == NCW - 1) lz_beta(X, j, now, xw);
+    named_sync(BAR_ALL, NCT);  // c is in shared memory
+    if (own.mode == 1) {
+      const int q = tid - own.kw;
+      if (q >= 0 && q < ncol) {
+        float ch = 0.f, cl = 0.f;
+#pragma unroll 8
+        for (int k = 0; k < j; ++k)
+          dot2_acc_df(ch, cl, dfv(Wm[(size_t)k * D + cbeg + q]), dfv(cs[k]));
+        a = df_sub(a, df_norm(ch, cl));
+        x_st(now + cbeg + q, x_pack(a));
+        x_st(old + cbeg + q, LZ_EMPTY);
+      }
+    } else {
+#pragma unroll 1
+      for (int q0 = 0; q0 < ncol; q0 += 2 * NCT) {
+        const int q = q0 + 2 * tid;  // this thread's columns cbeg + q, cbeg + q + 1
+        const bool live = q < ncol;
+        a = b = df_make(0.f, 0.f);
+#pragma unroll 1
+        for (int b0 = 0; b0 < g; b0 += 4) {
+          unsigned need = 0u;
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (live && b0 + u < g) need |= 1u << u;
+          unsigned long long va[4], vb[4];
+          unsigned long long* p0 = src + (size_t)b0 * own.WB + own.kw + q;
+          x_poll2<4>(p0, (size_t)own.WB, need, true, true, va, vb, xw);
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (need >> u & 1u) {
+              x_st2(p0 + (size_t)u * own.WB, LZ_EMPTY, LZ_EMPTY);
+              a = df_add(a, x_unpack(va[u]));
+              b = df_add(b, x_unpack(vb[u]));
+            }
+        }
+        if (live) {
+          float ch = 0.f, cl = 0.f, dh = 0.f, dl = 0.f;
+          const float4* wrow = reinterpret_cast<const float4*>(Wm + cbeg + q);
+#pragma unroll 8
+          for (int k = 0; k < j; ++k) {
+            const float4 w = wrow[(size_t)k * (D >> 1)];
+            const dfloat c = dfv(cs[k]);
+            dot2_acc_df(ch, cl, df_make(w.x, w.y), c);
+            dot2_acc_df(dh, dl, df_make(w.z, w.w), c);
+          }
+          a = df_sub(a, df_norm(ch, cl));
+          b = df_sub(b, df_norm(dh, dl));
+          x_st2(now + cbeg + q, x_pack(a), x_pack(b));
+          x_st2(old + cbeg + q, LZ_EMPTY, LZ_EMPTY);
+        }
+      }
+    }
+  }
+}
+
+// Exchange 3 of step j: Phi^T z1 of every CTA; w_j = Phi^T z1 / beta (into shared
+// memory when STAGE_W; this CTA's columns kept for the correction of later
+// steps) and alpha_j = |w_j|^2, returned packed; LZ_EMPTY when a wait of this CTA
+// has given up.
+template <bool STAGE_W>
+__device__ __noinline__ unsigned long long lz_exchange3(int j, unsigned x3) {
+  constexpr int NCW = LZ_NCW, NCT = LZ_NT;
+  LzXch& X = lz_xch();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (named_sync_any(BAR_ALL, NCT, X.err != 0)) {
+    if (tid == 0) atomicExch(X.poison, 0u);
+    return LZ_EMPTY;
+  }
+  if (warp == NCW - 1) lz_break_test(X, j);
+  const int D = X.D, cbeg = X.cbeg, cend = X.cend;
+  const dfloat invb = dfv(X.invb);
+  const unsigned long long* now = X.tot + (size_t)x3 * X.E;
+  float2* whs = reinterpret_cast<float2*>(lz_smem() + X.whs);
+  float2* wls = reinterpret_cast<float2*>(lz_smem() + X.wls);
+  XWait xw{X.poison, X.status, &X.err, 0ll, 0u};
+  dfloat sq = df_make(0.f, 0.f);
+  constexpr int B = 4;
+#pragma unroll 1
+  for (int p0 = 0; p0 < (D >> 1); p0 += B * NCT) {
+    unsigned need = 0u;
+#pragma unroll
+    for (int u = 0; u < B; ++u)
+      if (p0 + tid + u * NCT < (D >> 1)) need |= 1u << u;
+    unsigned long long va[B], vb[B];
+    x_poll2<B>(now + 2 * (p0 + tid), 2 * NCT, need, true, true, va, vb, xw);
+#pragma unroll
+    for (int u = 0; u < B; ++u)
+      if (need >> u & 1u) {
+        const int c = 2 * (p0 + tid + u * NCT);
+        const dfloat w0 = df_mul(x_unpack(va[u]), invb), w1 = df_mul(x_unpack(vb[u]), invb);
+        dot2_acc_df(sq.hi, sq.lo, w0, w0);
+        dot2_acc_df(sq.hi, sq.lo, w1, w1);
+        if (STAGE_W) {
+          whs[c >> 1] = make_float2(w0.hi, w1.hi);
+          wls[c >> 1] = make_float2(w0.lo, w1.lo);
+        }
+        if (c + 1 >= cbeg && c < cend) {
+          const bool by_col = X.own.mode == 0;
+          if (c >= cbeg) X.Wm[by_col ? (size_t)c * X.r + j : (size_t)j * D + c] = f2(w0);
+          if (c + 1 < cend) X.Wm[by_col ? (size_t)(c + 1) * X.r + j : (size_t)j * D + c + 1] = f2(w1);
+        }
+      }
+  }
+  sq = df_norm(sq.hi, sq.lo);
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) sq = df_add_fast(sq, shfl_xor_df(sq, o));
+  if (lane == 0) X.tmpw[warp] = f2(sq);
+  if (named_sync_any(BAR_ALL, NCT, X.err != 0)) {
+    if (tid == 0) atomicExch(X.poison, 0u);
+    return LZ_EMPTY;
+  }
+  dfloat a = (lane < NCW) ? dfv(X.tmpw[lane]) : df_make(0.f, 0.f);
+#pragma unroll 1
+  for (int o = 1; o < NCW; o <<= 1) a = df_add_fast(a, shfl_xor_df(a, o));
+  a.hi = __shfl_sync(0xffffffffu, a.hi, 0);
+  a.lo = __shfl_sync(0xffffffffu, a.lo, 0);
+  if (tid == (NCW - 1) * 32) {  // read by the break test of the next step
+    X.alpha = f2(a);
+    if (X.rank == 0 && !X.brk) X.alpha_out[j] = df_to_double(a);
+  }
+  return x_pack(a);
 }
 
 // Rows of one team in a ring: batches of R rows are numbered over the CTA's
@@ -431,13 +910,10 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
   using RV = RowVals<R>;
   // basis coefficients per lane: k = sub + LPR * (t * WPR + tw), t < KC
   constexpr int KC = (KT * 32 + LPR * WPR - 1) / (LPR * WPR);
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ float2 tmpw[NCW];
+  unsigned char* smem_raw = lz_smem();
+  LzXch& X = lz_xch();
+  volatile int& s_err = X.err;
   __shared__ float s_red1[NCW];  // per-warp max |Phi| (offset bounds)
-  __shared__ double shd[4];
-  __shared__ float2 sdf[3];  // 1 / beta, alpha, beta of the step as double-float
-  __shared__ int sflag, sbreak;
-  __shared__ volatile int s_err;      // a wait of this CTA gave up
 
   const int D = bt.D, r = bt.r, ldq = q_ld(bt.r);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -450,9 +926,13 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
 
   const unsigned phib = (unsigned)R * (unsigned)D * (unsigned)sizeof(PT);
   const unsigned stage = lz_stage_bytes(D, ldq, (int)sizeof(PT), R);
-  TeamRing ring{smem_raw + (size_t)team * ring_stages * stage, nullptr, (unsigned)ring_stages,
-                RingPos{0u, 0u}, RingPos{0u, 0u}};
-  float4* exch = reinterpret_cast<float4*>(smem_raw + (size_t)TEAMS * ring_stages * stage);
+  TeamRing ring{smem_raw + LZ_RING0 + (size_t)team * ring_stages * stage, nullptr,
+                (unsigned)ring_stages, RingPos{0u, 0u}, RingPos{0u, 0u}};
+  float* whs = reinterpret_cast<float*>(smem_raw + LZ_RING0 + (size_t)TEAMS * ring_stages * stage);
+  float* wls = whs + D;
+  const LzOwn own = lz_own(D, r, g);
+  float2* red = reinterpret_cast<float2*>(lz_stage_w(WPR) ? wls + D : whs);
+  float4* exch = reinterpret_cast<float4*>(red + lz_red_rows(own) * (own.mode < 2 ? own.WB : 0));
   float2* cs = reinterpret_cast<float2*>(exch + TEAMS * 2 * R * WPR);  // r + 1 (c = Q^T z')
   uint64_t* fullb = reinterpret_cast<uint64_t*>(
       (reinterpret_cast<uintptr_t>(cs + (r + 1)) + 15) & ~(uintptr_t)15);
@@ -461,24 +941,44 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
   // scratch of the pass ends, in the team's ring (idle then): its column sums,
   // its coefficient partials (k < r) and, at r, its part of |z'|^2
   const size_t tstride = (size_t)ring_stages * stage;
-  auto tcol = [&](int t) { return reinterpret_cast<float2*>(smem_raw + (size_t)t * tstride); };
+  auto tcol = [&](int t) {
+    return reinterpret_cast<float2*>(smem_raw + LZ_RING0 + (size_t)t * tstride);
+  };
   auto tco = [&](int t) { return tcol(t) + D; };
-
-  const LzLayout L = lz_layout(bt.nmax, D, r, g);
-  char* gb = scratch + (size_t)gi * gstride;
-  unsigned* barw = reinterpret_cast<unsigned*>(gb + L.bar);
-  double* acc = reinterpret_cast<double*>(gb + L.acc);
-  float2* wpart = reinterpret_cast<float2*>(gb + L.wpart);
-  float2* wred = reinterpret_cast<float2*>(gb + L.wred);
-  float2* Wm = reinterpret_cast<float2*>(gb + L.Wm);
-  const GroupBarrier bar{barw, barw + 32, (unsigned)g};
-  const int accs = lz_acc_stride(r);
   const uint64_t pol = l2_policy_evict_first();
 
   if (tid == 0) {
     for (int s = 0; s < TEAMS * ring_stages; ++s) mbar_init(&fullb[s], 1);
     mbar_fence_init();
-    s_err = 0;
+    const LzLayout L = lz_layout(bt.nmax, D, r, g);
+    char* gb = scratch + (size_t)gi * gstride;
+    auto offset = [&](const void* p) {
+      return (unsigned)(reinterpret_cast<const unsigned char*>(p) - smem_raw);
+    };
+    X.part = reinterpret_cast<unsigned long long*>(gb + L.part);
+    X.tot = reinterpret_cast<unsigned long long*>(gb + L.tot);
+    X.Wm = reinterpret_cast<float2*>(gb + L.Wm);
+    X.poison = reinterpret_cast<unsigned*>(gb + L.bar);
+    X.status = status;
+    X.own = own;
+    X.g = g;
+    X.rank = rank;
+    X.D = D;
+    X.r = r;
+    X.E = lz_exch_len(D, r);
+    X.cbeg = min(D, rank * own.cw);
+    X.cend = min(D, X.cbeg + own.cw);
+    X.kbeg = min(r + 1, (g - 1 - rank) * own.kw);
+    X.kend = min(r + 1, X.kbeg + own.kw);
+    X.cw_magic = 0xffffffffu / (unsigned)own.cw + 1u;
+    X.rings = LZ_RING0;
+    X.ring_bytes = (unsigned)tstride;
+    X.whs = offset(whs);
+    X.wls = offset(wls);
+    X.red = offset(red);
+    X.cs = offset(cs);
+    X.tol = f2(df_from_double(bt.tol));
+    X.err = 0;
   }
   __syncthreads();
 
@@ -505,8 +1005,9 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
   };
 
   const int nprob = nprob_of(bt);
-  unsigned lgen = 0;
-  unsigned gstep = 0;  // steps run by this group so far (parity of the group sums)
+  // exchanges run by this group so far: the partials' buffer (parity) and the
+  // totals' buffer (modulo 3) of the current one
+  unsigned xpar = 0u, x3 = 0u;
   for (int p = gi; p < nprob; p += ngroups) {
     const int64_t row0 = bt.row0 ? bt.row0[p] : 0;
     const int64_t n = bt.n ? (int64_t)bt.n[p] : bt.n_single;
@@ -521,21 +1022,14 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
     const int nb = nball > team ? (nball - team + TEAMS - 1) / TEAMS : 0;
     double* alpha_out = bt.alpha + (size_t)p * r;
     double* beta_out = bt.beta + (size_t)p * r;
-    const int cbeg = (int)((int64_t)rank * D / g), cend = (int)((int64_t)(rank + 1) * D / g);
-
-    double scale = 0.0, alpha_prev = 0.0;
-    // beta_{j-1} = 1 / e_inv and the break test of the step, in lane 0 of
-    // warp bw: the last warp during the slice phase when that warp sums no
-    // column there (measured 2% faster at the qwen7b shape), else warp 0
-    // after group barrier 2
-    double e_inv = 0.0, e_bnew = 0.0;
-    int e_brk = 0;
-    const bool beta_early = slice_last_warp_idle<NCW>(cend - cbeg);
-    const int bw = beta_early ? NCW - 1 : 0;
+    if (tid == 0) {  // read after the barriers of the prologue's end
+      X.alpha_out = alpha_out;
+      X.beta_out = beta_out;
+      X.scale = X.alpha = make_float2(0.f, 0.f);
+    }
     dfloat alpha_df = df_make(0.f, 0.f), beta_df = df_make(0.f, 0.f), invb_df;
     float phimax = 0.f;  // max |Phi| over this CTA's strip (prologue pass)
     int reff = 0;
-    sbreak = 0;
 
     // Row range of the team's batch b in pass `pass` (0 = the prologue;
     // passes alternate direction).
@@ -552,18 +1046,16 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
         ring_issue<PT>(ring, i0, min(R, nrows - i0), D, ldq, stage, phib, pass > 0, Phis, Qs, pol);
       }
     };
-    auto issue_pass_head = [&](int pass) {
+    // the batches [b0, min(b1, stages)) of a pass's head
+    auto issue_pass_head = [&](int pass, int b0, int b1) {
       if (leader)
-        for (int b = 0; b < (int)ring.S; ++b) issue(pass, b);
+        for (int b = b0; b < min(b1, (int)ring.S); ++b) issue(pass, b);
     };
 
-    // pass end: the column sums of the teams are added through their rings
-    // (idle now) and stored as the CTA's partials of Phi^T z'; the coefficient
-    // partials (k < K) and |z'|^2 join the group sums of parity `par` (float64
-    // atomics)
-    auto pass_end = [&](f32x2_t (&ah)[NC / 2], f32x2_t (&al)[NC / 2], dfloat (&cacc)[KC], int K,
-                        dfloat nacc,
-                        unsigned par) {
+    // The end of a pass: the team's column sums and coefficient partials (k < K)
+    // into its ring.
+    auto team_sums = [&](f32x2_t (&ah)[NC / 2], f32x2_t (&al)[NC / 2], dfloat (&cacc)[KC], int K,
+                         dfloat nacc) {
       if constexpr (WPR > 1) named_sync(bar_team, WPR * 32);  // the team is done with its ring
       else __syncwarp();
       {
@@ -602,42 +1094,14 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
         if (lane == 0) cw[r] = f2(nv);
       }
       // the columns of Q written in this pass reach the bulk reads of the next
-      // one, and the ring writes above are ordered before its bulk writes
-      // (async proxy)
+      // one, the ring writes above are ordered before its bulk writes (async
+      // proxy), and the slots emptied in the exchange before this pass before
+      // what is published after it
       asm volatile("fence.proxy.async;" ::: "memory");
-      named_sync(BAR_ALL, NCT);
-      {
-        float4* dst = reinterpret_cast<float4*>(wpart + (size_t)rank * D);
-        for (int c = tid; c < (D >> 1); c += NCT) {
-          float4 v[TEAMS];
-#pragma unroll
-          for (int t = 0; t < TEAMS; ++t) v[t] = reinterpret_cast<const float4*>(tcol(t))[c];
-#pragma unroll
-          for (int w = 1; w < TEAMS; w *= 2)
-#pragma unroll
-            for (int t = 0; t + w < TEAMS; t += 2 * w) {
-              const dfloat a = df_add_fast(df_make(v[t].x, v[t].y), df_make(v[t + w].x, v[t + w].y));
-              const dfloat b = df_add_fast(df_make(v[t].z, v[t].w), df_make(v[t + w].z, v[t + w].w));
-              v[t] = make_float4(a.hi, a.lo, b.hi, b.lo);
-            }
-          dst[c] = v[0];
-        }
-      }
-      // coefficient k (|z'|^2 at r): the TEAMS partials summed by two lanes
-      double* accn = acc + (size_t)(par & 1u) * accs;
-      for (int k0 = 0; k0 < K + 1; k0 += NCT / 2) {
-        const int e = k0 + tid / 2, part = tid & 1;
-        const int k = (e < K) ? e : r;
-        dfloat s = df_make(0.f, 0.f);
-        if (e <= K)
-          for (int t = part; t < TEAMS; t += 2) s = df_add(s, dfv(tco(t)[k]));
-        s = df_add_fast(s, shfl_xor_df(s, 1));
-        if (part == 0 && e <= K) red_add_f64(accn + (e < K ? e : r + 1), df_to_double(s));
-      }
-      named_sync(BAR_ALL, NCT);
+      __threadfence();
     };
 
-    issue_pass_head(0);
+    issue_pass_head(0, 0, (int)ring.S);
 
     // ---------------- prologue: z' = q1, |z'|^2 and Phi^T z' (pass 0) ------------
     {
@@ -684,119 +1148,35 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
       dfloat cacc0[KC];
 #pragma unroll
       for (int t = 0; t < KC; ++t) cacc0[t] = df_make(0.f, 0.f);
-      // |q1|^2 is the group sum of the first step
-      pass_end(ah, al, cacc0, 0, nacc, gstep);
-      if (r >= 2) issue_pass_head(1);
+      team_sums(ah, al, cacc0, 0, nacc);
+      if (bt.inject_fail && rank == 0 && tid == 0) lz_fail(status, &s_err);
+      // |q1|^2 is the sum of the first step
+      if (!lz_publish<TEAMS>(0, xpar)) {
+        drain();
+        return;
+      }
+      if (r >= 2) issue_pass_head(1, 0, 1);
     }
 
-    if (bt.inject_fail && rank == 0 && tid == 0) lz_fail(status, &s_err);
-    for (int j = 0; j < r; ++j, ++gstep) {
-      if (!group_sync_named(bar, lgen, status, &sflag, &s_err, BAR_ALL, NCT)) {
+    for (int j = 0; j < r; ++j) {
+      lz_exchange12(j, xpar, x3);
+      // the rest of the next pass's first batches, while the columns travel
+      if (j + 1 <= r - 1) issue_pass_head(j + 1, 1, (int)ring.S);
+      const unsigned long long alpha = lz_exchange3<lz_stage_w(WPR)>(j, x3);
+      if (alpha == LZ_EMPTY) {
         drain();
         return;
       }
-      const double* accj = acc + (size_t)(gstep & 1u) * accs;
-      // |z1|^2 = |z'|^2 - |c|^2 (Q orthonormal): beta_{j-1} and the break
-      // test (warp bw, once c is in shared memory)
-      auto beta_phase = [&]() {
-        const double zs = accj[r + 1];
-        dfloat cn = df_make(0.f, 0.f);
-#pragma unroll
-        for (int t2 = 0; t2 < KT; ++t2) {
-          const int k = lane + 32 * t2;
-          if (k < j) dot2_acc_df(cn.hi, cn.lo, dfv(cs[k]), dfv(cs[k]));
-        }
-        cn = df_norm(cn.hi, cn.lo);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) cn = df_add_fast(cn, shfl_xor_df(cn, o));
-        if (lane == 0) {
-          const double nrm2 = zs - df_to_double(cn);  // |z1|^2
-          // one reciprocal square root instead of a square root and two
-          // divides (float64 runs at a fraction of the float32 rate here)
-          e_inv = (nrm2 > 0.0) ? rsqrt(nrm2) : 0.0;  // 1 / beta
-          e_bnew = (nrm2 > 0.0) ? nrm2 * e_inv : 0.0;
-          e_brk = 0;
-          if (j > 0) {
-            scale = fmax(scale, fabs(alpha_prev) + e_bnew);
-            if (!(e_bnew > bt.tol * scale)) e_brk = 1;
-            else if (rank == 0) beta_out[j - 1] = e_bnew;
-          } else if (!(e_bnew > 0.0)) {
-            e_brk = 1;
-          }
-        }
-      };
-
-      // ---------------- slice phase: c, Phi^T z1 for this CTA's columns ----------
-      // c = Q^T z' (k < j) from the group sums; Phi^T z1 = Phi^T z' - sum_k
-      // c_k w_k with w_k = Phi^T q_k kept in Wm.  The group sums of the other
-      // parity were read in the previous step by every CTA (all of them have
-      // passed barrier 1 since): the first CTA clears them for the next step.
-      if (rank == 0) {
-        double* accz = acc + (size_t)((gstep + 1u) & 1u) * accs;
-        for (int k = tid; k < accs; k += NCT) accz[k] = 0.0;
-      }
-      {
-        // c is loaded by the last warp when it sums no column (it waits for
-        // beta there anyway), else by warp 0
-        bool synced = false;
-        dfloat sq = slice_columns<NCW>(wpart, Wm, wred, cs, accj, beta_early ? NCW - 1 : 0, g, D,
-                                       j, cbeg, cend, synced);
-        if (!synced) named_sync(BAR_ALL, NCT);
-        if (beta_early && warp == NCW - 1) beta_phase();
-        sq = df_norm(sq.hi, sq.lo);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sq = df_add_fast(sq, shfl_xor_df(sq, o));
-        if (lane == 0) tmpw[warp] = f2(sq);
-        named_sync(BAR_ALL, NCT);
-        if (warp == 0) {
-          // the NCW warp sums by a butterfly over the first NCW lanes
-          dfloat t = (lane < NCW) ? dfv(tmpw[lane]) : df_make(0.f, 0.f);
-#pragma unroll
-          for (int o = 1; o < NCW; o <<= 1) t = df_add_fast(t, shfl_xor_df(t, o));
-          if (lane == 0) red_add_f64(const_cast<double*>(accj) + r + 2, df_to_double(t));
-        }
-      }
-      if (!group_sync_named(bar, lgen, status, &sflag, &s_err, BAR_ALL, NCT)) {
-        drain();
-        return;
-      }
-
-      // ---------------- beta_{j-1}, alpha_j, break test; w_j gather ---------------
-      // this lane's columns of Phi^T z1 (loads in flight while the scalars are formed)
-      float4 wv[NV][2];
-#pragma unroll
-      for (int q = 0; q < NV; ++q) {
-        const int cg = lane + 32 * (q * WPR + tw);
-        wv[q][0] = wv[q][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (cg < C4) {
-          wv[q][0] = reinterpret_cast<const float4*>(wred)[2 * cg];
-          wv[q][1] = reinterpret_cast<const float4*>(wred)[2 * cg + 1];
-        }
-      }
-      if (!beta_early && warp == 0) beta_phase();
-      if (warp == bw && lane == 0) {
-        const double q = accj[r + 2];  // |Phi^T z1|^2
-        const double a = e_brk ? 0.0 : (q * e_inv) * e_inv;
-        if (!e_brk && rank == 0) alpha_out[j] = a;
-        shd[1] = e_brk ? 0.0 : e_inv;
-        shd[2] = a;
-        shd[3] = (j > 0) ? e_bnew : 0.0;
-        // converted once here: float64 runs at a small fraction of the
-        // float32 rate on this part, and every thread needs these
-        sdf[0] = f2(df_from_double(shd[1]));
-        sdf[1] = f2(df_from_double(a));
-        sdf[2] = f2(df_from_double(shd[3]));
-        sbreak = e_brk;
-      }
-      named_sync(BAR_ALL, NCT);
-      if (sbreak) {
+      const unsigned long long* now = X.tot + (size_t)x3 * X.E;
+      xpar ^= 1u;
+      x3 = x3 == 2u ? 0u : x3 + 1u;
+      if (X.brk) {
         reff = j;
         break;
       }
-      invb_df = dfv(sdf[0]);
-      alpha_prev = shd[2];
-      alpha_df = dfv(sdf[1]);
-      beta_df = dfv(sdf[2]);
+      invb_df = dfv(X.invb);
+      alpha_df = x_unpack(alpha);
+      beta_df = j > 0 ? dfv(X.beta) : df_make(0.f, 0.f);
       if (j == 0) {
 #pragma unroll
         for (int w = 0; w < NCW; ++w) phimax = fmaxf(phimax, s_red1[w]);
@@ -809,20 +1189,32 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
         break;
       }
 
-      // w_j = (Phi^T z1) / beta in registers; the CTA's slice of it is kept for
-      // the correction of later steps
-      for (int c = cbeg + tid; c < cend; c += NCT)
-        Wm[(size_t)j * D + c] = f2(df_mul(dfv(wred[c]), invb_df));
+      // this lane's columns of w_j
       f32x2_t wh[NC / 2], wl[NC / 2];
       float wt1 = 0.f;  // l1 norm of this lane's part of w_j
 #pragma unroll
-      for (int c = 0; c < NC / 2; ++c) {
-        const float4 v = wv[c / 2][c & 1];
-        const dfloat w0 = df_mul(df_make(v.x, v.y), invb_df);
-        const dfloat w1 = df_mul(df_make(v.z, v.w), invb_df);
-        wh[c] = pk2(w0.hi, w1.hi);
-        wl[c] = pk2(w0.lo, w1.lo);
-        wt1 += fabsf(w0.hi) + fabsf(w1.hi);
+      for (int q = 0; q < NV; ++q) {
+        const int cg = lane + 32 * (q * WPR + tw);
+        float4 h = make_float4(0.f, 0.f, 0.f, 0.f), l = h;
+        if (FULLD || cg < C4) {
+          if constexpr (lz_stage_w(WPR)) {
+            h = reinterpret_cast<const float4*>(whs)[cg];
+            l = reinterpret_cast<const float4*>(wls)[cg];
+          } else {
+            unsigned long long v[4];
+            x_ld2(now + 4 * cg, v[0], v[1]);
+            x_ld2(now + 4 * cg + 2, v[2], v[3]);
+            const dfloat w0 = df_mul(x_unpack(v[0]), invb_df), w1 = df_mul(x_unpack(v[1]), invb_df);
+            const dfloat w2 = df_mul(x_unpack(v[2]), invb_df), w3 = df_mul(x_unpack(v[3]), invb_df);
+            h = make_float4(w0.hi, w1.hi, w2.hi, w3.hi);
+            l = make_float4(w0.lo, w1.lo, w2.lo, w3.lo);
+          }
+        }
+        wh[2 * q] = pk2(h.x, h.y);
+        wh[2 * q + 1] = pk2(h.z, h.w);
+        wl[2 * q] = pk2(l.x, l.y);
+        wl[2 * q + 1] = pk2(l.z, l.w);
+        wt1 += (fabsf(h.x) + fabsf(h.y)) + (fabsf(h.z) + fabsf(h.w));
       }
       // Offset of the row dots: a power of two above eight times the largest
       // part a lane can hold, so that the sums of eight lanes' parts are exact
@@ -1099,27 +1491,23 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
       if (b0 < b1) full_batches(b0, b1);
       if (b1 < nb) lone_batch(nb - 1);
       if (Ca != 0.f) flush();
-      // partials for step j+1 (read after its barrier 1): Phi^T z', c, |z'|^2
-      pass_end(ah, al, cacc, j + 1, nacc, gstep + 1u);
-      if (pass + 1 <= r - 1) issue_pass_head(pass + 1);
+      // partials for step j+1: Phi^T z', c, |z'|^2
+      team_sums(ah, al, cacc, j + 1, nacc);
+      if (!lz_publish<TEAMS>(j + 1, xpar)) {
+        drain();
+        return;
+      }
+      if (pass + 1 <= r - 1) issue_pass_head(pass + 1, 0, 1);
     }
-    // the loop always ends in a break (the break test, or the last step) with
-    // gstep at that step; the slice phase of that step cleared the group sums
-    // of the next parity, where the next problem's prologue starts
-    ++gstep;
     // a break leaves the head of the next pass issued: wait for it to land and
     // count it as consumed
-    if (sbreak && !s_err && reff < r - 1)
+    if (reff < r - 1)
       for (int b = 0; b < min(nb, (int)ring.S); ++b) next_stage();
+    named_sync(BAR_ALL, NCT);  // every warp is done with the step's shared state
     if (rank == 0 && tid == 0) {
       bt.r_eff[p] = reff;
       for (int k = reff; k < r; ++k) alpha_out[k] = 0.0;
       for (int k = (reff > 0 ? reff - 1 : 0); k < r; ++k) beta_out[k] = 0.0;
-    }
-    // problems on the same group run back to back; keep them apart
-    if (!group_sync_named(bar, lgen, status, &sflag, &s_err, BAR_ALL, NCT)) {
-      drain();
-      return;
     }
   }
   drain();
@@ -1169,16 +1557,16 @@ int launch_lanczos_f32_3_1(SLS_LZ_LAUNCH_ARGS);
 int launch_lanczos_bf16_3_1(SLS_LZ_LAUNCH_ARGS);
 int launch_lanczos_f32_4_1(SLS_LZ_LAUNCH_ARGS);
 int launch_lanczos_bf16_4_1(SLS_LZ_LAUNCH_ARGS);
-int launch_lanczos_f32_6_1(SLS_LZ_LAUNCH_ARGS);
-int launch_lanczos_bf16_6_1(SLS_LZ_LAUNCH_ARGS);
-int launch_lanczos_f32_8_1(SLS_LZ_LAUNCH_ARGS);
-int launch_lanczos_bf16_8_1(SLS_LZ_LAUNCH_ARGS);
-int launch_lanczos_f32_6_2(SLS_LZ_LAUNCH_ARGS);
-int launch_lanczos_bf16_6_2(SLS_LZ_LAUNCH_ARGS);
-int launch_lanczos_f32_8_2(SLS_LZ_LAUNCH_ARGS);
-int launch_lanczos_bf16_8_2(SLS_LZ_LAUNCH_ARGS);
-int launch_lanczos_f32_8_4(SLS_LZ_LAUNCH_ARGS);
-int launch_lanczos_bf16_8_4(SLS_LZ_LAUNCH_ARGS);
+int launch_lanczos_f32_3_2(SLS_LZ_LAUNCH_ARGS);
+int launch_lanczos_bf16_3_2(SLS_LZ_LAUNCH_ARGS);
+int launch_lanczos_f32_4_2(SLS_LZ_LAUNCH_ARGS);
+int launch_lanczos_bf16_4_2(SLS_LZ_LAUNCH_ARGS);
+int launch_lanczos_f32_3_4(SLS_LZ_LAUNCH_ARGS);
+int launch_lanczos_bf16_3_4(SLS_LZ_LAUNCH_ARGS);
+int launch_lanczos_f32_4_4(SLS_LZ_LAUNCH_ARGS);
+int launch_lanczos_bf16_4_4(SLS_LZ_LAUNCH_ARGS);
+int launch_lanczos_f32_4_8(SLS_LZ_LAUNCH_ARGS);
+int launch_lanczos_bf16_4_8(SLS_LZ_LAUNCH_ARGS);
 int launch_lanczos_f32_8_8(SLS_LZ_LAUNCH_ARGS);
 int launch_lanczos_bf16_8_8(SLS_LZ_LAUNCH_ARGS);
 

@@ -9,7 +9,13 @@
 
 namespace {
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[SLS_NOALLOC_MAX_BYTES];
+// SLS_NOALLOC_MAX_BYTES bounds the problem (its basis, the coefficient rows and
+// one set of column partials per CTA); the Lanczos kernel's second set of
+// partials and its totals come on top, at most 2 * 152 * (D + r + 2) * 8 bytes
+// at D = 8192, r = 128 and as much again for more SMs.
+constexpr size_t kExchangeExtra = 24u << 20;
+static __device__ __align__(256) unsigned char
+    g_noalloc_scratch[SLS_NOALLOC_MAX_BYTES + kExchangeExtra];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_lock;
@@ -48,10 +54,12 @@ extern "C" int sls_lanczos_topr_noalloc(const float* Phi, int64_t N, int D, int 
     return SLS_ERR_INVALID_ARG;
   const size_t need = sls_lanczos_workspace_size(N, D, r);
   if (need == 0) return SLS_ERR_UNSUPPORTED;
-  if (need > (size_t)SLS_NOALLOC_MAX_BYTES) return SLS_ERR_WORKSPACE;
+  const size_t extra = sls::lanczos_exchange_extra(N, D, r);
+  if (need - extra > (size_t)SLS_NOALLOC_MAX_BYTES || need > sizeof(g_noalloc_scratch))
+    return SLS_ERR_WORKSPACE;
   void* ws = nullptr;
   const int st = scratch_address(&ws);
   if (st != SLS_OK) return st;
   return sls_lanczos_topr(Phi, N, D, r, q1, tol, theta, U, r_eff, alpha, beta, ws,
-                          (size_t)SLS_NOALLOC_MAX_BYTES, stream);
+                          sizeof(g_noalloc_scratch), stream);
 }
