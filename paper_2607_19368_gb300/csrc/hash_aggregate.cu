@@ -22,84 +22,190 @@ namespace sls {
 
 namespace {
 
-// SimHash of rows 0 .. n-1 with one lane per hyperplane: a warp takes
-// 32 / BP rows at a time (BP = bits rounded up to a power of two), lane
-// slot * BP + l forms row slot's dot with hyperplane l by the fixed float32
-// chain of the specification (acc = 0; for m = 0 .. k-1:
-// acc = fl(acc + fl(U[i,m] * R[l,m])), multiply and add rounded separately),
-// the row's elements read by every lane of its slot (the same addresses: one
-// transaction), R from shared memory with the padded row stride rs (no bank
-// conflicts between hyperplanes), and a ballot assembles the codes.  Warps
-// w0, w0 + wstride, ... of the launch.
-SLS_DEV void simhash_lanes(const float* __restrict__ U, int64_t n, int ldu, int kk,
-                           const float* __restrict__ Rs, int rs, int bits,
-                           uint32_t* __restrict__ codes, int64_t w0, int64_t wstride) {
-  int BP = 1;
-  while (BP < bits) BP <<= 1;
-  const int lane = threadIdx.x & 31;
-  const int slot = lane / BP, l = lane % BP, rpw = 32 / BP;
-  const float* rl = Rs + (size_t)min(l, max(bits, 1) - 1) * rs;
-  for (int64_t w = w0; w * rpw < n; w += wstride) {
-    const int64_t i = w * rpw + slot;
-    const bool live = i < n;
-    float acc = 0.0f;
-    if (live) {
-      const float* u = U + i * ldu;
-      for (int m = 0; m < kk; ++m) acc = __fadd_rn(acc, __fmul_rn(__ldg(u + m), rl[m]));
-    }
-    const unsigned ball = __ballot_sync(0xffffffffu, live && l < bits && acc > 0.0f);
-    if (live && l == 0) {
-      const unsigned mask = (BP == 32) ? 0xffffffffu : ((1u << BP) - 1u);
-      codes[i] = (ball >> (slot * BP)) & mask;
-    }
+// cp.async of 16 or 4 bytes (the first `bytes` of them, zeros after), and the
+// wait for all but the newest `pending` groups of a thread's copies.
+SLS_DEV void cp_async16(void* dst, const void* src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
+}
+SLS_DEV void cp_async4(void* dst, const void* src, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src),
+               "r"(bytes)
+               : "memory");
+}
+SLS_DEV void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+SLS_DEV void cp_async_wait_pending(int pending) {
+  switch (pending) {
+    case 0: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
+    case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
+    case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
+    case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
+    default: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
   }
 }
 
-// R (bits x kk) into shared memory with row stride kk + 1
-SLS_DEV void simhash_stage_R(const float* __restrict__ R, int ldr, int bits, int kk, float* Rs) {
-  for (int e = threadIdx.x; e < bits * kk; e += blockDim.x)
-    Rs[(e / kk) * (kk + 1) + e % kk] = R[(e / kk) * ldr + e % kk];
+// One tile of SimHash.  A thread forms the dots of RPT rows with eight
+// hyperplanes by the fixed float32 chain of the specification (acc = 0; for m =
+// 0 .. k-1: acc = fl(acc + fl(U[i,m] * R[l,m])), multiply and add rounded
+// separately; two hyperplanes per packed instruction); the 2^lg threads of a row
+// are neighbouring lanes and OR their bits.  The rows come through shared memory
+// by asynchronous copies in groups of SH_MC columns, all in flight at once, so
+// that the first groups' arithmetic hides the later groups' arrival.
+//
+// Bound by the packed multiplies and adds (N bits k / 2 each at two cycles a
+// warp: 6.7 us at N = 131060, k = 64, 16 bits, against 5 us for reading U).  The
+// former kernel, a lane per hyperplane with a row's elements read by every lane,
+// spent a load and an address per multiply; sls_simhash there 48 -> 18 us a call
+// (16 of them the host's, when nothing else runs), N = 32000, 20 bits 24 -> 17.
+constexpr int SH_T = 128;   // threads per CTA
+constexpr int SH_MC = 16;   // columns per copy group
+constexpr int SH_LMAX = 32; // row length of the transposed hyperplanes
+
+__host__ __device__ inline int sh_lg(int bits) { return bits <= 8 ? 0 : bits <= 16 ? 1 : 2; }
+__host__ __device__ inline int sh_rows(int bits, int rpt) { return (SH_T >> sh_lg(bits)) * rpt; }
+__host__ __device__ inline size_t sh_smem(int bits, int k, int rpt) {
+  const size_t k4 = (size_t)((k + 3) & ~3);
+  return sizeof(float) * (k4 * SH_LMAX + (size_t)sh_rows(bits, rpt) * (k4 + 4));
 }
 
-__global__ void __launch_bounds__(256)
+// R (bits x kk, row stride ldr) transposed into Rt[m][l], zero where there is
+// no hyperplane or column
+SLS_DEV void simhash_stage_R(const float* __restrict__ R, int ldr, int bits, int kk, float* Rt) {
+  const int k4 = (kk + 3) & ~3;
+  for (int e = threadIdx.x; e < k4 * SH_LMAX; e += SH_T) {
+    const int l = e & (SH_LMAX - 1), m = e / SH_LMAX;
+    Rt[e] = (l < bits && m < kk) ? R[(size_t)l * ldr + m] : 0.f;
+  }
+}
+
+template <int RPT>
+SLS_DEV void simhash_tile(const float* __restrict__ U, int64_t n, int64_t r0, int ldu, bool vec,
+                          int kk, const float* Rt, float* Us, int bits,
+                          uint32_t* __restrict__ codes) {
+  const int tid = threadIdx.x;
+  const int lg = sh_lg(bits), rows = sh_rows(bits, RPT);
+  const int k4 = (kk + 3) & ~3, us = k4 + 4;  // 16-byte rows, no bank conflicts
+  const int nch = (k4 + SH_MC - 1) / SH_MC;
+  for (int c = 0; c < nch; ++c) {
+    for (int e = tid; e < rows * (SH_MC / 4); e += SH_T) {
+      const int row = e / (SH_MC / 4), col = c * SH_MC + 4 * (e % (SH_MC / 4));
+      if (col < k4) {
+        const bool live = r0 + row < n;
+        const float* src = U + (live ? r0 + row : 0) * ldu;
+        const int left = live ? min(4, kk - col) : 0;  // elements of the quad that exist
+        float* dst = Us + row * us + col;
+        if (vec) {
+          cp_async16(dst, left ? src + col : src, 4 * left);
+        } else {
+#pragma unroll
+          for (int x = 0; x < 4; ++x) cp_async4(dst + x, x < left ? src + col + x : src, x < left ? 4 : 0);
+        }
+      }
+    }
+    cp_async_commit_group();
+  }
+  const int slot = tid >> lg, grp = tid & ((1 << lg) - 1);
+  f32x2_t acc[RPT][4];
+#pragma unroll
+  for (int s = 0; s < RPT; ++s)
+#pragma unroll
+    for (int h = 0; h < 4; ++h) acc[s][h] = 0ull;
+  const float* up = Us + slot * us;
+  const float* rp = Rt + grp * 8;
+  for (int c = 0; c < nch; ++c) {
+    cp_async_wait_pending(nch - 1 - c);
+    __syncthreads();
+    const int m1 = min(k4, (c + 1) * SH_MC);
+#pragma unroll 2
+    for (int m = c * SH_MC; m < m1; m += 4) {
+      float4 u[RPT];
+#pragma unroll
+      for (int s = 0; s < RPT; ++s)
+        u[s] = *reinterpret_cast<const float4*>(up + s * (SH_T >> lg) * us + m);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const float4 ra = *reinterpret_cast<const float4*>(rp + (m + x) * SH_LMAX);
+        const float4 rb = *reinterpret_cast<const float4*>(rp + (m + x) * SH_LMAX + 4);
+        const f32x2_t r0p = pk2(ra.x, ra.y), r1p = pk2(ra.z, ra.w);
+        const f32x2_t r2p = pk2(rb.x, rb.y), r3p = pk2(rb.z, rb.w);
+#pragma unroll
+        for (int s = 0; s < RPT; ++s) {
+          const float ux = x == 0 ? u[s].x : x == 1 ? u[s].y : x == 2 ? u[s].z : u[s].w;
+          const f32x2_t uu = pk2(ux, ux);
+          acc[s][0] = add2(acc[s][0], mul2(uu, r0p));
+          acc[s][1] = add2(acc[s][1], mul2(uu, r1p));
+          acc[s][2] = add2(acc[s][2], mul2(uu, r2p));
+          acc[s][3] = add2(acc[s][3], mul2(uu, r3p));
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int s = 0; s < RPT; ++s) {
+    unsigned code = 0u;
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      float a, b;
+      upk2(acc[s][h], a, b);
+      code |= (a > 0.f ? 1u : 0u) << (2 * h);
+      code |= (b > 0.f ? 1u : 0u) << (2 * h + 1);
+    }
+    code <<= 8 * grp;
+    if (lg > 0) code |= __shfl_xor_sync(0xffffffffu, code, 1);
+    if (lg > 1) code |= __shfl_xor_sync(0xffffffffu, code, 2);
+    const int64_t i = r0 + slot + s * (SH_T >> lg);
+    if (grp == 0 && i < n) codes[i] = code;
+  }
+}
+
+SLS_DEV bool simhash_vec(const float* U, int ldu) {
+  return (reinterpret_cast<uintptr_t>(U) & 15u) == 0 && (ldu & 3) == 0;
+}
+
+template <int RPT>
+__global__ void __launch_bounds__(SH_T)
 simhash_kernel(const float* __restrict__ U, int64_t N, int k, int ldu,
                const int32_t* __restrict__ k_dev, const float* __restrict__ R, int bits,
                int ldr, uint32_t* __restrict__ codes) {
-  extern __shared__ float Rs[];
+  extern __shared__ __align__(16) float sh_smem_f[];
   int kk = k;
   if (k_dev) kk = min(kk, max(0, (int)*k_dev));
-  simhash_stage_R(R, ldr, bits, kk, Rs);
+  simhash_stage_R(R, ldr, bits, kk, sh_smem_f);
   __syncthreads();
-  const int64_t wpb = blockDim.x >> 5;
-  simhash_lanes(U, N, ldu, kk, Rs, kk + 1, bits, codes,
-                (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5), (int64_t)gridDim.x * wpb);
+  simhash_tile<RPT>(U, N, (int64_t)blockIdx.x * sh_rows(bits, RPT), ldu, simhash_vec(U, ldu), kk,
+                    sh_smem_f, sh_smem_f + ((kk + 3) & ~3) * SH_LMAX, bits, codes);
 }
 
 // Batched over spectral problems: rows of problem p start at phi_row, k is
-// the problem's r_eff, bits its own bit count; simhash_lanes per problem.
-__global__ void __launch_bounds__(256)
+// the problem's r_eff, bits its own bit count; tiles of a problem over x.
+__global__ void __launch_bounds__(SH_T)
 simhash_batched_kernel(const ProbDesc* __restrict__ probs, const int* __restrict__ spec_list,
                        const int* __restrict__ nspec_dev, int nspec_max,
                        const int* __restrict__ r_eff, const float* __restrict__ U, int ldu,
                        const float* __restrict__ R, int ldr, uint32_t* __restrict__ codes) {
-  extern __shared__ float Rs[];
+  extern __shared__ __align__(16) float sh_smem_f[];
   const int s = blockIdx.y;
   int nspec = nspec_max;
   if (nspec_dev) nspec = min(nspec, *nspec_dev);
   if (s >= nspec) return;
   const ProbDesc P = probs[spec_list ? spec_list[s] : s];
+  const int rows = sh_rows(P.bits, 1);
+  if ((int64_t)blockIdx.x * rows >= P.n) return;
   const int kk = min(ldu, max(0, r_eff[s]));
-  simhash_stage_R(R, ldr, P.bits, kk, Rs);
+  simhash_stage_R(R, ldr, P.bits, kk, sh_smem_f);
   __syncthreads();
-  const int64_t wpb = blockDim.x >> 5;
-  simhash_lanes(U + (int64_t)P.phi_row * ldu, P.n, ldu, kk, Rs, kk + 1, P.bits,
-                codes + P.phi_row, (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5),
-                (int64_t)gridDim.x * wpb);
+  const float* Up = U + (int64_t)P.phi_row * ldu;
+  for (int64_t r0 = (int64_t)blockIdx.x * rows; r0 < P.n; r0 += (int64_t)gridDim.x * rows) {
+    simhash_tile<1>(Up, P.n, r0, ldu, simhash_vec(Up, ldu), kk, sh_smem_f,
+                    sh_smem_f + ((kk + 3) & ~3) * SH_LMAX, P.bits, codes + P.phi_row);
+    __syncthreads();
+  }
 }
 
 // Small problems (windows of at most SH_FLAT_MAX tokens): one thread per
 // (problem, row) over all spectral problems, R read through the read-only
-// cache (row l of R at R + l * ldr), the same float32 chain as simhash_lanes.
+// cache (row l of R at R + l * ldr), the same float32 chain as simhash_tile.
 constexpr int SH_FLAT_MAX = 64;
 
 __global__ void __launch_bounds__(256)
@@ -2209,15 +2315,19 @@ window_score_combine_kernel(int d, const ProbDesc* __restrict__ probs, int nprob
 int launch_simhash(const float* U, int64_t N, int k, int ldu, const int32_t* k_dev,
                    const float* R, int bits, int ldr, uint32_t* codes, cudaStream_t stream) {
   if (N == 0) return SLS_OK;
-  const size_t smem = sizeof(float) * bits * (k + 1);
-  int bp = 1;
-  while (bp < bits) bp <<= 1;
-  int64_t blocks = (N * bp + 255) / 256;  // 8 warps of 32 / bp rows
-  if (blocks > 4096) blocks = 4096;
+  int dev = 0, sms = 0;
+  SLS_CUDA_TRY(cudaGetDevice(&dev));
+  SLS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // two rows per thread (a hyperplane's load feeds both) once that still leaves
+  // every SM four tiles
+  const int rpt = N / sh_rows(bits, 2) >= 4 * (int64_t)sms ? 2 : 1;
+  auto fn = rpt == 2 ? simhash_kernel<2> : simhash_kernel<1>;
+  const size_t smem = sh_smem(bits, k, rpt);
+  const int64_t blocks = (N + sh_rows(bits, rpt) - 1) / sh_rows(bits, rpt);
+  if (blocks > 0x7fffffffLL) return SLS_ERR_UNSUPPORTED;
   if (smem > 48 * 1024)
-    SLS_CUDA_TRY(cudaFuncSetAttribute(simhash_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
-  simhash_kernel<<<(unsigned)blocks, 256, smem, stream>>>(U, N, k, ldu, k_dev, R, bits, ldr, codes);
+    SLS_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  fn<<<(unsigned)blocks, SH_T, smem, stream>>>(U, N, k, ldu, k_dev, R, bits, ldr, codes);
   SLS_LAUNCH_CHECK();
   return SLS_OK;
 }
@@ -2240,13 +2350,10 @@ int launch_simhash_problems(const ProbDesc* probs, const int* spec_list, const i
     SLS_LAUNCH_CHECK();
     return SLS_OK;
   }
-  const size_t smem = sizeof(float) * bits_max * (ldu + 1);
-  // warps of 32 / BP rows (BP: bits rounded up to a power of two): enough
-  // CTAs of 8 warps for the rows of the largest problem
-  int bpmax = 1;
-  while (bpmax < bits_max) bpmax <<= 1;
-  int64_t bx = (nmax * bpmax + 255) / 256;
-  if (bx > 1024) bx = 1024;
+  // shared memory for the widest tile of the problems' bit counts (bits <=
+  // bits_max; fewer bits per problem mean more rows per tile)
+  const size_t smem = sh_smem(1, ldu, 1);
+  int64_t bx = (nmax + sh_rows(bits_max, 1) - 1) / sh_rows(bits_max, 1);
   // at most about 8192 CTAs in all (the CTAs loop over their problem's
   // rows): the launch is sized by the bound on the spectral problems, most
   // of which may be empty at run time
@@ -2256,7 +2363,7 @@ int launch_simhash_problems(const ProbDesc* probs, const int* spec_list, const i
   if (smem > 48 * 1024)
     SLS_CUDA_TRY(cudaFuncSetAttribute(simhash_batched_kernel,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  simhash_batched_kernel<<<dim3((unsigned)bx, nspec_max), 256, smem, stream>>>(
+  simhash_batched_kernel<<<dim3((unsigned)bx, nspec_max), SH_T, smem, stream>>>(
       probs, spec_list, nspec_dev, nspec_max, r_eff, U, ldu, R, ldr, codes);
   SLS_LAUNCH_CHECK();
   return SLS_OK;
