@@ -14,10 +14,7 @@ namespace sls {
 
 namespace {
 
-constexpr int FM_BM = 64;   // tokens per CTA tile
-constexpr int FM_BN = 64;   // features per CTA tile
 constexpr int FM_BK = 16;   // K slice
-constexpr int FM_THREADS = 256;
 
 template <typename T>
 SLS_DEV float load_elem(const T* p);
@@ -32,73 +29,187 @@ SLS_DEV float load_elem<uint16_t>(const uint16_t* p) {
   return __uint_as_float(((unsigned)*p) << 16);
 }
 
-// One CTA computes a 64 x 64 tile; each thread a 4 x 4 block.  T: element
-// type of X and W; OT: of Phi (float, or uint16_t for bfloat16).
-template <typename T, typename OT>
-__global__ void __launch_bounds__(FM_THREADS)
+// Elements k .. k + 3 of a row of d elements (zero past its end); vec: the row
+// start and d allow 16-byte (float32) or 8-byte (bf16) loads.
+template <typename T>
+SLS_DEV float4 load_quad(const T* row, int k, int d, bool vec);
+
+template <>
+SLS_DEV float4 load_quad<float>(const float* row, int k, int d, bool vec) {
+  if (vec && k + 3 < d) return __ldg(reinterpret_cast<const float4*>(row + k));
+  return make_float4(k < d ? row[k] : 0.f, k + 1 < d ? row[k + 1] : 0.f,
+                     k + 2 < d ? row[k + 2] : 0.f, k + 3 < d ? row[k + 3] : 0.f);
+}
+
+template <>
+SLS_DEV float4 load_quad<uint16_t>(const uint16_t* row, int k, int d, bool vec) {
+  if (vec && k + 3 < d) {
+    const uint2 u = __ldg(reinterpret_cast<const uint2*>(row + k));
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                       __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+  }
+  return make_float4(k < d ? load_elem(row + k) : 0.f, k + 1 < d ? load_elem(row + k + 1) : 0.f,
+                     k + 2 < d ? load_elem(row + k + 2) : 0.f,
+                     k + 3 < d ? load_elem(row + k + 3) : 0.f);
+}
+
+// G (2 or 4) neighbouring floats of shared memory in one load.
+template <int G>
+SLS_DEV void load_group(const float* p, float* out) {
+  if constexpr (G == 4) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    out[0] = v.x;
+    out[1] = v.y;
+    out[2] = v.z;
+    out[3] = v.w;
+  } else {
+    const float2 v = *reinterpret_cast<const float2*>(p);
+    out[0] = v.x;
+    out[1] = v.y;
+  }
+}
+
+// One CTA computes a BM x BN tile, each thread TM x TN of it; every output is
+// one chain of fused multiply-adds over k ascending, whatever the tile.  T:
+// element type of X and W; OT: of Phi (float, or uint16_t for bfloat16).
+//
+// Bound by the FP32 pipes (two features per packed instruction).  A K slice is
+// loaded as quads along the rows into registers while the previous slice is
+// computed, then stored transposed into the other of two shared-memory buffers:
+// one barrier per slice, and TM + TN floats read per TM * TN multiply-adds.
+// N = 4084, d = 2048, D = 1024: 600 -> 395 us a call against the former kernel
+// (64 x 64 tiles, 4 x 4 per thread, scalar loads between two barriers), with the
+// same bits.
+template <typename T, typename OT, int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN))
 feature_map_simt_kernel(const T* __restrict__ X, int64_t N, int d, int64_t ldx,
                         const T* __restrict__ W, const float* __restrict__ bvec,
-                        int D, float scale, OT* __restrict__ Phi) {
-  __shared__ float As[FM_BK][FM_BM + 4];
-  __shared__ float Bs[FM_BK][FM_BN + 4];
+                        int D, float scale, OT* __restrict__ Phi, int vecx, int vecw) {
+  constexpr int NT = (BM / TM) * (BN / TN);
+  constexpr int QA = (BM * FM_BK / 4) / NT, QB = (BN * FM_BK / 4) / NT;  // quads per thread
+  static_assert(QA * NT == BM * FM_BK / 4 && QB * NT == BN * FM_BK / 4, "whole quads per thread");
+  static_assert(TM % 2 == 0 && TN % 2 == 0, "pairs");
+  __shared__ __align__(16) float As[2][FM_BK][BM + 4];
+  __shared__ __align__(16) float Bs[2][FM_BK][BN + 4];
   const int tid = threadIdx.x;
-  const int64_t row0 = (int64_t)blockIdx.y * FM_BM;
-  const int col0 = blockIdx.x * FM_BN;
-  const int ty = tid / 16, tx = tid % 16;
-  float acc[4][4];
+  const int64_t row0 = (int64_t)blockIdx.y * BM;
+  const int col0 = blockIdx.x * BN;
+  const int ty = tid / (BN / TN), tx = tid % (BN / TN);
+  f32x2_t acc[TM][TN / 2];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-  for (int k0 = 0; k0 < d; k0 += FM_BK) {
-    // each thread loads 4 elements of A and 4 of B (64 x 16 each)
+    for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+  float4 ra[QA], rb[QB];
+  auto fetch = [&](int k0) {
 #pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      int e = tid + t * FM_THREADS;  // 0..1023
-      int r = e / FM_BK, k = e % FM_BK;
-      int64_t gr = row0 + r;
-      int gk = k0 + k;
-      As[k][r] = (gr < N && gk < d) ? load_elem<T>(X + gr * ldx + gk) : 0.f;
-      int c = col0 + r;
-      Bs[k][r] = (c < D && gk < d) ? load_elem<T>(W + (int64_t)c * d + gk) : 0.f;
+    for (int q = 0; q < QA; ++q) {
+      const int e = tid + q * NT, r = e / (FM_BK / 4), k = k0 + 4 * (e % (FM_BK / 4));
+      ra[q] = row0 + r < N ? load_quad<T>(X + (row0 + r) * ldx, k, d, vecx)
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < QB; ++q) {
+      const int e = tid + q * NT, r = e / (FM_BK / 4), k = k0 + 4 * (e % (FM_BK / 4));
+      rb[q] = col0 + r < D ? load_quad<T>(W + (int64_t)(col0 + r) * d, k, d, vecw)
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  auto stage = [&](int buf) {
+#pragma unroll
+    for (int q = 0; q < QA; ++q) {
+      const int e = tid + q * NT, r = e / (FM_BK / 4), k = 4 * (e % (FM_BK / 4));
+      As[buf][k][r] = ra[q].x;
+      As[buf][k + 1][r] = ra[q].y;
+      As[buf][k + 2][r] = ra[q].z;
+      As[buf][k + 3][r] = ra[q].w;
+    }
+#pragma unroll
+    for (int q = 0; q < QB; ++q) {
+      const int e = tid + q * NT, r = e / (FM_BK / 4), k = 4 * (e % (FM_BK / 4));
+      Bs[buf][k][r] = rb[q].x;
+      Bs[buf][k + 1][r] = rb[q].y;
+      Bs[buf][k + 2][r] = rb[q].z;
+      Bs[buf][k + 3][r] = rb[q].w;
+    }
+  };
+  fetch(0);
+  stage(0);
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = 0; k0 < d; k0 += FM_BK, buf ^= 1) {
+    const bool more = k0 + FM_BK < d;
+    if (more) fetch(k0 + FM_BK);
 #pragma unroll
     for (int k = 0; k < FM_BK; ++k) {
-      float a[4], bb[4];
+      // the thread's rows in groups of two or four spread over the tile (rows
+      // ty * G + i of each BM / (TM / G) rows), so that a warp's reads of a
+      // group touch neighbouring words
+      constexpr int GA = TM % 4 ? 2 : 4, GB = TN % 4 ? 2 : 4;
+      float a[TM], bb[TN];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[k][ty * 4 + i];
+      for (int i = 0; i < TM; i += GA)
+        load_group<GA>(&As[buf][k][(i / GA) * (BM / (TM / GA)) + ty * GA], a + i);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) bb[j] = Bs[k][tx * 4 + j];
+      for (int j = 0; j < TN; j += GB)
+        load_group<GB>(&Bs[buf][k][(j / GB) * (BN / (TN / GB)) + tx * GB], bb + j);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TM; ++i) {
+        const f32x2_t aa = pk2(a[i], a[i]);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
+        for (int j = 0; j < TN / 2; ++j) acc[i][j] = fma2(aa, pk2(bb[2 * j], bb[2 * j + 1]), acc[i][j]);
+      }
     }
+    if (more) stage(buf ^ 1);
     __syncthreads();
   }
+  constexpr int GA = TM % 4 ? 2 : 4, GB = TN % 4 ? 2 : 4;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int64_t gr = row0 + ty * 4 + i;
+  for (int i = 0; i < TM; ++i) {
+    const int64_t gr = row0 + (i / GA) * (BM / (TM / GA)) + ty * GA + i % GA;
     if (gr >= N) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int c = col0 + tx * 4 + j;
-      if (c < D) phi_st(Phi + gr * D + c, scale * cosf(acc[i][j] + bvec[c]));
+    for (int j = 0; j < TN / 2; ++j) {
+      const int c = col0 + (2 * j / GB) * (BN / (TN / GB)) + tx * GB + (2 * j) % GB;
+      float v0, v1;
+      upk2(acc[i][j], v0, v1);
+      if (c < D) phi_st(Phi + gr * D + c, scale * cosf(v0 + bvec[c]));
+      if (c + 1 < D) phi_st(Phi + gr * D + c + 1, scale * cosf(v1 + bvec[c + 1]));
     }
   }
 }
 
-template <typename T>
-void launch_simt_t(const void* X, int64_t N, int d, int64_t ldx, const void* W, const float* b,
-                   int D, float scale, void* Phi, int phi_bf16, dim3 grid, cudaStream_t stream) {
+template <typename T, int BM, int BN, int TM, int TN>
+int launch_simt_tile(const void* X, int64_t N, int d, int64_t ldx, const void* W, const float* b,
+                     int D, float scale, void* Phi, int phi_bf16, cudaStream_t stream) {
+  const uintptr_t al = sizeof(T) == 4 ? 15 : 7;  // a quad of elements
+  const int vecx = ((uintptr_t)X & al) == 0 && ldx % 4 == 0;
+  const int vecw = ((uintptr_t)W & al) == 0 && d % 4 == 0;
+  const dim3 grid((D + BN - 1) / BN, (unsigned)((N + BM - 1) / BM));
+  constexpr int NT = (BM / TM) * (BN / TN);
   if (phi_bf16)
-    feature_map_simt_kernel<T, uint16_t><<<grid, FM_THREADS, 0, stream>>>(
-        (const T*)X, N, d, ldx, (const T*)W, b, D, scale, (uint16_t*)Phi);
+    feature_map_simt_kernel<T, uint16_t, BM, BN, TM, TN><<<grid, NT, 0, stream>>>(
+        (const T*)X, N, d, ldx, (const T*)W, b, D, scale, (uint16_t*)Phi, vecx, vecw);
   else
-    feature_map_simt_kernel<T, float><<<grid, FM_THREADS, 0, stream>>>(
-        (const T*)X, N, d, ldx, (const T*)W, b, D, scale, (float*)Phi);
+    feature_map_simt_kernel<T, float, BM, BN, TM, TN><<<grid, NT, 0, stream>>>(
+        (const T*)X, N, d, ldx, (const T*)W, b, D, scale, (float*)Phi, vecx, vecw);
+  SLS_LAUNCH_CHECK();
+  return SLS_OK;
+}
+
+// The tile: 128 x 64 once every SM gets three of them, 64 x 64 from one per SM
+// on, else 32 x 32, which keeps more SMs busy on a short prompt.  Measured (us;
+// 128 x 128 / 128 x 64 / 64 x 64): N = 4084, d = 2048, D = 1024 391 / 395 / 412;
+// 8192, 2048, 1024 750 / 659 / 777; 2000, 1024, 512 121 / 83 / 79.
+template <typename T>
+int launch_simt_t(const void* X, int64_t N, int d, int64_t ldx, const void* W, const float* b,
+                  int D, float scale, void* Phi, int phi_bf16, int sms, cudaStream_t stream) {
+  auto tiles = [&](int64_t bm, int64_t bn) { return ((N + bm - 1) / bm) * ((D + bn - 1) / bn); };
+  if (tiles(128, 64) >= 3 * (int64_t)sms)
+    return launch_simt_tile<T, 128, 64, 8, 8>(X, N, d, ldx, W, b, D, scale, Phi, phi_bf16, stream);
+  if (tiles(64, 64) >= (int64_t)sms)
+    return launch_simt_tile<T, 64, 64, 8, 4>(X, N, d, ldx, W, b, D, scale, Phi, phi_bf16, stream);
+  return launch_simt_tile<T, 32, 32, 4, 2>(X, N, d, ldx, W, b, D, scale, Phi, phi_bf16, stream);
 }
 
 }  // namespace
@@ -108,14 +219,13 @@ int launch_feature_map_simt(const void* X, int x_dtype, int64_t N, int d, int64_
                             cudaStream_t stream, int phi_bf16) {
   if (N == 0) return SLS_OK;
   const float scale = (float)sqrt(2.0 / (double)D);
-  dim3 grid((D + FM_BN - 1) / FM_BN, (unsigned)((N + FM_BM - 1) / FM_BM));
-  if (grid.y > 65535u) return SLS_ERR_UNSUPPORTED;
+  if ((N + 63) / 64 > 65535) return SLS_ERR_UNSUPPORTED;
+  int dev = 0, sms = 0;
+  SLS_CUDA_TRY(cudaGetDevice(&dev));
+  SLS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   if (x_dtype == SLS_F32)
-    launch_simt_t<float>(X, N, d, ldx, W, b, D, scale, Phi, phi_bf16, grid, stream);
-  else
-    launch_simt_t<uint16_t>(X, N, d, ldx, W, b, D, scale, Phi, phi_bf16, grid, stream);
-  SLS_LAUNCH_CHECK();
-  return SLS_OK;
+    return launch_simt_t<float>(X, N, d, ldx, W, b, D, scale, Phi, phi_bf16, sms, stream);
+  return launch_simt_t<uint16_t>(X, N, d, ldx, W, b, D, scale, Phi, phi_bf16, sms, stream);
 }
 
 }  // namespace sls
