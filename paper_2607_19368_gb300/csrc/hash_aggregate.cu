@@ -2061,21 +2061,42 @@ __host__ __device__ inline int chunk_parts_max(int64_t nmax) {
   return (int)((nmax + SCORE_PR / 2 - 1) / (SCORE_PR / 2));
 }
 
-// Element e of a 16-byte word of X as loaded: four floats, or eight bf16
-// values widened exactly.  Keeping the loaded rows as raw words halves their
-// registers for bf16 inputs.
+// Elements 2 p and 2 p + 1 of a 16-byte word of X as a packed pair.
 template <typename T>
-SLS_DEV float raw_elem(const uint4& r, int e);
+SLS_DEV f32x2_t raw_pair(const uint4& r, int p);
 template <>
-SLS_DEV float raw_elem<float>(const uint4& r, int e) {
-  const unsigned w = (e == 0) ? r.x : (e == 1) ? r.y : (e == 2) ? r.z : r.w;
-  return __uint_as_float(w);
+SLS_DEV f32x2_t raw_pair<float>(const uint4& r, int p) {
+  return p == 0 ? pk2(__uint_as_float(r.x), __uint_as_float(r.y))
+                : pk2(__uint_as_float(r.z), __uint_as_float(r.w));
 }
 template <>
-SLS_DEV float raw_elem<uint16_t>(const uint4& r, int e) {
-  const int k = e >> 1;
-  const unsigned w = (k == 0) ? r.x : (k == 1) ? r.y : (k == 2) ? r.z : r.w;
-  return (e & 1) ? __uint_as_float(w & 0xffff0000u) : __uint_as_float(w << 16);
+SLS_DEV f32x2_t raw_pair<uint16_t>(const uint4& r, int p) {
+  const unsigned w = (p == 0) ? r.x : (p == 1) ? r.y : (p == 2) ? r.z : r.w;
+  return pk2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
+// Sums over the warp of R values per lane (R a power of two up to 8) by a
+// transposed butterfly: lane L gets the sum of value L / (32 / R).
+template <int R>
+SLS_DEV float warp_sums(float (&v)[R]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int s = 0; s < 5; ++s) {
+    const int h = 16 >> s;
+    const int nv = (R >> s) > 1 ? (R >> s) : 1;
+    if (nv > 1) {
+      const bool up = (lane & h) != 0;
+#pragma unroll
+      for (int i = 0; i < nv / 2; ++i) {
+        const float send = up ? v[i] : v[i + nv / 2];
+        const float keep = up ? v[i + nv / 2] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], h);
+    }
+  }
+  return v[0];
 }
 
 // 16-byte asynchronous copy global -> shared (zero-filled when !live), and
@@ -2141,30 +2162,33 @@ window_score_chunk_kernel(const T* __restrict__ X, int d, int64_t ldx,
       const int g = (i < rem * (q + 1)) ? i / (q + 1) : rem + (i - rem * (q + 1)) / q;
       tok2macro[P.tok_row + i] = P.out_local + g;
     }
-    float cs[NV * V], ns[NV * V], gs[NV * V];
+    constexpr int PN = NV * V / 2;  // element pairs per thread
+    f32x2_t cs[PN], ns[PN], gs[PN];
 #pragma unroll
-    for (int e = 0; e < NV * V; ++e) cs[e] = ns[e] = gs[e] = 0.f;
+    for (int e = 0; e < PN; ++e) cs[e] = ns[e] = gs[e] = 0ull;
     int gcur = g0, gend = chunk_gstart(n, m, g0 + 1), gcnt = 0;  // before the barrier
     int pcur = g0, pend = gend, pcnt = 0;                          // after it
     float geta = 0.f;
     // the copies of batch s0 go to ring slot b; the next batch is in flight
     // while this one is processed
+    const T* xrow = X + (P.tok_row + r0) * ldx + tid * V;  // of the next batch to issue
     auto issue = [&](int s0, int b) {
 #pragma unroll
       for (int j = 0; j < MB; ++j) {
         const bool rl = s0 + j < r1;
-        const T* x = X + (P.tok_row + (rl ? s0 + j : r0)) * ldx;
 #pragma unroll
         for (int qv = 0; qv < NV; ++qv) {
-          const int c0 = (tid + qv * AGG_T) * V;
-          const bool live = rl && c0 < d;
-          cp16_async(&chk_ring[((b * MB + j) * NV + qv) * AGG_T + tid], live ? x + c0 : x, live);
+          const bool live = rl && (tid + qv * AGG_T) * V < d;
+          cp16_async(&chk_ring[((b * MB + j) * NV + qv) * AGG_T + tid],
+                     live ? xrow + j * ldx + qv * AGG_T * V : X, live);
         }
       }
+      xrow += MB * ldx;
       cp_async_commit();
     };
     issue(r0, 0);
     int buf = 0;
+    constexpr int LPR = 32 / MB;  // lanes that share a row's scalars
     for (int s0 = r0; s0 < r1; s0 += MB, buf ^= 1) {
       if (s0 + MB < r1) {
         issue(s0 + MB, buf ^ 1);
@@ -2181,56 +2205,68 @@ window_score_chunk_kernel(const T* __restrict__ X, int d, int64_t ldx,
       // before the barrier: row |x|^2 partials; the group sums, and for every
       // group that ends in this batch its mean (stored unscaled; a singleton is
       // its token) and the |mean|^2 partial
+      float sq[MB];
 #pragma unroll
       for (int j = 0; j < MB; ++j) {
-        float sq = 0.f;
+        f32x2_t q2 = 0ull;
 #pragma unroll
-        for (int e = 0; e < NV * V; ++e) {
-          const float x = raw_elem<T>(raw[j][e / V], e % V);
-          sq = fmaf(x, x, sq);
+        for (int e = 0; e < PN; ++e) {
+          const f32x2_t x = raw_pair<T>(raw[j][e / (V / 2)], e % (V / 2));
+          q2 = fma2(x, x, q2);
+          gs[e] = add2(gs[e], x);  // a row past the part is zero
         }
-        sq = warp_sum_f(sq);
-        if (lane == 0) shq[buf][j][warp] = sq;
+        float qa, qb;
+        upk2(q2, qa, qb);
+        sq[j] = qa + qb;
         if (s0 + j < r1) {
-#pragma unroll
-          for (int e = 0; e < NV * V; ++e) gs[e] += raw_elem<T>(raw[j][e / V], e % V);
           ++gcnt;
           if (s0 + j + 1 == gend) {
             const float ginv = (gcnt > 1) ? 1.0f / (float)gcnt : 1.0f;
-            float gq = 0.f;
+            float gq = 0.f, mean[NV * V];
 #pragma unroll
-            for (int e = 0; e < NV * V; ++e) {
-              if (gcnt > 1) gs[e] *= ginv;
-              gq = fmaf(gs[e], gs[e], gq);
+            for (int e = 0; e < PN; ++e) {
+              cs[e] = add2(cs[e], gs[e]);
+              upk2(gs[e], mean[2 * e], mean[2 * e + 1]);
+              if (gcnt > 1) {
+                mean[2 * e] *= ginv;
+                mean[2 * e + 1] *= ginv;
+              }
+              gq = fmaf(mean[2 * e], mean[2 * e], gq);
+              gq = fmaf(mean[2 * e + 1], mean[2 * e + 1], gq);
+              gs[e] = 0ull;
             }
             gq = warp_sum_f(gq);
             if (lane == 0) shg[buf][j][warp] = gq;
-            store_row<V, NV>(gs, 1.0f, d, Xt + (P.out0 + gcur) * (int64_t)d);
-#pragma unroll
-            for (int e = 0; e < NV * V; ++e) gs[e] = 0.f;
+            store_row<V, NV>(mean, 1.0f, d, Xt + (P.out0 + gcur) * (int64_t)d);
             gcnt = 0;
             ++gcur;
             gend = chunk_gstart(n, m, gcur + 1);
           }
         }
       }
+      {
+        const float t = warp_sums<MB>(sq);
+        if (lane % LPR == 0) shq[buf][lane / LPR][warp] = t;
+      }
       __syncthreads();
       // after it: the score sums, and each finished group's mean rescaled in
-      // place to the mean member norm (Eq. macro_embed)
+      // place to the mean member norm (Eq. macro_embed).  LPR lanes add a row's
+      // warp sums and form its norm; shuffles hand it to the others.
+      float tq = 0.f;
+#pragma unroll
+      for (int w = lane % LPR; w < NW; w += LPR) tq += shq[buf][lane / LPR][w];
+#pragma unroll
+      for (int o = 1; o < LPR && o < NW; o <<= 1) tq += __shfl_xor_sync(0xffffffffu, tq, o);
+      const float nrm_l = sqrtf(tq), inv_l = (tq > 0.f) ? 1.0f / nrm_l : 0.f;
 #pragma unroll
       for (int j = 0; j < MB; ++j) {
         if (s0 + j >= r1) break;
-        float tq = 0.f;
+        const float nrm = __shfl_sync(0xffffffffu, nrm_l, j * LPR);
+        const float inv = __shfl_sync(0xffffffffu, inv_l, j * LPR);
+        const f32x2_t inv2 = pk2(inv, inv);
 #pragma unroll
-        for (int w = 0; w < NW; ++w) tq += shq[buf][j][w];
-        const float nrm = sqrtf(tq);
-        const float inv = (tq > 0.f) ? 1.0f / nrm : 0.f;
-#pragma unroll
-        for (int e = 0; e < NV * V; ++e) {
-          const float x = raw_elem<T>(raw[j][e / V], e % V);
-          cs[e] += x;
-          ns[e] = fmaf(x, inv, ns[e]);
-        }
+        for (int e = 0; e < PN; ++e)
+          ns[e] = fma2(raw_pair<T>(raw[j][e / (V / 2)], e % (V / 2)), inv2, ns[e]);
         geta += nrm;
         ++pcnt;
         if (s0 + j + 1 == pend) {
@@ -2269,10 +2305,13 @@ window_score_chunk_kernel(const T* __restrict__ X, int d, int64_t ldx,
       if (c0 < d)
 #pragma unroll
         for (int e = 0; e < V; e += 4) {
-          store_vec4(dst + c0 + e, cs[qv * V + e], cs[qv * V + e + 1], cs[qv * V + e + 2],
-                     cs[qv * V + e + 3]);
-          store_vec4(dst + d + c0 + e, ns[qv * V + e], ns[qv * V + e + 1], ns[qv * V + e + 2],
-                     ns[qv * V + e + 3]);
+          float a0, a1, a2, a3;
+          upk2(cs[(qv * V + e) / 2], a0, a1);
+          upk2(cs[(qv * V + e) / 2 + 1], a2, a3);
+          store_vec4(dst + c0 + e, a0, a1, a2, a3);
+          upk2(ns[(qv * V + e) / 2], a0, a1);
+          upk2(ns[(qv * V + e) / 2 + 1], a2, a3);
+          store_vec4(dst + d + c0 + e, a0, a1, a2, a3);
         }
     }
     __syncthreads();
@@ -2289,15 +2328,19 @@ window_score_combine_kernel(int d, const ProbDesc* __restrict__ probs, int nprob
     const int n = probs[p].n;
     const int kp = chunked ? chunk_nparts(n, probs[p].m) : score_parts(n);
     float dot = 0.f, cc = 0.f;
-    for (int c = threadIdx.x; c < d; c += AGG_T) {
-      float cs = 0.f, ns = 0.f;
-      for (int k = 0; k < kp; ++k) {
-        const float* src = part + ((size_t)p * KP + k) * 2 * d;
-        cs += src[c];
-        ns += src[d + c];
+    // four columns per thread (d % 4 == 0), several parts' loads in flight
+    for (int c = 4 * threadIdx.x; c < d; c += 4 * AGG_T) {
+      float4 cs = make_float4(0.f, 0.f, 0.f, 0.f), ns = cs;
+      const float* src = part + (size_t)p * KP * 2 * d + c;
+#pragma unroll 4
+      for (int k = 0; k < kp; ++k, src += 2 * d) {
+        const float4 a = *reinterpret_cast<const float4*>(src);
+        const float4 b = *reinterpret_cast<const float4*>(src + d);
+        cs = make_float4(cs.x + a.x, cs.y + a.y, cs.z + a.z, cs.w + a.w);
+        ns = make_float4(ns.x + b.x, ns.y + b.y, ns.z + b.z, ns.w + b.w);
       }
-      dot = fmaf(ns, cs, dot);
-      cc = fmaf(cs, cs, cc);
+      dot = fmaf(ns.x, cs.x, fmaf(ns.y, cs.y, fmaf(ns.z, cs.z, fmaf(ns.w, cs.w, dot))));
+      cc = fmaf(cs.x, cs.x, fmaf(cs.y, cs.y, fmaf(cs.z, cs.z, fmaf(cs.w, cs.w, cc))));
     }
     dot = agg_block_sum(dot, sh);
     cc = agg_block_sum(cc, sh);
