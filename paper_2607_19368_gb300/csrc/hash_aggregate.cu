@@ -691,7 +691,19 @@ segment_kernel(const ProbDesc* __restrict__ probs, int nprob, const uint32_t* __
 // ============================================================================
 
 constexpr int SEGG_MAX = 256;           // CTAs of the grid segment kernel, at most
-constexpr int64_t SEG_GRID_MIN_N = 8192;  // tokens from which one problem uses the grid kernel
+
+// One problem of at least SEG_CLUSTER_MIN_N tokens runs on a cluster of SEG_CL
+// CTAs (N = 1500: 148 us on a cluster of eight, 124 on one CTA with its sort in
+// shared memory), above SEG_CLUSTER_MAX_N on a cooperative grid.
+constexpr int SEG_CL = 16;
+constexpr int64_t SEG_CLUSTER_MIN_N = 4096, SEG_CLUSTER_MAX_N = 1 << 18;
+
+// All CTAs of one thread-block cluster meet (arrive: release, wait: acquire, at
+// cluster scope, global memory included).
+SLS_DEV void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 
 struct GridSync {
   GroupBarrier bar;
@@ -699,9 +711,14 @@ struct GridSync {
   int* status;
   int* sflag;
   volatile int* serr;
+  bool cluster;  // the grid is one cluster: its hardware barrier
 };
 
 SLS_DEV bool gsync(GridSync& gs) {
+  if (gs.cluster) {
+    cluster_sync_all();
+    return true;
+  }
   return group_sync_named(gs.bar, gs.lgen, gs.status, gs.sflag, gs.serr, 1, SEG_T);
 }
 
@@ -831,7 +848,7 @@ segment_grid_kernel(const ProbDesc* __restrict__ probs, const uint32_t* __restri
                     int pos_scheme, int pos_mode, char* sb, int64_t nmax, int64_t mmax,
                     int* __restrict__ perm, int* __restrict__ mstart, int* __restrict__ mlen,
                     int32_t* __restrict__ pos_out, int32_t* __restrict__ tok2macro,
-                    int* status, int chunk_done) {
+                    int* status, int chunk_done, int cluster) {
   __shared__ int sh_sort[512 + SEG_W * 256];
   __shared__ long long sh_ll[SEG_W + 1];
   __shared__ int sh_i[SEG_W + 1];
@@ -843,7 +860,7 @@ segment_grid_kernel(const ProbDesc* __restrict__ probs, const uint32_t* __restri
   __syncthreads();
   GridSync gs{GroupBarrier{reinterpret_cast<unsigned*>(sb + L.gbar),
                            reinterpret_cast<unsigned*>(sb + L.gbar) + 32, (unsigned)G},
-              0u, status, &sflag, &serr};
+              0u, status, &sflag, &serr, cluster != 0};
   const ProbDesc P = probs[0];
   const int n = P.n, M = P.m;
   if (n <= 0 || M <= 0) return;
@@ -897,9 +914,10 @@ segment_grid_kernel(const ProbDesc* __restrict__ probs, const uint32_t* __restri
         const int gp = (t == 0) ? -1 : (int)(((long long)(t - 1) * M) / C);
         if (g != gp) gst[g] = cst[t];
       }
-    } else if (b == 0) {
+    } else {
       // split: D'Hondt seats, one guaranteed per cluster, ties to the lower
-      // code (few clusters: one CTA)
+      // code.  The K-th quotient by multisection: every CTA counts the
+      // quotients at or above its own threshold, one grid barrier per round.
       const long long K = (long long)(M - C);
       int maxn = 0;
       for (int t = tid; t < C; t += SEG_T) maxn = max(maxn, cst[t + 1] - cst[t]);
@@ -910,41 +928,55 @@ segment_grid_kernel(const ProbDesc* __restrict__ probs, const uint32_t* __restri
       maxn = sh_i[0];
       __syncthreads();
       long long lo = 0, hi = ((long long)maxn) << 40;
-      while (hi - lo > 1) {
-        const long long mid = lo + (hi - lo) / 2;
+      long long* cnt = reinterpret_cast<long long*>(hist);  // 2 x G counts by round parity
+      for (int round = 0; hi - lo > 1; ++round) {
+        // threshold x (1 <= x <= G): lo + x (hi - lo) / (G + 1), the quotient and
+        // remainder apart so that nothing overflows
+        const long long w = hi - lo, wq = w / (G + 1), wr = w % (G + 1);
+        auto thr = [&](int x) { return lo + wq * x + wr * x / (G + 1); };
+        const long long mine = thr(b + 1);
         long long c = 0;
-        for (int t = tid; t < C; t += SEG_T) c += dhondt_count_ge(cst[t + 1] - cst[t], mid);
+        for (int t = tid; t < C; t += SEG_T) c += dhondt_count_ge(cst[t + 1] - cst[t], mine);
         c = block_sum<long long>(c, sh_ll);
-        if (c >= K) lo = mid;
-        else hi = mid;
+        if (tid == 0) cnt[(round & 1) * G + b] = c;
+        if (!gsync(gs)) return;
+        // counts fall with the threshold: the last one still at K or above
+        int ok = 0;
+        for (int x = tid; x < G; x += SEG_T) ok += cnt[(round & 1) * G + x] >= K ? 1 : 0;
+        const int nok = block_sum<int>(ok, sh_i);
+        const long long nlo = nok > 0 ? thr(nok) : lo, nhi = nok < G ? thr(nok + 1) : hi;
+        lo = nlo;
+        hi = nhi;
       }
-      long long gt_sum = 0;
-      for (int t = tid; t < C; t += SEG_T) {
-        const long long nt = cst[t + 1] - cst[t];
-        const long long ge = dhondt_count_ge(nt, lo);
-        const long long gt = dhondt_count_ge(nt, lo + 1);
-        seat[t] = (int)gt;
-        f[t] = (int)(ge - gt);
-        gt_sum += gt;
-      }
-      gt_sum = block_sum<long long>(gt_sum, sh_ll);
-      const int R = (int)(K - gt_sum);
-      __syncthreads();
-      int* eqs = grp;  // scratch (size >= C)
-      block_scan_array<int>(f, eqs, C, sh_i);
-      for (int t = tid; t < C; t += SEG_T) {
-        const int extra = (f[t] && eqs[t] < R) ? 1 : 0;
-        seat[t] = 1 + seat[t] + extra;
-      }
-      __syncthreads();
-      int* so = f;
-      block_scan_array<int>(seat, so, C, sh_i);
-      for (int t = tid; t < C; t += SEG_T) {
-        const int nt = cst[t + 1] - cst[t], pt = seat[t];
-        const int q = nt / pt, rem = nt % pt;
-        for (int k = 0; k < pt; ++k) {
-          const int off = (k < rem) ? k * (q + 1) : rem * (q + 1) + (k - rem) * q;
-          gst[so[t] + k] = cst[t] + off;
+      if (b == 0) {
+        long long gt_sum = 0;
+        for (int t = tid; t < C; t += SEG_T) {
+          const long long nt = cst[t + 1] - cst[t];
+          const long long ge = dhondt_count_ge(nt, lo);
+          const long long gt = dhondt_count_ge(nt, lo + 1);
+          seat[t] = (int)gt;
+          f[t] = (int)(ge - gt);
+          gt_sum += gt;
+        }
+        gt_sum = block_sum<long long>(gt_sum, sh_ll);
+        const int R = (int)(K - gt_sum);
+        __syncthreads();
+        int* eqs = grp;  // scratch (size >= C)
+        block_scan_array<int>(f, eqs, C, sh_i);
+        for (int t = tid; t < C; t += SEG_T) {
+          const int extra = (f[t] && eqs[t] < R) ? 1 : 0;
+          seat[t] = 1 + seat[t] + extra;
+        }
+        __syncthreads();
+        int* so = f;
+        block_scan_array<int>(seat, so, C, sh_i);
+        for (int t = tid; t < C; t += SEG_T) {
+          const int nt = cst[t + 1] - cst[t], pt = seat[t];
+          const int q = nt / pt, rem = nt % pt;
+          for (int k = 0; k < pt; ++k) {
+            const int off = (k < rem) ? k * (q + 1) : rem * (q + 1) + (k - rem) * q;
+            gst[so[t] + k] = cst[t] + off;
+          }
         }
       }
     }
@@ -2429,22 +2461,44 @@ int launch_segment(const ProbDesc* probs, int nprob, const uint32_t* codes, int 
     SLS_LAUNCH_CHECK();
     return SLS_OK;
   }
-  if (nprob == 1 && nmax >= SEG_GRID_MIN_N && status) {
-    // one large problem: spread it over a cooperative grid
+  if (nprob == 1 && nmax >= SEG_CLUSTER_MIN_N && status) {
+    char* sb = (char*)scratch;
+    if (nmax <= SEG_CLUSTER_MAX_N) {
+      // one problem on one cluster: its hardware barrier costs 0.2 us, the
+      // cooperative grid's 2.5 us, and the computation holds about thirty
+      // (N = 8180: 82 -> 50 us, N = 32756: 132 -> 70)
+      const int G = SEG_CL;
+      SLS_CUDA_TRY(cudaFuncSetAttribute(segment_grid_kernel,
+                                        cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(G);
+      cfg.blockDim = dim3(SEG_T);
+      cfg.stream = stream;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = G;
+      at[0].val.clusterDim.y = 1;
+      at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      SLS_CUDA_TRY(cudaLaunchKernelEx(&cfg, segment_grid_kernel, probs, codes, pos_scheme,
+                                      pos_mode, sb, nmax, mmax, perm, mstart, mlen, pos_out,
+                                      tok2macro, status, chunk_done, 1));
+      count_launch(1);
+      return SLS_OK;
+    }
+    // a larger one: a cooperative grid
     int dev = 0, sms = 0;
     SLS_CUDA_TRY(cudaGetDevice(&dev));
     SLS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     int G = sms < SEGG_MAX ? sms : SEGG_MAX;
-    const int64_t want = (nmax + 255) / 256;
-    if (want < G) G = (int)want;
-    if (G < 1) G = 1;
-    char* sb = (char*)scratch;
     SLS_CUDA_TRY(cudaMemsetAsync(sb + L.gbar, 0, 256, stream));
     int64_t nm = nmax, mm = mmax;
+    int cluster = 0;
     void* args[] = {(void*)&probs, (void*)&codes, (void*)&pos_scheme, (void*)&pos_mode,
                     (void*)&sb, (void*)&nm, (void*)&mm, (void*)&perm, (void*)&mstart,
                     (void*)&mlen, (void*)&pos_out, (void*)&tok2macro, (void*)&status,
-                    (void*)&chunk_done};
+                    (void*)&chunk_done, (void*)&cluster};
     SLS_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)segment_grid_kernel, dim3(G), dim3(SEG_T),
                                              args, 0, stream));
     count_launch(1);

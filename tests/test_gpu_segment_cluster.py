@@ -1,0 +1,60 @@
+"""Clusters, exact-length adjustment and macro-tokens (Sec. 3.3-3.4) of one prompt
+at the edges of the cluster launch (from 4096 tokens) and of the cooperative grid
+above 262144, against the oracle: maps bit for bit.  Embeddings within 1e-4: a
+member sum adds 64 rows in order and then N / 64 partial sums, so its error per
+member is below (64 + N / 64) 2^-24 max |x| (N = 9001: 205 x 6e-8 x 5 = 6e-5; the
+larger N have at most a few hundred members in a macro-token).  The code distributions cover merging (more
+clusters than groups), the D'Hondt split with ties (fewer), one cluster, and
+macro-tokens of hundreds of work items."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+POS = {"max": 0, "median": 1, "mean": 2}
+
+
+@pytest.fixture(scope="module")
+def sls():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2607_19368_gb300 as m
+    m.lib()
+    return m
+
+
+def _codes(g, N, kind):
+    if kind == "one":
+        return np.full(N, 3, np.uint32)
+    if kind == "ties":                       # equal cluster sizes
+        return (np.arange(N) % 16).astype(np.uint32)
+    if kind == "few":                        # uneven, fewer than the groups
+        return np.minimum(g.zipf(1.3, N) - 1, 200).astype(np.uint32)
+    c = np.minimum(g.zipf(1.2, N) - 1, 60000).astype(np.uint32)   # many
+    return c ^ (g.integers(0, 2, N).astype(np.uint32) << 31 if kind == "wide" else 0)
+
+
+@pytest.mark.parametrize("N,d,M,kind,scheme", [
+    (1023, 40, 100, "many", "max"), (1024, 40, 100, "many", "median"),
+    (1025, 32, 300, "few", "mean"), (4095, 24, 1000, "ties", "max"),
+    (4096, 264, 17, "many", "max"), (8180, 2056, 511, "many", "max"),
+    (9001, 24, 4000, "few", "median"), (9001, 24, 5, "one", "max"),
+    (9001, 24, 900, "one", "mean"), (40000, 16, 2500, "wide", "mean"),
+    (262144, 8, 16384, "many", "max"), (262145, 8, 16384, "few", "max")])
+def test_aggregate_cluster_matches_oracle(sls, N, d, M, kind, scheme):
+    g = np.random.default_rng(N + M)
+    codes = _codes(g, N, kind)
+    X = g.standard_normal((N, d)).astype(np.float32)
+    groups = O.adjust_groups(O.bucket(codes), M)
+    order = O.order_groups(groups, getattr(O, "POS_" + scheme.upper()))
+    want = np.empty(N, dtype=np.int64)
+    for i, k in enumerate(order):
+        want[groups[k]] = i
+    Xt_o = O.aggregate_groups(X.astype(np.float64), [groups[k] for k in order])
+    Xt, pos, t2m = sls.aggregate(torch.from_numpy(X).cuda(),
+                                 torch.from_numpy(codes.view(np.int32)).cuda(), M, POS[scheme])
+    assert np.array_equal(t2m.cpu().numpy(), want)
+    assert float(np.max(np.abs(Xt.cpu().numpy() - Xt_o))) <= 1e-4
