@@ -1333,139 +1333,81 @@ __global__ void identity_kernel(const T* __restrict__ X, int64_t B, int64_t N, i
 // ============================================================================
 
 constexpr int AGG_T = 256;
-constexpr int AGG_CH = 64;      // members per work item
+constexpr int AGG_CH = 64;      // members per work item, at most
 
 // Work items: macro-token m is split into ceil(len / AGG_CH) items, listed in
-// macro order.  Three grid-wide passes: per-block totals over the macro
-// lengths; per macro its item offset, member-row offset, partial-sum slot and
-// (for macros spanning several items) its place in a compact list; then one
-// thread per item finds its macro by binary search over the increasing item
-// offsets, writes the item and, for each of the G member-pass CTAs whose
-// balanced row boundary falls inside the item, that CTA's first item.
-constexpr int AI_BLOCK = SEG_T;           // macros per block (one per thread)
-constexpr int AGG_MAX_GRID = 2048;        // member-pass CTAs at most
+// macro order.  One cluster of AI_CL CTAs: each thread takes a run of macros and
+// adds up its items, the partial-sum slots and the macros that span several
+// items; scans over the CTA and (through distributed shared memory) the cluster
+// turn the counts into offsets, and the thread writes its items.
+constexpr int AI_CL = 8;
 
-// Auxiliary integers of the aggregation: counts (16), block totals (4 per
-// block), CTA range starts (AGG_MAX_GRID + 1), multi-item macro list, and per
-// macro its first item and first member row.
+// Auxiliary integers of the aggregation: counts (16) and the multi-item macros.
 struct AggAux {
-  int* counts;  // [0] items, [1] partial slots, [2] multi-item macros, [3] member rows
-  int4* btot;
-  int* cta_first;
+  int* counts;  // [0] items, [1] partial slots, [2] multi-item macros
   int* multi;
-  int* it_start;
-  int* r_start;
 };
 
-__host__ __device__ inline int64_t agg_blocks(int64_t Mtot) { return (Mtot + AI_BLOCK - 1) / AI_BLOCK; }
-
-__host__ __device__ inline AggAux agg_aux(int* base, int64_t Mtot, int64_t Ntot) {
-  AggAux A;
-  A.counts = base;
-  A.btot = reinterpret_cast<int4*>(base + 16);
-  A.cta_first = base + 16 + 4 * agg_blocks(Mtot);
-  A.multi = A.cta_first + AGG_MAX_GRID + 1;
-  A.it_start = A.multi + Ntot / AGG_CH + 2;
-  A.r_start = A.it_start + Mtot;
-  return A;
-}
+__host__ __device__ inline AggAux agg_aux(int* base) { return AggAux{base, base + 16}; }
 
 SLS_DEV int nchunks(int len) { return (len + AGG_CH - 1) / AGG_CH; }
 
-__global__ void __launch_bounds__(SEG_T)
-agg_count_kernel(const int* __restrict__ mlen, int64_t Mtot, int64_t Ntot, int* __restrict__ aux) {
-  __shared__ int sh[SEG_W + 1];
-  const AggAux A = agg_aux(aux, Mtot, Ntot);
-  const int64_t m = (int64_t)blockIdx.x * AI_BLOCK + threadIdx.x;
-  const int len = (m < Mtot) ? mlen[m] : 0, nch = nchunks(len);
-  int t0, t1, t2, t3;
-  block_excl_scan<int>(nch, sh, &t0);
-  block_excl_scan<int>((nch > 1) ? nch : 0, sh, &t1);
-  block_excl_scan<int>((nch > 1) ? 1 : 0, sh, &t2);
-  block_excl_scan<int>(len, sh, &t3);
-  if (threadIdx.x == 0) A.btot[blockIdx.x] = make_int4(t0, t1, t2, t3);
+SLS_DEV uint32_t cluster_addr(const void* p, unsigned rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
 }
 
-__global__ void __launch_bounds__(SEG_T)
-agg_offsets_kernel(const int* __restrict__ mlen, int64_t Mtot, int64_t Ntot,
-                   int* __restrict__ aux, int* __restrict__ pt_start) {
+__global__ void __cluster_dims__(AI_CL, 1, 1) __launch_bounds__(SEG_T)
+agg_items_kernel(const int* __restrict__ mlen, int64_t Mtot, int* __restrict__ aux,
+                 int2* __restrict__ items, int* __restrict__ pt_start) {
   __shared__ int sh[SEG_W + 1];
-  const AggAux A = agg_aux(aux, Mtot, Ntot);
-  const int nb = (int)agg_blocks(Mtot);
-  // offsets of this block (sum over the blocks before it) and the totals
-  int b0 = 0, b1 = 0, b2 = 0, b3 = 0, a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-  for (int k = threadIdx.x; k < nb; k += SEG_T) {
-    const int4 v = A.btot[k];
-    if (k < (int)blockIdx.x) {
-      b0 += v.x;
-      b1 += v.y;
-      b2 += v.z;
-      b3 += v.w;
+  __shared__ int s_tot[3], s_pre[3];
+  const AggAux A = agg_aux(aux);
+  const int tid = threadIdx.x, rank = blockIdx.x;
+  const int64_t K = (Mtot + (int64_t)AI_CL * SEG_T - 1) / ((int64_t)AI_CL * SEG_T);
+  const int64_t b = min(Mtot, ((int64_t)rank * SEG_T + tid) * K), e = min(Mtot, b + K);
+  int c0 = 0, c1 = 0, c2 = 0;
+  for (int64_t m = b; m < e; ++m) {
+    const int nch = nchunks(mlen[m]);
+    c0 += nch;
+    c1 += nch > 1 ? nch : 0;
+    c2 += nch > 1 ? 1 : 0;
+  }
+  int t0, t1, t2;
+  int o0 = block_excl_scan<int>(c0, sh, &t0);
+  int o1 = block_excl_scan<int>(c1, sh, &t1);
+  int o2 = block_excl_scan<int>(c2, sh, &t2);
+  if (tid == 0) {
+    s_tot[0] = t0;
+    s_tot[1] = t1;
+    s_tot[2] = t2;
+  }
+  cluster_sync_all();
+  if (tid < 3) {
+    int pre = 0;
+    for (int r = 0; r < rank; ++r) {
+      int v;
+      asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v)
+                   : "r"(cluster_addr(&s_tot[tid], (unsigned)r)) : "memory");
+      pre += v;
     }
-    a0 += v.x;
-    a1 += v.y;
-    a2 += v.z;
-    a3 += v.w;
+    s_pre[tid] = pre;
+    if (rank == AI_CL - 1) A.counts[tid] = pre + s_tot[tid];
   }
-  int o0, o1, o2, o3, n0, n1, n2, n3;
-  block_excl_scan<int>(b0, sh, &o0);
-  block_excl_scan<int>(b1, sh, &o1);
-  block_excl_scan<int>(b2, sh, &o2);
-  block_excl_scan<int>(b3, sh, &o3);
-  block_excl_scan<int>(a0, sh, &n0);
-  block_excl_scan<int>(a1, sh, &n1);
-  block_excl_scan<int>(a2, sh, &n2);
-  block_excl_scan<int>(a3, sh, &n3);
-  const int64_t m = (int64_t)blockIdx.x * AI_BLOCK + threadIdx.x;
-  const int len = (m < Mtot) ? mlen[m] : 0, nch = nchunks(len);
-  int tt;
-  const int ito = o0 + block_excl_scan<int>(nch, sh, &tt);
-  const int pto = o1 + block_excl_scan<int>((nch > 1) ? nch : 0, sh, &tt);
-  const int muo = o2 + block_excl_scan<int>((nch > 1) ? 1 : 0, sh, &tt);
-  const int ro = o3 + block_excl_scan<int>(len, sh, &tt);
-  if (m < Mtot) {
-    A.it_start[m] = ito;
-    A.r_start[m] = ro;
-    pt_start[m] = (nch > 1) ? pto : -1;
-    if (nch > 1) A.multi[muo] = (int)m;
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    A.cta_first[0] = 0;
-    A.counts[0] = n0;
-    A.counts[1] = n1;
-    A.counts[2] = n2;
-    A.counts[3] = n3;
-  }
-}
-
-__global__ void __launch_bounds__(256)
-agg_fill_kernel(const int* __restrict__ mlen, int64_t Mtot, int64_t Ntot, int G,
-                int* __restrict__ aux, int2* __restrict__ items) {
-  const AggAux A = agg_aux(aux, Mtot, Ntot);
-  const int nitems = A.counts[0];
-  const int64_t rtot = A.counts[3];
-  // no items (every macro-token already written elsewhere): every CTA range
-  // is empty
-  if (nitems == 0 && blockIdx.x == 0)
-    for (int t = threadIdx.x; t <= G; t += blockDim.x) A.cta_first[t] = 0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nitems; i += gridDim.x * blockDim.x) {
-    // the macro of item i: the last m with it_start[m] <= i
-    int lo = 0, hi = (int)Mtot - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (A.it_start[mid] <= i)
-        lo = mid;
-      else
-        hi = mid - 1;
+  cluster_sync_all();  // s_pre is ready, and every CTA has read the totals
+  o0 += s_pre[0];
+  o1 += s_pre[1];
+  o2 += s_pre[2];
+  for (int64_t m = b; m < e; ++m) {
+    const int nch = nchunks(mlen[m]);
+    for (int c = 0; c < nch; ++c) items[o0 + c] = make_int2((int)m, c);
+    pt_start[m] = nch > 1 ? o1 : -1;
+    o0 += nch;
+    if (nch > 1) {
+      A.multi[o2++] = (int)m;
+      o1 += nch;
     }
-    const int m = lo, c = i - A.it_start[m], len = mlen[m];
-    items[i] = make_int2(m, c);
-    // CTA t starts at the first item whose first row is at or past
-    // t * rtot / G: the item after the last one starting before it
-    const int64_t rs = (int64_t)A.r_start[m] + (int64_t)c * AGG_CH;
-    const int64_t re = (int64_t)A.r_start[m] + min((int64_t)len, (int64_t)(c + 1) * AGG_CH);
-    const int64_t tlo = rs * G / rtot + 1, thi = re * G / rtot;
-    for (int64_t t = tlo; t <= thi && t <= G; ++t) A.cta_first[t] = i + 1;
   }
 }
 
@@ -1532,37 +1474,6 @@ SLS_DEV void store_row(const float (&acc)[NV * V], float scale, int d, float* __
   }
 }
 
-// Finalise one macro-token row from the member sum `acc` (per thread), the
-// member count and the sum of member norms: mean, then rescale to the mean
-// norm (Eq. macro_embed); a singleton is its token unchanged.
-template <int V, int NV>
-SLS_DEV void agg_finalize(float (&acc)[NV * V], int len, float eta_sum, int renorm, int d,
-                          float* __restrict__ out, float* sh) {
-  if (len == 1) {
-    store_row<V, NV>(acc, 1.0f, d, out);
-    return;
-  }
-  const int tid = threadIdx.x;
-  const float inv = 1.0f / (float)len;
-  float sq = 0.f;
-#pragma unroll
-  for (int q = 0; q < NV; ++q) {
-    const int c0 = (tid + q * AGG_T) * V;
-    if (c0 < d)
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        acc[q * V + v] *= inv;
-        sq = fmaf(acc[q * V + v], acc[q * V + v], sq);
-      }
-  }
-  float scale = 1.0f;
-  if (renorm) {
-    const float nrm = sqrtf(agg_block_sum(sq, sh));
-    if (nrm >= 1e-30f) scale = (eta_sum * inv) / nrm;
-  }
-  store_row<V, NV>(acc, scale, d, out);
-}
-
 // Member rows loaded per batch, so that about eight 16-byte loads per thread
 // are in flight.
 template <int NV>
@@ -1571,396 +1482,247 @@ constexpr int agg_batch() {
 }
 
 // The macro-tokens whose members span several items: sum their partial rows
-// and finalise (one CTA per macro-token of the compact list).
-template <int V, int NV>
-__global__ void __launch_bounds__(AGG_T)
+// and finalise (Eq. macro_embed), a cluster of AF_CL CTAs per macro-token of the
+// compact list, each CTA a slice of its columns with the rows split over its
+// threads; the slices' |sum|^2 meet through distributed shared memory.  Latency
+// bound: one CTA per macro-token summed a frequent token's sixty partial rows
+// four at a time (N = 32756, d = 3584: 38 -> 8 us).
+constexpr int AF_CL = 8;
+
+SLS_DEV float ld_cluster_f32(const float* p, unsigned rank) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr(p, rank)) : "memory");
+  return v;
+}
+
+__global__ void __cluster_dims__(AF_CL, 1, 1) __launch_bounds__(AGG_T)
 agg_final_kernel(int d, const int* __restrict__ mlen, const int* __restrict__ pt_start,
-                 int64_t Mtot, int64_t Ntot, int renorm, const int* __restrict__ aux,
-                 const float* __restrict__ part, const float* __restrict__ part_eta,
-                 float* __restrict__ Xt) {
+                 int renorm, const int* __restrict__ aux, const float* __restrict__ part,
+                 const float* __restrict__ part_eta, float* __restrict__ Xt) {
   __shared__ float sh[AGG_T / 32];
+  __shared__ float s_sq;
+  __shared__ float4 red[AGG_T];
   const int tid = threadIdx.x;
-  const AggAux A = agg_aux(const_cast<int*>(aux), Mtot, Ntot);
+  const AggAux A = agg_aux(const_cast<int*>(aux));
   const int nmulti = A.counts[2];
-  for (int t = blockIdx.x; t < nmulti; t += gridDim.x) {
+  const int rank = blockIdx.x % AF_CL;
+  const int wq = (d / 4 + AF_CL - 1) / AF_CL;          // float4 columns per slice (<= AGG_T)
+  const int q0 = rank * wq, nq = max(0, min(d / 4 - q0, wq));
+  const int RG = AGG_T / wq;                           // rows summed side by side
+  const int cq = tid % wq, rg = tid / wq;
+  for (int t = blockIdx.x / AF_CL; t < nmulti; t += gridDim.x / AF_CL) {
     const int64_t m = A.multi[t];
     const int ps = pt_start[m];
     const int len = mlen[m];
     const int nch = (len + AGG_CH - 1) / AGG_CH;
-    float acc[NV * V];
-#pragma unroll
-    for (int k = 0; k < NV * V; ++k) acc[k] = 0.f;
-    float eta = 0.f;
-    // AF_B partial rows in flight per thread (the chunks are independent)
-    constexpr int AF_B = (NV * V <= 16) ? 4 : 2;
-    for (int cb = 0; cb < nch; cb += AF_B) {
-      float4 buf[AF_B][NV * V / 4];
-#pragma unroll
-      for (int j = 0; j < AF_B; ++j) {
-        const float* src = part + (int64_t)(ps + cb + j) * d;
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
-          const int c0 = (tid + q * AGG_T) * V;
-#pragma unroll
-          for (int k = 0; k < V; k += 4) {
-            float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (cb + j < nch && c0 < d) f = *reinterpret_cast<const float4*>(src + c0 + k);
-            buf[j][(q * V + k) / 4] = f;
-          }
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < AF_B; ++j) {
-        if (cb + j < nch) eta += part_eta[ps + cb + j];
-#pragma unroll
-        for (int e = 0; e < NV * V / 4; ++e) {
-          acc[4 * e] += buf[j][e].x;
-          acc[4 * e + 1] += buf[j][e].y;
-          acc[4 * e + 2] += buf[j][e].z;
-          acc[4 * e + 3] += buf[j][e].w;
-        }
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (rg < RG && cq < nq) {
+      const float4* src = reinterpret_cast<const float4*>(part + (int64_t)ps * d) + q0 + cq;
+#pragma unroll 8
+      for (int c = rg; c < nch; c += RG) {
+        const float4 v = src[(int64_t)c * (d / 4)];
+        acc = make_float4(acc.x + v.x, acc.y + v.y, acc.z + v.z, acc.w + v.w);
       }
     }
-    agg_finalize<V, NV>(acc, len, eta, renorm, d, Xt + m * d, sh);
+    float eta = 0.f;
+    for (int c = tid; c < nch; c += AGG_T) eta += part_eta[ps + c];
+    red[tid] = acc;
+    eta = agg_block_sum(eta, sh);  // (its barriers also publish red)
+    float sq = 0.f;
+    if (rg == 0 && cq < nq) {
+      for (int g = 1; g < RG; ++g) {
+        const float4 v = red[g * wq + cq];
+        acc = make_float4(acc.x + v.x, acc.y + v.y, acc.z + v.z, acc.w + v.w);
+      }
+      const float inv = 1.0f / (float)len;
+      acc = make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv);
+      sq = fmaf(acc.x, acc.x, fmaf(acc.y, acc.y, fmaf(acc.z, acc.z, acc.w * acc.w)));
+    }
+    float scale = 1.0f;
+    if (renorm) {
+      sq = agg_block_sum(sq, sh);
+      if (tid == 0) s_sq = sq;
+      cluster_sync_all();
+      float tot = 0.f;
+      for (int r = 0; r < AF_CL; ++r) tot += ld_cluster_f32(&s_sq, (unsigned)r);
+      const float nrm = sqrtf(tot);
+      if (nrm >= 1e-30f) scale = (eta / (float)len) / nrm;
+      cluster_sync_all();  // every CTA has read the sums
+    }
+    if (rg == 0 && cq < nq)
+      store_vec4(Xt + m * d + 4 * (q0 + cq), acc.x * scale, acc.y * scale, acc.z * scale,
+                 acc.w * scale);
     __syncthreads();
   }
 }
 
-// ---------------------------------------------------------------------------
-// Member pass with a shared-memory row ring.  Warp 0 is the producer: it walks
-// this CTA's contiguous range of work items (balanced by member rows), loads each
-// item's descriptor and member ids one item ahead, and streams every member
-// row into an S-stage ring with one bulk async copy per row (mbarrier
-// complete_tx); the item descriptor travels with the item's first row.  Warps
-// 1..8 consume the rows in the same order: each consumer thread owns the
-// column groups c0 = (ct + q * 256) * V, sums them and the row's |x|^2, and
-// releases the stage.  At the end of an item the consumers meet at a named
-// barrier (which also ORs their failure flags), form the sum of member norms
-// and finalise the macro-token (Eq. macro_embed) or store a partial sum.
-// Every wait is bounded; a wait that gives up records SLS_ERR_TIMEOUT, the
-// other roles stop at their next check, and in-flight copies are drained.
-// ---------------------------------------------------------------------------
-
-constexpr int AGR_CW = 8;                    // consumer warps
-constexpr int AGR_CT = AGR_CW * 32;          // consumer threads
-constexpr int AGR_THREADS = AGR_CT + 32;     // + producer warp
-constexpr int AGR_MAX_STAGES = 16;
-constexpr int AGR_BAR = 1;                   // named barrier of the consumers
-
-struct AggDesc {
-  int m, c, n, len, ps, pad0, pad1, pad2;
-};
-
-SLS_DEV bool named_sync_or(unsigned id, unsigned nthreads, bool pred) {
-  unsigned r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n"
-      " bar.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r)
-      : "r"((unsigned)pred), "r"(id), "r"(nthreads)
-      : "memory");
-  return r != 0;
-}
-
+// Elements 2 p and 2 p + 1 of a 16-byte word of X as a packed pair.
 template <typename T>
-SLS_DEV void load_vec_smem(const T* p, float* out);
+SLS_DEV f32x2_t raw_pair(const uint4& r, int p);
 template <>
-SLS_DEV void load_vec_smem<float>(const float* p, float* out) {
-  const float4 v = *reinterpret_cast<const float4*>(p);
-  out[0] = v.x;
-  out[1] = v.y;
-  out[2] = v.z;
-  out[3] = v.w;
+SLS_DEV f32x2_t raw_pair<float>(const uint4& r, int p) {
+  return p == 0 ? pk2(__uint_as_float(r.x), __uint_as_float(r.y))
+                : pk2(__uint_as_float(r.z), __uint_as_float(r.w));
 }
 template <>
-SLS_DEV void load_vec_smem<uint16_t>(const uint16_t* p, float* out) {
-  const uint4 v = *reinterpret_cast<const uint4*>(p);
-  const unsigned w[4] = {v.x, v.y, v.z, v.w};
+SLS_DEV f32x2_t raw_pair<uint16_t>(const uint4& r, int p) {
+  const unsigned w = (p == 0) ? r.x : (p == 1) ? r.y : (p == 2) ? r.z : r.w;
+  return pk2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
+// Sums over the warp of R values per lane (R a power of two up to 8) by a
+// transposed butterfly: lane L gets the sum of value L / (32 / R).
+template <int R>
+SLS_DEV float warp_sums(float (&v)[R]) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    out[2 * k] = __uint_as_float(w[k] << 16);
-    out[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
-  }
-}
-
-// Bounded wait (about a second of clock cycles) that also returns early once
-// another role has aborted.  The producer polls without sleeping so that it
-// refills a stage as soon as it is released; the eight consumer warps back
-// off after a few polls so that their polling does not take the producer's
-// issue slots.
-template <bool BACKOFF>
-SLS_DEV bool agr_wait(uint64_t* bar, unsigned parity, volatile int* abort_flag) {
-  const long long t0 = clock64();
-  for (unsigned it = 0;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 63) == 63 && (*abort_flag || clock64() - t0 > SLS_WAIT_CYCLES)) return false;
-    if (BACKOFF && it > 64) __nanosleep(32);
-  }
-}
-
-// Descriptor of the local item kidx of this CTA (item i0 + kidx of its
-// contiguous range [i0, i1)), or an empty one past the end.
-struct LaneDesc {
-  int m, c, n, len, ps, off;
-};
-
-SLS_DEV LaneDesc agr_lane_desc(const int2* __restrict__ items, const int* __restrict__ mlen,
-                               const int* __restrict__ mstart, const int* __restrict__ pt_start,
-                               int i0, int i1, int kidx) {
-  LaneDesc L{0, 0, 0, 0, -1, 0};
-  const int it = i0 + kidx;
-  if (it < i1) {
-    const int2 item = items[it];
-    L.m = item.x;
-    L.c = item.y;
-    L.len = mlen[L.m];
-    L.n = min(L.len - L.c * AGG_CH, AGG_CH);
-    L.ps = pt_start[L.m];
-    L.off = mstart[L.m] + L.c * AGG_CH;
-  }
-  return L;
-}
-
-// Member row f (flattened over the 32 items of a batch whose inclusive row
-// prefix is `pre`): its item j, index s inside the item and token row id.
-SLS_DEV void agr_fetch_row(const int* __restrict__ perm, int pre, int nrows, int off, int f0,
-                           int lane, int& rid, int& rj, int& rs) {
-  const int f = f0 + lane;
-  int j = 0;
+  for (int s = 0; s < 5; ++s) {
+    const int h = 16 >> s;
+    const int nv = (R >> s) > 1 ? (R >> s) : 1;
+    if (nv > 1) {
+      const bool up = (lane & h) != 0;
 #pragma unroll
-  for (int step = 16; step >= 1; step >>= 1) {
-    const int pv = __shfl_sync(0xffffffffu, pre, j + step - 1);
-    if (pv <= f) j += step;
+      for (int i = 0; i < nv / 2; ++i) {
+        const float send = up ? v[i] : v[i + nv / 2];
+        const float keep = up ? v[i + nv / 2] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], h);
+    }
   }
-  j = min(j, 31);
-  const int base = __shfl_sync(0xffffffffu, pre, j > 0 ? j - 1 : 0);
-  const int off_j = __shfl_sync(0xffffffffu, off, j);
-  rs = f - (j > 0 ? base : 0);
-  rj = j;
-  rid = (f < nrows) ? perm[off_j + rs] : 0;
+  return v[0];
 }
+
+// ---------------------------------------------------------------------------
+// Member pass: a CTA per work item, its member rows by plain 16-byte loads in
+// batches of MB rows per thread (about eight loads in flight each).  A thread
+// owns the column groups c0 = (tid + q * AGG_T) * V, sums them and the rows'
+// |x|^2 on packed pairs; one barrier per item publishes the row norms and the
+// sum's own, and every thread finalises its columns of the macro-token (Eq.
+// macro_embed) or stores them as a partial sum.
+//
+// Bound by reading X: four or more CTAs per SM keep 100 KB of rows in flight, and
+// an item's chain of descriptor, member ids and rows hides behind the others'.
+// The former pass streamed each row through a shared-memory ring with one bulk
+// copy per row; issuing those took a producer warp about 1000 cycles per row
+// (N = 32756, d = 3584: 90 -> 58 us, against 35 us for the bytes; N = 8180,
+// d = 4096: 43 -> 29).
+// ---------------------------------------------------------------------------
 
 template <typename T, int NV>
-__global__ void __launch_bounds__(AGR_THREADS, 2)
-agg_ring_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __restrict__ perm,
-                const int* __restrict__ mstart, const int* __restrict__ mlen,
-                const int2* __restrict__ items, const int* __restrict__ cta_first,
-                const int* __restrict__ pt_start, int renorm, float* __restrict__ Xt,
-                float* __restrict__ part, float* __restrict__ part_eta, int S, int stage_bytes,
-                int* status, int64_t ntot) {
+__global__ void __launch_bounds__(AGG_T, NV <= 2 ? 4 : 2)
+agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __restrict__ perm,
+                  const int* __restrict__ mstart, const int* __restrict__ mlen,
+                  const int2* __restrict__ items, const int* __restrict__ aux,
+                  const int* __restrict__ pt_start, int renorm, float* __restrict__ Xt,
+                  float* __restrict__ part, float* __restrict__ part_eta, int* status,
+                  int64_t ntot) {
   constexpr int V = VecOf<T>::V;
-  extern __shared__ __align__(128) unsigned char agr_smem[];
+  constexpr int PN = NV * V / 2;  // element pairs per thread
+  constexpr int MB = agg_batch<NV>();
+  constexpr int NW = AGG_T / 32, LPR = 32 / MB;
+  __shared__ float shq[2][AGG_CH][NW];  // row |x|^2 by warp
+  __shared__ float shm[2][NW];          // |member sum|^2 by warp
+  (void)status;
   (void)ntot;  // bounds of the member rows (debug-build checks)
-  __shared__ uint64_t fullb[AGR_MAX_STAGES], emptyb[AGR_MAX_STAGES];
-  __shared__ AggDesc dring[AGR_MAX_STAGES + 2];
-  __shared__ float shq[2][AGR_CW][AGG_CH];
-  __shared__ float shm[2][AGR_CW];  // per-warp |member sum|^2 of the item
-  __shared__ volatile int s_abort;
-  const int DQ = S + 2;
-  const int i0 = cta_first[blockIdx.x], i1 = cta_first[blockIdx.x + 1];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned row_bytes = (unsigned)d * sizeof(T);
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < S; ++s) {
-      mbar_init(&fullb[s], 1);
-      mbar_init(&emptyb[s], AGR_CW);
-    }
-    mbar_fence_init();
-    s_abort = 0;
-  }
-  __syncthreads();
-
-  if (warp == 0) {
-    // ------------------------------ producer ------------------------------
-    // Lane j holds the descriptor of local item kb + j; the member ids of the
-    // batch are fetched 32 rows at a time, one chunk ahead of the copies.
-    const uint64_t pol = l2_policy_evict_first();
-    const int GP = S / 2 < 8 ? (S / 2 < 1 ? 1 : S / 2) : 8;  // rows issued together
-    unsigned issued = 0;
-    bool ok = true;
-    int kb = 0;
-    LaneDesc cd = agr_lane_desc(items, mlen, mstart, pt_start, i0, i1, kb + lane);
-    while (ok) {
-      int pre = cd.n;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nitems = agg_aux(const_cast<int*>(aux)).counts[0];
+  int buf = 0;
+  for (int it = blockIdx.x; it < nitems; it += gridDim.x, buf ^= 1) {
+    const int2 item = items[it];
+    const int m = item.x, c = item.y;
+    const int len = mlen[m], ps = pt_start[m];
+    const int n = min(len - c * AGG_CH, AGG_CH);
+    const int* ids = perm + mstart[m] + c * AGG_CH;
+    f32x2_t acc[PN];
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, pre, o);
-        if (lane >= o) pre += t;
-      }
-      const int nrows = __shfl_sync(0xffffffffu, pre, 31);
-      if (nrows == 0) break;
-      const LaneDesc nd = agr_lane_desc(items, mlen, mstart, pt_start, i0, i1, kb + 32 + lane);
-      int rid, rj, rs;
-      agr_fetch_row(perm, pre, nrows, cd.off, 0, lane, rid, rj, rs);
-      for (int f0 = 0; f0 < nrows && ok; f0 += 32) {
-        int nrid = 0, nrj = 0, nrs = 0;
-        if (f0 + 32 < nrows) agr_fetch_row(perm, pre, nrows, cd.off, f0 + 32, lane, nrid, nrj, nrs);
-        const int cnt = min(32, nrows - f0);
-        // rows g0 .. g0 + GP - 1 of the batch go out together, one per lane:
-        // each lane waits for its own ring stage, then issues its copy (a
-        // thread issuing a bulk copy is held for a few hundred cycles, so
-        // one lane issuing every row made the producer the bottleneck)
-        for (int g0 = 0; g0 < cnt; g0 += GP) {
-          const int gn = min(GP, cnt - g0);
-          const bool act = lane < gn;
-          const int row = __shfl_sync(0xffffffffu, rid, (g0 + lane) & 31);
-          const int j = __shfl_sync(0xffffffffu, rj, (g0 + lane) & 31);
-          const int s = __shfl_sync(0xffffffffu, rs, (g0 + lane) & 31);
-          AggDesc D;
-          D.m = __shfl_sync(0xffffffffu, cd.m, j);
-          D.c = __shfl_sync(0xffffffffu, cd.c, j);
-          D.n = __shfl_sync(0xffffffffu, cd.n, j);
-          D.len = __shfl_sync(0xffffffffu, cd.len, j);
-          D.ps = __shfl_sync(0xffffffffu, cd.ps, j);
-          D.pad0 = D.pad1 = D.pad2 = 0;
-          const unsigned mine = issued + (unsigned)lane;
-          const int st = (int)(mine % (unsigned)S);
-          const unsigned par = (mine / (unsigned)S) & 1u;
-          bool w_ok = true;
-          if (act) w_ok = agr_wait<false>(&emptyb[st], par ^ 1u, &s_abort);
-          if (!__all_sync(0xffffffffu, w_ok)) {
-            ok = false;
-            if (lane == 0) {
-              s_abort = 1;
-              atomicExch(status, SLS_ERR_TIMEOUT);
-            }
-            break;
-          }
-          if (act) {
-            if (s == 0) dring[(kb + j) % DQ] = D;
-            unsigned char* dst = agr_smem + (size_t)st * stage_bytes;
-            mbar_expect_tx(&fullb[st], row_bytes);
-            int64_t src_row = row;
+    for (int e = 0; e < PN; ++e) acc[e] = 0ull;
+    int id = 0;
+    for (int s = 0; s < n; s += MB) {
+      if ((s & 31) == 0) id = s + lane < n ? ids[s + lane] : 0;  // MB divides 32
+      uint4 raw[MB][NV];
+#pragma unroll
+      for (int j = 0; j < MB; ++j) {
+        int64_t row = __shfl_sync(0xffffffffu, id, (s + j) & 31);
 #ifdef SLS_DEBUG
-            // a member row outside the token set is not fetched: the stage
-            // gets row 0 instead and the status records SLS_ERR_BOUNDS
-            if (!(row >= 0 && (int64_t)row < ntot)) {
-              atomicExch(status, SLS_ERR_BOUNDS);
-              src_row = 0;
-            }
+        // a member row outside the token set is not read: row 0 instead, and
+        // the status records SLS_ERR_BOUNDS
+        if (!(row >= 0 && row < ntot)) {
+          atomicExch(status, SLS_ERR_BOUNDS);
+          row = 0;
+        }
 #endif
-            bulk_g2s(dst, X + src_row * ldx, row_bytes, &fullb[st], pol);
-          }
-          issued += (unsigned)gn;
+        const T* x = X + row * ldx;
+#pragma unroll
+        for (int q = 0; q < NV; ++q) {
+          const int c0 = (tid + q * AGG_T) * V;
+          raw[j][q] = make_uint4(0u, 0u, 0u, 0u);
+          if (s + j < n && c0 < d) raw[j][q] = __ldcs(reinterpret_cast<const uint4*>(x + c0));
         }
-        rid = nrid;
-        rj = nrj;
-        rs = nrs;
       }
-      kb += 32;
-      cd = nd;
+      float sq[MB];
+#pragma unroll
+      for (int j = 0; j < MB; ++j) {
+        f32x2_t q2 = 0ull;
+#pragma unroll
+        for (int e = 0; e < PN; ++e) {
+          const f32x2_t x = raw_pair<T>(raw[j][e / (V / 2)], e % (V / 2));
+          acc[e] = add2(acc[e], x);
+          q2 = fma2(x, x, q2);
+        }
+        float qa, qb;
+        upk2(q2, qa, qb);
+        sq[j] = qa + qb;
+      }
+      const float t = warp_sums<MB>(sq);
+      if (lane % LPR == 0 && s + lane / LPR < n) shq[buf][s + lane / LPR][warp] = t;
     }
-    // every issued copy has landed before the CTA may exit
-    if (lane == 0) {
-      const unsigned first = issued > (unsigned)S ? issued - (unsigned)S : 0u;
-      for (unsigned c = first; c < issued; ++c) {
-        for (unsigned w = 0; w < (1u << 25); ++w) {
-          if (mbar_try_wait(&fullb[c % (unsigned)S], (c / (unsigned)S) & 1u)) break;
-          __nanosleep(32);
-        }
-      }
+    float v[NV * V];
+    float msq = 0.f;
+#pragma unroll
+    for (int e = 0; e < PN; ++e) {
+      upk2(acc[e], v[2 * e], v[2 * e + 1]);
+      msq = fmaf(v[2 * e], v[2 * e], msq);
+      msq = fmaf(v[2 * e + 1], v[2 * e + 1], msq);
     }
-  } else {
-    // ------------------------------ consumers -----------------------------
-    const int cw = warp - 1, ct = threadIdx.x - 32;
-    unsigned consumed = 0;
-    bool ok = true;
-    int k = 0;
-    for (int it = i0; it < i1; ++it, ++k) {
-      float acc[NV * V];
+    msq = warp_sum_f(msq);
+    if (lane == 0) shm[buf][warp] = msq;
+    __syncthreads();
+    // sum of member norms (every warp forms the same total)
+    float eta = 0.f;
 #pragma unroll
-      for (int e = 0; e < NV * V; ++e) acc[e] = 0.f;
-      AggDesc D{};
-      D.n = 1;
-      float* q = &shq[k & 1][cw][0];
-      for (int s = 0; s < D.n && ok; ++s) {
-        const int st = (int)(consumed % (unsigned)S);
-        const unsigned par = (consumed / (unsigned)S) & 1u;
-        if (!agr_wait<true>(&fullb[st], par, &s_abort)) {
-          ok = false;
-          if (lane == 0) {
-            s_abort = 1;
-            atomicExch(status, SLS_ERR_TIMEOUT);
-          }
-          break;
-        }
-        if (s == 0) D = dring[k % DQ];
-        const T* rowp = reinterpret_cast<const T*>(agr_smem + (size_t)st * stage_bytes);
-        float sq = 0.f;
+    for (int h = 0; h < AGG_CH / 32; ++h) {
+      const int r = lane + 32 * h;
+      if (r < n) {
+        float t = 0.f;
 #pragma unroll
-        for (int qv = 0; qv < NV; ++qv) {
-          const int c0 = (ct + qv * AGR_CT) * V;
-          if (c0 < d) {
-            float v[V];
-            load_vec_smem<T>(rowp + c0, v);
-#pragma unroll
-            for (int e = 0; e < V; ++e) {
-              acc[qv * V + e] += v[e];
-              sq = fmaf(v[e], v[e], sq);
-            }
-          }
-        }
-        sq = warp_sum_f(sq);
-        __syncwarp();
-        if (lane == 0) {
-          q[s] = sq;
-          mbar_arrive(&emptyb[st]);
-        }
-        ++consumed;
-      }
-      // this warp's share of |sum of the members|^2, published with the
-      // item-end barrier (the renorm needs no barrier of its own)
-      {
-        float msq = 0.f;
-#pragma unroll
-        for (int e = 0; e < NV * V; ++e) msq = fmaf(acc[e], acc[e], msq);
-        msq = warp_sum_f(msq);
-        if (lane == 0) shm[k & 1][cw] = msq;
-      }
-      if (named_sync_or(AGR_BAR, AGR_CT, !ok)) break;
-      // sum of member norms (every warp forms the same total)
-      float eta = 0.f;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int s = lane + 32 * h;
-        if (s < D.n) {
-          float t = 0.f;
-#pragma unroll
-          for (int w = 0; w < AGR_CW; ++w) t += shq[k & 1][w][s];
-          eta += sqrtf(t);
-        }
-      }
-      eta = warp_sum_f(eta);
-      float scale = 1.0f;
-      float* dst;
-      if (D.ps < 0) {
-        dst = Xt + (int64_t)D.m * d;
-        if (D.len > 1) {
-          // mean = sum / len, rescaled to the mean member norm
-          const float inv = 1.0f / (float)D.len;
-          scale = inv;
-          if (renorm) {
-            float tot = 0.f;
-#pragma unroll
-            for (int w = 0; w < AGR_CW; ++w) tot += shm[k & 1][w];
-            const float nrm = sqrtf(tot) * inv;
-            if (nrm >= 1e-30f) scale = inv * ((eta * inv) / nrm);
-          }
-        }
-      } else {
-        dst = part + (int64_t)(D.ps + D.c) * d;
-        if (ct == 0) part_eta[D.ps + D.c] = eta;
-      }
-#pragma unroll
-      for (int qv = 0; qv < NV; ++qv) {
-        const int c0 = (ct + qv * AGR_CT) * V;
-        if (c0 < d)
-#pragma unroll
-          for (int e = 0; e < V; e += 4)
-            store_vec4(dst + c0 + e, acc[qv * V + e] * scale, acc[qv * V + e + 1] * scale,
-                       acc[qv * V + e + 2] * scale, acc[qv * V + e + 3] * scale);
+        for (int w = 0; w < NW; ++w) t += shq[buf][r][w];
+        eta += sqrtf(t);
       }
     }
+    eta = warp_sum_f(eta);
+    float scale = 1.0f;
+    float* dst;
+    if (ps < 0) {
+      dst = Xt + (int64_t)m * d;
+      if (len > 1) {
+        // mean = sum / len, rescaled to the mean member norm
+        const float inv = 1.0f / (float)len;
+        scale = inv;
+        if (renorm) {
+          float tot = 0.f;
+#pragma unroll
+          for (int w = 0; w < NW; ++w) tot += shm[buf][w];
+          const float nrm = sqrtf(tot) * inv;
+          if (nrm >= 1e-30f) scale = inv * ((eta * inv) / nrm);
+        }
+      }
+    } else {
+      dst = part + (int64_t)(ps + c) * d;
+      if (tid == 0) part_eta[ps + c] = eta;
+    }
+    store_row<V, NV>(v, scale, d, dst);
   }
 }
 
@@ -2091,44 +1853,6 @@ __host__ __device__ inline int chunk_nparts(int n, int m) {
 // the last holds at least SCORE_PR / 2 rows
 __host__ __device__ inline int chunk_parts_max(int64_t nmax) {
   return (int)((nmax + SCORE_PR / 2 - 1) / (SCORE_PR / 2));
-}
-
-// Elements 2 p and 2 p + 1 of a 16-byte word of X as a packed pair.
-template <typename T>
-SLS_DEV f32x2_t raw_pair(const uint4& r, int p);
-template <>
-SLS_DEV f32x2_t raw_pair<float>(const uint4& r, int p) {
-  return p == 0 ? pk2(__uint_as_float(r.x), __uint_as_float(r.y))
-                : pk2(__uint_as_float(r.z), __uint_as_float(r.w));
-}
-template <>
-SLS_DEV f32x2_t raw_pair<uint16_t>(const uint4& r, int p) {
-  const unsigned w = (p == 0) ? r.x : (p == 1) ? r.y : (p == 2) ? r.z : r.w;
-  return pk2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-}
-
-// Sums over the warp of R values per lane (R a power of two up to 8) by a
-// transposed butterfly: lane L gets the sum of value L / (32 / R).
-template <int R>
-SLS_DEV float warp_sums(float (&v)[R]) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int s = 0; s < 5; ++s) {
-    const int h = 16 >> s;
-    const int nv = (R >> s) > 1 ? (R >> s) : 1;
-    if (nv > 1) {
-      const bool up = (lane & h) != 0;
-#pragma unroll
-      for (int i = 0; i < nv / 2; ++i) {
-        const float send = up ? v[i] : v[i + nv / 2];
-        const float keep = up ? v[i + nv / 2] : v[i];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
-      }
-    } else {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], h);
-    }
-  }
-  return v[0];
 }
 
 // 16-byte asynchronous copy global -> shared (zero-filled when !live), and
@@ -2550,7 +2274,8 @@ int launch_identity(const void* X, int x_dtype, int64_t B, int64_t N, int d, int
 
 size_t agg_item_capacity(int64_t Mtot, int64_t Ntot) { return (size_t)(Mtot + Ntot / AGG_CH + 2); }
 size_t agg_aux_ints(int64_t Mtot, int64_t Ntot) {
-  return (size_t)(16 + 4 * agg_blocks(Mtot) + (AGG_MAX_GRID + 1) + Ntot / AGG_CH + 2 + 2 * Mtot);
+  (void)Mtot;
+  return (size_t)(16 + Ntot / AGG_CH + 2);
 }
 size_t agg_part_capacity(int64_t Ntot) { return (size_t)(2 * (Ntot / AGG_CH) + 2); }
 
@@ -2561,47 +2286,25 @@ int launch_agg_t(const void* X, int d, int64_t ldx, const int* perm, const int* 
                  float* Xt,
                  int* pt_start, int2* items, int* aux, float* part, float* part_eta,
                  int* status, cudaStream_t stream) {
-  constexpr int V = VecOf<T>::V;
-  const int stage = (int)(((size_t)d * sizeof(T) + 127) & ~(size_t)127);
-  // two CTAs per SM when each still gets at least 6 ring stages in ~100 KB
-  int per_sm = 2;
-  int S = (100 * 1024) / stage;
-  if (S < 6) {
-    per_sm = 1;
-    S = (200 * 1024) / stage;
-  }
-  if (S > AGR_MAX_STAGES) S = AGR_MAX_STAGES;
-  if (S < 2) return SLS_ERR_UNSUPPORTED;
-  const size_t smem = (size_t)S * stage;
-  SLS_CUDA_TRY(cudaFuncSetAttribute(agg_ring_kernel<T, NV>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int occ = 0;
-  SLS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, agg_ring_kernel<T, NV>,
-                                                             AGR_THREADS, smem));
-  if (occ < 1) return SLS_ERR_UNSUPPORTED;
-  if (occ < per_sm) per_sm = occ;
   int dev = 0, sms = 0;
   SLS_CUDA_TRY(cudaGetDevice(&dev));
   SLS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  int grid = sms * per_sm;
-  if (grid > AGG_MAX_GRID) grid = AGG_MAX_GRID;
-  // work items, partial slots and the balanced CTA ranges
-  const unsigned nb = (unsigned)agg_blocks(Mtot);
-  agg_count_kernel<<<nb, SEG_T, 0, stream>>>(mlen, Mtot, Ntot, aux);
+  agg_items_kernel<<<AI_CL, SEG_T, 0, stream>>>(mlen, Mtot, aux, items, pt_start);
   SLS_LAUNCH_CHECK();
-  agg_offsets_kernel<<<nb, SEG_T, 0, stream>>>(mlen, Mtot, Ntot, aux, pt_start);
+  // CTAs that fit the GPU at once (NV <= 2: four per SM), each every grid-th item
+  int occ = 0;
+  SLS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, agg_member_kernel<T, NV>,
+                                                             AGG_T, 0));
+  int64_t grid = (int64_t)sms * (occ < 1 ? 1 : occ);
+  const int64_t most = Mtot + Ntot / AGG_CH;  // items at most
+  if (grid > most) grid = most;
+  agg_member_kernel<T, NV><<<(unsigned)grid, AGG_T, 0, stream>>>(
+      (const T*)X, d, ldx, perm, mstart, mlen, items, aux, pt_start, renorm, Xt, part, part_eta,
+      status, Ntot);
   SLS_LAUNCH_CHECK();
-  int64_t fill = (Mtot + Ntot / AGG_CH + 255) / 256;
-  if (fill > 8 * (int64_t)sms) fill = 8 * (int64_t)sms;
-  agg_fill_kernel<<<(unsigned)fill, 256, 0, stream>>>(mlen, Mtot, Ntot, grid, aux, items);
-  SLS_LAUNCH_CHECK();
-  const AggAux A = agg_aux(aux, Mtot, Ntot);
-  agg_ring_kernel<T, NV><<<grid, AGR_THREADS, smem, stream>>>(
-      (const T*)X, d, ldx, perm, mstart, mlen, items, A.cta_first, pt_start, renorm, Xt, part,
-      part_eta, S, stage, status, Ntot);
-  SLS_LAUNCH_CHECK();
-  agg_final_kernel<V, NV><<<(unsigned)fblocks, AGG_T, 0, stream>>>(
-      d, mlen, pt_start, Mtot, Ntot, renorm, aux, part, part_eta, Xt);
+  const int64_t clusters = fblocks < 64 ? fblocks : 64;
+  agg_final_kernel<<<(unsigned)(clusters * AF_CL), AGG_T, 0, stream>>>(
+      d, mlen, pt_start, renorm, aux, part, part_eta, Xt);
   SLS_LAUNCH_CHECK();
   return SLS_OK;
 }
@@ -2613,7 +2316,7 @@ int launch_agg_dtype(const void* X, int d, int64_t ldx, const int* perm, const i
                      int* pt_start, int2* items, int* aux, float* part, float* part_eta,
                      int* status, cudaStream_t stream) {
   constexpr int V = VecOf<T>::V;
-  const int nv = (d / V + AGR_CT - 1) / AGR_CT;
+  const int nv = (d / V + AGG_T - 1) / AGG_T;
 #define SLS_AGG_NV(N)                                                                       \
   return launch_agg_t<T, N>(X, d, ldx, perm, mstart, mlen, Mtot, Ntot, fblocks, renorm, Xt, \
                             pt_start, items, aux, part, part_eta, status, stream)
