@@ -198,6 +198,11 @@ SLS_DEV bool fm_tile_live(const FmJob& J, int b, int mb) {
   return false;
 }
 
+// Live tiles of a CTA (its i-th tile is blockIdx.x + i gridDim.x) as a bit mask
+// in shared memory, filled by all threads at once: every role walked the route
+// table by itself before, a dependent load per tile (21 us for 8192 dead tiles).
+constexpr int TC_MASK_TILES = 4096;
+
 // Four consecutive bfloat16 features, rounded to nearest even: one 8-byte
 // store.
 SLS_DEV void store4(uint16_t* p, float4 o) {
@@ -218,6 +223,7 @@ feature_map_tc_kernel(const __grid_constant__ CUtensorMap tmX,
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ uint64_t full_bar[TC_STAGES], empty_bar[TC_STAGES], tfull[2], tempty[2], done_bar;
   __shared__ uint32_t tmem_holder;
+  __shared__ uint32_t s_live[TC_MASK_TILES / 32];
   __shared__ volatile int s_abort;
 
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -243,6 +249,22 @@ feature_map_tc_kernel(const __grid_constant__ CUtensorMap tmX,
     mbar_fence_init();
     s_abort = 0;
   }
+  if (J.live) {
+    const int mine = (num_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    for (int i0 = 32 * warp; i0 < min(mine, TC_MASK_TILES); i0 += TC_THREADS) {
+      const int tile = blockIdx.x + (i0 + lane) * gridDim.x;
+      const bool live =
+          tile < num_tiles && fm_tile_live(J, tile / per_prompt, (tile % per_prompt) / n_tiles);
+      const unsigned m = __ballot_sync(0xffffffffu, live);
+      if (lane == 0) s_live[i0 / 32] = m;
+    }
+  }
+  // whether the CTA's i-th tile is computed
+  auto tile_live = [&](int i, int tile) {
+    if (!J.live) return true;
+    if (i < TC_MASK_TILES) return (s_live[i >> 5] >> (i & 31) & 1u) != 0u;
+    return fm_tile_live(J, tile / per_prompt, (tile % per_prompt) / n_tiles);
+  };
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_holder)),
@@ -265,10 +287,11 @@ feature_map_tc_kernel(const __grid_constant__ CUtensorMap tmX,
     if (lane == 0) {
       unsigned it = 0;
       bool ok = true;
+      int i = -1;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+        if (!tile_live(++i, tile)) continue;
         const int pb = tile / per_prompt, rem = tile % per_prompt;
         const int mb = rem / n_tiles, nb = rem % n_tiles;
-        if (!fm_tile_live(J, pb, mb)) continue;
         const int y = pb * J.x_stride + mb * TC_BM;
         for (int kb = 0; kb < k_blocks; ++kb, ++it) {
           const int s = it % TC_STAGES;
@@ -299,8 +322,9 @@ feature_map_tc_kernel(const __grid_constant__ CUtensorMap tmX,
     if (lane == 0) {
       unsigned it = 0, acc_it = 0;
       bool ok = true;
+      int i = -1;
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-        if (!fm_tile_live(J, tile / per_prompt, (tile % per_prompt) / n_tiles)) continue;
+        if (!tile_live(++i, tile)) continue;
         const int acc = acc_it & 1;
         const unsigned apar = (acc_it >> 1) & 1u;
         if (!tc_wait(&tempty[acc], apar ^ 1u, &s_abort)) {
@@ -346,10 +370,11 @@ feature_map_tc_kernel(const __grid_constant__ CUtensorMap tmX,
                           (uint32_t)((warp - 2) * 2 * TC_OUT_BYTES);
     unsigned char* stg0p = smem + TC_STAGES * TC_STAGE_BYTES + (warp - 2) * 2 * TC_OUT_BYTES;
     unsigned acc_it = 0, blk = 0;
+    int i = -1;
     for (int tile = blockIdx.x; tile < num_tiles; tile += gridDim.x) {
+      if (!tile_live(++i, tile)) continue;
       const int pb = tile / per_prompt, rem = tile % per_prompt;
       const int mb = rem / n_tiles, nb = rem % n_tiles;
-      if (!fm_tile_live(J, pb, mb)) continue;
       const int acc = acc_it & 1;
       const unsigned apar = (acc_it >> 1) & 1u;
       if (!tc_wait(&tfull[acc], apar, &s_abort)) {
