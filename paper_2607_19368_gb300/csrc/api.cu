@@ -335,7 +335,7 @@ struct CompressWs {
   int64_t* lz_q1off;
   int* nspec;
   float* score;
-  float* score_part;  // window-score partial sums (adaptive backend)
+  float* score_part;  // window-score sums of short windows (adaptive backend)
   float2* norm_scratch;  // row-normalised operator: column sums
   int32_t* route;  // spectral flag per problem
   void* Phi;  // float32, or bfloat16 bits when the plan stores Phi as bf16
@@ -488,7 +488,7 @@ size_t tail_bytes(const CompressPlan& P, int64_t toks, int d, int backend) {
   Carver cv(nullptr);
   cv.take<float>(agg_part_capacity(toks) * (size_t)d);
   cv.take<float>(agg_part_capacity(toks));
-  if (backend == SLS_BACKEND_ADAPTIVE) cv.take<float>(score_part_floats(P.nprob, P.nmax, d));
+  if (backend == SLS_BACKEND_ADAPTIVE) cv.take<float>(score_part_floats(P.nprob, toks, d));
   return cv.off;
 }
 
@@ -872,7 +872,7 @@ int sls_compress(const sls_config_t* cfg, const void* X, int x_dtype, int64_t B,
     W.part = tail.take<float>(agg_part_capacity(B * N) * (size_t)d);
     W.part_eta = tail.take<float>(agg_part_capacity(B * N));
     W.score_part = (cfg->backend == SLS_BACKEND_ADAPTIVE)
-                       ? tail.take<float>(score_part_floats(P.nprob, P.nmax, d))
+                       ? tail.take<float>(score_part_floats(P.nprob, B * N, d))
                        : nullptr;
     W.tail = tail;
   }
@@ -900,9 +900,9 @@ int sls_compress(const sls_config_t* cfg, const void* X, int x_dtype, int64_t B,
     // below rho = 16 the score pass also writes every window's chunk-path
     // output, so the segment and aggregation steps only see spectral windows
     if (cfg->rho < 16.0 &&
-        (st = launch_window_score_chunk(X, x_dtype, d, ldx, W.probs, nprob, P.nmax,
-                                        W.score_part, W.score, cfg->pos_scheme, cfg->pos_mode,
-                                        cfg->renorm, Xt, pos, tok2macro, s)) != SLS_OK)
+        (st = launch_window_score_chunk(X, x_dtype, d, ldx, W.probs, nprob, P.nmax, P.mmax, B * N,
+                                        W.part, W.score_part, W.score, cfg->pos_scheme,
+                                        cfg->pos_mode, cfg->renorm, Xt, pos, tok2macro, s)) != SLS_OK)
       return st;
   }
   double tau = cfg->tau;

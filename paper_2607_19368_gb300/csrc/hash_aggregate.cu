@@ -1732,94 +1732,10 @@ agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __rest
 
 // score = (1/L) sum_i cos(x_i, c) with c the window centroid; computed in one
 // pass over X as (sum_i x_i/|x_i|) . (sum_i x_i) / (L |sum_i x_i|).  Zero rows
-// add 0.  Every window is cut into parts of SCORE_PR rows (so that a batch of
-// windows spreads evenly over the SMs); a CTA takes a part at a time, gathers
-// its rows in batches of agg_batch<NV>(), reduces each row's |x|^2 from the
-// same registers (per warp, then across warps through a double-buffered
-// shared array, one barrier per batch) and writes the part's sums of x and of
-// x/|x|; window_score_combine_kernel adds a window's parts and forms the
-// score.
-constexpr int SCORE_PR = 512;  // rows per part
-
-__host__ __device__ inline int score_parts(int64_t nmax) {
-  return (int)((nmax + SCORE_PR - 1) / SCORE_PR);
-}
-
-template <typename T, int NV>
-__global__ void __launch_bounds__(AGG_T, 2)
-window_score_kernel(const T* __restrict__ X, int d, int64_t ldx,
-                    const ProbDesc* __restrict__ probs, int nprob, int KP,
-                    float* __restrict__ part) {
-  constexpr int V = VecOf<T>::V;
-  constexpr int MB = agg_batch<NV>();
-  constexpr int NW = AGG_T / 32;
-  __shared__ float shq[2][MB][NW];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int units = nprob * KP;
-  for (int u = blockIdx.x; u < units; u += gridDim.x) {
-    const int p = u / KP, k = u % KP;
-    const ProbDesc P = probs[p];
-    const int r0 = min(P.n, k * SCORE_PR), r1 = min(P.n, r0 + SCORE_PR);
-    if (r0 >= r1) continue;
-    float cs[NV * V], ns[NV * V];
-#pragma unroll
-    for (int e = 0; e < NV * V; ++e) cs[e] = ns[e] = 0.f;
-    int buf = 0;
-    for (int s0 = r0; s0 < r1; s0 += MB, buf ^= 1) {
-      float v[MB][NV * V];
-#pragma unroll
-      for (int j = 0; j < MB; ++j) {
-        const bool live = s0 + j < r1;
-        const T* x = X + (P.tok_row + s0 + j) * ldx;
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
-          const int c0 = (tid + q * AGG_T) * V;
-          if (live && c0 < d) {
-            load_vec<T>(x + c0, &v[j][q * V]);
-          } else {
-#pragma unroll
-            for (int e = 0; e < V; ++e) v[j][q * V + e] = 0.f;
-          }
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < MB; ++j) {
-        float sq = 0.f;
-#pragma unroll
-        for (int e = 0; e < NV * V; ++e) sq = fmaf(v[j][e], v[j][e], sq);
-        sq = warp_sum_f(sq);
-        if (lane == 0) shq[buf][j][warp] = sq;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int j = 0; j < MB; ++j) {
-        float t = 0.f;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) t += shq[buf][j][w];
-        const float inv = (t > 0.f) ? 1.0f / sqrtf(t) : 0.f;
-#pragma unroll
-        for (int e = 0; e < NV * V; ++e) {
-          cs[e] += v[j][e];
-          ns[e] = fmaf(v[j][e], inv, ns[e]);
-        }
-      }
-    }
-    float* dst = part + (size_t)u * 2 * d;
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      const int c0 = (tid + q * AGG_T) * V;
-      if (c0 < d)
-#pragma unroll
-        for (int e = 0; e < V; e += 4) {
-          store_vec4(dst + c0 + e, cs[q * V + e], cs[q * V + e + 1], cs[q * V + e + 2],
-                     cs[q * V + e + 3]);
-          store_vec4(dst + d + c0 + e, ns[q * V + e], ns[q * V + e + 1], ns[q * V + e + 2],
-                     ns[q * V + e + 3]);
-        }
-    }
-    __syncthreads();
-  }
-}
+// add 0.  Every window is cut into parts; a CTA takes a part, reduces each row's
+// |x|^2 (per warp, then across warps through a double-buffered shared array, one
+// barrier per batch of agg_batch<NV>() rows) and writes the part's sums of x and
+// of x/|x|; window_score_combine_kernel adds a window's parts and forms the score.
 
 // ---------------------------------------------------------------------------
 // The score pass with the chunk path folded in (adaptive backend below rho =
@@ -1830,9 +1746,9 @@ window_score_kernel(const T* __restrict__ X, int d, int64_t ldx,
 // routed to the chunk path -- renormalised means (Eq. macro_embed), their
 // positions and the token map -- and the segment and aggregation steps then
 // handle the spectral windows only, whose outputs replace these.  Parts are
-// cut on group boundaries (about SCORE_PR rows each), so no group spans two
-// CTAs; a batch's shared-memory reduction carries, besides the row norms,
-// the squared norms of the group means that end in the batch.
+// cut on group boundaries, so no group spans two CTAs; a batch's shared-memory
+// reduction carries, besides the row norms, the squared norms of the group means
+// that end in the batch.
 // ---------------------------------------------------------------------------
 
 // first token of chunk group g (g <= m; group m starts at n)
@@ -1840,20 +1756,8 @@ __host__ __device__ inline int chunk_gstart(int n, int m, int g) {
   const int q = n / m, rem = n % m;
   return (g < rem) ? g * (q + 1) : rem * (q + 1) + (g - rem) * q;
 }
-// groups per part: about SCORE_PR rows, at least one group
-__host__ __device__ inline int chunk_gpp(int n, int m) {
-  const int gp = SCORE_PR / (n / m + 1);
-  return gp < 1 ? 1 : gp;
-}
-__host__ __device__ inline int chunk_nparts(int n, int m) {
-  const int gp = chunk_gpp(n, m);
-  return (m + gp - 1) / gp;
-}
-// a bound on chunk_nparts over windows of at most nmax tokens: every part but
-// the last holds at least SCORE_PR / 2 rows
-__host__ __device__ inline int chunk_parts_max(int64_t nmax) {
-  return (int)((nmax + SCORE_PR / 2 - 1) / (SCORE_PR / 2));
-}
+// groups per part when m groups are cut into at most np parts
+__host__ __device__ inline int chunk_gpp(int m, int np) { return (m + np - 1) / np; }
 
 // 16-byte asynchronous copy global -> shared (zero-filled when !live), and
 // the wait for all but the newest `pending` groups of a thread's copies.
@@ -1894,7 +1798,7 @@ window_score_chunk_kernel(const T* __restrict__ X, int d, int64_t ldx,
     const ProbDesc P = probs[p];
     const int n = P.n, m = P.m;
     if (n <= 0 || m <= 0) continue;
-    const int gp = chunk_gpp(n, m);
+    const int gp = chunk_gpp(m, KP);
     if (k >= (m + gp - 1) / gp) continue;
     const int g0 = k * gp, g1 = min(m, g0 + gp);
     const int r0 = chunk_gstart(n, m, g0), r1 = chunk_gstart(n, m, g1);
@@ -2074,21 +1978,26 @@ window_score_chunk_kernel(const T* __restrict__ X, int d, int64_t ldx,
   }
 }
 
-// score[p] = (sum of the parts' x / |x|) . (sum of the parts' x) / (n |sum x|)
-__global__ void __launch_bounds__(AGG_T)
+// score[p] = (sum of the parts' x / |x|) . (sum of the parts' x) / (n |sum x|):
+// a cluster of SC_CL CTAs per window, four columns per thread (d % 4 == 0) with
+// several parts' loads in flight; latency bound (one CTA per window took twice
+// the time).
+constexpr int SC_CL = 4;
+
+__global__ void __cluster_dims__(SC_CL, 1, 1) __launch_bounds__(AGG_T)
 window_score_combine_kernel(int d, const ProbDesc* __restrict__ probs, int nprob, int KP,
-                            int chunked, const float* __restrict__ part,
-                            float* __restrict__ score) {
+                            const float* __restrict__ part, float* __restrict__ score) {
   __shared__ float sh[AGG_T / 32];
-  for (int p = blockIdx.x; p < nprob; p += gridDim.x) {
-    const int n = probs[p].n;
-    const int kp = chunked ? chunk_nparts(n, probs[p].m) : score_parts(n);
+  __shared__ float s_sum[2];
+  const int rank = blockIdx.x % SC_CL;
+  for (int p = blockIdx.x / SC_CL; p < nprob; p += gridDim.x / SC_CL) {
+    const int n = probs[p].n, m = max(probs[p].m, 1);
+    const int gp = chunk_gpp(m, KP), kp = (m + gp - 1) / gp;
     float dot = 0.f, cc = 0.f;
-    // four columns per thread (d % 4 == 0), several parts' loads in flight
-    for (int c = 4 * threadIdx.x; c < d; c += 4 * AGG_T) {
+    for (int c = 4 * (rank * AGG_T + threadIdx.x); c < d; c += 4 * AGG_T * SC_CL) {
       float4 cs = make_float4(0.f, 0.f, 0.f, 0.f), ns = cs;
       const float* src = part + (size_t)p * KP * 2 * d + c;
-#pragma unroll 4
+#pragma unroll 8
       for (int k = 0; k < kp; ++k, src += 2 * d) {
         const float4 a = *reinterpret_cast<const float4*>(src);
         const float4 b = *reinterpret_cast<const float4*>(src + d);
@@ -2100,8 +2009,17 @@ window_score_combine_kernel(int d, const ProbDesc* __restrict__ probs, int nprob
     }
     dot = agg_block_sum(dot, sh);
     cc = agg_block_sum(cc, sh);
-    if (threadIdx.x == 0) score[p] = (cc > 0.f) ? dot / ((float)n * sqrtf(cc)) : 0.f;
-    __syncthreads();
+    if (threadIdx.x == 0) s_sum[0] = dot, s_sum[1] = cc;
+    cluster_sync_all();
+    if (rank == 0 && threadIdx.x == 0) {
+      dot = cc = 0.f;
+      for (int r = 0; r < SC_CL; ++r) {
+        dot += ld_cluster_f32(&s_sum[0], (unsigned)r);
+        cc += ld_cluster_f32(&s_sum[1], (unsigned)r);
+      }
+      score[p] = (cc > 0.f) ? dot / ((float)n * sqrtf(cc)) : 0.f;
+    }
+    cluster_sync_all();  // the sums have been read
   }
 }
 
@@ -2344,101 +2262,82 @@ int launch_aggregate(const void* X, int x_dtype, int d, int64_t ldx, const int* 
 }
 
 namespace {
-template <typename T>
-int launch_score_dtype(const void* X, int d, int64_t ldx, const ProbDesc* probs, int nprob,
-                       int64_t nmax, float* part, float* score, cudaStream_t stream) {
-  constexpr int V = VecOf<T>::V;
-  const int nv = (d / V + AGG_T - 1) / AGG_T;
-  const int KP = score_parts(nmax);
+// Parts per window: the count that makes the slowest CTA's share of rows least,
+// with `slots` CTAs resident and 16 rows' worth of time to start and end a part
+// (eight equal parts of a 2048-token window: 128 windows on 304 CTAs took three
+// rounds of 448 rows, and seven take three of 296).
+int score_parts(int64_t nprob, int64_t nmax, int64_t mmax, int64_t np_cap, int64_t slots) {
+  const int64_t q = (nmax + mmax - 1) / mmax;  // rows of a group
+  int64_t best = 1, cost_best = 0;
+  for (int64_t np = 1; np == 1 || (np <= np_cap && np <= mmax && np * 64 <= nmax); ++np) {
+    const int64_t cost = ((nprob * np + slots - 1) / slots) * (chunk_gpp((int)mmax, (int)np) * q + 16);
+    if (np == 1 || cost < cost_best) best = np, cost_best = cost;
+  }
+  return (int)best;
+}
+
+template <typename T, int NV>
+int launch_score_chunk_nv(const T* X, int d, int64_t ldx, const ProbDesc* probs, int nprob,
+                          int64_t nmax, int64_t mmax, int64_t np_cap, float* part, float* score,
+                          int pos_scheme, int pos_mode, int renorm, float* Xt, int32_t* pos,
+                          int32_t* tok2macro, cudaStream_t stream) {
+  auto fn = window_score_chunk_kernel<T, NV>;
+  int dev = 0, sms = 0, occ = 0;
+  SLS_CUDA_TRY(cudaGetDevice(&dev));
+  SLS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  SLS_CUDA_TRY(
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, CHK_RING_BYTES));
+  SLS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, AGG_T, CHK_RING_BYTES));
+  const int KP = score_parts(nprob, nmax, mmax, np_cap, (int64_t)(occ < 1 ? 1 : occ) * sms);
   const int64_t units = (int64_t)nprob * KP;
   const int blocks = (int)(units < 65535 ? units : 65535);
-#define SLS_SCORE_NV(N)                                                                    \
-  window_score_kernel<T, N><<<blocks, AGG_T, 0, stream>>>((const T*)X, d, ldx, probs, nprob, \
-                                                          KP, part)
-  if (nv <= 1)
-    SLS_SCORE_NV(1);
-  else if (nv <= 2)
-    SLS_SCORE_NV(2);
-  else if (nv <= 4)
-    SLS_SCORE_NV(4);
-  else if (nv <= 8)
-    SLS_SCORE_NV(8);
-  else
-    return SLS_ERR_UNSUPPORTED;
-#undef SLS_SCORE_NV
+  fn<<<blocks, AGG_T, CHK_RING_BYTES, stream>>>(X, d, ldx, probs, nprob, KP, part, pos_scheme,
+                                                pos_mode, renorm, Xt, pos, tok2macro);
   SLS_LAUNCH_CHECK();
   const int cb = nprob < 4096 ? nprob : 4096;
-  window_score_combine_kernel<<<cb, AGG_T, 0, stream>>>(d, probs, nprob, KP, 0, part, score);
+  window_score_combine_kernel<<<cb * SC_CL, AGG_T, 0, stream>>>(d, probs, nprob, KP, part, score);
   SLS_LAUNCH_CHECK();
   return SLS_OK;
 }
-}  // namespace
 
-namespace {
 template <typename T>
 int launch_score_chunk_dtype(const void* X, int d, int64_t ldx, const ProbDesc* probs, int nprob,
-                             int64_t nmax, float* part, float* score, int pos_scheme,
-                             int pos_mode, int renorm, float* Xt, int32_t* pos,
-                             int32_t* tok2macro, cudaStream_t stream) {
-  constexpr int V = VecOf<T>::V;
-  const int nv = (d / V + AGG_T - 1) / AGG_T;
-  const int KP = chunk_parts_max(nmax);
-  const int64_t units = (int64_t)nprob * KP;
-  const int blocks = (int)(units < 65535 ? units : 65535);
-#define SLS_SCORE_NV(N)                                                                   \
-  do {                                                                                     \
-    SLS_CUDA_TRY(cudaFuncSetAttribute(window_score_chunk_kernel<T, N>,                      \
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize,          \
-                                      CHK_RING_BYTES));                                     \
-    window_score_chunk_kernel<T, N><<<blocks, AGG_T, CHK_RING_BYTES, stream>>>(             \
-        (const T*)X, d, ldx, probs, nprob, KP, part, pos_scheme, pos_mode, renorm, Xt, pos, \
-        tok2macro);                                                                        \
-  } while (0)
-  if (nv <= 1)
-    SLS_SCORE_NV(1);
-  else if (nv <= 2)
-    SLS_SCORE_NV(2);
-  else if (nv <= 4)
-    SLS_SCORE_NV(4);
-  else if (nv <= 8)
-    SLS_SCORE_NV(8);
-  else
-    return SLS_ERR_UNSUPPORTED;
-#undef SLS_SCORE_NV
-  SLS_LAUNCH_CHECK();
-  const int cb = nprob < 4096 ? nprob : 4096;
-  window_score_combine_kernel<<<cb, AGG_T, 0, stream>>>(d, probs, nprob, KP, 1, part, score);
-  SLS_LAUNCH_CHECK();
-  return SLS_OK;
+                             int64_t nmax, int64_t mmax, int64_t np_cap, float* part,
+                             float* score, int pos_scheme, int pos_mode, int renorm, float* Xt,
+                             int32_t* pos, int32_t* tok2macro, cudaStream_t stream) {
+  const int nv = (d / VecOf<T>::V + AGG_T - 1) / AGG_T;
+  auto fn = nv <= 1   ? launch_score_chunk_nv<T, 1>
+            : nv <= 2 ? launch_score_chunk_nv<T, 2>
+            : nv <= 4 ? launch_score_chunk_nv<T, 4>
+                      : launch_score_chunk_nv<T, 8>;
+  if (nv > 8) return SLS_ERR_UNSUPPORTED;
+  return fn((const T*)X, d, ldx, probs, nprob, nmax, mmax, np_cap, part, score, pos_scheme,
+            pos_mode, renorm, Xt, pos, tok2macro, stream);
 }
 }  // namespace
 
-size_t score_part_floats(int64_t nprob, int64_t nmax, int d) {
-  const int64_t kp = chunk_parts_max(nmax) > score_parts(nmax) ? chunk_parts_max(nmax)
-                                                                 : score_parts(nmax);
-  return (size_t)nprob * (size_t)kp * 2 * (size_t)d;
+// Part sums go to the aggregation's partial rows, idle at that time; only windows
+// of fewer than 64 tokens (more windows than row pairs there) need room of their
+// own, one part each.
+size_t score_part_floats(int64_t nprob, int64_t Ntot, int d) {
+  return nprob > (int64_t)agg_part_capacity(Ntot) / 2 ? (size_t)nprob * 2 * (size_t)d : 0;
 }
 
 int launch_window_score_chunk(const void* X, int x_dtype, int d, int64_t ldx,
-                              const ProbDesc* probs, int nprob, int64_t nmax, float* part,
-                              float* score, int pos_scheme, int pos_mode, int renorm, float* Xt,
-                              int32_t* pos, int32_t* tok2macro, cudaStream_t stream) {
+                              const ProbDesc* probs, int nprob, int64_t nmax, int64_t mmax,
+                              int64_t Ntot, float* agg_part, float* own_part, float* score,
+                              int pos_scheme, int pos_mode, int renorm, float* Xt, int32_t* pos,
+                              int32_t* tok2macro, cudaStream_t stream) {
   if (nprob <= 0) return SLS_OK;
+  const int64_t np_cap = (int64_t)agg_part_capacity(Ntot) / 2 / nprob;
+  float* part = np_cap > 0 ? agg_part : own_part;
   if (x_dtype == SLS_F32)
-    return launch_score_chunk_dtype<float>(X, d, ldx, probs, nprob, nmax, part, score,
-                                           pos_scheme, pos_mode, renorm, Xt, pos, tok2macro,
-                                           stream);
-  return launch_score_chunk_dtype<uint16_t>(X, d, ldx, probs, nprob, nmax, part, score,
-                                            pos_scheme, pos_mode, renorm, Xt, pos, tok2macro,
-                                            stream);
-}
-
-int launch_window_score(const void* X, int x_dtype, int d, int64_t ldx, const ProbDesc* probs,
-                        int nprob, int64_t nmax, float* part, float* score, cudaStream_t stream) {
-  if (nprob <= 0) return SLS_OK;
-  if (x_dtype == SLS_F32)
-    return launch_score_dtype<float>(X, d, ldx, probs, nprob, nmax, part, score, stream);
-  return launch_score_dtype<uint16_t>(X, d, ldx, probs, nprob, nmax, part, score, stream);
+    return launch_score_chunk_dtype<float>(X, d, ldx, probs, nprob, nmax, mmax, np_cap, part,
+                                           score, pos_scheme, pos_mode, renorm, Xt, pos,
+                                           tok2macro, stream);
+  return launch_score_chunk_dtype<uint16_t>(X, d, ldx, probs, nprob, nmax, mmax, np_cap, part,
+                                            score, pos_scheme, pos_mode, renorm, Xt, pos,
+                                            tok2macro, stream);
 }
 
 }  // namespace sls

@@ -137,17 +137,17 @@ int launch_aggregate(const void* X, int x_dtype, int d, int64_t ldx, const int* 
                      const int* mstart, const int* mlen, int64_t Mtot, int64_t Ntot, int renorm,
                      float* Xt, int* pt_start, int2* items, int* aux, float* part,
                      float* part_eta, int* status, cudaStream_t stream);
-// Redundancy score of every window (Sec. 3.6, Eq. redundancy); part holds
-// score_part_floats(nprob, nmax, d) floats of scratch.
-size_t score_part_floats(int64_t nprob, int64_t nmax, int d);
-int launch_window_score(const void* X, int x_dtype, int d, int64_t ldx, const ProbDesc* probs,
-                        int nprob, int64_t nmax, float* part, float* score, cudaStream_t stream);
-// The same score pass, which also writes every window's chunk-path output
-// (array_split groups of its m macro-tokens: renormalised means into Xt,
-// positions, token map) -- final for the windows the router sends to the
-// chunk path, replaced by the spectral path for the others.
+// Redundancy score of every window (Sec. 3.6, Eq. redundancy); the same pass
+// writes every window's chunk-path output (array_split groups of its m
+// macro-tokens: renormalised means into Xt, positions, token map) -- final for
+// the windows the router sends to the chunk path, replaced by the spectral path
+// for the others.  Scratch: agg_part, the aggregation's partial rows
+// (agg_part_capacity(Ntot) * d floats, Ntot at least the windows' tokens), and
+// own_part, score_part_floats(nprob, Ntot, d) floats.
+size_t score_part_floats(int64_t nprob, int64_t Ntot, int d);
 int launch_window_score_chunk(const void* X, int x_dtype, int d, int64_t ldx,
-                              const ProbDesc* probs, int nprob, int64_t nmax, float* part,
-                              float* score, int pos_scheme, int pos_mode, int renorm, float* Xt,
-                              int32_t* pos, int32_t* tok2macro, cudaStream_t stream);
+                              const ProbDesc* probs, int nprob, int64_t nmax, int64_t mmax,
+                              int64_t Ntot, float* agg_part, float* own_part, float* score,
+                              int pos_scheme, int pos_mode, int renorm, float* Xt, int32_t* pos,
+                              int32_t* tok2macro, cudaStream_t stream);
 }  // namespace sls
