@@ -1344,7 +1344,7 @@ constexpr int AI_CL = 8;
 
 // Auxiliary integers of the aggregation: counts (16) and the multi-item macros.
 struct AggAux {
-  int* counts;  // [0] items, [1] partial slots, [2] multi-item macros
+  int* counts;  // [0] items, [1] partial slots, [2] multi-item macros, [3] item ticket
   int* multi;
 };
 
@@ -1395,6 +1395,7 @@ agg_items_kernel(const int* __restrict__ mlen, int64_t Mtot, int* __restrict__ a
     s_pre[tid] = pre;
     if (rank == AI_CL - 1) A.counts[tid] = pre + s_tot[tid];
   }
+  if (rank == 0 && tid == 3) A.counts[3] = 0;
   cluster_sync_all();  // s_pre is ready, and every CTA has read the totals
   o0 += s_pre[0];
   o1 += s_pre[1];
@@ -1614,7 +1615,7 @@ template <typename T, int NV>
 __global__ void __launch_bounds__(AGG_T, NV <= 2 ? 4 : 2)
 agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __restrict__ perm,
                   const int* __restrict__ mstart, const int* __restrict__ mlen,
-                  const int2* __restrict__ items, const int* __restrict__ aux,
+                  const int2* __restrict__ items, int* __restrict__ aux,
                   const int* __restrict__ pt_start, int renorm, float* __restrict__ Xt,
                   float* __restrict__ part, float* __restrict__ part_eta, int* status,
                   int64_t ntot) {
@@ -1624,13 +1625,17 @@ agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __rest
   constexpr int NW = AGG_T / 32, LPR = 32 / MB;
   __shared__ float shq[2][AGG_CH][NW];  // row |x|^2 by warp
   __shared__ float shm[2][NW];          // |member sum|^2 by warp
+  __shared__ int s_next[2];
   (void)status;
   (void)ntot;  // bounds of the member rows (debug-build checks)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int nitems = agg_aux(const_cast<int*>(aux)).counts[0];
+  int* counts = agg_aux(aux).counts;
+  const int nitems = counts[0];
   int buf = 0;
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x, buf ^= 1) {
+  for (int it = blockIdx.x; it < nitems; it = s_next[buf], buf ^= 1) {
     const int2 item = items[it];
+    // the next item, handed out by a ticket (read after the item's barrier)
+    if (tid == 0) s_next[buf] = (int)gridDim.x + atomicAdd(&counts[3], 1);
     const int m = item.x, c = item.y;
     const int len = mlen[m], ps = pt_start[m];
     const int n = min(len - c * AGG_CH, AGG_CH);
