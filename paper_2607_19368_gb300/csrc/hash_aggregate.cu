@@ -1597,14 +1597,14 @@ SLS_DEV float warp_sums(float (&v)[R]) {
 
 // ---------------------------------------------------------------------------
 // Member pass: a CTA per work item, its member rows by plain 16-byte loads in
-// batches of MB rows per thread (about eight loads in flight each).  A thread
+// batches of MB rows per thread (eight or more loads in flight each).  A thread
 // owns the column groups c0 = (tid + q * AGG_T) * V, sums them and the rows'
 // |x|^2 on packed pairs; one barrier per item publishes the row norms and the
 // sum's own, and every thread finalises its columns of the macro-token (Eq.
 // macro_embed) or stores them as a partial sum.
 //
-// Bound by reading X: four or more CTAs per SM keep 100 KB of rows in flight, and
-// an item's chain of descriptor, member ids and rows hides behind the others'.
+// Bound by reading X: an SM keeps 100 KB of rows in flight, and an item's chain of
+// descriptor, member ids and rows hides behind the other CTAs'.
 // The former pass streamed each row through a shared-memory ring with one bulk
 // copy per row; issuing those took a producer warp about 1000 cycles per row
 // (N = 32756, d = 3584: 90 -> 58 us, against 35 us for the bytes; N = 8180,
@@ -1612,7 +1612,7 @@ SLS_DEV float warp_sums(float (&v)[R]) {
 // ---------------------------------------------------------------------------
 
 template <typename T, int NV>
-__global__ void __launch_bounds__(AGG_T, NV <= 2 ? 4 : 2)
+__global__ void __launch_bounds__(AGG_T, NV == 1 ? 4 : 2)
 agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __restrict__ perm,
                   const int* __restrict__ mstart, const int* __restrict__ mlen,
                   const int2* __restrict__ items, int* __restrict__ aux,
@@ -1621,7 +1621,10 @@ agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __rest
                   int64_t ntot) {
   constexpr int V = VecOf<T>::V;
   constexpr int PN = NV * V / 2;  // element pairs per thread
-  constexpr int MB = agg_batch<NV>();
+  // NV = 2 (d up to 4096 in bf16): twice the rows in flight on half the CTAs, so
+  // that a long item ends sooner (N = 8180, d = 4096: 31 -> 26 us); NV = 1 keeps
+  // four CTAs (N = 20000, d = 512: 198 us for the call against 227).
+  constexpr int MB = NV == 2 ? 8 : agg_batch<NV>();
   constexpr int NW = AGG_T / 32, LPR = 32 / MB;
   __shared__ float shq[2][AGG_CH][NW];  // row |x|^2 by warp
   __shared__ float shm[2][NW];          // |member sum|^2 by warp
