@@ -29,15 +29,21 @@ SLS_DEV int reff_clamped(const LanczosBatch& bt, int p) {
 // a serial recurrence pays at every step.
 // ----------------------------------------------------------------------------
 
-// Ritz values of few problems: one CTA per eigenvalue, 256 shifts per round
-// (fewer, longer rounds: the faster form when the launch has few eigenvalues)
+// Ritz values of few problems: one CTA per eigenvalue, a shift per thread and
+// round.  Bound by the double-float recurrence (about 70 instructions and a chain
+// of 20 per row of T).  Three rounds in float32 come first and are widened by their
+// error, and the first double-float round spans the widened interval ends
+// included, so an eigenvalue outside it is found all the same.  r = 32: 33 -> 26 us,
+// r = 64: 58 -> 46 (128 threads: the same).
 constexpr int EIG_THREADS = 256;  // shifts per multisection round
 constexpr float kInvShiftsF = 1.0f / (float)(EIG_THREADS + 1);
+constexpr int EIG_F32_ROUNDS = 3;
+constexpr float EIG_F32_MARGIN = 0x1p-18f;
 
 __global__ void __launch_bounds__(EIG_THREADS)
 tridiag_eigvals_cta_kernel(LanczosBatch bt) {
   __shared__ float2 sa[SLS_MAX_R], sb2[SLS_MAX_R];
-  __shared__ int s_first[EIG_THREADS / 32];
+  __shared__ int s_first[2][EIG_THREADS / 32];
   __shared__ double s_sc;
   __shared__ float2 s_lo, s_hi;  // the interval, double-float
   const int m = blockIdx.x, p = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -90,28 +96,53 @@ tridiag_eigvals_cta_kernel(LanczosBatch bt) {
   }
   __syncthreads();
   const int k = n - 1 - m;  // ascending index of the wanted eigenvalue
+  int buf = 0;
+  // first shift whose count exceeds k (EIG_THREADS: none), the same in every thread
+  auto first_above = [&](int c) {
+    const unsigned ball = __ballot_sync(0xffffffffu, c > k);
+    if (lane == 0) s_first[buf][warp] = ball ? warp * 32 + __ffs(ball) - 1 : EIG_THREADS;
+    __syncthreads();
+    int f = EIG_THREADS;
+#pragma unroll
+    for (int w2 = 0; w2 < EIG_THREADS / 32; ++w2) f = min(f, s_first[buf][w2]);
+    buf ^= 1;
+    return f;
+  };
+  const dfloat lo0 = dfv(s_lo), hi0 = dfv(s_hi);
+  dfloat lo = lo0, hi = hi0;
+  {
+    float fl = lo0.hi, fh = hi0.hi;
+    for (int round = 0; round < EIG_F32_ROUNDS; ++round) {
+      const float step = (fh - fl) * kInvShiftsF;
+      const int f = first_above(sturm_count_f32(sa, sb2, n, fmaf(step, (float)(tid + 1), fl)));
+      const float nl = fmaf(step, (float)f, fl);
+      if (f < EIG_THREADS) fh = fmaf(step, (float)(f + 1), fl);
+      fl = nl;
+    }
+    lo = df_make(fl - EIG_F32_MARGIN, 0.f);
+    hi = df_make(fh + EIG_F32_MARGIN, 0.f);
+    // shifts lo + t (hi - lo) / (EIG_THREADS - 1), both ends among them
+    const dfloat step = df_mul_f(df_sub(hi, lo), 1.0f / (float)(EIG_THREADS - 1));
+    const int f = first_above(sturm_count(sa, sb2, n, df_add(lo, df_mul_f(step, (float)tid))));
+    const dfloat base = lo;
+    lo = f > 0 ? df_add(base, df_mul_f(step, (float)(f - 1))) : lo0;
+    hi = f < EIG_THREADS ? df_add(base, df_mul_f(step, (float)f)) : hi0;
+  }
   for (int round = 0; round < 40; ++round) {
-    const dfloat lo = dfv(s_lo), hi = dfv(s_hi);
     const dfloat w = df_sub(hi, lo);
     // 2^-46 relative, or one float64 unit of the scaled |T| <= 1
     if (w.hi <= 0x1p-46f * fmaxf(fabsf(lo.hi), fabsf(hi.hi)) || w.hi <= 0x1p-52f) break;
     // shift t: lo + (t + 1) (hi - lo) / (EIG_THREADS + 1), in double-float on
     // the float32 pipes (every thread computes one per round)
     const dfloat step = df_mul_f(w, kInvShiftsF);
-    const int c = sturm_count(sa, sb2, n, df_add(lo, df_mul_f(step, (float)(tid + 1))));
-    const unsigned ball = __ballot_sync(0xffffffffu, c > k);
-    if (lane == 0) s_first[warp] = ball ? warp * 32 + __ffs(ball) - 1 : EIG_THREADS;
-    __syncthreads();
-    if (tid == 0) {
-      int f = EIG_THREADS;
-      for (int w2 = 0; w2 < EIG_THREADS / 32; ++w2) f = min(f, s_first[w2]);
-      // count(x_t) is non-decreasing in t: the eigenvalue lies in (x_{f-1}, x_f]
-      if (f < EIG_THREADS) s_hi = f2(df_add(lo, df_mul_f(step, (float)(f + 1))));
-      if (f > 0) s_lo = f2(df_add(lo, df_mul_f(step, (float)f)));
-    }
-    __syncthreads();
+    const int f =
+        first_above(sturm_count(sa, sb2, n, df_add(lo, df_mul_f(step, (float)(tid + 1)))));
+    // count(x_t) is non-decreasing in t: the eigenvalue lies in (x_{f-1}, x_f]
+    const dfloat nlo = f > 0 ? df_add(lo, df_mul_f(step, (float)f)) : lo;
+    if (f < EIG_THREADS) hi = df_add(lo, df_mul_f(step, (float)(f + 1)));
+    lo = nlo;
   }
-  if (tid == 0) theta[m] = (0.5 * df_to_double(df_add(dfv(s_lo), dfv(s_hi)))) / sc;
+  if (tid == 0) theta[m] = (0.5 * df_to_double(df_add(lo, hi))) / sc;
 }
 
 constexpr int EIG_WARPS = 8;  // eigenvalues per CTA (one warp each)
@@ -203,13 +234,15 @@ tridiag_eigvals_kernel(LanczosBatch bt) {
 // Eigenvectors of one cluster [first, last] of nearly equal Ritz values of
 // problem p (n = r_eff), written as columns of S: inverse iteration with
 // partial-pivoting LU of T - shift I in double-float, two iterations, each
-// followed by modified Gram-Schmidt against the cluster members already
-// found.  One thread; the work arrays (n entries each) belong to the caller.
-// The recurrences carry their running values in registers (the factorisation
-// the current pivot row, the solves the last one or two entries), so a step's
-// dependent chain holds no memory access, and the back substitution
-// multiplies by the pivots' reciprocals, formed during the factorisation off
-// that chain; sums over n run as four interleaved partial sums.
+// followed by modified Gram-Schmidt against the cluster members already found.
+// The recurrences carry their running values in registers (the factorisation the
+// current pivot row, the solves the last one or two entries), so a step's
+// dependent chain holds no memory access; pivoting selects operands instead of
+// branching; the first forward solve rides along the factorisation; and the back
+// substitution multiplies by the pivots' reciprocals.  The work arrays (n entries
+// each) belong to the caller.  WARP: the lanes of a warp run the recurrences
+// alike, on arrays in shared memory, and share the loops over entries; else one
+// thread computes the cluster (sums over n as four interleaved partial sums).
 SLS_DEV dfloat sum4_df(dfloat (&acc)[4]) {
   return df_add(df_add(acc[0], acc[1]), df_add(acc[2], acc[3]));
 }
@@ -239,6 +272,74 @@ SLS_DEV void eig_scaled_T(const LanczosBatch& bt, int p, int n, double sc, int t
   }
 }
 
+// LU of T - shift I with the forward solve of the running right-hand side y:
+// d the pivots' reciprocals, du and du2 the rows of U, dl the multipliers, piv the
+// interchanges.  Returns the last entry of the solved right-hand side.
+template <typename Y0>
+SLS_DEV dfloat eig_factor(int n, dfloat shift, dfloat pert, Y0 y0, const float2* __restrict__ sa,
+                          const float2* __restrict__ sb, float2* __restrict__ d,
+                          float2* __restrict__ du, float2* __restrict__ du2,
+                          float2* __restrict__ dl, float2* __restrict__ y,
+                          unsigned char* __restrict__ piv) {
+  const dfloat one = df_make(1.f, 0.f), zero = df_make(0.f, 0.f);
+  // cd, cu: the current pivot row's diagonal and superdiagonal entries as the
+  // elimination has left them; cy: the running right-hand side
+  dfloat cd = df_sub(dfv(sa[0]), shift), cu = dfv(sb[0]), cy = df_make(y0(0), 0.f);
+  for (int i = 0; i < n - 1; ++i) {
+    const dfloat li = dfv(sb[i]);
+    const dfloat dn = df_sub(dfv(sa[i + 1]), shift);
+    const dfloat un = (i < n - 2) ? dfv(sb[i + 1]) : zero;
+    const dfloat yn = df_make(y0(i + 1), 0.f);
+    const bool sw = !(fabsf(cd.hi) >= fabsf(li.hi));
+    if (!sw && cd.hi == 0.f) cd = pert;
+    const dfloat den = sw ? li : cd;
+    const dfloat f = df_div(sw ? cd : li, den);
+    const dfloat u1 = sw ? dn : cu, u2 = sw ? un : zero, ya = sw ? yn : cy;
+    d[i] = f2(df_div(one, den));
+    dl[i] = f2(f);
+    du[i] = f2(u1);
+    du2[i] = f2(u2);
+    y[i] = f2(ya);
+    piv[i] = sw ? 1 : 0;
+    cd = df_sub(sw ? cu : dn, df_mul(f, u1));
+    cy = df_sub(sw ? cy : yn, df_mul(f, ya));
+    cu = sw ? df_neg(df_mul(f, un)) : un;
+  }
+  if (cd.hi == 0.f) cd = pert;
+  d[n - 1] = f2(df_div(one, cd));
+  return cy;
+}
+
+// Forward solve with the row interchanges; returns the last entry.
+SLS_DEV dfloat eig_forward(int n, const float2* __restrict__ dl, float2* __restrict__ y,
+                           const unsigned char* __restrict__ piv) {
+  dfloat cy = dfv(y[0]);
+  for (int i = 0; i < n - 1; ++i) {
+    const dfloat yn = dfv(y[i + 1]);
+    const bool sw = piv[i] != 0;
+    const dfloat ya = sw ? yn : cy;
+    y[i] = f2(ya);
+    cy = df_sub(sw ? cy : yn, df_mul(dfv(dl[i]), ya));
+  }
+  return cy;
+}
+
+// Back substitution from the last entry cy; c1, c2: y[i + 1], y[i + 2].
+SLS_DEV void eig_back(int n, dfloat cy, const float2* __restrict__ d,
+                      const float2* __restrict__ du, const float2* __restrict__ du2,
+                      float2* __restrict__ y) {
+  dfloat c1 = df_mul(cy, dfv(d[n - 1])), c2 = df_make(0.f, 0.f);
+  y[n - 1] = f2(c1);
+  for (int i = n - 2; i >= 0; --i) {
+    dfloat t = dfv(y[i]);
+    if (i < n - 2) t = df_sub(t, df_mul(dfv(du2[i]), c2));
+    c2 = c1;
+    c1 = df_mul(df_sub(t, df_mul(dfv(du[i]), c1)), dfv(d[i]));
+    y[i] = f2(c1);
+  }
+}
+
+template <bool WARP>
 SLS_DEV void eigvec_cluster(const LanczosBatch& bt, int p, int n, int first, int last,
                             double sc, double tnorm, const float2* __restrict__ sa,
                             const float2* __restrict__ sb, float2* __restrict__ d,
@@ -248,121 +349,81 @@ SLS_DEV void eigvec_cluster(const LanczosBatch& bt, int p, int n, int first, int
   const int r = bt.r;
   double* S = bt.S + (size_t)p * r * r;
   const double* th = bt.theta + (size_t)p * r;
-  const double pert = 0x1p-44 * tnorm * sc;
-  const dfloat pert_df = df_from_double(pert);
-  const dfloat one = df_make(1.f, 0.f);
+  const double pert = 0x1p-44 * tnorm;
+  const dfloat pert_df = df_from_double(pert * sc);
+  const int i0 = WARP ? (threadIdx.x & 31) : 0;
+  constexpr int di = WARP ? 32 : 1;
+  // lanes that hold alike what each has written meet before and after a loop
+  // that they share
+  auto meet = [] {
+    if (WARP) __syncwarp();
+  };
+  auto dot_all = [&](auto term) {  // sum of term(i) over i < n
+    if constexpr (WARP) {
+      dfloat acc = df_make(0.f, 0.f);
+      for (int i = i0; i < n; i += di) acc = df_add(acc, term(i));
+      return warp_sum_df(acc);
+    } else {
+      dfloat acc[4] = {df_make(0.f, 0.f), df_make(0.f, 0.f), df_make(0.f, 0.f),
+                       df_make(0.f, 0.f)};
+      for (int i = 0; i < n; ++i) acc[i & 3] = df_add(acc[i & 3], term(i));
+      return sum4_df(acc);
+    }
+  };
   for (int mm = first; mm <= last; ++mm) {
     // distinct shifts inside a cluster
-    const dfloat shift = df_from_double((th[mm] - (double)(mm - first) * 4.0 * (pert / sc)) * sc);
-    // the diagonal of T - shift I (d) and the off-diagonal (dl), unfactored
-    for (int i = 0; i < n; ++i) {
-      d[i] = f2(df_sub(dfv(sa[i]), shift));
-      if (i < n - 1) dl[i] = sb[i];
-    }
+    const dfloat shift = df_from_double((th[mm] - (double)(mm - first) * 4.0 * pert) * sc);
     if (n == 1) {
       y[0] = make_float2(1.f, 0.f);
     } else {
-      // LU with partial pivoting of T - shift I; cd, cu: the current pivot
-      // row's diagonal and superdiagonal entries as the elimination has left
-      // them.  d[i] then holds the reciprocal of pivot i.
-      dfloat cd = dfv(d[0]), cu = dfv(dl[0]);
-      for (int i = 0; i < n - 1; ++i) {
-        const dfloat li = dfv(dl[i]);
-        const dfloat dn0 = dfv(d[i + 1]);
-        const dfloat un0 = (i < n - 2) ? dfv(dl[i + 1]) : df_make(0.f, 0.f);
-        if (fabsf(cd.hi) >= fabsf(li.hi)) {
-          if (cd.hi == 0.f) cd = pert_df;
-          const dfloat f = df_div(li, cd);
-          d[i] = f2(df_div(one, cd));
-          dl[i] = f2(f);
-          du[i] = f2(cu);
-          du2[i] = make_float2(0.f, 0.f);
-          cd = df_sub(dn0, df_mul(f, cu));
-          cu = un0;
-          piv[i] = 0;
-        } else {
-          const dfloat f = df_div(cd, li);
-          d[i] = f2(df_div(one, li));
-          dl[i] = f2(f);
-          du[i] = f2(dn0);
-          du2[i] = f2(un0);
-          cd = df_sub(cu, df_mul(f, dn0));
-          cu = df_neg(df_mul(f, un0));
-          piv[i] = 1;
-        }
-      }
-      if (cd.hi == 0.f) cd = pert_df;
-      d[n - 1] = f2(df_div(one, cd));
       // deterministic start vector
-      for (int i = 0; i < n; ++i) {
+      auto y0 = [mm](int i) {
         unsigned h = (unsigned)(i + 1) * 2654435761u ^ (unsigned)(mm + 7) * 40503u;
         h ^= h >> 13;
         h *= 0x5bd1e995u;
         h ^= h >> 15;
-        y[i] = make_float2(0.5f + (float)(h & 0xffffu) / 65536.f, 0.f);
-      }
+        return 0.5f + (float)(h & 0xffffu) / 65536.f;
+      };
       for (int it = 0; it < 2; ++it) {
-        // forward substitution with the row interchanges; cy: the running y[i]
-        dfloat cy = dfv(y[0]);
-        for (int i = 0; i < n - 1; ++i) {
-          const dfloat yn = dfv(y[i + 1]);
-          const dfloat li = dfv(dl[i]);
-          if (!piv[i]) {
-            y[i] = f2(cy);
-            cy = df_sub(yn, df_mul(li, cy));
-          } else {
-            y[i] = f2(yn);
-            cy = df_sub(cy, df_mul(li, yn));
-          }
-        }
-        // back substitution; c1, c2: y[i + 1], y[i + 2]
-        dfloat c1 = df_mul(cy, dfv(d[n - 1]));
-        y[n - 1] = f2(c1);
-        dfloat c2 = c1;
-        c1 = df_mul(df_sub(dfv(y[n - 2]), df_mul(dfv(du[n - 2]), c1)), dfv(d[n - 2]));
-        y[n - 2] = f2(c1);
-        for (int i = n - 3; i >= 0; --i) {
-          const dfloat t = df_sub(df_sub(dfv(y[i]), df_mul(dfv(du[i]), c1)),
-                                  df_mul(dfv(du2[i]), c2));
-          c2 = c1;
-          c1 = df_mul(t, dfv(d[i]));
-          y[i] = f2(c1);
-        }
+        const dfloat cy = it == 0
+                              ? eig_factor(n, shift, pert_df, y0, sa, sb, d, du, du2, dl, y, piv)
+                              : eig_forward(n, dl, y, piv);
+        eig_back(n, cy, d, du, du2, y);
+        meet();
         // keep the iterate in range: divide by its largest entry (a power of two)
         float ymax = 0.f;
-        for (int i = 0; i < n; ++i) ymax = fmaxf(ymax, fabsf(y[i].x));
+        for (int i = i0; i < n; i += di) ymax = fmaxf(ymax, fabsf(y[i].x));
+        if (WARP)
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) ymax = fmaxf(ymax, __shfl_xor_sync(0xffffffffu, ymax, o));
         if (ymax > 0.f && isfinite(ymax)) {
           int e2 = 0;
           frexpf(ymax, &e2);
           const float s2 = ldexpf(1.f, -e2);
-          for (int i = 0; i < n; ++i) y[i] = f2(df_scale(dfv(y[i]), s2));
+          for (int i = i0; i < n; i += di) y[i] = f2(df_scale(dfv(y[i]), s2));
         }
         // orthogonalise against the cluster members found so far
         for (int pm = first; pm < mm; ++pm) {
-          dfloat acc[4] = {df_make(0.f, 0.f), df_make(0.f, 0.f), df_make(0.f, 0.f),
-                           df_make(0.f, 0.f)};
-          for (int i = 0; i < n; ++i)
-            acc[i & 3] = df_add(acc[i & 3],
-                                df_mul(df_from_double(S[(size_t)i * r + pm]), dfv(y[i])));
-          const dfloat dot = sum4_df(acc);
-          for (int i = 0; i < n; ++i)
+          const dfloat dot = dot_all(
+              [&](int i) { return df_mul(df_from_double(S[(size_t)i * r + pm]), dfv(y[i])); });
+          for (int i = i0; i < n; i += di)
             y[i] = f2(df_sub(dfv(y[i]), df_mul(dot, df_from_double(S[(size_t)i * r + pm]))));
         }
-        dfloat acc[4] = {df_make(0.f, 0.f), df_make(0.f, 0.f), df_make(0.f, 0.f),
-                         df_make(0.f, 0.f)};
-        for (int i = 0; i < n; ++i) acc[i & 3] = df_add(acc[i & 3], df_mul(dfv(y[i]), dfv(y[i])));
-        const double nr = sqrt(df_to_double(sum4_df(acc)));
+        const double nr =
+            sqrt(df_to_double(dot_all([&](int i) { return df_mul(dfv(y[i]), dfv(y[i])); })));
         if (!(nr > 0.0) || !isfinite(nr)) {
-          for (int i = 0; i < n; ++i) y[i] = make_float2((i == mm) ? 1.f : 0.f, 0.f);
+          for (int i = i0; i < n; i += di) y[i] = make_float2((i == mm) ? 1.f : 0.f, 0.f);
         } else {
           const dfloat inv = df_from_double(1.0 / nr);
-          for (int i = 0; i < n; ++i) y[i] = f2(df_mul(dfv(y[i]), inv));
+          for (int i = i0; i < n; i += di) y[i] = f2(df_mul(dfv(y[i]), inv));
         }
+        meet();
       }
     }
     const double sg = (y[0].x < 0.f) ? -1.0 : 1.0;
 #pragma unroll 4
-    for (int i = 0; i < n; ++i) S[(size_t)i * r + mm] = sg * df_to_double(dfv(y[i]));
+    for (int i = i0; i < n; i += di) S[(size_t)i * r + mm] = sg * df_to_double(dfv(y[i]));
+    meet();
   }
 }
 
@@ -377,8 +438,8 @@ SLS_DEV void eig_cluster(const double* th, int n, int m, int& first, int& last) 
   while (last + 1 < n && th[last] - th[last + 1] <= ctol) ++last;
 }
 
-// One CTA (lane 0 working) per Ritz value: the CTA of a cluster's first
-// member computes the whole cluster.
+// One warp per Ritz value: the warp of a cluster's first member computes the whole
+// cluster.
 __global__ void __launch_bounds__(32)
 tridiag_eigvecs_kernel(LanczosBatch bt) {
   __shared__ float2 d[SLS_MAX_R], du[SLS_MAX_R], du2[SLS_MAX_R], dl[SLS_MAX_R];
@@ -404,15 +465,17 @@ tridiag_eigvecs_kernel(LanczosBatch bt) {
   const double sc = eig_scale(bt.theta + (size_t)p * r, n, &tnorm);
   eig_scaled_T(bt, p, n, sc, lane, 32, sa, sb);
   __syncwarp();
-  if (lane != 0) return;
-  eigvec_cluster(bt, p, n, first, last, sc, tnorm, sa, sb, d, du, du2, dl, y, piv);
+  eigvec_cluster<true>(bt, p, n, first, last, sc, tnorm, sa, sb, d, du, du2, dl, y, piv);
 }
 
-// Small problems (r <= 32): one warp per problem, one lane per Ritz value;
+// Many small problems (r <= 32): one warp per problem, one lane per Ritz value;
 // the lane of a cluster's first member computes the whole cluster, with its
 // work arrays in local memory.
 constexpr int EIGW_WARPS = 1;  // one problem per CTA: the fewest idle SMs at the end
 constexpr int EIGW_MAXR = 32;
+// Ritz values up to which a warp computes each eigenvector (32 values: 22 us, a
+// lane each 31; 2048 values: 39 us either way)
+constexpr int64_t EIGV_WARPS_MAX = 2048;
 
 __global__ void __launch_bounds__(EIGW_WARPS * 32)
 tridiag_eigvecs_warp_kernel(LanczosBatch bt) {
@@ -442,7 +505,8 @@ tridiag_eigvecs_warp_kernel(LanczosBatch bt) {
   if (first != lane) return;
   float2 d[EIGW_MAXR], du[EIGW_MAXR], du2[EIGW_MAXR], dl[EIGW_MAXR], y[EIGW_MAXR];
   unsigned char piv[EIGW_MAXR];
-  eigvec_cluster(bt, p, n, first, last, sc, tnorm, sa[warp], sb[warp], d, du, du2, dl, y, piv);
+  eigvec_cluster<false>(bt, p, n, first, last, sc, tnorm, sa[warp], sb[warp], d, du, du2, dl, y,
+                        piv);
 }
 
 // ----------------------------------------------------------------------------
@@ -633,7 +697,7 @@ int launch_tridiag_eigen(const LanczosBatch& bt, cudaStream_t stream, bool value
     }
     SLS_LAUNCH_CHECK();
   }
-  if (bt.r <= EIGW_MAXR) {
+  if (bt.r <= EIGW_MAXR && (int64_t)bt.r * bt.nprob_max > EIGV_WARPS_MAX) {
     const int blocks = (bt.nprob_max + EIGW_WARPS - 1) / EIGW_WARPS;
     tridiag_eigvecs_warp_kernel<<<blocks, EIGW_WARPS * 32, 0, stream>>>(bt);
   } else {

@@ -18,10 +18,20 @@ SLS_DEV dfloat df_div(dfloat a, dfloat b) {
 
 SLS_DEV dfloat df_scale(dfloat a, float s) { return df_make(a.hi * s, a.lo * s); }
 
+// a - b with an error of 2^-47 (|a| + |b|) at most (df_sub: of the result), a
+// third shorter.
+SLS_DEV dfloat df_sub_abs(dfloat a, dfloat b) {
+  float s, e;
+  two_sum(a.hi, -b.hi, s, e);
+  return df_norm(s, __fadd_rn(e, __fsub_rn(a.lo, b.lo)));
+}
+
 // Number of eigenvalues of the (scaled) tridiagonal below x, from the signs of
 // the leading principal minors p_i(x) (three-term recurrence, Sturm sequence).
 // Powers of two rescale the pair (p_{i-1}, p_i) to keep it in range; a zero
-// minor takes the sign opposite to its predecessor.
+// minor takes the sign opposite to its predecessor.  An error in a minor that is
+// small beside its two terms acts as a relative change of b_{i-1}^2 and a_i - x,
+// which is why their difference needs no more than df_sub_abs.
 SLS_DEV int sturm_count(const float2* __restrict__ a, const float2* __restrict__ b2, int n,
                         dfloat x) {
   dfloat pm = df_make(1.f, 0.f), pc = df_sub(dfv(a[0]), x);
@@ -32,7 +42,7 @@ SLS_DEV int sturm_count(const float2* __restrict__ a, const float2* __restrict__
   for (int i = 1; i < n; ++i) {
     const dfloat d = df_sub(dfv(a[i]), x);
     const dfloat t = df_mul(dfv(b2[i - 1]), pm);
-    const dfloat pn = df_sub(df_mul(d, pc), t);
+    const dfloat pn = df_sub_abs(df_mul(d, pc), t);
     pm = pc;
     pc = pn;
     const float mg = fmaxf(fabsf(pc.hi), fabsf(pm.hi));
@@ -44,6 +54,34 @@ SLS_DEV int sturm_count(const float2* __restrict__ a, const float2* __restrict__
       pm = df_scale(pm, 0x1p60f);
     }
     s = (pc.hi < 0.f) ? 1 : ((pc.hi > 0.f) ? 0 : 1 - sprev);
+    cnt += (s != sprev);
+    sprev = s;
+  }
+  return cnt;
+}
+
+// The same count in float32, exact for a T whose entries differ by a few
+// float32 units (|T| <= 1: eigenvalues that move by less than 2^-20).
+SLS_DEV int sturm_count_f32(const float2* __restrict__ a, const float2* __restrict__ b2, int n,
+                            float x) {
+  float pm = 1.f, pc = a[0].x - x;
+  int sprev = 0;
+  int s = (pc < 0.f) ? 1 : ((pc > 0.f) ? 0 : 1);
+  int cnt = (s != sprev);
+  sprev = s;
+  for (int i = 1; i < n; ++i) {
+    const float pn = fmaf(a[i].x - x, pc, -(b2[i - 1].x * pm));
+    pm = pc;
+    pc = pn;
+    const float mg = fmaxf(fabsf(pc), fabsf(pm));
+    if (mg > 0x1p60f) {
+      pc *= 0x1p-60f;
+      pm *= 0x1p-60f;
+    } else if (mg < 0x1p-60f && mg > 0.f) {
+      pc *= 0x1p60f;
+      pm *= 0x1p60f;
+    }
+    s = (pc < 0.f) ? 1 : ((pc > 0.f) ? 0 : 1 - sprev);
     cnt += (s != sprev);
     sprev = s;
   }
