@@ -331,10 +331,10 @@ SLS_DEV void eig_back(int n, dfloat cy, const float2* __restrict__ d,
   dfloat c1 = df_mul(cy, dfv(d[n - 1])), c2 = df_make(0.f, 0.f);
   y[n - 1] = f2(c1);
   for (int i = n - 2; i >= 0; --i) {
-    dfloat t = dfv(y[i]);
+    dfloat t = df_sub(dfv(y[i]), df_mul(dfv(du[i]), c1));
     if (i < n - 2) t = df_sub(t, df_mul(dfv(du2[i]), c2));
     c2 = c1;
-    c1 = df_mul(df_sub(t, df_mul(dfv(du[i]), c1)), dfv(d[i]));
+    c1 = df_mul(t, dfv(d[i]));
     y[i] = f2(c1);
   }
 }

@@ -18,20 +18,10 @@ SLS_DEV dfloat df_div(dfloat a, dfloat b) {
 
 SLS_DEV dfloat df_scale(dfloat a, float s) { return df_make(a.hi * s, a.lo * s); }
 
-// a - b with an error of 2^-47 (|a| + |b|) at most (df_sub: of the result), a
-// third shorter.
-SLS_DEV dfloat df_sub_abs(dfloat a, dfloat b) {
-  float s, e;
-  two_sum(a.hi, -b.hi, s, e);
-  return df_norm(s, __fadd_rn(e, __fsub_rn(a.lo, b.lo)));
-}
-
 // Number of eigenvalues of the (scaled) tridiagonal below x, from the signs of
 // the leading principal minors p_i(x) (three-term recurrence, Sturm sequence).
 // Powers of two rescale the pair (p_{i-1}, p_i) to keep it in range; a zero
-// minor takes the sign opposite to its predecessor.  An error in a minor that is
-// small beside its two terms acts as a relative change of b_{i-1}^2 and a_i - x,
-// which is why their difference needs no more than df_sub_abs.
+// minor takes the sign opposite to its predecessor.
 SLS_DEV int sturm_count(const float2* __restrict__ a, const float2* __restrict__ b2, int n,
                         dfloat x) {
   dfloat pm = df_make(1.f, 0.f), pc = df_sub(dfv(a[0]), x);
@@ -42,7 +32,7 @@ SLS_DEV int sturm_count(const float2* __restrict__ a, const float2* __restrict__
   for (int i = 1; i < n; ++i) {
     const dfloat d = df_sub(dfv(a[i]), x);
     const dfloat t = df_mul(dfv(b2[i - 1]), pm);
-    const dfloat pn = df_sub_abs(df_mul(d, pc), t);
+    const dfloat pn = df_sub(df_mul(d, pc), t);
     pm = pc;
     pc = pn;
     const float mg = fmaxf(fabsf(pc.hi), fabsf(pm.hi));
