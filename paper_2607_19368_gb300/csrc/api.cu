@@ -586,6 +586,9 @@ int sls_feature_map(const void* X, int x_dtype, int64_t N, int d, int64_t ldx, c
   if (x_dtype == SLS_BF16) {
     const int st = launch_feature_map_tc(X, N, d, ldx, W, b, D, Phi, s);
     if (st != SLS_ERR_UNSUPPORTED) return st;
+  } else {
+    const int st = launch_feature_map_tf32(X, N, d, ldx, W, b, D, Phi, s, 0);
+    if (st != SLS_ERR_UNSUPPORTED) return st;
   }
   return launch_feature_map_simt(X, x_dtype, N, d, ldx, W, b, D, Phi, s);
 }
@@ -602,6 +605,9 @@ int sls_feature_map_ex(const void* X, int x_dtype, int64_t N, int d, int64_t ldx
   cudaStream_t s = (cudaStream_t)stream;
   if (x_dtype == SLS_BF16) {
     const int st = launch_feature_map_tc(X, N, d, ldx, W, b, D, Phi, s, nullptr, 1);
+    if (st != SLS_ERR_UNSUPPORTED) return st;
+  } else {
+    const int st = launch_feature_map_tf32(X, N, d, ldx, W, b, D, Phi, s, 1);
     if (st != SLS_ERR_UNSUPPORTED) return st;
   }
   return launch_feature_map_simt(X, x_dtype, N, d, ldx, W, b, D, Phi, s, 1);

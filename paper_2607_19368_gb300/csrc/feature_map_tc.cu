@@ -161,6 +161,16 @@ SLS_DEV float rff_cos_fast(float x) {
   return __uint_as_float(__float_as_uint(v) ^ ((unsigned)((q + 1) & 2) << 30));
 }
 
+// th = scale * cos(th) for a warp's rows, amax the largest |th| of the thread
+SLS_DEV void rff_cos_block(float (&th)[32], float amax, float scale) {
+  if (__all_sync(0xffffffffu, amax <= RFF_COS_FAST_MAX)) {
+#pragma unroll
+    for (int e = 0; e < 32; ++e) th[e] = scale * rff_cos_fast(th[e]);
+  } else {
+    for (int e = 0; e < 32; ++e) th[e] = scale * rff_cos_wide(th[e]);
+  }
+}
+
 // TMA tensor store of a 32 x 32 float32 block (3-d map: feature, row, prompt)
 // from shared memory, tracked as a bulk async group of the issuing thread.
 SLS_DEV void tma_store_3d(const CUtensorMap* map, uint32_t src, int x, int y, int z) {
@@ -403,12 +413,7 @@ feature_map_tc_kernel(const __grid_constant__ CUtensorMap tmX,
           amax = fmaxf(amax, fmaxf(fmaxf(fabsf(th[e]), fabsf(th[e + 1])),
                                    fmaxf(fabsf(th[e + 2]), fabsf(th[e + 3]))));
         }
-        if (__all_sync(0xffffffffu, amax <= RFF_COS_FAST_MAX)) {
-#pragma unroll
-          for (int e = 0; e < 32; ++e) th[e] = scale * rff_cos_fast(th[e]);
-        } else {
-          for (int e = 0; e < 32; ++e) th[e] = scale * rff_cos_wide(th[e]);
-        }
+        rff_cos_block(th, amax, scale);
         if constexpr (sizeof(OT) == 4) {
           // row `lane` of the block: its eight 16-byte pieces at the swizzled
           // positions (piece c of row l goes to c ^ (l mod 8))
@@ -452,6 +457,303 @@ feature_map_tc_kernel(const __grid_constant__ CUtensorMap tmX,
   }
 }
 
+// ---------------------------------------------------------------------------
+// Float32 inputs on the tensor cores.  Each float32 is split into a tf32 part
+// (its upper 11 significand bits: what kind::tf32 reads of a float32) and a tf32
+// remainder, and X W^T is the sum of three products, hi hi + lo hi + hi lo; the
+// parts left out are below 2^-20 of a product.  The tensor core adds into its
+// float32 accumulator with truncation, so only the hi hi products of TF_CH slices
+// of K go into one accumulator, which the epilogue warps add into float32
+// registers; the small products of all of K have their own.  The error against
+// float64 stays below that of one chain of float32 multiply-adds over K (N(0,1)
+// inputs, K = 512 / 1024 / 2048 / 4096: rms of the feature 2.2 / 2.2 / 2.3 / 2.4 e-7
+// against 3.0 / 4.1 / 5.8 / 8.1, largest 1.7 / 1.7 / 2.3 / 2.1 e-6 against 3.8 / 5.1 /
+// 10 / 9.4; four slices per accumulator would exceed it at K = 512).
+//
+// 128 x 128 tiles, one CTA per SM: warp 0 copies the 128 x 32 float32 tiles of X
+// and W (three stages), warps 2-7 write each stage's remainders beside it (same
+// swizzled offsets), warp 1 issues the MMAs, warps 8-15 add up the slices (a row
+// quarter and half the columns each) and store.  Bound by shared memory: an MMA
+// of K = 8 reads 8 KB at 128 bytes a cycle, and the copy and the split move
+// another 96 KB per stage.  N = 4084, d = 2048, D = 1024 395 -> 122 us; N = 8192,
+// d = 1024, D = 512 209 -> 67; N = 1000, d = 2048, D = 1024 147 -> 65.
+// ---------------------------------------------------------------------------
+constexpr int TF_BM = 128, TF_BN = 128, TF_BK = 32, TF_STAGES = 3;
+constexpr int TF_CH = 2;             // K slices of TF_BK per accumulator
+constexpr int TF_TILE = 128 * 128;   // bytes of one 128 x 32 float32 tile
+constexpr int TF_STAGE_BYTES = 4 * TF_TILE;  // X, W, and their remainders
+constexpr int TF_THREADS = 512, TF_SPLIT_WARPS = 6, TF_EPI_WARPS = 8;
+constexpr int TF_TMEM_COLS = 512;    // two accumulators of hi hi products, two of small ones
+constexpr size_t TF_SMEM =
+    (size_t)TF_STAGES * TF_STAGE_BYTES + (size_t)TF_EPI_WARPS * TC_OUT_BYTES + 1024;
+// kind::tf32: float32 accumulator, tf32 A and B, both K-major, M = N = 128
+constexpr uint32_t TF_IDESC = (1u << 4) | (2u << 7) | (2u << 10) |
+                              ((uint32_t)(TF_BN >> 3) << 17) | ((uint32_t)(TF_BM >> 4) << 24);
+
+SLS_DEV void tf_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
+      "l"(adesc), "l"(bdesc), "r"(TF_IDESC), "r"(accumulate)
+      : "memory");
+}
+
+// What x exceeds its tf32 part by, set up to be read as tf32 rounded to nearest
+// (the part itself is read truncated).  An infinity or NaN is carried by its
+// tf32 part alone.
+SLS_DEV float tf_rest(float x) {
+  const float lo = x - __uint_as_float(__float_as_uint(x) & 0xffffe000u);
+  return __uint_as_float(__float_as_uint(lo) + 0x1000u);
+}
+
+template <typename OT>
+__global__ void __launch_bounds__(TF_THREADS, 1)
+feature_map_tf32_kernel(const __grid_constant__ CUtensorMap tmX,
+                        const __grid_constant__ CUtensorMap tmW,
+                        const __grid_constant__ CUtensorMap tmPhi, const float* __restrict__ bvec,
+                        OT* __restrict__ Phi, int rows, int D, int K, float scale, int* status) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  __shared__ uint64_t full_bar[TF_STAGES], split_bar[TF_STAGES], empty_bar[TF_STAGES], tfull[2],
+      tempty[2], done_bar;
+  __shared__ uint32_t tmem_holder;
+  __shared__ volatile int s_abort;
+  unsigned char* smem = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const uint32_t smem_base = smem_u32(smem);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n_tiles = (D + TF_BN - 1) / TF_BN;
+  const int num_tiles = ((rows + TF_BM - 1) / TF_BM) * n_tiles;
+  const int k_blocks = (K + TF_BK - 1) / TF_BK;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < TF_STAGES; ++s) {
+      mbar_init(&full_bar[s], 1);
+      mbar_init(&split_bar[s], TF_SPLIT_WARPS);
+      mbar_init(&empty_bar[s], 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(&tfull[a], 1);
+      mbar_init(&tempty[a], TF_EPI_WARPS);
+    }
+    mbar_init(&done_bar, 1);
+    mbar_fence_init();
+    s_abort = 0;
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_holder)),
+                 "r"(TF_TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_holder;
+  auto fail = [&]() {
+    s_abort = 1;
+    atomicExch(status, SLS_ERR_TIMEOUT);
+  };
+
+  if (warp == 0) {
+    // ------------------------------ TMA producer ------------------------------
+    if (lane == 0) {
+      unsigned it = 0;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+        const int mb = tile / n_tiles, nb = tile % n_tiles;
+        for (int kb = 0; kb < k_blocks; ++kb, ++it) {
+          const int s = it % TF_STAGES;
+          if (!tc_wait(&empty_bar[s], ((it / TF_STAGES) & 1u) ^ 1u, &s_abort)) {
+            fail();
+            ok = false;
+            break;
+          }
+          const uint32_t dst = smem_base + s * TF_STAGE_BYTES;
+          mbar_expect_tx(&full_bar[s], 2 * TF_TILE);
+          tma_load_2d(dst, &tmX, kb * TF_BK, mb * TF_BM, smem_u32(&full_bar[s]));
+          tma_load_2d(dst + TF_TILE, &tmW, kb * TF_BK, nb * TF_BN, smem_u32(&full_bar[s]));
+        }
+      }
+      // drain: every issued stage has landed before the CTA may exit
+      const unsigned first = it > TF_STAGES ? it - TF_STAGES : 0;
+      for (unsigned c = first; c < it; ++c) {
+        for (unsigned w = 0; w < (1u << 25); ++w) {
+          if (mbar_try_wait(&full_bar[c % TF_STAGES], (c / TF_STAGES) & 1u)) break;
+          __nanosleep(20);
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------ MMA issuer --------------------------------
+    if (lane == 0) {
+      unsigned it = 0, ch = 0, tl = 0;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++tl) {
+        // (the accumulator of the tile before last: its reader is past it, for it
+        // has released a slice of the last tile)
+        const uint32_t d_low = tmem_base + (uint32_t)((2 + (tl & 1)) * TF_BN);
+        for (int k0 = 0; k0 < k_blocks && ok; k0 += TF_CH, ++ch) {
+          const int acc = ch & 1;
+          if (!tc_wait(&tempty[acc], ((ch >> 1) & 1u) ^ 1u, &s_abort)) {
+            fail();
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t d_main = tmem_base + (uint32_t)(acc * TF_BN);
+          const int k1 = min(k0 + TF_CH, k_blocks);
+          for (int kb = k0; kb < k1; ++kb, ++it) {
+            const int s = it % TF_STAGES;
+            const unsigned par = (it / TF_STAGES) & 1u;
+            if (!tc_wait(&full_bar[s], par, &s_abort) || !tc_wait(&split_bar[s], par, &s_abort)) {
+              fail();
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t ah = smem_base + s * TF_STAGE_BYTES, bh = ah + TF_TILE;
+            const uint32_t al = ah + 2 * TF_TILE, bl = ah + 3 * TF_TILE;
+#pragma unroll
+            for (int kk = 0; kk < TF_BK / 8; ++kk) {
+              const uint32_t o = kk * 32, more = (kb > k0 || kk > 0) ? 1u : 0u;
+              tf_mma(d_main, sw128_desc(ah + o), sw128_desc(bh + o), more);
+              tf_mma(d_low, sw128_desc(al + o), sw128_desc(bh + o), kb > 0 || kk > 0 ? 1u : 0u);
+              tf_mma(d_low, sw128_desc(ah + o), sw128_desc(bl + o), 1u);
+            }
+            tc_commit(smem_u32(&empty_bar[s]));
+          }
+          if (ok) tc_commit(smem_u32(&tfull[acc]));
+        }
+      }
+      // all MMAs issued by this thread have completed before TMEM is freed
+      tc_commit(smem_u32(&done_bar));
+      for (unsigned w = 0; w < (1u << 25); ++w) {
+        if (mbar_try_wait(&done_bar, 0)) break;
+        __nanosleep(20);
+      }
+    }
+  } else if (warp < 2 + TF_SPLIT_WARPS) {
+    // ------------------------------ split -------------------------------------
+    const int t = threadIdx.x - 64;
+    unsigned it = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
+      for (int kb = 0; kb < k_blocks; ++kb, ++it) {
+        const int s = it % TF_STAGES;
+        if (!tc_wait(&full_bar[s], (it / TF_STAGES) & 1u, &s_abort)) {
+          if (lane == 0) fail();
+          ok = false;
+          break;
+        }
+        const float4* src = reinterpret_cast<const float4*>(smem + s * TF_STAGE_BYTES);
+        float4* dst = reinterpret_cast<float4*>(smem + s * TF_STAGE_BYTES + 2 * TF_TILE);
+        // (all loads before the stores: N = 4084, d = 2048, D = 1024 in 13% less time)
+        constexpr int NX = 2 * TF_TILE / 16, ST = 32 * TF_SPLIT_WARPS;
+        float4 x[(NX + ST - 1) / ST];
+#pragma unroll
+        for (int j = 0; j < (NX + ST - 1) / ST; ++j)
+          if (t + j * ST < NX) x[j] = src[t + j * ST];
+#pragma unroll
+        for (int j = 0; j < (NX + ST - 1) / ST; ++j)
+          if (t + j * ST < NX)
+            dst[t + j * ST] =
+                make_float4(tf_rest(x[j].x), tf_rest(x[j].y), tf_rest(x[j].z), tf_rest(x[j].w));
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&split_bar[s]);
+      }
+    }
+  } else {
+    // ------------------------------ epilogue ----------------------------------
+    const int q = warp & 3, half = (warp - 8) >> 2;  // TMEM lane quarter, column half
+    unsigned char* stg = smem + TF_STAGES * TF_STAGE_BYTES + (warp - 8) * TC_OUT_BYTES;
+    const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 64);
+    unsigned ch = 0, tl = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++tl) {
+      const int mb = tile / n_tiles, nb = tile % n_tiles;
+      float sum[2][32];
+#pragma unroll
+      for (int e = 0; e < 32; ++e) sum[0][e] = sum[1][e] = 0.f;
+      for (int k0 = 0; k0 < k_blocks; k0 += TF_CH, ++ch) {
+        const int acc = ch & 1;
+        if (!tc_wait(&tfull[acc], (ch >> 1) & 1u, &s_abort)) {
+          if (lane == 0) fail();
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        auto add = [&](int at) {  // the warp's columns of the accumulator at column `at`
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            uint32_t v[32];
+            tc_ld32(lane_base + (uint32_t)(at + c * 32), v);
+#pragma unroll
+            for (int e = 0; e < 32; ++e) sum[c][e] += __uint_as_float(v[e]);
+          }
+        };
+        add(acc * TF_BN);
+        if (k0 + TF_CH >= k_blocks) add((2 + (int)(tl & 1)) * TF_BN);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tempty[acc]);
+      }
+      if (!ok) break;
+      const int row = mb * TF_BM + q * 32 + lane;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int col = nb * TF_BN + half * 64 + c * 32;
+        if (col >= D) break;
+        float amax = 0.f;
+#pragma unroll
+        for (int e = 0; e < 32; e += 4) {
+          const float4 bq = col + e < D ? __ldg(reinterpret_cast<const float4*>(bvec + col + e))
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+          sum[c][e] += bq.x;
+          sum[c][e + 1] += bq.y;
+          sum[c][e + 2] += bq.z;
+          sum[c][e + 3] += bq.w;
+          amax = fmaxf(amax, fmaxf(fmaxf(fabsf(sum[c][e]), fabsf(sum[c][e + 1])),
+                                   fmaxf(fabsf(sum[c][e + 2]), fabsf(sum[c][e + 3]))));
+        }
+        // (a NaN fails no comparison of amax and comes out as NaN either way)
+        rff_cos_block(sum[c], amax, scale);
+        if constexpr (sizeof(OT) == 4) {
+          if (lane == 0) bulk_wait_all();  // the previous block has left the buffer
+          __syncwarp();
+#pragma unroll
+          for (int g = 0; g < 8; ++g)
+            *reinterpret_cast<float4*>(stg + lane * 128 + ((g ^ (lane & 7)) << 4)) = make_float4(
+                sum[c][4 * g], sum[c][4 * g + 1], sum[c][4 * g + 2], sum[c][4 * g + 3]);
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0 && mb * TF_BM + q * 32 < rows)
+            tma_store_3d(&tmPhi, smem_u32(stg), col, mb * TF_BM + q * 32, 0);
+        } else {
+          if (row < rows) {
+            OT* out = Phi + (int64_t)row * D + col;
+#pragma unroll
+            for (int e = 0; e < 32; e += 4)
+              if (col + e < D)
+                store4(out + e,
+                       make_float4(sum[c][e], sum[c][e + 1], sum[c][e + 2], sum[c][e + 3]));
+          }
+        }
+      }
+    }
+    if (lane == 0) bulk_wait_all();
+    __syncwarp();
+  }
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                 "r"(TF_TMEM_COLS)
+                 : "memory");
+  }
+}
+
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
                                   const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -472,16 +774,17 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
+// 128-byte wide boxes (64 bf16 or 32 float32 columns)
 bool make_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint64_t ld,
-              uint32_t box_rows) {
+              uint32_t box_rows, bool f32 = false) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[2] = {cols, rows};
-  const cuuint64_t strides[1] = {ld * 2};
-  const cuuint32_t box[2] = {(cuuint32_t)TC_BK, box_rows};
+  const cuuint64_t strides[1] = {ld * (f32 ? 4 : 2)};
+  const cuuint32_t box[2] = {(cuuint32_t)(f32 ? TF_BK : TC_BK), box_rows};
   const cuuint32_t estr[2] = {1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+  return fn(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+            const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -564,6 +867,46 @@ int launch_feature_map_tc(const void* X, int64_t N, int d, int64_t ldx, const vo
                           int* status, int phi_bf16) {
   return launch_feature_map_tc_batched(X, 1, N, N, d, ldx, W, b, D, Phi, nullptr, 0, 0, stream,
                                        status, phi_bf16);
+}
+
+// Depth and tiles from which float32 inputs go to the tensor cores.  Below K = 512
+// a chain of float32 multiply-adds is as exact; few tiles leave most SMs idle (us,
+// float32 kernel / this one: 8 tiles, d = 512 19 / 25; 12 tiles, d = 2048 70 / 71;
+// 24 tiles, d = 2048 89 / 65; 32 tiles, d = 512 32 / 24).
+constexpr int TF_MIN_K = 512;
+constexpr int64_t TF_MIN_TILES = 24;
+
+int launch_feature_map_tf32(const void* X, int64_t N, int d, int64_t ldx, const void* W,
+                            const float* b, int D, void* Phi, cudaStream_t stream, int phi_bf16) {
+  const int64_t tiles = ((N + TF_BM - 1) / TF_BM) * ((D + TF_BN - 1) / TF_BN);
+  if (d < TF_MIN_K || tiles < TF_MIN_TILES || N > (int64_t)INT32_MAX - TF_BM ||
+      tiles > (int64_t)INT32_MAX || D % 4 != 0 || d % 4 != 0 || ldx % 4 != 0)
+    return SLS_ERR_UNSUPPORTED;
+  if (((uintptr_t)X & 15) || ((uintptr_t)W & 15) || ((uintptr_t)b & 15) || ((uintptr_t)Phi & 15))
+    return SLS_ERR_UNSUPPORTED;
+  CUtensorMap mx, mw, mp;
+  memset(&mp, 0, sizeof(mp));
+  if (!make_map(&mx, X, (uint64_t)N, (uint64_t)d, (uint64_t)ldx, TF_BM, true) ||
+      !make_map(&mw, W, (uint64_t)D, (uint64_t)d, (uint64_t)d, TF_BN, true) ||
+      (!phi_bf16 && !make_out_map(&mp, Phi, (uint64_t)D, (uint64_t)N, 1)))
+    return SLS_ERR_UNSUPPORTED;
+  int* st = nullptr;
+  SLS_CUDA_TRY(cudaGetSymbolAddress((void**)&st, g_fm_status));
+  const int grid = tiles < sm_count() ? (int)tiles : sm_count();
+  const float scale = (float)sqrt(2.0 / (double)D);
+  if (phi_bf16) {
+    SLS_CUDA_TRY(cudaFuncSetAttribute(feature_map_tf32_kernel<uint16_t>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TF_SMEM));
+    feature_map_tf32_kernel<uint16_t><<<grid, TF_THREADS, TF_SMEM, stream>>>(
+        mx, mw, mp, b, (uint16_t*)Phi, (int)N, D, d, scale, st);
+  } else {
+    SLS_CUDA_TRY(cudaFuncSetAttribute(feature_map_tf32_kernel<float>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TF_SMEM));
+    feature_map_tf32_kernel<float><<<grid, TF_THREADS, TF_SMEM, stream>>>(
+        mx, mw, mp, b, (float*)Phi, (int)N, D, d, scale, st);
+  }
+  SLS_LAUNCH_CHECK();
+  return SLS_OK;
 }
 
 }  // namespace sls
