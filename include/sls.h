@@ -447,14 +447,13 @@ int sls_selftest_wait_limit(int which, void* workspace, size_t workspace_bytes,
 /*
  * Self-test of the Lanczos kernel's failure path (the paper has no
  * counterpart): sls_lanczos_topr (float32 Phi, tol = 1e-10, same arguments
- * and workspace) with its first CTA reporting, at its first barrier, a wait
+ * and workspace) with its first CTA reporting, at its first exchange, a wait
  * that gave up.  The kernel then takes the path of a real give-up: the other
- * CTAs are released at once, the copy warps stop after their own bounded
- * wait (about a second), the status word reads SLS_ERR_TIMEOUT, *r_eff stays
+ * CTAs' polls stop at once, every copy in flight lands, the status word reads SLS_ERR_TIMEOUT, *r_eff stays
  * -1, theta and U are zero, and the context stays usable.  No fault, trap or
  * hang is involved.  Errors: those of sls_lanczos_topr; UNSUPPORTED when the
  * problem runs on the one-warp small-window kernel (N <= 32), which has no
- * barrier to fail.
+ * exchange to fail.
  */
 int sls_selftest_lanczos_giveup(const float* Phi, int64_t N, int D, int r, const double* q1,
                                 double* theta, float* U, int32_t* r_eff, void* workspace,

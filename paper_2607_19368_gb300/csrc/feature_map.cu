@@ -2,9 +2,9 @@
 //   Phi[i, c] = sqrt(2/D) * cos( X[i, :] . W[c, :] + b[c] ),  W = Omega^T (D x d).
 //
 // The contraction X W^T is GEMM-shaped (M = tokens, N = features, K = d).
-// This file holds the fp32 SIMT kernel (used for float32 embeddings and as
-// the reference path for small shapes); the bf16 tcgen05 kernel lives in
-// feature_map_tc.cu.  Both fuse the bias, cosine and scale into the epilogue,
+// This file holds the fp32 SIMT kernel (shallow or small float32 contractions,
+// unaligned or odd shapes); the tcgen05 kernels for bf16 and for deep float32
+// inputs live in feature_map_tc.cu.  All fuse the bias, cosine and scale into the epilogue,
 // so Phi is written exactly once, as float32 or (opt-in) as bfloat16 rounded
 // to nearest even from the float32 value.
 #include "common.cuh"

@@ -1,4 +1,5 @@
-// Random Fourier feature map on the 5th-generation tensor cores (sm_103a):
+// Random Fourier feature map on the 5th-generation tensor cores (sm_103a), bf16
+// inputs (float32 inputs: feature_map_tf32_kernel below):
 //   Phi = sqrt(2/D) * cos(X W^T + b)      (Sec. 3.2, Eq. rff_map)
 // X (N x d) and W = Omega^T (D x d) are bf16, K-major (row-major, K = d
 // contiguous); the contraction accumulates in fp32 in tensor memory; the

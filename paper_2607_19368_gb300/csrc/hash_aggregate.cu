@@ -6,7 +6,8 @@
 // segment.cuh).  The per-problem bookkeeping -- a stable radix sort of
 // (code, token), cluster boundaries, the merge or D'Hondt split to exactly m
 // groups, group positions and the ordering of groups by position -- runs in
-// one 1024-thread CTA per problem and touches only integers.  Reading X and
+// one 1024-thread CTA per problem (a cluster of them for one large problem, a
+// warp for windows of at most 32 tokens) and touches only integers.  Reading X and
 // writing the macro-token embeddings is spread over the whole GPU.
 #include <climits>
 
@@ -2217,7 +2218,7 @@ int launch_agg_t(const void* X, int d, int64_t ldx, const int* perm, const int* 
   SLS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   agg_items_kernel<<<AI_CL, SEG_T, 0, stream>>>(mlen, Mtot, aux, items, pt_start);
   SLS_LAUNCH_CHECK();
-  // CTAs that fit the GPU at once (NV <= 2: four per SM), each every grid-th item
+  // CTAs that fit the GPU at once; items by ticket
   int occ = 0;
   SLS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, agg_member_kernel<T, NV>,
                                                              AGG_T, 0));
