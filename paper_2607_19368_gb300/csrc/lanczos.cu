@@ -240,9 +240,9 @@ tridiag_eigvals_kernel(LanczosBatch bt) {
 // dependent chain holds no memory access; pivoting selects operands instead of
 // branching; the first forward solve rides along the factorisation; and the back
 // substitution multiplies by the pivots' reciprocals.  The work arrays (n entries
-// each) belong to the caller.  WARP: the lanes of a warp run the recurrences
-// alike, on arrays in shared memory, and share the loops over entries; else one
-// thread computes the cluster (sums over n as four interleaved partial sums).
+// each) belong to the caller.  WARP: a warp's lanes share the loops over entries of
+// arrays in shared memory; else one thread runs them (sums over n as four
+// interleaved partial sums).
 SLS_DEV dfloat sum4_df(dfloat (&acc)[4]) {
   return df_add(df_add(acc[0], acc[1]), df_add(acc[2], acc[3]));
 }
@@ -339,25 +339,46 @@ SLS_DEV void eig_back(int n, dfloat cy, const float2* __restrict__ d,
   }
 }
 
+// Deterministic start vector of column mm, entry i.
+SLS_DEV float eig_start(int mm, int i) {
+  unsigned h = (unsigned)(i + 1) * 2654435761u ^ (unsigned)(mm + 7) * 40503u;
+  h ^= h >> 13;
+  h *= 0x5bd1e995u;
+  h ^= h >> 15;
+  return 0.5f + (float)(h & 0xffffu) / 65536.f;
+}
+
+// The shift of column mm of the cluster that starts at column first: distinct
+// inside a cluster.
+SLS_DEV dfloat eig_shift(const double* th, int mm, int first, double pert, double sc) {
+  return df_from_double((th[mm] - (double)(mm - first) * 4.0 * pert) * sc);
+}
+
+// Keep the iterate y in range (divide by its largest entry, a power of two).
 template <bool WARP>
-SLS_DEV void eigvec_cluster(const LanczosBatch& bt, int p, int n, int first, int last,
-                            double sc, double tnorm, const float2* __restrict__ sa,
-                            const float2* __restrict__ sb, float2* __restrict__ d,
-                            float2* __restrict__ du, float2* __restrict__ du2,
-                            float2* __restrict__ dl, float2* __restrict__ y,
-                            unsigned char* __restrict__ piv) {
-  const int r = bt.r;
-  double* S = bt.S + (size_t)p * r * r;
-  const double* th = bt.theta + (size_t)p * r;
-  const double pert = 0x1p-44 * tnorm;
-  const dfloat pert_df = df_from_double(pert * sc);
+SLS_DEV void eig_rescale(int n, float2* __restrict__ y) {
   const int i0 = WARP ? (threadIdx.x & 31) : 0;
   constexpr int di = WARP ? 32 : 1;
-  // lanes that hold alike what each has written meet before and after a loop
-  // that they share
-  auto meet = [] {
-    if (WARP) __syncwarp();
-  };
+  float ymax = 0.f;
+  for (int i = i0; i < n; i += di) ymax = fmaxf(ymax, fabsf(y[i].x));
+  if (WARP)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ymax = fmaxf(ymax, __shfl_xor_sync(0xffffffffu, ymax, o));
+  if (ymax > 0.f && isfinite(ymax)) {
+    int e2 = 0;
+    frexpf(ymax, &e2);
+    const float s2 = ldexpf(1.f, -e2);
+    for (int i = i0; i < n; i += di) y[i] = f2(df_scale(dfv(y[i]), s2));
+  }
+}
+
+// Orthogonalise y against columns first .. mm - 1 of S, the cluster members found
+// so far, and normalise it.
+template <bool WARP>
+SLS_DEV void eig_orthonormalise(int n, int r, int first, int mm, const double* __restrict__ S,
+                                float2* __restrict__ y) {
+  const int i0 = WARP ? (threadIdx.x & 31) : 0;
+  constexpr int di = WARP ? 32 : 1;
   auto dot_all = [&](auto term) {  // sum of term(i) over i < n
     if constexpr (WARP) {
       dfloat acc = df_make(0.f, 0.f);
@@ -370,60 +391,63 @@ SLS_DEV void eigvec_cluster(const LanczosBatch& bt, int p, int n, int first, int
       return sum4_df(acc);
     }
   };
+  for (int pm = first; pm < mm; ++pm) {
+    const dfloat dot =
+        dot_all([&](int i) { return df_mul(df_from_double(S[(size_t)i * r + pm]), dfv(y[i])); });
+    for (int i = i0; i < n; i += di)
+      y[i] = f2(df_sub(dfv(y[i]), df_mul(dot, df_from_double(S[(size_t)i * r + pm]))));
+  }
+  const double nr =
+      sqrt(df_to_double(dot_all([&](int i) { return df_mul(dfv(y[i]), dfv(y[i])); })));
+  if (!(nr > 0.0) || !isfinite(nr)) {
+    for (int i = i0; i < n; i += di) y[i] = make_float2((i == mm) ? 1.f : 0.f, 0.f);
+  } else {
+    const dfloat inv = df_from_double(1.0 / nr);
+    for (int i = i0; i < n; i += di) y[i] = f2(df_mul(dfv(y[i]), inv));
+  }
+}
+
+// Column mm of S from y, its first entry made non-negative.
+template <bool WARP>
+SLS_DEV void eig_store(int n, int r, int mm, const float2* __restrict__ y,
+                       double* __restrict__ S) {
+  const double sg = (y[0].x < 0.f) ? -1.0 : 1.0;
+#pragma unroll 4
+  for (int i = WARP ? (threadIdx.x & 31) : 0; i < n; i += WARP ? 32 : 1)
+    S[(size_t)i * r + mm] = sg * df_to_double(dfv(y[i]));
+}
+
+// The cluster [first, last] by one warp, on arrays in shared memory: the lanes run
+// the recurrences alike and share the loops over entries, meeting between the two.
+SLS_DEV void eigvec_cluster(const LanczosBatch& bt, int p, int n, int first, int last,
+                            double sc, double tnorm, const float2* __restrict__ sa,
+                            const float2* __restrict__ sb, float2* __restrict__ d,
+                            float2* __restrict__ du, float2* __restrict__ du2,
+                            float2* __restrict__ dl, float2* __restrict__ y,
+                            unsigned char* __restrict__ piv) {
+  const int r = bt.r;
+  double* S = bt.S + (size_t)p * r * r;
+  const double pert = 0x1p-44 * tnorm;
+  const dfloat pert_df = df_from_double(pert * sc);
   for (int mm = first; mm <= last; ++mm) {
-    // distinct shifts inside a cluster
-    const dfloat shift = df_from_double((th[mm] - (double)(mm - first) * 4.0 * pert) * sc);
+    const dfloat shift = eig_shift(bt.theta + (size_t)p * r, mm, first, pert, sc);
     if (n == 1) {
       y[0] = make_float2(1.f, 0.f);
     } else {
-      // deterministic start vector
-      auto y0 = [mm](int i) {
-        unsigned h = (unsigned)(i + 1) * 2654435761u ^ (unsigned)(mm + 7) * 40503u;
-        h ^= h >> 13;
-        h *= 0x5bd1e995u;
-        h ^= h >> 15;
-        return 0.5f + (float)(h & 0xffffu) / 65536.f;
-      };
       for (int it = 0; it < 2; ++it) {
-        const dfloat cy = it == 0
-                              ? eig_factor(n, shift, pert_df, y0, sa, sb, d, du, du2, dl, y, piv)
-                              : eig_forward(n, dl, y, piv);
+        const dfloat cy = it == 0 ? eig_factor(n, shift, pert_df,
+                                               [mm](int i) { return eig_start(mm, i); }, sa, sb,
+                                               d, du, du2, dl, y, piv)
+                                  : eig_forward(n, dl, y, piv);
         eig_back(n, cy, d, du, du2, y);
-        meet();
-        // keep the iterate in range: divide by its largest entry (a power of two)
-        float ymax = 0.f;
-        for (int i = i0; i < n; i += di) ymax = fmaxf(ymax, fabsf(y[i].x));
-        if (WARP)
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) ymax = fmaxf(ymax, __shfl_xor_sync(0xffffffffu, ymax, o));
-        if (ymax > 0.f && isfinite(ymax)) {
-          int e2 = 0;
-          frexpf(ymax, &e2);
-          const float s2 = ldexpf(1.f, -e2);
-          for (int i = i0; i < n; i += di) y[i] = f2(df_scale(dfv(y[i]), s2));
-        }
-        // orthogonalise against the cluster members found so far
-        for (int pm = first; pm < mm; ++pm) {
-          const dfloat dot = dot_all(
-              [&](int i) { return df_mul(df_from_double(S[(size_t)i * r + pm]), dfv(y[i])); });
-          for (int i = i0; i < n; i += di)
-            y[i] = f2(df_sub(dfv(y[i]), df_mul(dot, df_from_double(S[(size_t)i * r + pm]))));
-        }
-        const double nr =
-            sqrt(df_to_double(dot_all([&](int i) { return df_mul(dfv(y[i]), dfv(y[i])); })));
-        if (!(nr > 0.0) || !isfinite(nr)) {
-          for (int i = i0; i < n; i += di) y[i] = make_float2((i == mm) ? 1.f : 0.f, 0.f);
-        } else {
-          const dfloat inv = df_from_double(1.0 / nr);
-          for (int i = i0; i < n; i += di) y[i] = f2(df_mul(dfv(y[i]), inv));
-        }
-        meet();
+        __syncwarp();
+        eig_rescale<true>(n, y);
+        eig_orthonormalise<true>(n, r, first, mm, S, y);
+        __syncwarp();
       }
     }
-    const double sg = (y[0].x < 0.f) ? -1.0 : 1.0;
-#pragma unroll 4
-    for (int i = i0; i < n; i += di) S[(size_t)i * r + mm] = sg * df_to_double(dfv(y[i]));
-    meet();
+    eig_store<true>(n, r, mm, y, S);
+    __syncwarp();
   }
 }
 
@@ -465,12 +489,13 @@ tridiag_eigvecs_kernel(LanczosBatch bt) {
   const double sc = eig_scale(bt.theta + (size_t)p * r, n, &tnorm);
   eig_scaled_T(bt, p, n, sc, lane, 32, sa, sb);
   __syncwarp();
-  eigvec_cluster<true>(bt, p, n, first, last, sc, tnorm, sa, sb, d, du, du2, dl, y, piv);
+  eigvec_cluster(bt, p, n, first, last, sc, tnorm, sa, sb, d, du, du2, dl, y, piv);
 }
 
 // Many small problems (r <= 32): one warp per problem, one lane per Ritz value;
-// the lane of a cluster's first member computes the whole cluster, with its
-// work arrays in local memory.
+// every lane factors and solves once, then a cluster's members take turns at the
+// rest, which needs the finished ones (2048 windows of 16 tokens: 12 us less than
+// with the whole cluster on its first member's lane).  Work arrays in local memory.
 constexpr int EIGW_WARPS = 1;  // one problem per CTA: the fewest idle SMs at the end
 constexpr int EIGW_MAXR = 32;
 // Ritz values up to which a warp computes each eigenvector (32 values: 22 us, a
@@ -499,14 +524,39 @@ tridiag_eigvecs_warp_kernel(LanczosBatch bt) {
     eig_scaled_T(bt, p, n, sc, lane, 32, sa[warp], sb[warp]);
   }
   __syncwarp();
-  if (lane >= n) return;
-  int first, last;
-  eig_cluster(bt.theta + (size_t)p * r, n, lane, first, last);
-  if (first != lane) return;
+  int first = lane, last = lane;
   float2 d[EIGW_MAXR], du[EIGW_MAXR], du2[EIGW_MAXR], dl[EIGW_MAXR], y[EIGW_MAXR];
   unsigned char piv[EIGW_MAXR];
-  eigvec_cluster<false>(bt, p, n, first, last, sc, tnorm, sa[warp], sb[warp], d, du, du2, dl, y,
-                        piv);
+  const double pert = 0x1p-44 * tnorm;
+  if (lane < n) {
+    const double* th = bt.theta + (size_t)p * r;
+    eig_cluster(th, n, lane, first, last);
+    if (n == 1) {
+      y[0] = make_float2(1.f, 0.f);
+    } else {
+      const dfloat cy = eig_factor(n, eig_shift(th, lane, first, pert, sc),
+                                   df_from_double(pert * sc),
+                                   [lane](int i) { return eig_start(lane, i); }, sa[warp],
+                                   sb[warp], d, du, du2, dl, y, piv);
+      eig_back(n, cy, d, du, du2, y);
+      eig_rescale<false>(n, y);
+    }
+  }
+  // then the members of a cluster in turn, the clusters side by side
+  const int turns = (int)__reduce_max_sync(0xffffffffu, (unsigned)(lane - first)) + 1;
+  for (int k = 0; k < turns; ++k) {
+    if (lane < n && lane - first == k) {
+      if (n > 1) {
+        eig_orthonormalise<false>(n, r, first, lane, S, y);
+        const dfloat cy = eig_forward(n, dl, y, piv);
+        eig_back(n, cy, d, du, du2, y);
+        eig_rescale<false>(n, y);
+        eig_orthonormalise<false>(n, r, first, lane, S, y);
+      }
+      eig_store<false>(n, r, lane, y, S);
+    }
+    __syncwarp();
+  }
 }
 
 // ----------------------------------------------------------------------------
