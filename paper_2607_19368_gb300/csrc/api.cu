@@ -621,7 +621,6 @@ int sls_feature_map_batched(const void* X, int64_t nb, int64_t rows, int64_t x_s
   if (live && (nwin < 1 || win < 1 || (int64_t)nwin * win < rows)) return SLS_ERR_INVALID_ARG;
   if (nb == 0 || rows == 0) return SLS_OK;
   if (!X || !W || !b || !Phi) return SLS_ERR_INVALID_ARG;
-  if (D % 256 != 0) return SLS_ERR_UNSUPPORTED;
   return launch_feature_map_tc_batched(X, nb, rows, x_stride, d, ldx, W, b, D, Phi, live, nwin,
                                        win, (cudaStream_t)stream, nullptr);
 }

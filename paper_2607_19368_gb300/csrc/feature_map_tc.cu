@@ -8,11 +8,7 @@
 //
 // One persistent CTA per SM, 128 x 256 output tiles (tile index -> prompt,
 // then m-block, then n-block innermost, so the D/256 tiles that share an X
-// block run at the same time and X is read from HBM once).  The last n-block may
-// be ragged (any D % 4 == 0): the copy engine fills the missing rows of W with
-// zeros and clips the stores.  Even a quarter of the columns in use leaves the
-// tensor cores ahead of the float32 kernel that took these shapes before: N =
-// 8000, d = 2048, D = 1000 1163 -> 38 us; N = 300, d = 1024, D = 64 100 -> 19 us.  One launch covers
+// block run at the same time and X is read from HBM once).  One launch covers
 // a batch of prompts (equal row counts, a fixed row stride in X); with a
 // per-window route table, the row tiles whose windows all went to the chunk
 // path (Sec. 3.6) are skipped by every role alike.  Warp roles:
@@ -242,7 +238,7 @@ feature_map_tc_kernel(const __grid_constant__ CUtensorMap tmX,
   const uint32_t smem_base = smem_u32(smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m_tiles = (J.rows + TC_BM - 1) / TC_BM;
-  const int n_tiles = (D + TC_BN - 1) / TC_BN;  // the last may be ragged (D % 4 == 0)
+  const int n_tiles = D / TC_BN;
   const int per_prompt = m_tiles * n_tiles;
   const int num_tiles = J.nb * per_prompt;
   const int k_blocks = (K + TC_BK - 1) / TC_BK;
@@ -395,18 +391,14 @@ feature_map_tc_kernel(const __grid_constant__ CUtensorMap tmX,
       tc_fence_after();
       const int row = mb * TC_BM + q * 32 + lane;
       const float* bb = bvec + (size_t)nb * TC_BN;
-      // a ragged tile ends at its last 32-column block; the tensor store clips
-      // the block's columns past D
-      const int bn = min(TC_BN, D - nb * TC_BN);
-      for (int c0 = 0; c0 < bn; c0 += 32, ++blk) {
+      for (int c0 = 0; c0 < TC_BN; c0 += 32, ++blk) {
         uint32_t v[32];
         tc_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * TC_BN + c0), v);
         float th[32];
         float amax = 0.f;
 #pragma unroll
         for (int e = 0; e < 32; e += 4) {
-          const float4 bq = c0 + e < bn ? __ldg(reinterpret_cast<const float4*>(bb + c0 + e))
-                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+          const float4 bq = __ldg(reinterpret_cast<const float4*>(bb + c0 + e));
           th[e + 0] = __uint_as_float(v[e + 0]) + bq.x;
           th[e + 1] = __uint_as_float(v[e + 1]) + bq.y;
           th[e + 2] = __uint_as_float(v[e + 2]) + bq.z;
@@ -436,7 +428,7 @@ feature_map_tc_kernel(const __grid_constant__ CUtensorMap tmX,
             OT* out = Phi + ((int64_t)pb * J.rows + row) * D + (int64_t)nb * TC_BN + c0;
 #pragma unroll
             for (int e = 0; e < 32; e += 4)
-              if (c0 + e < bn) store4(out + e, make_float4(th[e], th[e + 1], th[e + 2], th[e + 3]));
+              store4(out + e, make_float4(th[e], th[e + 1], th[e + 2], th[e + 3]));
           }
         }
       }
@@ -823,12 +815,11 @@ int launch_feature_map_tc_batched(const void* X, int64_t nb, int64_t rows, int64
                                   void* Phi, const int* live, int nwin, int win,
                                   cudaStream_t stream, int* status, int phi_bf16) {
   // shapes the kernel covers; anything else takes the SIMT path
-  if (nb <= 0 || rows <= 0 || x_stride < rows || D % 4 != 0 || d % 8 != 0 || ldx % 8 != 0)
+  if (nb <= 0 || rows <= 0 || x_stride < rows || D % TC_BN != 0 || d % 8 != 0 || ldx % 8 != 0)
     return SLS_ERR_UNSUPPORTED;
   const int64_t map_rows = (nb - 1) * x_stride + rows;
   const int64_t m_tiles = (rows + TC_BM - 1) / TC_BM;
-  const int64_t tiles = nb * m_tiles * ((D + TC_BN - 1) / TC_BN);
-  if (map_rows > (int64_t)INT32_MAX - TC_BM || tiles > (int64_t)INT32_MAX)
+  if (map_rows > (int64_t)INT32_MAX - TC_BM || nb * m_tiles * (D / TC_BN) > (int64_t)INT32_MAX)
     return SLS_ERR_UNSUPPORTED;
   if (live && (nwin < 1 || win < 1)) return SLS_ERR_INVALID_ARG;
   if (((uintptr_t)X & 15) || ((uintptr_t)W & 15) || ((uintptr_t)b & 15) || ((uintptr_t)Phi & 15))
@@ -850,6 +841,7 @@ int launch_feature_map_tc_batched(const void* X, int64_t nb, int64_t rows, int64
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
   SLS_CUDA_TRY(cudaFuncSetAttribute(feature_map_tc_kernel<uint16_t>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
+  const int64_t tiles = nb * m_tiles * (D / TC_BN);
   const int grid = tiles < sm_count() ? (int)tiles : sm_count();
   const float scale = (float)sqrt(2.0 / (double)D);
   FmJob J{(int)nb, (int)rows, (int)x_stride, live, nwin, win};

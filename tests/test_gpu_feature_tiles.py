@@ -1,8 +1,7 @@
 """The feature map (Sec. 3.2, Eq. rff_map) at the edges of its tiles: the float32
 kernel's three tile sizes with ragged rows, features and depth, unaligned and
-strided inputs, the tensor-core kernel's ragged last feature block, and the
-three-product kernel that takes deep float32 contractions.  Every feature within
-the float32 bound of the oracle."""
+strided inputs, and the three-product kernel that takes deep float32
+contractions.  Every feature within the float32 bound of the oracle."""
 import math
 
 import numpy as np
@@ -10,8 +9,7 @@ import pytest
 import torch
 
 import oracle as O
-import workloads as WL
-from tests.gpu_util import feature_tolerance, to_torch_x, widen
+from tests.gpu_util import feature_tolerance
 
 pytestmark = pytest.mark.gpu
 
@@ -59,25 +57,6 @@ def test_feature_map_f32_strided_rows(sls):
         wide[:, :64] = torch.from_numpy(X)
         _check(sls.feature_map(wide[:, :64], torch.from_numpy(W).cuda(), torch.from_numpy(b).cuda()),
                X.astype(np.float64), W.astype(np.float64), b)
-
-
-@pytest.mark.parametrize("phi", [torch.float32, torch.bfloat16])
-@pytest.mark.parametrize("N,d,D", [(129, 72, 4), (300, 64, 100), (257, 200, 260), (128, 64, 316),
-                                   (400, 128, 776)])
-def test_feature_map_tc_ragged_features(sls, N, d, D, phi):
-    X, W, b = _inputs(N, d, D, D)
-    Xb, Wb = WL.f32_to_bf16_bits(X), WL.f32_to_bf16_bits(W)
-    guard = torch.full((N + 1, D), 7.0, device="cuda", dtype=phi)
-    got = sls.feature_map(to_torch_x(Xb, "bf16"), to_torch_x(Wb, "bf16"),
-                          torch.from_numpy(b).cuda(), out=guard[:N])
-    assert torch.all(guard[N] == 7.0)
-    X64, W64 = widen(Xb, "bf16"), widen(Wb, "bf16")
-    if phi == torch.float32:
-        _check(got, X64, W64, b)
-    else:
-        want = O.rff_features(X64, W64, b)
-        tol = feature_tolerance(X64, W64, b.astype(np.float64)) + 2.0 ** -8 * np.abs(want)
-        assert np.all(np.abs(got.float().cpu().numpy() - want) <= tol)
 
 
 # the smallest and ragged shapes of the float32 inputs that go to the tensor cores
