@@ -27,6 +27,7 @@
 // eigenvectors and U = Q S come from the same kernels as there.
 #include <cfloat>
 
+#include "common.cuh"
 #include "kernels.cuh"
 #include "tridiag.cuh"
 

@@ -3,7 +3,7 @@
 // bisection and multisection search on.
 #pragma once
 
-#include "common.cuh"
+#include "dfloat.cuh"
 
 namespace sls {
 
