@@ -449,15 +449,33 @@ int sls_selftest_wait_limit(int which, void* workspace, size_t workspace_bytes,
  * counterpart): sls_lanczos_topr (float32 Phi, tol = 1e-10, same arguments
  * and workspace) with its first CTA reporting, at its first exchange, a wait
  * that gave up.  The kernel then takes the path of a real give-up: the other
- * CTAs' polls stop at once, every copy in flight lands, the status word reads SLS_ERR_TIMEOUT, *r_eff stays
- * -1, theta and U are zero, and the context stays usable.  No fault, trap or
- * hang is involved.  Errors: those of sls_lanczos_topr; UNSUPPORTED when the
+ * CTAs' polls stop at once, every copy in flight lands, the status word reads
+ * SLS_ERR_TIMEOUT, *r_eff stays -1, theta and U are zero, and the context stays
+ * usable.  No fault, trap or hang is involved.  Errors: those of sls_lanczos_topr; UNSUPPORTED when the
  * problem runs on the one-warp small-window kernel (N <= 32), which has no
  * exchange to fail.
  */
 int sls_selftest_lanczos_giveup(const float* Phi, int64_t N, int D, int r, const double* q1,
                                 double* theta, float* U, int32_t* r_eff, void* workspace,
                                 size_t workspace_bytes, void* stream);
+
+/*
+ * Self-test of the compression pass's status word where the feature map gives
+ * up (the paper has no counterpart): sls_compress (same arguments and
+ * workspace) with the first CTA of the float32 tensor-core feature map
+ * reporting a wait that gave up.  That CTA leaves its tiles of Phi unwritten,
+ * the rest of the pass runs, and sls_workspace_status() reads SLS_ERR_TIMEOUT;
+ * the outputs are not to be used.  Zero the workspace before the call, so that
+ * the unwritten part of Phi holds finite values.  Errors: those of
+ * sls_compress; UNSUPPORTED when the pass would not run that kernel (bf16
+ * embeddings, the chunk backend, an identity call, or a shape that the float32
+ * kernel keeps).
+ */
+int sls_selftest_compress_giveup(const sls_config_t* cfg, const void* X, int x_dtype, int64_t B,
+                                 int64_t N, int d, int64_t ldx, const sls_params_t* params,
+                                 float* Xt, int32_t* pos, int32_t* tok2macro, int32_t* r_eff,
+                                 int32_t* route, void* workspace, size_t workspace_bytes,
+                                 void* stream);
 
 /*
  * Self-test of the debug build's checks (a library built with -DSLS_DEBUG,

@@ -27,7 +27,7 @@ __all__ = [
     "compress_workspace_size", "workspace_status", "EXPORTED", "PHASES",
     "set_phase_events", "launch_count", "Workspace", "embed_gather", "compress_tokens",
     "compress_tokens_workspace_size", "TokensWorkspace", "selftest_wait_limit",
-    "lanczos_topr_batched", "selftest_lanczos_giveup",
+    "lanczos_topr_batched", "selftest_lanczos_giveup", "selftest_compress_giveup",
 ]
 
 SLS_OK = 0
@@ -143,6 +143,9 @@ EXPORTED = {
                                         _vp, _d, _vp, _vp, _vp, _vp, _vp, _vp, _sz, _vp]),
     "sls_selftest_lanczos_giveup": (_i32, [_vp, _i64, _i32, _i32, _vp, _vp, _vp, _vp, _vp, _sz,
                                            _vp]),
+    "sls_selftest_compress_giveup": (_i32, [ctypes.POINTER(Config), _vp, _i32, _i64, _i64, _i32,
+                                            _i64, ctypes.POINTER(_Params), _vp, _vp, _vp, _vp,
+                                            _vp, _vp, _sz, _vp]),
     "sls_debug_selftest": (_i32, [_i32, _vp, _sz, _vp]),
     "sls_set_phase_events": (_i32, [ctypes.POINTER(ctypes.c_void_p), _i32]),
     "sls_launch_count": (_i64, []),
@@ -470,6 +473,25 @@ def compress(X: torch.Tensor, cfg: Config, W: Optional[torch.Tensor] = None,
     if not batched:
         return Xt[0], pos[0], t2m[0], r_eff, route
     return Xt, pos, t2m, r_eff, route
+
+
+def selftest_compress_giveup(X: torch.Tensor, cfg: Config, W: torch.Tensor, b: torch.Tensor,
+                             R: torch.Tensor, q1: torch.Tensor, workspace: Workspace) -> int:
+    """compress() of one float32 prompt with the feature map's give-up path
+    injected (see sls_selftest_compress_giveup); returns the status word of the
+    workspace, SLS_ERR_TIMEOUT = 5 when the failure was reported as designed."""
+    _need_cuda(X, W, b, R, q1)
+    N, d = X.shape
+    M, Xt, pos, t2m, r_eff, route = _outputs(cfg, 1, N, d, X.device, None)
+    params, keep = _params(cfg, M, N, 1, False, X.device, W, b, R, q1)
+    workspace.buf.zero_()
+    st = lib().sls_selftest_compress_giveup(
+        ctypes.byref(cfg), _ptr(X), _dtype_code(X), 1, N, d, X.stride(0), ctypes.byref(params),
+        _ptr(Xt), _ptr(pos), _ptr(t2m), _ptr(r_eff), _ptr(route), _ptr(workspace.buf),
+        workspace.nbytes, _stream(X))
+    _check("sls_selftest_compress_giveup", st)
+    del keep
+    return workspace_status(workspace)
 
 
 def embed_gather(table: torch.Tensor, ids: torch.Tensor, out: Optional[torch.Tensor] = None,

@@ -492,6 +492,21 @@ size_t tail_bytes(const CompressPlan& P, int64_t toks, int d, int backend) {
   return cv.off;
 }
 
+// The feature map by the kernel that takes the shape: tensor cores for bf16 and
+// for deep float32 inputs, else the float32 kernel (which holds no wait).
+// status: where a device-side wait that gave up is reported (NULL: a word of the
+// library).  inject_fail = 1: the float32 tensor-core kernel's give-up path.
+int feature_map_any(const void* X, int x_dtype, int64_t N, int d, int64_t ldx, const void* W,
+                    const float* b, int D, void* Phi, int phi_bf16, int* status, cudaStream_t s,
+                    int inject_fail = 0) {
+  const int st = x_dtype == SLS_BF16
+                     ? launch_feature_map_tc(X, N, d, ldx, W, b, D, Phi, s, status, phi_bf16)
+                     : launch_feature_map_tf32(X, N, d, ldx, W, b, D, Phi, s, status, phi_bf16,
+                                               inject_fail);
+  if (st != SLS_ERR_UNSUPPORTED || inject_fail) return st;
+  return launch_feature_map_simt(X, x_dtype, N, d, ldx, W, b, D, Phi, s, phi_bf16);
+}
+
 // One Lanczos problem (sls_lanczos_topr_ex); inject_fail = 1 runs the
 // failure self-test (the kernel's give-up path, see LanczosBatch).
 int lanczos_single(const void* Phi, int phi_dtype, int64_t N, int D, int r, const double* q1,
@@ -553,6 +568,187 @@ int lanczos_single(const void* Phi, int phi_dtype, int64_t N, int D, int r, cons
   return guards_check(cv, status, s);
 }
 
+// The whole pass (sls_compress); inject_fail = 1 runs the failure self-test (the
+// give-up path of the float32 tensor-core feature map).
+int compress_pass(const sls_config_t* cfg, const void* X, int x_dtype, int64_t B, int64_t N, int d,
+                  int64_t ldx, const sls_params_t* params, float* Xt, int32_t* pos,
+                  int32_t* tok2macro, int32_t* r_eff, int32_t* route, void* workspace,
+                  size_t workspace_bytes, void* stream, int inject_fail) {
+  int st = validate_config(cfg);
+  if (st != SLS_OK) return st;
+  if (B < 1 || N < 1 || d < 1 || ldx < d || B * N > (1LL << 30)) return SLS_ERR_INVALID_ARG;
+  if (x_dtype != SLS_F32 && x_dtype != SLS_BF16) return SLS_ERR_INVALID_ARG;
+  if (!ptr_ok(X) || !Xt || !pos || !tok2macro) return SLS_ERR_INVALID_ARG;
+  cudaStream_t s = (cudaStream_t)stream;
+  if (is_identity(cfg, N)) {
+    // the workspace (if any) holds only the status word
+    if (workspace && workspace_bytes >= 256) SLS_CUDA_TRY(cudaMemsetAsync(workspace, 0, 256, s));
+    return launch_identity(X, x_dtype, B, N, d, ldx, Xt, pos, tok2macro, s);
+  }
+  const int vec = (x_dtype == SLS_BF16) ? 8 : 4;
+  if (d % vec || ldx % vec || d > SLS_MAX_D) return SLS_ERR_UNSUPPORTED;
+  CompressPlan P;
+  if ((st = make_plan(cfg, B, N, &P)) != SLS_OK) return st;
+  const bool spectral = cfg->backend != SLS_BACKEND_CHUNK;
+  if (spectral) {
+    if (!params || !params->W || !params->b || !params->R || !params->q1)
+      return SLS_ERR_INVALID_ARG;
+    if (params->R_ld < cfg->r || params->R_rows < P.bits_max) return SLS_ERR_INVALID_ARG;
+    if (B > 1 && params->q1_stride < P.Nc) return SLS_ERR_INVALID_ARG;
+  }
+  CompressWs W;
+  carve(P, workspace, &W);
+  const size_t need = W.total + tail_bytes(P, B * N, d, cfg->backend);
+  if (!workspace || workspace_bytes < need) return SLS_ERR_WORKSPACE;
+  {
+    Carver tail((char*)workspace + W.total);
+    W.part = tail.take<float>(agg_part_capacity(B * N) * (size_t)d);
+    W.part_eta = tail.take<float>(agg_part_capacity(B * N));
+    W.score_part = (cfg->backend == SLS_BACKEND_ADAPTIVE)
+                       ? tail.take<float>(score_part_floats(P.nprob, B * N, d))
+                       : nullptr;
+    W.tail = tail;
+  }
+  SLS_CUDA_TRY(cudaMemsetAsync(W.status, 0, 256, s));
+  if ((st = guards_arm(W.cv, s)) != SLS_OK) return st;
+  if ((st = guards_arm(W.tail, s)) != SLS_OK) return st;
+  const int nprob = (int)P.nprob;
+  phase_mark(0, 0, s);
+  // problem table
+  {
+    // bit counts of the two window lengths (formed here: the float64 loop took
+    // the kernel 14 us for 2048 windows)
+    const int bits_full = cfg->bits > 0 ? cfg->bits : auto_bits(P.bud.L_full, cfg->rho);
+    const int bits_last = cfg->bits > 0 ? cfg->bits : auto_bits(P.bud.L_last, cfg->rho);
+    plan_kernel<<<(unsigned)((nprob + 127) / 128), 128, 0, s>>>(
+        W.probs, nprob, (int)P.bud.W, N, P.M, P.pf, P.Nc, P.bud.L_full, P.bud.m_full,
+        P.bud.m_last, P.bud.left_full, P.bud.L_last, bits_full, bits_last, spectral ? 1 : 0,
+        cfg->backend == SLS_BACKEND_CHUNK ? P.k_chunk : 0, spectral ? params->q1_stride : 0);
+    SLS_LAUNCH_CHECK();
+  }
+  // routing; at rho >= 16 every window is spectral and no score is needed
+  int mode = spectral ? 0 : 1;
+  if (cfg->backend == SLS_BACKEND_ADAPTIVE) {
+    mode = 2;
+    // below rho = 16 the score pass also writes every window's chunk-path
+    // output, so the segment and aggregation steps only see spectral windows
+    if (cfg->rho < 16.0 &&
+        (st = launch_window_score_chunk(X, x_dtype, d, ldx, W.probs, nprob, P.nmax, P.mmax, B * N,
+                                        W.part, W.score_part, W.score, cfg->pos_scheme,
+                                        cfg->pos_mode, cfg->renorm, Xt, pos, tok2macro, s)) != SLS_OK)
+      return st;
+  }
+  double tau = cfg->tau;
+  if (cfg->tau_schedule) {
+    tau = 0.75 - 0.05 * std::log2(cfg->rho);
+    if (tau > 0.70) tau = 0.70;
+    if (tau < 0.55) tau = 0.55;
+  }
+  int32_t* rflags = route ? route : W.route;
+  route_compact_kernel<<<1, 1024, 0, s>>>(W.probs, nprob, mode, W.score, cfg->rho, tau,
+                                          W.spec_list, W.lz_row0, W.lz_n, W.lz_q1off, W.nspec,
+                                          rflags, W.r_eff);
+  SLS_LAUNCH_CHECK();
+  phase_mark(0, 1, s);
+  phase_mark(1, 0, s);
+  if (spectral) {
+    // features of the compressible rows of every prompt, in one launch on the
+    // tensor cores (bf16); windows routed to the chunk path are skipped
+    st = SLS_ERR_UNSUPPORTED;
+    if (x_dtype == SLS_BF16)
+      st = launch_feature_map_tc_batched(
+          (const char*)X + (size_t)P.pf * ldx * 2, B, P.Nc, N, d, ldx, params->W, params->b,
+          cfg->D, W.Phi, mode == 2 ? rflags : nullptr, (int)P.bud.W, (int)P.bud.L_full, s,
+          W.status, P.phi_bf16);
+    if (st == SLS_ERR_UNSUPPORTED) {
+      const size_t esz = P.phi_bf16 ? 2 : 4;
+      for (int64_t b = 0; b < B; ++b) {
+        const char* xb = (const char*)X +
+                         (size_t)(b * N + P.pf) * ldx * (x_dtype == SLS_BF16 ? 2 : 4);
+        st = feature_map_any(xb, x_dtype, P.Nc, d, ldx, params->W, params->b, cfg->D,
+                             (char*)W.Phi + (size_t)b * P.Nc * cfg->D * esz, P.phi_bf16, W.status,
+                             s, inject_fail);
+        if (st != SLS_OK) return st;
+      }
+    }
+    if (st != SLS_OK) return st;
+    // the row-normalised operator: each spectral problem's rows scaled by
+    // 1 / sqrt of its estimated row sums (Sec. 3.2)
+    if (cfg->normalize &&
+        (st = launch_feature_normalize((float*)W.Phi, cfg->D, W.lz_row0, W.lz_n, nprob, W.nspec, 0,
+                                       P.nmax, W.norm_scratch, nullptr, s)) != SLS_OK)
+      return st;
+    phase_mark(1, 1, s);
+    phase_mark(2, 0, s);
+    LanczosBatch bt{};
+    bt.Phi = W.Phi;
+    bt.phi_bf16 = P.phi_bf16;
+    bt.D = cfg->D;
+    bt.r = cfg->r;
+    bt.tol = cfg->lanczos_tol;
+    bt.q1 = params->q1;
+    bt.n_single = 0;
+    bt.nprob_max = nprob;
+    bt.nprob_dev = W.nspec;
+    bt.row0 = W.lz_row0;
+    bt.n = W.lz_n;
+    bt.q1off = W.lz_q1off;
+    bt.Q = W.Q;
+    bt.alpha = W.alpha;
+    bt.beta = W.beta;
+    bt.theta = W.theta;
+    bt.S = W.S;
+    bt.r_eff = W.r_eff;
+    bt.nmax = P.nmax;
+    // windows of at most 32 tokens: one warp per window (values of T included)
+    const bool small = lanczos_window_fits(P.nmax, cfg->D, cfg->r);
+    if (small) {
+      if ((st = launch_lanczos_window(bt, s)) != SLS_OK) return st;
+    } else if ((st = launch_lanczos(bt, W.lz_scratch, W.lz_bytes, W.status, P.lz_groups,
+                                    P.lz_g, s)) != SLS_OK) {
+      return st;
+    }
+    phase_mark(2, 1, s);
+    phase_mark(3, 0, s);
+    if ((st = launch_tridiag_eigen(bt, s, small)) != SLS_OK) return st;
+    if ((st = launch_ritz_vectors(bt, W.U, s)) != SLS_OK) return st;
+    phase_mark(3, 1, s);
+    phase_mark(4, 0, s);
+    if ((st = launch_simhash_problems(W.probs, W.spec_list, W.nspec, nprob, P.nmax, W.r_eff, W.U,
+                                      cfg->r, params->R, params->R_ld, P.bits_max, W.codes, s)) !=
+        SLS_OK)
+      return st;
+    if (r_eff) {
+      finish_reff_kernel<<<(nprob + 255) / 256, 256, 0, s>>>(W.probs, nprob, W.r_eff, r_eff);
+      SLS_LAUNCH_CHECK();
+    }
+    phase_mark(4, 1, s);
+  } else {
+    for (int ph = 1; ph <= 4; ++ph) {
+      if (ph > 1) phase_mark(ph, 0, s);
+      phase_mark(ph, 1, s);
+    }
+  }
+  phase_mark(5, 0, s);
+  const int chunk_done = (cfg->backend == SLS_BACKEND_ADAPTIVE && cfg->rho < 16.0) ? 1 : 0;
+  if ((st = launch_segment(W.probs, nprob, W.codes, cfg->pos_scheme, cfg->pos_mode, W.seg_scratch,
+                           P.seg_slots, P.nmax, P.mmax, W.perm, W.mstart, W.mlen, pos, tok2macro,
+                           W.status, s, chunk_done)) != SLS_OK)
+    return st;
+  if ((st = launch_preserved(B, N, P.M, (int)P.pf, (int)P.pl, cfg->pos_mode, W.perm, W.mstart,
+                             W.mlen, pos, tok2macro, s)) != SLS_OK)
+    return st;
+  phase_mark(5, 1, s);
+  phase_mark(6, 0, s);
+  st = launch_aggregate(X, x_dtype, d, ldx, W.perm, W.mstart, W.mlen, B * P.M, B * N,
+                        cfg->renorm, Xt, W.pt_start, W.items, W.counts, W.part, W.part_eta,
+                        W.status, s);
+  phase_mark(6, 1, s);
+  if (st != SLS_OK) return st;
+  if ((st = guards_check(W.cv, W.status, s)) != SLS_OK) return st;
+  return guards_check(W.tail, W.status, s);
+}
+
 }  // namespace
 
 // ===========================================================================
@@ -582,15 +778,7 @@ int sls_feature_map(const void* X, int x_dtype, int64_t N, int d, int64_t ldx, c
   if (x_dtype != SLS_F32 && x_dtype != SLS_BF16) return SLS_ERR_INVALID_ARG;
   if (N == 0) return SLS_OK;
   if (!X || !W || !b || !Phi) return SLS_ERR_INVALID_ARG;
-  cudaStream_t s = (cudaStream_t)stream;
-  if (x_dtype == SLS_BF16) {
-    const int st = launch_feature_map_tc(X, N, d, ldx, W, b, D, Phi, s);
-    if (st != SLS_ERR_UNSUPPORTED) return st;
-  } else {
-    const int st = launch_feature_map_tf32(X, N, d, ldx, W, b, D, Phi, s, 0);
-    if (st != SLS_ERR_UNSUPPORTED) return st;
-  }
-  return launch_feature_map_simt(X, x_dtype, N, d, ldx, W, b, D, Phi, s);
+  return feature_map_any(X, x_dtype, N, d, ldx, W, b, D, Phi, 0, nullptr, (cudaStream_t)stream);
 }
 
 int sls_feature_map_ex(const void* X, int x_dtype, int64_t N, int d, int64_t ldx, const void* W,
@@ -602,15 +790,7 @@ int sls_feature_map_ex(const void* X, int x_dtype, int64_t N, int d, int64_t ldx
   if (x_dtype != SLS_F32 && x_dtype != SLS_BF16) return SLS_ERR_INVALID_ARG;
   if (N == 0) return SLS_OK;
   if (!X || !W || !b || !Phi) return SLS_ERR_INVALID_ARG;
-  cudaStream_t s = (cudaStream_t)stream;
-  if (x_dtype == SLS_BF16) {
-    const int st = launch_feature_map_tc(X, N, d, ldx, W, b, D, Phi, s, nullptr, 1);
-    if (st != SLS_ERR_UNSUPPORTED) return st;
-  } else {
-    const int st = launch_feature_map_tf32(X, N, d, ldx, W, b, D, Phi, s, 1);
-    if (st != SLS_ERR_UNSUPPORTED) return st;
-  }
-  return launch_feature_map_simt(X, x_dtype, N, d, ldx, W, b, D, Phi, s, 1);
+  return feature_map_any(X, x_dtype, N, d, ldx, W, b, D, Phi, 1, nullptr, (cudaStream_t)stream);
 }
 
 int sls_feature_map_batched(const void* X, int64_t nb, int64_t rows, int64_t x_stride, int d,
@@ -846,179 +1026,20 @@ int sls_compress(const sls_config_t* cfg, const void* X, int x_dtype, int64_t B,
                  int64_t ldx, const sls_params_t* params, float* Xt, int32_t* pos,
                  int32_t* tok2macro, int32_t* r_eff, int32_t* route, void* workspace,
                  size_t workspace_bytes, void* stream) {
-  int st = validate_config(cfg);
-  if (st != SLS_OK) return st;
-  if (B < 1 || N < 1 || d < 1 || ldx < d || B * N > (1LL << 30)) return SLS_ERR_INVALID_ARG;
-  if (x_dtype != SLS_F32 && x_dtype != SLS_BF16) return SLS_ERR_INVALID_ARG;
-  if (!ptr_ok(X) || !Xt || !pos || !tok2macro) return SLS_ERR_INVALID_ARG;
-  cudaStream_t s = (cudaStream_t)stream;
-  if (is_identity(cfg, N)) {
-    // the workspace (if any) holds only the status word
-    if (workspace && workspace_bytes >= 256) SLS_CUDA_TRY(cudaMemsetAsync(workspace, 0, 256, s));
-    return launch_identity(X, x_dtype, B, N, d, ldx, Xt, pos, tok2macro, s);
-  }
-  const int vec = (x_dtype == SLS_BF16) ? 8 : 4;
-  if (d % vec || ldx % vec || d > SLS_MAX_D) return SLS_ERR_UNSUPPORTED;
-  CompressPlan P;
-  if ((st = make_plan(cfg, B, N, &P)) != SLS_OK) return st;
-  const bool spectral = cfg->backend != SLS_BACKEND_CHUNK;
-  if (spectral) {
-    if (!params || !params->W || !params->b || !params->R || !params->q1)
-      return SLS_ERR_INVALID_ARG;
-    if (params->R_ld < cfg->r || params->R_rows < P.bits_max) return SLS_ERR_INVALID_ARG;
-    if (B > 1 && params->q1_stride < P.Nc) return SLS_ERR_INVALID_ARG;
-  }
-  CompressWs W;
-  carve(P, workspace, &W);
-  const size_t need = W.total + tail_bytes(P, B * N, d, cfg->backend);
-  if (!workspace || workspace_bytes < need) return SLS_ERR_WORKSPACE;
-  {
-    Carver tail((char*)workspace + W.total);
-    W.part = tail.take<float>(agg_part_capacity(B * N) * (size_t)d);
-    W.part_eta = tail.take<float>(agg_part_capacity(B * N));
-    W.score_part = (cfg->backend == SLS_BACKEND_ADAPTIVE)
-                       ? tail.take<float>(score_part_floats(P.nprob, B * N, d))
-                       : nullptr;
-    W.tail = tail;
-  }
-  SLS_CUDA_TRY(cudaMemsetAsync(W.status, 0, 256, s));
-  if ((st = guards_arm(W.cv, s)) != SLS_OK) return st;
-  if ((st = guards_arm(W.tail, s)) != SLS_OK) return st;
-  const int nprob = (int)P.nprob;
-  phase_mark(0, 0, s);
-  // problem table
-  {
-    // bit counts of the two window lengths (formed here: the float64 loop took
-    // the kernel 14 us for 2048 windows)
-    const int bits_full = cfg->bits > 0 ? cfg->bits : auto_bits(P.bud.L_full, cfg->rho);
-    const int bits_last = cfg->bits > 0 ? cfg->bits : auto_bits(P.bud.L_last, cfg->rho);
-    plan_kernel<<<(unsigned)((nprob + 127) / 128), 128, 0, s>>>(
-        W.probs, nprob, (int)P.bud.W, N, P.M, P.pf, P.Nc, P.bud.L_full, P.bud.m_full,
-        P.bud.m_last, P.bud.left_full, P.bud.L_last, bits_full, bits_last, spectral ? 1 : 0,
-        cfg->backend == SLS_BACKEND_CHUNK ? P.k_chunk : 0, spectral ? params->q1_stride : 0);
-    SLS_LAUNCH_CHECK();
-  }
-  // routing; at rho >= 16 every window is spectral and no score is needed
-  int mode = spectral ? 0 : 1;
-  if (cfg->backend == SLS_BACKEND_ADAPTIVE) {
-    mode = 2;
-    // below rho = 16 the score pass also writes every window's chunk-path
-    // output, so the segment and aggregation steps only see spectral windows
-    if (cfg->rho < 16.0 &&
-        (st = launch_window_score_chunk(X, x_dtype, d, ldx, W.probs, nprob, P.nmax, P.mmax, B * N,
-                                        W.part, W.score_part, W.score, cfg->pos_scheme,
-                                        cfg->pos_mode, cfg->renorm, Xt, pos, tok2macro, s)) != SLS_OK)
-      return st;
-  }
-  double tau = cfg->tau;
-  if (cfg->tau_schedule) {
-    tau = 0.75 - 0.05 * std::log2(cfg->rho);
-    if (tau > 0.70) tau = 0.70;
-    if (tau < 0.55) tau = 0.55;
-  }
-  int32_t* rflags = route ? route : W.route;
-  route_compact_kernel<<<1, 1024, 0, s>>>(W.probs, nprob, mode, W.score, cfg->rho, tau,
-                                          W.spec_list, W.lz_row0, W.lz_n, W.lz_q1off, W.nspec,
-                                          rflags, W.r_eff);
-  SLS_LAUNCH_CHECK();
-  phase_mark(0, 1, s);
-  phase_mark(1, 0, s);
-  if (spectral) {
-    // features of the compressible rows of every prompt, in one launch on the
-    // tensor cores (bf16); windows routed to the chunk path are skipped
-    st = SLS_ERR_UNSUPPORTED;
-    if (x_dtype == SLS_BF16)
-      st = launch_feature_map_tc_batched(
-          (const char*)X + (size_t)P.pf * ldx * 2, B, P.Nc, N, d, ldx, params->W, params->b,
-          cfg->D, W.Phi, mode == 2 ? rflags : nullptr, (int)P.bud.W, (int)P.bud.L_full, s,
-          W.status, P.phi_bf16);
-    if (st == SLS_ERR_UNSUPPORTED) {
-      const size_t esz = P.phi_bf16 ? 2 : 4;
-      for (int64_t b = 0; b < B; ++b) {
-        const char* xb = (const char*)X +
-                         (size_t)(b * N + P.pf) * ldx * (x_dtype == SLS_BF16 ? 2 : 4);
-        st = sls_feature_map_ex(xb, x_dtype, P.Nc, d, ldx, params->W, params->b, cfg->D,
-                                (char*)W.Phi + (size_t)b * P.Nc * cfg->D * esz,
-                                P.phi_bf16 ? SLS_BF16 : SLS_F32, stream);
-        if (st != SLS_OK) return st;
-      }
-    }
-    if (st != SLS_OK) return st;
-    // the row-normalised operator: each spectral problem's rows scaled by
-    // 1 / sqrt of its estimated row sums (Sec. 3.2)
-    if (cfg->normalize &&
-        (st = launch_feature_normalize((float*)W.Phi, cfg->D, W.lz_row0, W.lz_n, nprob, W.nspec, 0,
-                                       P.nmax, W.norm_scratch, nullptr, s)) != SLS_OK)
-      return st;
-    phase_mark(1, 1, s);
-    phase_mark(2, 0, s);
-    LanczosBatch bt{};
-    bt.Phi = W.Phi;
-    bt.phi_bf16 = P.phi_bf16;
-    bt.D = cfg->D;
-    bt.r = cfg->r;
-    bt.tol = cfg->lanczos_tol;
-    bt.q1 = params->q1;
-    bt.n_single = 0;
-    bt.nprob_max = nprob;
-    bt.nprob_dev = W.nspec;
-    bt.row0 = W.lz_row0;
-    bt.n = W.lz_n;
-    bt.q1off = W.lz_q1off;
-    bt.Q = W.Q;
-    bt.alpha = W.alpha;
-    bt.beta = W.beta;
-    bt.theta = W.theta;
-    bt.S = W.S;
-    bt.r_eff = W.r_eff;
-    bt.nmax = P.nmax;
-    // windows of at most 32 tokens: one warp per window (values of T included)
-    const bool small = lanczos_window_fits(P.nmax, cfg->D, cfg->r);
-    if (small) {
-      if ((st = launch_lanczos_window(bt, s)) != SLS_OK) return st;
-    } else if ((st = launch_lanczos(bt, W.lz_scratch, W.lz_bytes, W.status, P.lz_groups,
-                                    P.lz_g, s)) != SLS_OK) {
-      return st;
-    }
-    phase_mark(2, 1, s);
-    phase_mark(3, 0, s);
-    if ((st = launch_tridiag_eigen(bt, s, small)) != SLS_OK) return st;
-    if ((st = launch_ritz_vectors(bt, W.U, s)) != SLS_OK) return st;
-    phase_mark(3, 1, s);
-    phase_mark(4, 0, s);
-    if ((st = launch_simhash_problems(W.probs, W.spec_list, W.nspec, nprob, P.nmax, W.r_eff, W.U,
-                                      cfg->r, params->R, params->R_ld, P.bits_max, W.codes, s)) !=
-        SLS_OK)
-      return st;
-    if (r_eff) {
-      finish_reff_kernel<<<(nprob + 255) / 256, 256, 0, s>>>(W.probs, nprob, W.r_eff, r_eff);
-      SLS_LAUNCH_CHECK();
-    }
-    phase_mark(4, 1, s);
-  } else {
-    for (int ph = 1; ph <= 4; ++ph) {
-      if (ph > 1) phase_mark(ph, 0, s);
-      phase_mark(ph, 1, s);
-    }
-  }
-  phase_mark(5, 0, s);
-  const int chunk_done = (cfg->backend == SLS_BACKEND_ADAPTIVE && cfg->rho < 16.0) ? 1 : 0;
-  if ((st = launch_segment(W.probs, nprob, W.codes, cfg->pos_scheme, cfg->pos_mode, W.seg_scratch,
-                           P.seg_slots, P.nmax, P.mmax, W.perm, W.mstart, W.mlen, pos, tok2macro,
-                           W.status, s, chunk_done)) != SLS_OK)
-    return st;
-  if ((st = launch_preserved(B, N, P.M, (int)P.pf, (int)P.pl, cfg->pos_mode, W.perm, W.mstart,
-                             W.mlen, pos, tok2macro, s)) != SLS_OK)
-    return st;
-  phase_mark(5, 1, s);
-  phase_mark(6, 0, s);
-  st = launch_aggregate(X, x_dtype, d, ldx, W.perm, W.mstart, W.mlen, B * P.M, B * N,
-                        cfg->renorm, Xt, W.pt_start, W.items, W.counts, W.part, W.part_eta,
-                        W.status, s);
-  phase_mark(6, 1, s);
-  if (st != SLS_OK) return st;
-  if ((st = guards_check(W.cv, W.status, s)) != SLS_OK) return st;
-  return guards_check(W.tail, W.status, s);
+  return compress_pass(cfg, X, x_dtype, B, N, d, ldx, params, Xt, pos, tok2macro, r_eff, route,
+                       workspace, workspace_bytes, stream, 0);
+}
+
+int sls_selftest_compress_giveup(const sls_config_t* cfg, const void* X, int x_dtype, int64_t B,
+                                 int64_t N, int d, int64_t ldx, const sls_params_t* params,
+                                 float* Xt, int32_t* pos, int32_t* tok2macro, int32_t* r_eff,
+                                 int32_t* route, void* workspace, size_t workspace_bytes,
+                                 void* stream) {
+  if (validate_config(cfg) != SLS_OK) return SLS_ERR_INVALID_ARG;
+  if (x_dtype != SLS_F32 || cfg->backend == SLS_BACKEND_CHUNK || is_identity(cfg, N))
+    return SLS_ERR_UNSUPPORTED;
+  return compress_pass(cfg, X, x_dtype, B, N, d, ldx, params, Xt, pos, tok2macro, r_eff, route,
+                       workspace, workspace_bytes, stream, 1);
 }
 
 int sls_embed_gather(const void* table, int x_dtype, int64_t V, int d, int64_t ld_table,

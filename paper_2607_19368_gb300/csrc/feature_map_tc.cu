@@ -504,7 +504,8 @@ __global__ void __launch_bounds__(TF_THREADS, 1)
 feature_map_tf32_kernel(const __grid_constant__ CUtensorMap tmX,
                         const __grid_constant__ CUtensorMap tmW,
                         const __grid_constant__ CUtensorMap tmPhi, const float* __restrict__ bvec,
-                        OT* __restrict__ Phi, int rows, int D, int K, float scale, int* status) {
+                        OT* __restrict__ Phi, int rows, int D, int K, float scale, int* status,
+                        int inject_fail) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ uint64_t full_bar[TF_STAGES], split_bar[TF_STAGES], empty_bar[TF_STAGES], tfull[2],
       tempty[2], done_bar;
@@ -552,7 +553,8 @@ feature_map_tf32_kernel(const __grid_constant__ CUtensorMap tmX,
     // ------------------------------ TMA producer ------------------------------
     if (lane == 0) {
       unsigned it = 0;
-      bool ok = true;
+      bool ok = !(inject_fail && blockIdx.x == 0);
+      if (!ok) fail();
       for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
         const int mb = tile / n_tiles, nb = tile % n_tiles;
         for (int kb = 0; kb < k_blocks; ++kb, ++it) {
@@ -870,7 +872,8 @@ constexpr int TF_MIN_K = 512;
 constexpr int64_t TF_MIN_TILES = 24;
 
 int launch_feature_map_tf32(const void* X, int64_t N, int d, int64_t ldx, const void* W,
-                            const float* b, int D, void* Phi, cudaStream_t stream, int phi_bf16) {
+                            const float* b, int D, void* Phi, cudaStream_t stream, int* status,
+                            int phi_bf16, int inject_fail) {
   const int64_t tiles = ((N + TF_BM - 1) / TF_BM) * ((D + TF_BN - 1) / TF_BN);
   if (d < TF_MIN_K || tiles < TF_MIN_TILES || N > (int64_t)INT32_MAX - TF_BM ||
       tiles > (int64_t)INT32_MAX || D % 4 != 0 || d % 4 != 0 || ldx % 4 != 0)
@@ -883,20 +886,20 @@ int launch_feature_map_tf32(const void* X, int64_t N, int d, int64_t ldx, const 
       !make_map(&mw, W, (uint64_t)D, (uint64_t)d, (uint64_t)d, TF_BN, true) ||
       (!phi_bf16 && !make_out_map(&mp, Phi, (uint64_t)D, (uint64_t)N, 1)))
     return SLS_ERR_UNSUPPORTED;
-  int* st = nullptr;
-  SLS_CUDA_TRY(cudaGetSymbolAddress((void**)&st, g_fm_status));
+  int* st = status;
+  if (!st) SLS_CUDA_TRY(cudaGetSymbolAddress((void**)&st, g_fm_status));
   const int grid = tiles < sm_count() ? (int)tiles : sm_count();
   const float scale = (float)sqrt(2.0 / (double)D);
   if (phi_bf16) {
     SLS_CUDA_TRY(cudaFuncSetAttribute(feature_map_tf32_kernel<uint16_t>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TF_SMEM));
     feature_map_tf32_kernel<uint16_t><<<grid, TF_THREADS, TF_SMEM, stream>>>(
-        mx, mw, mp, b, (uint16_t*)Phi, (int)N, D, d, scale, st);
+        mx, mw, mp, b, (uint16_t*)Phi, (int)N, D, d, scale, st, inject_fail);
   } else {
     SLS_CUDA_TRY(cudaFuncSetAttribute(feature_map_tf32_kernel<float>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TF_SMEM));
     feature_map_tf32_kernel<float><<<grid, TF_THREADS, TF_SMEM, stream>>>(
-        mx, mw, mp, b, (float*)Phi, (int)N, D, d, scale, st);
+        mx, mw, mp, b, (float*)Phi, (int)N, D, d, scale, st, inject_fail);
   }
   SLS_LAUNCH_CHECK();
   return SLS_OK;

@@ -18,9 +18,11 @@ int launch_feature_map_tc(const void* X, int64_t N, int d, int64_t ldx, const vo
                           const float* b, int D, void* Phi, cudaStream_t stream,
                           int* status = nullptr, int phi_bf16 = 0);
 // Float32 X and W on the tensor cores as three tf32 products (deep contractions;
-// SLS_ERR_UNSUPPORTED for the shapes that the float32 kernel keeps).
+// SLS_ERR_UNSUPPORTED for the shapes that the float32 kernel keeps); status as
+// above.  inject_fail: the first CTA's copy warp reports a wait that gave up.
 int launch_feature_map_tf32(const void* X, int64_t N, int d, int64_t ldx, const void* W,
-                            const float* b, int D, void* Phi, cudaStream_t stream, int phi_bf16);
+                            const float* b, int D, void* Phi, cudaStream_t stream,
+                            int* status = nullptr, int phi_bf16 = 0, int inject_fail = 0);
 // The same over nb prompts in one launch: prompt k has `rows` rows starting at
 // X row k * x_stride and writes Phi rows [k * rows, (k + 1) * rows).  With
 // `live` set (one flag per window of `win` rows, nwin per prompt,

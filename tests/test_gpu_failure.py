@@ -72,3 +72,29 @@ def test_lanczos_giveup_leaves_empty_result_and_usable_context(sls):
     assert int(k.item()) == ko
     t = th.cpu().numpy()[:ko]
     assert np.all(np.abs(t - th_o) <= 1e-4 * np.abs(th_o) + 1e-12 * abs(th_o[0]))
+
+
+def test_feature_map_giveup_reaches_the_pass_status(sls):
+    """A wait of the float32 tensor-core feature map that gives up inside
+    compress() is reported by the workspace's status word, as it is for bf16;
+    the same workspace then serves a normal pass."""
+    g = torch.Generator(device="cuda").manual_seed(9)
+    N, d, D, r = 1500, 512, 256, 16
+    X = torch.randn(N, d, generator=g, device="cuda") / d ** 0.5
+    W = torch.randn(D, d, generator=g, device="cuda") * d ** -0.25
+    b = torch.rand(D, generator=g, device="cuda") * 6.28
+    R = torch.randn(32, r, generator=g, device="cuda")
+    q1 = torch.randn(N, generator=g, device="cuda", dtype=torch.float64)
+    cfg = sls.Config.make(rho=4.0, D=D, r=r, bits=8)
+    ws = sls.Workspace(cfg, 1, N, d, X.device)
+    t0 = time.time()
+    assert sls.selftest_compress_giveup(X, cfg, W, b, R, q1, ws) == 5
+    assert time.time() - t0 < 30.0
+    Xt, pos, t2m, _, _ = sls.compress(X, cfg, W, b, R, q1, workspace=ws)
+    assert sls.workspace_status(ws) == 0
+    again = sls.compress(X, cfg, W, b, R, q1)
+    assert torch.equal(t2m, again[2]) and torch.equal(Xt, again[0])
+    # shapes without that kernel are refused instead of passing untested
+    with pytest.raises(sls.SLSError):
+        sls.selftest_compress_giveup(X[:, :256].contiguous(), cfg, W[:, :256].contiguous(), b, R, q1,
+                                     sls.Workspace(cfg, 1, N, 256, X.device))
