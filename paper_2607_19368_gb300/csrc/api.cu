@@ -317,6 +317,8 @@ struct CompressPlan {
   Budgets bud;
   int64_t nprob;     // problems (B * W)
   int64_t nmax, mmax;
+  int64_t nlong;     // tokens of the longest window (nmax is the window length, which
+                     // a short prompt does not fill)
   int D, r;
   int bits_max;
   int lz_groups, lz_g;
@@ -335,7 +337,7 @@ struct CompressWs {
   int64_t* lz_q1off;
   int* nspec;
   float* score;
-  float* score_part;  // window-score sums of short windows (adaptive backend)
+  float* score_part;  // window-score sums that the partial rows cannot hold (adaptive)
   float2* norm_scratch;  // row-normalised operator: column sums
   int32_t* route;  // spectral flag per problem
   void* Phi;  // float32, or bfloat16 bits when the plan stores Phi as bf16
@@ -399,6 +401,7 @@ int make_plan(const sls_config_t* c, int64_t B, int64_t N, CompressPlan* P,
   P->nmax = P->bud.L_full > P->bud.L_last ? P->bud.L_full : P->bud.L_last;
   P->mmax = P->bud.m_full + 1 > P->bud.m_last ? P->bud.m_full + 1 : P->bud.m_last;
   if (P->mmax > P->nmax) P->mmax = P->nmax;
+  P->nlong = P->nmax < R.Nc ? P->nmax : R.Nc;
   if (c->bits > 0) {
     P->bits_max = c->bits;
   } else {
@@ -488,7 +491,8 @@ size_t tail_bytes(const CompressPlan& P, int64_t toks, int d, int backend) {
   Carver cv(nullptr);
   cv.take<float>(agg_part_capacity(toks) * (size_t)d);
   cv.take<float>(agg_part_capacity(toks));
-  if (backend == SLS_BACKEND_ADAPTIVE) cv.take<float>(score_part_floats(P.nprob, toks, d));
+  if (backend == SLS_BACKEND_ADAPTIVE)
+    cv.take<float>(score_part_floats(P.nprob, P.nlong, toks, d));
   return cv.off;
 }
 
@@ -605,7 +609,7 @@ int compress_pass(const sls_config_t* cfg, const void* X, int x_dtype, int64_t B
     W.part = tail.take<float>(agg_part_capacity(B * N) * (size_t)d);
     W.part_eta = tail.take<float>(agg_part_capacity(B * N));
     W.score_part = (cfg->backend == SLS_BACKEND_ADAPTIVE)
-                       ? tail.take<float>(score_part_floats(P.nprob, B * N, d))
+                       ? tail.take<float>(score_part_floats(P.nprob, P.nlong, B * N, d))
                        : nullptr;
     W.tail = tail;
   }
@@ -633,7 +637,7 @@ int compress_pass(const sls_config_t* cfg, const void* X, int x_dtype, int64_t B
     // below rho = 16 the score pass also writes every window's chunk-path
     // output, so the segment and aggregation steps only see spectral windows
     if (cfg->rho < 16.0 &&
-        (st = launch_window_score_chunk(X, x_dtype, d, ldx, W.probs, nprob, P.nmax, P.mmax, B * N,
+        (st = launch_window_score_chunk(X, x_dtype, d, ldx, W.probs, nprob, P.nlong, B * N,
                                         W.part, W.score_part, W.score, cfg->pos_scheme,
                                         cfg->pos_mode, cfg->renorm, Xt, pos, tok2macro, s)) != SLS_OK)
       return st;

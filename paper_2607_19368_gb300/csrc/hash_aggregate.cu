@@ -1744,7 +1744,13 @@ agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __rest
 // add 0.  Every window is cut into parts; a CTA takes a part, reduces each row's
 // |x|^2 (per warp, then across warps through a double-buffered shared array, one
 // barrier per batch of agg_batch<NV>() rows) and writes the part's sums of x and
-// of x/|x|; window_score_combine_kernel adds a window's parts and forms the score.
+// of x/|x|; window_score_combine_kernel adds a window's parts in order and forms
+// the score.  The parts are a function of the window and the row width alone, so a
+// window's score, and with it its route, has the same bits alone, in any batch and
+// on any number of SMs, and no chain of sums grows with the batch.  About 128 rows
+// each (64 of rows wider than 4096): parts that fill the GPU evenly for the batch at
+// hand are a little faster (16 prompts of 16384 tokens, d = 4096: the pass in 572 us
+// against 599; one prompt 132 against 141), parts of 256 rows slower (607; 189).
 
 // ---------------------------------------------------------------------------
 // The score pass with the chunk path folded in (adaptive backend below rho =
@@ -1765,8 +1771,14 @@ __host__ __device__ inline int chunk_gstart(int n, int m, int g) {
   const int q = n / m, rem = n % m;
   return (g < rem) ? g * (q + 1) : rem * (q + 1) + (g - rem) * q;
 }
-// groups per part when m groups are cut into at most np parts
-__host__ __device__ inline int chunk_gpp(int m, int np) { return (m + np - 1) / np; }
+// parts of a window of n tokens, at most, and groups per part
+__host__ __device__ inline int score_parts(int64_t n, int d) {
+  const int rows = d > 4096 ? 64 : 128;
+  return n < rows ? 1 : (int)(n / rows);
+}
+__host__ __device__ inline int score_gpp(int n, int m, int d) {
+  return (m + score_parts(n, d) - 1) / score_parts(n, d);
+}
 
 // 16-byte asynchronous copy global -> shared (zero-filled when !live), and
 // the wait for all but the newest `pending` groups of a thread's copies.
@@ -1807,7 +1819,7 @@ window_score_chunk_kernel(const T* __restrict__ X, int d, int64_t ldx,
     const ProbDesc P = probs[p];
     const int n = P.n, m = P.m;
     if (n <= 0 || m <= 0) continue;
-    const int gp = chunk_gpp(m, KP);
+    const int gp = score_gpp(n, m, d);
     if (k >= (m + gp - 1) / gp) continue;
     const int g0 = k * gp, g1 = min(m, g0 + gp);
     const int r0 = chunk_gstart(n, m, g0), r1 = chunk_gstart(n, m, g1);
@@ -2001,7 +2013,7 @@ window_score_combine_kernel(int d, const ProbDesc* __restrict__ probs, int nprob
   const int rank = blockIdx.x % SC_CL;
   for (int p = blockIdx.x / SC_CL; p < nprob; p += gridDim.x / SC_CL) {
     const int n = probs[p].n, m = max(probs[p].m, 1);
-    const int gp = chunk_gpp(m, KP), kp = (m + gp - 1) / gp;
+    const int gp = score_gpp(n, m, d), kp = (m + gp - 1) / gp;
     float dot = 0.f, cc = 0.f;
     for (int c = 4 * (rank * AGG_T + threadIdx.x); c < d; c += 4 * AGG_T * SC_CL) {
       float4 cs = make_float4(0.f, 0.f, 0.f, 0.f), ns = cs;
@@ -2271,33 +2283,15 @@ int launch_aggregate(const void* X, int x_dtype, int d, int64_t ldx, const int* 
 }
 
 namespace {
-// Parts per window: the count that makes the slowest CTA's share of rows least,
-// with `slots` CTAs resident and 16 rows' worth of time to start and end a part
-// (eight equal parts of a 2048-token window: 128 windows on 304 CTAs took three
-// rounds of 448 rows, and seven take three of 296).
-int score_parts(int64_t nprob, int64_t nmax, int64_t mmax, int64_t np_cap, int64_t slots) {
-  const int64_t q = (nmax + mmax - 1) / mmax;  // rows of a group
-  int64_t best = 1, cost_best = 0;
-  for (int64_t np = 1; np == 1 || (np <= np_cap && np <= mmax && np * 64 <= nmax); ++np) {
-    const int64_t cost = ((nprob * np + slots - 1) / slots) * (chunk_gpp((int)mmax, (int)np) * q + 16);
-    if (np == 1 || cost < cost_best) best = np, cost_best = cost;
-  }
-  return (int)best;
-}
-
 template <typename T, int NV>
 int launch_score_chunk_nv(const T* X, int d, int64_t ldx, const ProbDesc* probs, int nprob,
-                          int64_t nmax, int64_t mmax, int64_t np_cap, float* part, float* score,
-                          int pos_scheme, int pos_mode, int renorm, float* Xt, int32_t* pos,
-                          int32_t* tok2macro, cudaStream_t stream) {
+                          int64_t nmax, float* part, float* score, int pos_scheme, int pos_mode,
+                          int renorm, float* Xt, int32_t* pos, int32_t* tok2macro,
+                          cudaStream_t stream) {
   auto fn = window_score_chunk_kernel<T, NV>;
-  int dev = 0, sms = 0, occ = 0;
-  SLS_CUDA_TRY(cudaGetDevice(&dev));
-  SLS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   SLS_CUDA_TRY(
       cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, CHK_RING_BYTES));
-  SLS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, AGG_T, CHK_RING_BYTES));
-  const int KP = score_parts(nprob, nmax, mmax, np_cap, (int64_t)(occ < 1 ? 1 : occ) * sms);
+  const int KP = score_parts(nmax, d);
   const int64_t units = (int64_t)nprob * KP;
   const int blocks = (int)(units < 65535 ? units : 65535);
   fn<<<blocks, AGG_T, CHK_RING_BYTES, stream>>>(X, d, ldx, probs, nprob, KP, part, pos_scheme,
@@ -2311,42 +2305,42 @@ int launch_score_chunk_nv(const T* X, int d, int64_t ldx, const ProbDesc* probs,
 
 template <typename T>
 int launch_score_chunk_dtype(const void* X, int d, int64_t ldx, const ProbDesc* probs, int nprob,
-                             int64_t nmax, int64_t mmax, int64_t np_cap, float* part,
-                             float* score, int pos_scheme, int pos_mode, int renorm, float* Xt,
-                             int32_t* pos, int32_t* tok2macro, cudaStream_t stream) {
+                             int64_t nmax, float* part, float* score, int pos_scheme,
+                             int pos_mode, int renorm, float* Xt, int32_t* pos,
+                             int32_t* tok2macro, cudaStream_t stream) {
   const int nv = (d / VecOf<T>::V + AGG_T - 1) / AGG_T;
   auto fn = nv <= 1   ? launch_score_chunk_nv<T, 1>
             : nv <= 2 ? launch_score_chunk_nv<T, 2>
             : nv <= 4 ? launch_score_chunk_nv<T, 4>
                       : launch_score_chunk_nv<T, 8>;
   if (nv > 8) return SLS_ERR_UNSUPPORTED;
-  return fn((const T*)X, d, ldx, probs, nprob, nmax, mmax, np_cap, part, score, pos_scheme,
-            pos_mode, renorm, Xt, pos, tok2macro, stream);
+  return fn((const T*)X, d, ldx, probs, nprob, nmax, part, score, pos_scheme, pos_mode, renorm,
+            Xt, pos, tok2macro, stream);
 }
 }  // namespace
 
-// Part sums go to the aggregation's partial rows, idle at that time; only windows
-// of fewer than 64 tokens (more windows than row pairs there) need room of their
-// own, one part each.
-size_t score_part_floats(int64_t nprob, int64_t Ntot, int d) {
-  return nprob > (int64_t)agg_part_capacity(Ntot) / 2 ? (size_t)nprob * 2 * (size_t)d : 0;
+// Part sums go to the aggregation's partial rows, idle at that time; where those are
+// too few (windows of fewer than 64 tokens; some short prompts of wide rows) they
+// have room of their own.
+size_t score_part_floats(int64_t nprob, int64_t nmax, int64_t Ntot, int d) {
+  const int64_t pairs = nprob * score_parts(nmax, d);
+  return 2 * pairs > (int64_t)agg_part_capacity(Ntot) ? (size_t)pairs * 2 * (size_t)d : 0;
 }
 
 int launch_window_score_chunk(const void* X, int x_dtype, int d, int64_t ldx,
-                              const ProbDesc* probs, int nprob, int64_t nmax, int64_t mmax,
-                              int64_t Ntot, float* agg_part, float* own_part, float* score,
-                              int pos_scheme, int pos_mode, int renorm, float* Xt, int32_t* pos,
+                              const ProbDesc* probs, int nprob, int64_t nmax, int64_t Ntot,
+                              float* agg_part, float* own_part, float* score, int pos_scheme,
+                              int pos_mode, int renorm, float* Xt, int32_t* pos,
                               int32_t* tok2macro, cudaStream_t stream) {
   if (nprob <= 0) return SLS_OK;
-  const int64_t np_cap = (int64_t)agg_part_capacity(Ntot) / 2 / nprob;
-  float* part = np_cap > 0 ? agg_part : own_part;
+  float* part = score_part_floats(nprob, nmax, Ntot, d) == 0 ? agg_part : own_part;
   if (x_dtype == SLS_F32)
-    return launch_score_chunk_dtype<float>(X, d, ldx, probs, nprob, nmax, mmax, np_cap, part,
-                                           score, pos_scheme, pos_mode, renorm, Xt, pos,
-                                           tok2macro, stream);
-  return launch_score_chunk_dtype<uint16_t>(X, d, ldx, probs, nprob, nmax, mmax, np_cap, part,
-                                            score, pos_scheme, pos_mode, renorm, Xt, pos,
-                                            tok2macro, stream);
+    return launch_score_chunk_dtype<float>(X, d, ldx, probs, nprob, nmax, part, score,
+                                           pos_scheme, pos_mode, renorm, Xt, pos, tok2macro,
+                                           stream);
+  return launch_score_chunk_dtype<uint16_t>(X, d, ldx, probs, nprob, nmax, part, score,
+                                            pos_scheme, pos_mode, renorm, Xt, pos, tok2macro,
+                                            stream);
 }
 
 }  // namespace sls

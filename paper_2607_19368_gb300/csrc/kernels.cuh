@@ -149,11 +149,12 @@ int launch_aggregate(const void* X, int x_dtype, int d, int64_t ldx, const int* 
 // the windows the router sends to the chunk path, replaced by the spectral path
 // for the others.  Scratch: agg_part, the aggregation's partial rows
 // (agg_part_capacity(Ntot) * d floats, Ntot at least the windows' tokens), and
-// own_part, score_part_floats(nprob, Ntot, d) floats.
-size_t score_part_floats(int64_t nprob, int64_t Ntot, int d);
+// own_part, score_part_floats(nprob, nmax, Ntot, d) floats; nmax: the longest
+// window's tokens.
+size_t score_part_floats(int64_t nprob, int64_t nmax, int64_t Ntot, int d);
 int launch_window_score_chunk(const void* X, int x_dtype, int d, int64_t ldx,
-                              const ProbDesc* probs, int nprob, int64_t nmax, int64_t mmax,
-                              int64_t Ntot, float* agg_part, float* own_part, float* score,
-                              int pos_scheme, int pos_mode, int renorm, float* Xt, int32_t* pos,
+                              const ProbDesc* probs, int nprob, int64_t nmax, int64_t Ntot,
+                              float* agg_part, float* own_part, float* score, int pos_scheme,
+                              int pos_mode, int renorm, float* Xt, int32_t* pos,
                               int32_t* tok2macro, cudaStream_t stream);
 }  // namespace sls
