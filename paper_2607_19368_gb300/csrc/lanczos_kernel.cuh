@@ -39,9 +39,10 @@
 // re-orthogonalised Lanczos run stays at rounding level, so a second pass
 // would change z1 only in the second order of the rounding unit.  Passes
 // alternate direction so each starts on the rows the previous one left in
-// L2.  Vectors are double-float (two float32) and every sum over N or D is
-// compensated; every sum over the CTAs runs in a fixed order (c and |z'|^2 in
-// float64).  Waits poll without sleeping and give up after about a second of
+// L2.  Vectors are double-float (two float32), every sum over N or D is
+// compensated, and the sums over the CTAs are double-float in a fixed order;
+// |z1|^2 = |z'|^2 - |c|^2, beta, its reciprocal, alpha and the break test are
+// float64.  Waits poll without sleeping and give up after about a second of
 // clock cycles, reporting SLS_ERR_TIMEOUT through the status word.
 //
 // The exchanges.  The CTAs of a group hold no barrier: a value is published as
@@ -74,10 +75,10 @@
 // chain is hidden behind the sweeps of the others, and inside a warp behind the
 // row dots of the next R rows.  Measured against the CTA-wide form with two
 // group barriers per step (whole sls_lanczos_topr calls, both built and timed
-// alternately): 64 windows of 2048 rows at D = 1024, r = 32 5.91 -> 3.87 ms;
-// N = 32756, D = 2048, r = 64 4.57 -> 3.82 ms; N = 8180, D = 1024, r = 32 0.750 ->
-// 0.600 ms; windows of 1024 rows at D = 256 2.95 -> 1.01 ms; N = 12000, D = 1536,
-// r = 48 2.10 -> 1.46 ms; N = 488, D = 256, r = 16 0.308 -> 0.223 ms.
+// alternately): 64 windows of 2048 rows at D = 1024, r = 32 5.92 -> 3.93 ms;
+// N = 32756, D = 2048, r = 64 4.58 -> 3.90 ms; N = 8180, D = 1024, r = 32 0.750 ->
+// 0.596 ms; 64 windows of 1024 rows at D = 256, r = 16 2.99 -> 1.22 ms; N = 488,
+// D = 256, r = 16 0.308 -> 0.231 ms.
 //
 // The kernel is a template over NV (float4 column groups of Phi per lane), WPR,
 // KT (32-wide tiles of the basis index k < r), FULLD (D = 128 NV WPR, no ragged
@@ -251,8 +252,10 @@ struct LzXch {
   unsigned cw_magic;            // c / cw = umulhi(c, cw_magic)
   unsigned rings, ring_bytes;   // offsets: the teams' rings (column sums, coefficients),
   unsigned whs, wls, red, cs;   // w_j, sums of a block, c
-  float2 tol, scale;            // of the break test
-  float2 invb, beta, alpha;     // of the step
+  double tol, scale;            // of the break test
+  double nrm2, inv64, alpha64;  // |z1|^2, 1 / beta and alpha of the step
+  float2 invb, beta;            // 1 / beta and beta as double-float
+  float2 q2;                    // |Phi^T z1|^2 of the step
   float2 tmpw[LZ_NCW];
   int brk;
   volatile int err;             // a wait of this CTA gave up
@@ -301,6 +304,14 @@ SLS_DEV float transpose_sum8(float (&v)[R]) {
   return v[0];
 }
 
+// Whether the sweeps add by Dot2 (10 operations per element) instead of against an
+// offset (5).  An offset is several times the largest sum it may carry, and the low
+// parts round at its scale: over rows of up to 512 columns the plain Dot2 sums leave
+// alpha and beta ten times closer to float64 (N = 1000, D = 256, r = 24: 3e-15 of |T|
+// against 7e-14; 64 windows of 1024 rows there 1.03 -> 1.21 ms).  From D = 1024 on the
+// kernel has always added against offsets (of 512 < D < 1024 a former one lost rows).
+__host__ __device__ constexpr bool lz_dot2(int wpr) { return wpr == 1; }
+
 // Double-float sum without the second renormalisation (11 operations): the
 // error is a few units of the low part, enough for partial sums that are
 // combined once.
@@ -311,6 +322,28 @@ SLS_DEV dfloat df_add_fast(dfloat a, dfloat b) {
   float h, l;
   fast_two_sum(s, e, h, l);
   return df_make(h, l);
+}
+
+// The butterfly of transpose_sum8 on double-floats (any values).
+template <int R>
+SLS_DEV dfloat transpose_sum8_df(float (&h)[R], float (&l)[R]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int s = 0; s < 3; ++s) {
+    const int m = 16 >> s;
+    const int nv = (R >> s) > 1 ? (R >> s) : 1;
+    const bool up = (lane & m) != 0;
+#pragma unroll
+    for (int i = 0; i < (nv > 1 ? nv / 2 : 1); ++i) {
+      const int k = nv > 1 ? i + nv / 2 : i;
+      const dfloat send = nv > 1 && !up ? df_make(h[k], l[k]) : df_make(h[i], l[i]);
+      const dfloat keep = nv > 1 && up ? df_make(h[k], l[k]) : df_make(h[i], l[i]);
+      const dfloat t = df_add_fast(keep, shfl_xor_df(send, m));
+      h[i] = t.hi;
+      l[i] = t.lo;
+    }
+  }
+  return df_make(h[0], l[0]);
 }
 
 // The last step: z1 = z' - Q c (the re-orthogonalisation with c = Q^T z' of
@@ -335,32 +368,8 @@ SLS_DEV void last_row_phase(float2* __restrict__ Qs, int ldq, int nrows, int j,
   }
 }
 
-// 1 / sqrt(x), x > 0: the float32 reciprocal square root y and the correction
-// y (h / 2 + 3 h^2 / 8) with h = 1 - x y^2 formed to double-float precision;
-// |h| < 2^-21, so the series ends below 2^-62 and the rounding of the
-// correction stays near 2^-46 of the result.
-SLS_DEV dfloat df_rsqrt(dfloat x) {
-  // x in the float32 range; a power of four keeps x y^2 clear of its ends
-  float sc = 1.f, scy = 1.f;
-  if (x.hi < 0x1p-90f) {
-    sc = 0x1p60f;
-    scy = 0x1p30f;
-  }
-  x = df_make(x.hi * sc, x.lo * sc);
-  const float y = rsqrtf(x.hi);
-  float p, e;
-  two_prod(y, y, p, e);
-  const dfloat t = df_mul(x, df_make(p, e));
-  const float h = __fsub_rn(__fsub_rn(1.f, t.hi), t.lo);
-  const float corr = y * (h * __fmaf_rn(0.375f, h, 0.5f));
-  const dfloat r = df_norm(y, corr);
-  return df_make(r.hi * scy, r.lo * scy);
-}
-
-// a < b (false if either is NaN)
-SLS_DEV bool df_less(dfloat a, dfloat b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
-
-// A wait of this CTA gave up: report it and leave at the next group barrier.
+// A wait of this CTA gave up: report it; the CTA leaves at its next barrier that
+// reads the flag.
 SLS_DEV void lz_fail(int* status, volatile int* err) {
   atomicExch(status, SLS_ERR_TIMEOUT);
   *err = 1;
@@ -519,10 +528,11 @@ __device__ __noinline__ bool lz_publish(int K, unsigned xpar) {
 
 // c (into shared memory) and beta_{j-1} = |z1|, by one warp: |z1|^2 = |z'|^2 -
 // |c|^2 (Q orthonormal; |c|^2 is below the rounding of |z'|^2 until a
-// breakdown, so its sum over the lanes is plain).  The whole group waits for
-// this chain: double-float (float64 has a long dependent latency on this part)
-// and as few instructions as it takes, since they run cold after each pass.
-SLS_DEV void lz_beta(LzXch& X, int j, const unsigned long long* now, XWait& xw) {
+// breakdown, so its sum over the lanes is plain).  The difference, beta and its
+// reciprocal are float64: q_j is scaled by that reciprocal, and a double-float
+// reciprocal square root, off by up to 2^-46, left that error in every alpha and
+// beta (N = 1000, D = 256: alpha off by 7e-15 of |T| instead of 2e-15).
+SLS_DEV void lz_beta(LzXch& X, const unsigned long long* now, XWait& xw) {
   const int lane = threadIdx.x & 31;
   const int D = X.D, r = X.r;
   float2* cs = reinterpret_cast<float2*>(lz_smem() + X.cs);
@@ -541,34 +551,34 @@ SLS_DEV void lz_beta(LzXch& X, int j, const unsigned long long* now, XWait& xw) 
     cn.lo += __shfl_xor_sync(0xffffffffu, cn.lo, o);
   }
   if (__any_sync(0xffffffffu, n0 == LZ_EMPTY)) n0 = x_poll(now + D + r, true, xw);
-  const dfloat nrm2 = df_sub(x_unpack(n0), df_norm(cn.hi, cn.lo));  // |z1|^2
-  const bool pos = nrm2.hi > 0.f;
-  const dfloat inv = pos ? df_rsqrt(nrm2) : df_make(0.f, 0.f);  // 1 / beta
-  const dfloat bnew = pos ? df_mul(nrm2, inv) : df_make(0.f, 0.f);
   if (lane == 0) {
-    X.invb = f2(inv);
-    X.beta = f2(bnew);
+    const double nrm2 = df_to_double(x_unpack(n0)) - df_to_double(cn);  // |z1|^2
+    const double inv = nrm2 > 0.0 ? rsqrt(nrm2) : 0.0;
+    X.nrm2 = nrm2;
+    X.inv64 = inv;
+    X.invb = f2(df_from_double(inv));
   }
-  (void)j;
 }
 
-// The break test of step j, by the warp that formed beta, while the columns of
-// exchange 3 travel.
+// alpha_j = |Phi^T z1|^2 / beta^2, by the lane that formed 1 / beta.
+SLS_DEV void lz_alpha(LzXch& X, int j) {
+  X.alpha64 = df_to_double(dfv(X.q2)) * X.inv64 * X.inv64;
+  if (X.rank == 0) X.alpha_out[j] = X.alpha64;
+}
+
+// beta_{j-1} and the break test of step j, by one lane of the warp that formed
+// 1 / beta, while the columns of exchange 3 travel.
 SLS_DEV void lz_break_test(LzXch& X, int j) {
-  const dfloat bnew = dfv(X.beta);
-  dfloat scale = dfv(X.scale);
-  bool brk = !(bnew.hi > 0.f);
-  if (j > 0) {
-    const dfloat a = dfv(X.alpha);  // of step j - 1
-    const dfloat sc = df_add(a.hi < 0.f ? df_neg(a) : a, bnew);
-    if (df_less(scale, sc)) scale = sc;
-    brk = !df_less(df_mul(dfv(X.tol), scale), bnew);
-  }
-  __syncwarp();
   if ((threadIdx.x & 31) == 0) {
-    X.scale = f2(scale);
+    const double bnew = X.nrm2 > 0.0 ? X.nrm2 * X.inv64 : 0.0;
+    bool brk = !(bnew > 0.0);
+    if (j > 0) {
+      X.scale = fmax(X.scale, fabs(X.alpha64) + bnew);  // (alpha of step j - 1)
+      brk = !(bnew > X.tol * X.scale);
+    }
     X.brk = brk;
-    if (X.rank == 0 && j > 0 && !brk) X.beta_out[j - 1] = df_to_double(bnew);
+    X.beta = f2(df_from_double(bnew));
+    if (X.rank == 0 && j > 0 && !brk) X.beta_out[j - 1] = bnew;
   }
 }
 
@@ -586,6 +596,7 @@ __device__ __noinline__ void lz_exchange12(int j, unsigned xpar, unsigned x3) {
   const float2* cs = reinterpret_cast<const float2*>(lz_smem() + X.cs);
   const float2* Wm = X.Wm;
   XWait xw{X.poison, X.status, &X.err, 0ll, 0u};
+  if (tid == (NCW - 1) * 32 && j > 0) lz_alpha(X, j - 1);
   unsigned long long* src = X.part + ((size_t)xpar * g + X.rank) * g * own.WB;  // my block
   unsigned long long* now = X.tot + (size_t)x3 * X.E;
   unsigned long long* old = X.tot + (size_t)(x3 == 0u ? 2u : x3 - 1u) * X.E;
@@ -657,7 +668,7 @@ __device__ __noinline__ void lz_exchange12(int j, unsigned xpar, unsigned x3) {
         x_st(old + at, LZ_EMPTY);
       }
     }
-    if (warp == NCW - 1) lz_beta(X, j, now, xw);
+    if (warp == NCW - 1) lz_beta(X, now, xw);
   } else {
     dfloat a = df_make(0.f, 0.f), b = a;
     if (own.mode == 1) {
@@ -686,7 +697,7 @@ __device__ __noinline__ void lz_exchange12(int j, unsigned xpar, unsigned x3) {
         }
       }
     }
-    if (warp == NCW - 1) lz_beta(X, j, now, xw);
+    if (warp == NCW - 1) lz_beta(X, now, xw);
     named_sync(BAR_ALL, NCT);  // c is in shared memory
     if (own.mode == 1) {
       const int q = tid - own.kw;
@@ -744,7 +755,7 @@ __device__ __noinline__ void lz_exchange12(int j, unsigned xpar, unsigned x3) {
 
 // Exchange 3 of step j: Phi^T z1 of every CTA; w_j = Phi^T z1 / beta (into shared
 // memory when STAGE_W; this CTA's columns kept for the correction of later
-// steps) and alpha_j = |w_j|^2, returned packed; LZ_EMPTY when a wait of this CTA
+// steps) and alpha_j = |w_j|^2 = |Phi^T z1|^2 / beta^2, returned packed; LZ_EMPTY when a wait of this CTA
 // has given up.
 template <bool STAGE_W>
 __device__ __noinline__ unsigned long long lz_exchange3(int j, unsigned x3) {
@@ -776,9 +787,10 @@ __device__ __noinline__ unsigned long long lz_exchange3(int j, unsigned x3) {
     for (int u = 0; u < B; ++u)
       if (need >> u & 1u) {
         const int c = 2 * (p0 + tid + u * NCT);
-        const dfloat w0 = df_mul(x_unpack(va[u]), invb), w1 = df_mul(x_unpack(vb[u]), invb);
-        dot2_acc_df(sq.hi, sq.lo, w0, w0);
-        dot2_acc_df(sq.hi, sq.lo, w1, w1);
+        const dfloat z0 = x_unpack(va[u]), z1 = x_unpack(vb[u]);
+        const dfloat w0 = df_mul(z0, invb), w1 = df_mul(z1, invb);
+        dot2_acc_df(sq.hi, sq.lo, z0, z0);
+        dot2_acc_df(sq.hi, sq.lo, z1, z1);
         if (STAGE_W) {
           whs[c >> 1] = make_float2(w0.hi, w1.hi);
           wls[c >> 1] = make_float2(w0.lo, w1.lo);
@@ -803,11 +815,11 @@ __device__ __noinline__ unsigned long long lz_exchange3(int j, unsigned x3) {
   for (int o = 1; o < NCW; o <<= 1) a = df_add_fast(a, shfl_xor_df(a, o));
   a.hi = __shfl_sync(0xffffffffu, a.hi, 0);
   a.lo = __shfl_sync(0xffffffffu, a.lo, 0);
-  if (tid == (NCW - 1) * 32) {  // read by the break test of the next step
-    X.alpha = f2(a);
-    if (X.rank == 0 && !X.brk) X.alpha_out[j] = df_to_double(a);
-  }
-  return x_pack(a);
+  // alpha_j: double-float for the recurrence (whose z' is orthogonalised against q_j
+  // again), float64 as the result and for the break test, formed while the partials
+  // of the next step travel
+  if (tid == (NCW - 1) * 32) X.q2 = f2(a);
+  return x_pack(df_mul(df_mul(a, invb), invb));
 }
 
 // Rows of one team in a ring: batches of R rows are numbered over the CTA's
@@ -907,6 +919,7 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
   constexpr int LPR = 32 / R;               // lanes per row in the row work
   constexpr int TEAMS = NCW / WPR;
   constexpr int NC = 4 * NV;                // columns per lane
+  constexpr bool DOT2 = lz_dot2(WPR);
   using RV = RowVals<R>;
   // basis coefficients per lane: k = sub + LPR * (t * WPR + tw), t < KC
   constexpr int KC = (KT * 32 + LPR * WPR - 1) / (LPR * WPR);
@@ -977,7 +990,7 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
     X.wls = offset(wls);
     X.red = offset(red);
     X.cs = offset(cs);
-    X.tol = f2(df_from_double(bt.tol));
+    X.tol = bt.tol;
     X.err = 0;
   }
   __syncthreads();
@@ -1025,7 +1038,7 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
     if (tid == 0) {  // read after the barriers of the prologue's end
       X.alpha_out = alpha_out;
       X.beta_out = beta_out;
-      X.scale = X.alpha = make_float2(0.f, 0.f);
+      X.scale = 0.0;
     }
     dfloat alpha_df = df_make(0.f, 0.f), beta_df = df_make(0.f, 0.f), invb_df;
     float phimax = 0.f;  // max |Phi| over this CTA's strip (prologue pass)
@@ -1184,6 +1197,7 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
 
       if (j == r - 1) {
         // the last step needs no pass over Phi: q_{r-1} = z1 / beta_{r-2}
+        if (tid == (NCW - 1) * 32) lz_alpha(X, j);
         last_row_phase(Qs, ldq, nrows, j, cs, invb_df);
         reff = r;
         break;
@@ -1222,7 +1236,7 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
       float wtm = wt1;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) wtm = fmaxf(wtm, __shfl_xor_sync(0xffffffffu, wtm, o));
-      const float Ct = ofs_pow2(4.f * (phimax * wtm));
+      const float Ct = DOT2 ? 0.f : ofs_pow2(4.f * (phimax * wtm));
 
       // ---------------- fused pass j+1 over Phi ----------------------------------
       // The team's batches run as a pipeline inside each warp: while a batch's
@@ -1231,7 +1245,7 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
       // issue slots, and the butterfly of those dots runs beside the column
       // sums of the batch before.
       const int pass = j + 1;
-      f32x2_t ah[NC / 2], al[NC / 2], sa[NC / 2];
+      f32x2_t ah[NC / 2], al[NC / 2], sa[NC / 2];  // (sa, Ca, room: not with DOT2)
 #pragma unroll
       for (int c = 0; c < NC / 2; ++c) ah[c] = al[c] = sa[c] = 0ull;
       float Ca = 0.f;    // offset of the column sums (0: none yet)
@@ -1271,8 +1285,9 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
       // against the offset Ct (5 operations per element, common.cuh).  Every
       // part and every sum of up to eight lanes' parts is a multiple of
       // Ct 2^-24 below Ct, so the first three butterfly steps are exact; the
-      // rounding errors travel in the low parts.  And this warp's part of
-      // the re-orthogonalisation (Q c)_i of the lane's row.
+      // rounding errors travel in the low parts.  (DOT2: both are double-float
+      // sums.)  And this warp's part of the re-orthogonalisation (Q c)_i of the
+      // lane's row.
       auto front = [&](auto rows_c, const unsigned char* st, int nr, RV& vh, RV& vl, float& corr) {
         constexpr bool FULL = decltype(rows_c)::value;
         const PT* phi = reinterpret_cast<const PT*>(st);
@@ -1284,15 +1299,28 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
 #pragma unroll
             for (int q = 0; q < NV; ++q) {
               const float4 f = phi_ld4(phi, (size_t)i * C4 + colgroup(q));
-              ofs_step<LZ_PK>(s0, l0, pk2(f.x, f.y), wh[2 * q], wl[2 * q]);
-              ofs_step<LZ_PK>(s0, l0, pk2(f.z, f.w), wh[2 * q + 1], wl[2 * q + 1]);
+              if constexpr (DOT2) {
+                dot2_acc2(s0, l0, pk2(f.x, f.y), wh[2 * q], wl[2 * q]);
+                dot2_acc2(s0, l0, pk2(f.z, f.w), wh[2 * q + 1], wl[2 * q + 1]);
+              } else {
+                ofs_step<LZ_PK>(s0, l0, pk2(f.x, f.y), wh[2 * q], wl[2 * q]);
+                ofs_step<LZ_PK>(s0, l0, pk2(f.z, f.w), wh[2 * q + 1], wl[2 * q + 1]);
+              }
             }
           }
           float sx, sy, lx, ly;
           upk2(s0, sx, sy);
           upk2(l0, lx, ly);
-          vh.v[i] = (sx - Ct) + (sy - Ct);
-          vl.v[i] = lx + ly;
+          if constexpr (DOT2) {
+            float e;
+            two_sum(sx, sy, sx, e);
+            const dfloat t = df_norm(sx, e + (lx + ly));
+            vh.v[i] = t.hi;
+            vl.v[i] = t.lo;
+          } else {
+            vh.v[i] = (sx - Ct) + (sy - Ct);
+            vl.v[i] = lx + ly;
+          }
         }
         const float2* qrow = reinterpret_cast<const float2*>(st + phib) + (size_t)ri * ldq;
         corr = 0.f;
@@ -1312,9 +1340,13 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
       // other warps (the half of the buffer in use was read before the last
       // team barrier)
       auto middle = [&](RV& vh, RV& vl, float& corr, dfloat& s) {
-        const float th = transpose_sum8<R>(vh.v);
-        const float tl = transpose_sum8<R>(vl.v);
-        two_sum(th, tl, s.hi, s.lo);
+        if constexpr (DOT2) {
+          s = transpose_sum8_df<R>(vh.v, vl.v);
+        } else {
+          const float th = transpose_sum8<R>(vh.v);
+          const float tl = transpose_sum8<R>(vl.v);
+          two_sum(th, tl, s.hi, s.lo);
+        }
 #pragma unroll
         for (int o = 2; o > 0; o >>= 1) s = df_add_fast(s, shfl_xor_df(s, o));
 #pragma unroll
@@ -1383,6 +1415,7 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
       // times the l1 norm of the z' accumulated under it stays below Ca / 2
       // (about eight rows of like size)
       auto offset = [&](const RV& uh) {
+        if constexpr (DOT2) return;
         float l1 = 0.f;
 #pragma unroll
         for (int i = 0; i < R; ++i) l1 += fabsf(uh.v[i]);
@@ -1413,8 +1446,13 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
           for (int i = 0; i < R; ++i) {
             if (FULL || i < nr) {
               const float4 f = phi_ld4(phi, (size_t)i * C4 + colgroup(q));
-              ofs_step<LZ_PK>(sa[2 * q], al[2 * q], pk2(f.x, f.y), uhp[i], ulp[i]);
-              ofs_step<LZ_PK>(sa[2 * q + 1], al[2 * q + 1], pk2(f.z, f.w), uhp[i], ulp[i]);
+              if constexpr (DOT2) {
+                dot2_acc2(ah[2 * q], al[2 * q], pk2(f.x, f.y), uhp[i], ulp[i]);
+                dot2_acc2(ah[2 * q + 1], al[2 * q + 1], pk2(f.z, f.w), uhp[i], ulp[i]);
+              } else {
+                ofs_step<LZ_PK>(sa[2 * q], al[2 * q], pk2(f.x, f.y), uhp[i], ulp[i]);
+                ofs_step<LZ_PK>(sa[2 * q + 1], al[2 * q + 1], pk2(f.z, f.w), uhp[i], ulp[i]);
+              }
             }
           }
         }
