@@ -132,9 +132,14 @@ int sls_version(void);
  *   Phi[i, c] = sqrt(2/D) * cos( sum_k X[i, k] * W[c, k] + b[c] ).
  * X: N x d (row stride ldx elements), W: D x d, both of dtype x_dtype;
  * b: D floats; Phi: N x D floats (output, row stride D).
- * bf16 inputs use the tcgen05 tensor cores (fp32 accumulation); fp32 inputs
- * use an fp32 SIMT path.  N may be 0.  Errors: INVALID_ARG for negative or
- * zero sizes, NULL pointers, D % 4 != 0 or D > SLS_MAX_D.
+ * bf16 inputs with D % 256 == 0 and d % 8 == 0 use the tcgen05 tensor cores (fp32
+ * accumulation), fp32 inputs with d >= 512 and d % 4 == 0 too (as three tf32
+ * products, closer to the exact sum than a chain of fp32 multiply-adds); every
+ * other shape, and rows or pointers that are not 16-byte aligned, an fp32 SIMT
+ * path.  The kernels round differently; which one runs depends on d, D and the
+ * alignment, not on N, so a row's features do not depend on the rows beside it.
+ * N may be 0.  Errors: INVALID_ARG for negative or zero sizes, NULL pointers,
+ * D % 4 != 0 or D > SLS_MAX_D; UNSUPPORTED for more than 64 * 65535 fp32 rows.
  */
 int sls_feature_map(const void* X, int x_dtype, int64_t N, int d, int64_t ldx,
                     const void* W, const float* b, int D, float* Phi,

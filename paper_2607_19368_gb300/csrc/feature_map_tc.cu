@@ -158,13 +158,17 @@ SLS_DEV float rff_cos_fast(float x) {
   return __uint_as_float(__float_as_uint(v) ^ ((unsigned)((q + 1) & 2) << 30));
 }
 
-// th = scale * cos(th) for a warp's rows, amax the largest |th| of the thread
+// th = scale * cos(th) for a warp's rows, amax the largest |th| of the thread.  Every
+// element takes the cosine of its own size: a row's bits do not depend on the rows
+// beside it.
 SLS_DEV void rff_cos_block(float (&th)[32], float amax, float scale) {
   if (__all_sync(0xffffffffu, amax <= RFF_COS_FAST_MAX)) {
 #pragma unroll
     for (int e = 0; e < 32; ++e) th[e] = scale * rff_cos_fast(th[e]);
   } else {
-    for (int e = 0; e < 32; ++e) th[e] = scale * rff_cos_wide(th[e]);
+#pragma unroll
+    for (int e = 0; e < 32; ++e)
+      th[e] = scale * (fabsf(th[e]) <= RFF_COS_FAST_MAX ? rff_cos_fast(th[e]) : rff_cos_wide(th[e]));
   }
 }
 
@@ -864,20 +868,20 @@ int launch_feature_map_tc(const void* X, int64_t N, int d, int64_t ldx, const vo
                                        status, phi_bf16);
 }
 
-// Depth and tiles from which float32 inputs go to the tensor cores.  Below K = 512
-// a chain of float32 multiply-adds is as exact; few tiles leave most SMs idle (us,
-// float32 kernel / this one: 8 tiles, d = 512 19 / 25; 12 tiles, d = 2048 70 / 71;
-// 24 tiles, d = 2048 89 / 65; 32 tiles, d = 512 32 / 24).
+// Depth from which float32 inputs go to the tensor cores: below K = 512 a chain of
+// float32 multiply-adds is as exact.  The row count does not enter: the two kernels
+// round differently, and a row's features, whose signs become codes, keep their bits
+// whatever prompt the row is in.  Few tiles leave most SMs idle either way (us, float32
+// kernel / this one: 1 tile, d = 512 18 / 21, d = 2048 59 / 62; 12 tiles, d = 2048
+// 68 / 62; 16 tiles, d = 512 21 / 23; 24 tiles, d = 2048 89 / 65).
 constexpr int TF_MIN_K = 512;
-constexpr int64_t TF_MIN_TILES = 24;
 
 int launch_feature_map_tf32(const void* X, int64_t N, int d, int64_t ldx, const void* W,
                             const float* b, int D, void* Phi, cudaStream_t stream, int* status,
                             int phi_bf16, int inject_fail) {
   const int64_t tiles = ((N + TF_BM - 1) / TF_BM) * ((D + TF_BN - 1) / TF_BN);
-  if (d < TF_MIN_K || tiles < TF_MIN_TILES || N > (int64_t)INT32_MAX - TF_BM ||
-      tiles > (int64_t)INT32_MAX || D % 4 != 0 || d % 4 != 0 || ldx % 4 != 0)
-    return SLS_ERR_UNSUPPORTED;
+  if (d < TF_MIN_K || D % 4 != 0 || d % 4 != 0 || ldx % 4 != 0) return SLS_ERR_UNSUPPORTED;
+  if ((N + 63) / 64 > 65535) return SLS_ERR_UNSUPPORTED;  // the float32 kernel's limit too
   if (((uintptr_t)X & 15) || ((uintptr_t)W & 15) || ((uintptr_t)b & 15) || ((uintptr_t)Phi & 15))
     return SLS_ERR_UNSUPPORTED;
   CUtensorMap mx, mw, mp;

@@ -37,7 +37,7 @@ def _check(phi, X64, W64, b):
     assert np.all(err <= tol), float(np.max(err / tol))
 
 
-# 32 x 32, 64 x 64 and 128 x 128 tiles (by the number of tiles), the depth a
+# 32 x 32, 64 x 64 and 128 x 64 tiles (by the number of tiles), the depth a
 # multiple of the 16-wide slice, of four, and odd
 @pytest.mark.parametrize("N,d,D", [(31, 16, 32), (33, 17, 36), (65, 5, 100), (1500, 31, 1300),
                                    (1793, 40, 1028), (2500, 36, 3076), (3000, 7, 2560)])
