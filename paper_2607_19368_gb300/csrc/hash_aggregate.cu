@@ -9,6 +9,7 @@
 // one 1024-thread CTA per problem (a cluster of them for one large problem, a
 // warp for windows of at most 32 tokens) and touches only integers.  Reading X and
 // writing the macro-token embeddings is spread over the whole GPU.
+#include <atomic>
 #include <climits>
 
 #include "common.cuh"
@@ -692,12 +693,6 @@ segment_kernel(const ProbDesc* __restrict__ probs, int nprob, const uint32_t* __
 // ============================================================================
 
 constexpr int SEGG_MAX = 256;           // CTAs of the grid segment kernel, at most
-
-// One problem of at least SEG_CLUSTER_MIN_N tokens runs on a cluster of SEG_CL
-// CTAs (N = 1500: 148 us on a cluster of eight, 124 on one CTA with its sort in
-// shared memory), above SEG_CLUSTER_MAX_N on a cooperative grid.
-constexpr int SEG_CL = 16;
-constexpr int64_t SEG_CLUSTER_MIN_N = 4096, SEG_CLUSTER_MAX_N = 1 << 18;
 
 // All CTAs of one thread-block cluster meet (arrive: release, wait: acquire, at
 // cluster scope, global memory included).
@@ -2107,6 +2102,50 @@ int launch_simhash_problems(const ProbDesc* probs, const int* spec_list, const i
   return SLS_OK;
 }
 
+namespace {
+// The launch of segment_grid_kernel as one cluster.
+cudaLaunchConfig_t segment_cluster_config(cudaLaunchAttribute* at, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(SEG_CL);
+  cfg.blockDim = dim3(SEG_T);
+  cfg.stream = stream;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = SEG_CL;
+  at->val.clusterDim.y = 1;
+  at->val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Whether the current device can place that cluster (asked once per device).
+cudaError_t segment_cluster_fits(bool* fits) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices];  // 0: not asked yet, 1: no, 2: yes
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int k = dev < kDevices ? known[dev].load() : 0;
+  if (k == 0) {
+    if ((e = cudaFuncSetAttribute(segment_grid_kernel,
+                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) ==
+        cudaSuccess) {
+      cudaLaunchAttribute at;
+      const cudaLaunchConfig_t cfg = segment_cluster_config(&at, nullptr);
+      int clusters = 0;
+      e = cudaOccupancyMaxActiveClusters(&clusters, segment_grid_kernel, &cfg);
+      k = e == cudaSuccess && clusters > 0 ? 2 : 1;
+    } else {
+      k = 1;
+    }
+    if (e != cudaSuccess) (void)cudaGetLastError();  // a device without it: the other kernels
+    if (dev < kDevices) known[dev].store(k);
+  }
+  *fits = k == 2;
+  return cudaSuccess;
+}
+}  // namespace
+
 int launch_segment(const ProbDesc* probs, int nprob, const uint32_t* codes, int pos_scheme,
                    int pos_mode, void* scratch, int slots, int64_t nmax, int64_t mmax, int* perm,
                    int* mstart, int* mlen, int32_t* pos_out, int32_t* tok2macro, int* status,
@@ -2114,7 +2153,11 @@ int launch_segment(const ProbDesc* probs, int nprob, const uint32_t* codes, int 
   if (nprob <= 0) return SLS_OK;
   const SegLayout L = seg_layout(nmax, mmax);
   const size_t stride = L.total;
-  if (nmax <= 32) {
+  bool fits = false;
+  if (segment_route(nprob, nmax, status != nullptr, true) == SegRoute::cluster)
+    SLS_CUDA_TRY(segment_cluster_fits(&fits));
+  const SegRoute route = segment_route(nprob, nmax, status != nullptr, fits);
+  if (route == SegRoute::warp) {
     // windows of at most 32 tokens: one warp per window
     int64_t blocks = ((int64_t)nprob + SEGW_WARPS - 1) / SEGW_WARPS;
     if (blocks > 65535) blocks = 65535;
@@ -2124,33 +2167,19 @@ int launch_segment(const ProbDesc* probs, int nprob, const uint32_t* codes, int 
     SLS_LAUNCH_CHECK();
     return SLS_OK;
   }
-  if (nprob == 1 && nmax >= SEG_CLUSTER_MIN_N && status) {
+  if (route == SegRoute::cluster) {
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg = segment_cluster_config(&at, stream);
+    SLS_CUDA_TRY(cudaFuncSetAttribute(segment_grid_kernel,
+                                      cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    SLS_CUDA_TRY(cudaLaunchKernelEx(&cfg, segment_grid_kernel, probs, codes, pos_scheme, pos_mode,
+                                    (char*)scratch, nmax, mmax, perm, mstart, mlen, pos_out,
+                                    tok2macro, status, chunk_done, 1));
+    count_launch(1);
+    return SLS_OK;
+  }
+  if (route == SegRoute::grid) {
     char* sb = (char*)scratch;
-    if (nmax <= SEG_CLUSTER_MAX_N) {
-      // one problem on one cluster: its hardware barrier costs 0.2 us, the
-      // cooperative grid's 2.5 us, and the computation holds about thirty
-      // (N = 8180: 82 -> 50 us, N = 32756: 132 -> 70)
-      const int G = SEG_CL;
-      SLS_CUDA_TRY(cudaFuncSetAttribute(segment_grid_kernel,
-                                        cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(G);
-      cfg.blockDim = dim3(SEG_T);
-      cfg.stream = stream;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = G;
-      at[0].val.clusterDim.y = 1;
-      at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      SLS_CUDA_TRY(cudaLaunchKernelEx(&cfg, segment_grid_kernel, probs, codes, pos_scheme,
-                                      pos_mode, sb, nmax, mmax, perm, mstart, mlen, pos_out,
-                                      tok2macro, status, chunk_done, 1));
-      count_launch(1);
-      return SLS_OK;
-    }
-    // a larger one: a cooperative grid
     int dev = 0, sms = 0;
     SLS_CUDA_TRY(cudaGetDevice(&dev));
     SLS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

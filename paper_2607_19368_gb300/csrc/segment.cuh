@@ -23,4 +23,32 @@ struct ProbDesc {
   int out_local;     // first output macro index inside its prompt
 };
 
+// Which kernel segments the problems of a launch.
+enum class SegRoute {
+  warp,     // a warp per problem of at most 32 tokens
+  cluster,  // one problem on a thread-block cluster of SEG_CL CTAs
+  grid,     // one problem on a cooperative grid
+  cta       // a CTA per problem
+};
+
+// A cluster of 16 CTAs of 1024 threads is more than every device must place (the
+// portable size is 8): cluster_fits says whether this one does.  Its hardware
+// barrier costs 0.2 us, the grid's 2.5 us, and the computation holds about thirty
+// (N = 8180: 82 -> 50 us, N = 32756: 132 -> 70); below 4096 tokens a CTA by itself,
+// its sort in shared memory, is faster (N = 1500: 124 us against 148), above 262144
+// the grid's SMs are worth their barriers.  Without the cluster the grid starts
+// where it beats one CTA.
+constexpr int SEG_CL = 16;
+constexpr int64_t SEG_CLUSTER_MIN_N = 4096, SEG_CLUSTER_MAX_N = 1 << 18, SEG_GRID_MIN_N = 8192;
+
+inline SegRoute segment_route(int nprob, int64_t nmax, bool has_status, bool cluster_fits) {
+  if (nmax <= 32) return SegRoute::warp;
+  if (nprob == 1 && has_status) {
+    if (cluster_fits && nmax >= SEG_CLUSTER_MIN_N && nmax <= SEG_CLUSTER_MAX_N)
+      return SegRoute::cluster;
+    if (nmax >= SEG_GRID_MIN_N) return SegRoute::grid;
+  }
+  return SegRoute::cta;
+}
+
 }  // namespace sls
