@@ -394,12 +394,12 @@ int sls_compress_tokens(const sls_config_t* cfg, const void* table, int x_dtype,
  * sls_lanczos_topr (the caller still passes Phi, q1 and the output arrays).
  *
  * Scratch lives in one statically sized device array inside the library
- * (SLS_NOALLOC_MAX_BYTES and 24 MiB for the kernel's exchange slots); every
- * GPU that loads the library holds it until the process exits.  No cudaMalloc, cudaFree or allocating
- * library routine is called.  The first call on a device (with that device
- * current) looks up the array's device address once; make that first call
- * before any stream capture.  All calls share the array and it keeps the
- * previous call's contents (what must start at zero is cleared by each
+ * (SLS_NOALLOC_MAX_BYTES and 26 MiB for the kernel's exchange slots); every
+ * GPU that loads the library holds it until the process exits.  No cudaMalloc,
+ * cudaFree or allocating library routine is called.  The first call on a
+ * device (with that device current) looks up the array's device address once;
+ * make that first call before any stream capture.  All calls share the array and it keeps the
+ * previous call's contents (what must start empty is cleared by each
  * call), so calls that overlap on the GPU -- on different streams, or from
  * different host threads -- race and must be serialised by the caller.
  * The looked-up address is cached for the life of the process: after a

@@ -10,10 +10,11 @@
 namespace {
 
 // SLS_NOALLOC_MAX_BYTES bounds the problem (its basis, the coefficient rows and
-// one set of column partials per CTA); the Lanczos kernel's second set of
-// partials and its totals come on top, at most 2 * 152 * (D + r + 2) * 8 bytes
-// at D = 8192, r = 128 and as much again for more SMs.
-constexpr size_t kExchangeExtra = 24u << 20;
+// one set of column partials per CTA); the rest of the Lanczos kernel's exchange
+// slots comes on top.  Two buffers of g x g blocks, a block padded to a power of two
+// of slots: at most 26,223,616 bytes more over every N, D and r and up to 160 SMs
+// (130 CTAs, D = 8192, r = 128: 64 + 1 slots padded to 128).
+constexpr size_t kExchangeExtra = 26u << 20;
 static __device__ __align__(256) unsigned char
     g_noalloc_scratch[SLS_NOALLOC_MAX_BYTES + kExchangeExtra];
 
