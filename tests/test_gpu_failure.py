@@ -44,10 +44,10 @@ def test_stuck_wait_ends_with_timeout_status(sls, which):
 
 def test_lanczos_giveup_leaves_empty_result_and_usable_context(sls):
     """The persistent Lanczos kernel's own give-up path: one CTA reports a
-    failed wait at its first group barrier (as a wait that ran out would), so
-    the group is released, the copy warps stop after their bounded wait, the
-    status reads SLS_ERR_TIMEOUT, r_eff stays -1 and the later kernels treat
-    the problem as empty (theta and U zero) instead of reading stale values.
+    failed wait at its first exchange (as a wait that ran out would), so the
+    other CTAs' polls stop, every copy in flight lands, the status reads
+    SLS_ERR_TIMEOUT, r_eff stays -1 and the later kernels treat the problem as
+    empty (theta and U zero) instead of reading stale values.
     The same problem then runs normally and matches the oracle."""
     g = np.random.default_rng(5)
     N, D, r = 3000, 512, 24

@@ -79,3 +79,17 @@ def test_lanczos_batched_uneven_problems_match_oracle(sls, sizes, D, r):
     theta, U, k = theta.cpu().numpy(), U.cpu().numpy(), k.cpu().numpy()
     for p, (s, n) in enumerate(zip(row0, sizes)):
         _check(theta[p], U[s:s + n], int(k[p]), phi[s:s + n].astype(np.float64), q1[s:s + n], r)
+
+
+@pytest.mark.parametrize("N,D,r", [(7677, 768, 16), (5823, 1024, 16), (14000, 512, 24)])
+def test_lanczos_bf16_full_grid_matches_oracle(sls, N, D, r):
+    """Every SM's CTA at work and rings deeper than a team's batches: the whole next
+    pass is issued ahead while the exchanges run."""
+    phi, q1 = _phi(N, D, N + D)
+    phib = torch.from_numpy(phi).cuda().to(torch.bfloat16)
+    theta, U, k, alpha, _ = sls.lanczos_topr(phib, torch.from_numpy(q1).cuda(), r)
+    phi64 = phib.double().cpu().numpy()
+    _check(theta.cpu().numpy(), U.cpu().numpy(), int(k.item()), phi64, q1, r)
+    # (a row left out of a pass would show in the first step already)
+    a = O.lanczos(phi64, q1, 2)[0]
+    assert np.all(np.abs(alpha.cpu().numpy()[:2] - a) <= 1e-12 * np.abs(a).max())
