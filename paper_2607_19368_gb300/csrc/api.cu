@@ -447,7 +447,7 @@ void carve(const CompressPlan& P, void* ws, CompressWs* W) {
   W->r_eff = cv.take<int>(np);
   W->U = cv.take<float>(spectral ? (size_t)rows * P.r : 0);
   W->codes = cv.take<uint32_t>(spectral ? (size_t)rows : 0);
-  W->lz_bytes = spectral ? lanczos_scratch_bytes(P.nmax, P.D, P.r, P.lz_groups, P.lz_g) : 0;
+  W->lz_bytes = spectral ? lanczos_scratch_bytes(P.D, P.r, P.lz_groups, P.lz_g) : 0;
   W->lz_scratch = cv.take<char>(W->lz_bytes);
   W->seg_scratch = cv.take<char>(segment_scratch_bytes(P.nmax, P.mmax, P.seg_slots));
   W->perm = cv.take<int>(toks);
@@ -535,7 +535,7 @@ int lanczos_single(const void* Phi, int phi_dtype, int64_t N, int D, int r, cons
   double* al = cv.take<double>(r);
   double* be = cv.take<double>(r);
   double* S = cv.take<double>((size_t)r * r);
-  const size_t lzb = lanczos_scratch_bytes(N, D, r, groups, g);
+  const size_t lzb = lanczos_scratch_bytes(D, r, groups, g);
   void* lz = cv.take<char>(lzb);
   SLS_CUDA_TRY(cudaMemsetAsync(status, 0, 256, s));
   if ((st = guards_arm(cv, s)) != SLS_OK) return st;
@@ -835,7 +835,7 @@ size_t sls_lanczos_workspace_size(int64_t N, int D, int r) {
   cv.take<double>(r);
   cv.take<double>(r);
   cv.take<double>((size_t)r * r);
-  cv.take<char>(lanczos_scratch_bytes(N, D, r, groups, g));
+  cv.take<char>(lanczos_scratch_bytes(D, r, groups, g));
   return cv.off;
 }
 
@@ -871,7 +871,7 @@ size_t sls_lanczos_batched_workspace_size(int64_t rows, int64_t nmax, int D, int
   cv.take<double>((size_t)nprob * r);
   cv.take<double>((size_t)nprob * r);
   cv.take<double>((size_t)nprob * r * r);
-  cv.take<char>(lanczos_scratch_bytes(nmax, D, r, groups, g));
+  cv.take<char>(lanczos_scratch_bytes(D, r, groups, g));
   return cv.off;
 }
 
@@ -900,7 +900,7 @@ int sls_lanczos_topr_batched(const void* Phi, int phi_dtype, int D, int r, int n
   double* al = cv.take<double>((size_t)nprob * r);
   double* be = cv.take<double>((size_t)nprob * r);
   double* S = cv.take<double>((size_t)nprob * r * r);
-  const size_t lzb = lanczos_scratch_bytes(nmax, D, r, groups, g);
+  const size_t lzb = lanczos_scratch_bytes(D, r, groups, g);
   void* lz = cv.take<char>(lzb);
   SLS_CUDA_TRY(cudaMemsetAsync(status, 0, 256, s));
   if ((st = guards_arm(cv, s)) != SLS_OK) return st;

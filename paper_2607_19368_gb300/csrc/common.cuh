@@ -204,22 +204,9 @@ SLS_DEV uint64_t l2_policy_evict_first() {
   return p;
 }
 
-SLS_DEV uint64_t l2_policy_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-
-SLS_DEV uint64_t l2_policy_normal() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-
 SLS_DEV void named_sync(unsigned id, unsigned nthreads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
 }
-
 
 // ---------------------------------------------------------------------------
 // memory-model helpers
@@ -229,10 +216,6 @@ SLS_DEV unsigned ld_relaxed_gpu(const unsigned* p) {
   unsigned v;
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
-}
-
-SLS_DEV void st_release_gpu(unsigned* p, unsigned v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 SLS_DEV unsigned atom_add_acq_rel_gpu(unsigned* p, unsigned v) {

@@ -1419,27 +1419,6 @@ struct VecOf<uint16_t> {
   static constexpr int V = 8;
 };
 
-template <typename T>
-SLS_DEV void load_vec(const T* p, float* out);
-template <>
-SLS_DEV void load_vec<float>(const float* p, float* out) {
-  const float4 v = __ldg(reinterpret_cast<const float4*>(p));
-  out[0] = v.x;
-  out[1] = v.y;
-  out[2] = v.z;
-  out[3] = v.w;
-}
-template <>
-SLS_DEV void load_vec<uint16_t>(const uint16_t* p, float* out) {
-  const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
-  const unsigned w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    out[2 * k] = __uint_as_float(w[k] << 16);
-    out[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
-  }
-}
-
 SLS_DEV float agg_block_sum(float v, float* sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   v = warp_sum_f(v);
@@ -1775,19 +1754,6 @@ __host__ __device__ inline int score_gpp(int n, int m, int d) {
   return (m + score_parts(n, d) - 1) / score_parts(n, d);
 }
 
-// 16-byte asynchronous copy global -> shared (zero-filled when !live), and
-// the wait for all but the newest `pending` groups of a thread's copies.
-SLS_DEV void cp16_async(void* dst, const void* src, bool live) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
-               "r"(live ? 16 : 0)
-               : "memory");
-}
-SLS_DEV void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int PENDING>
-SLS_DEV void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
-}
-
 // Rows of a batch staged per thread: slot [buffer][row][column group][thread];
 // two batches of MB * NV = 8 words, the next in flight while one is used (a
 // third stage measured slower: its registers spill).
@@ -1855,12 +1821,12 @@ window_score_chunk_kernel(const T* __restrict__ X, int d, int64_t ldx,
 #pragma unroll
         for (int qv = 0; qv < NV; ++qv) {
           const bool live = rl && (tid + qv * AGG_T) * V < d;
-          cp16_async(&chk_ring[((b * MB + j) * NV + qv) * AGG_T + tid],
-                     live ? xrow + j * ldx + qv * AGG_T * V : X, live);
+          cp_async16(&chk_ring[((b * MB + j) * NV + qv) * AGG_T + tid],
+                     live ? xrow + j * ldx + qv * AGG_T * V : X, live ? 16 : 0);
         }
       }
       xrow += MB * ldx;
-      cp_async_commit();
+      cp_async_commit_group();
     };
     issue(r0, 0);
     int buf = 0;
@@ -1868,9 +1834,9 @@ window_score_chunk_kernel(const T* __restrict__ X, int d, int64_t ldx,
     for (int s0 = r0; s0 < r1; s0 += MB, buf ^= 1) {
       if (s0 + MB < r1) {
         issue(s0 + MB, buf ^ 1);
-        cp_async_wait<1>();
+        cp_async_wait_pending(1);
       } else {
-        cp_async_wait<0>();
+        cp_async_wait_pending(0);
       }
       uint4 raw[MB][NV];
 #pragma unroll

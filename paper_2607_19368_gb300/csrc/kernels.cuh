@@ -92,7 +92,7 @@ struct LanczosBatch {
   int inject_fail;
 };
 
-size_t lanczos_scratch_bytes(int64_t nmax, int D, int r, int groups, int ctas_per_group);
+size_t lanczos_scratch_bytes(int D, int r, int groups, int ctas_per_group);
 // Scratch of one problem's exchange slots beyond one g x D set of column
 // partials, one D-wide total and the scalars' sums (what
 // SLS_NOALLOC_MAX_BYTES counts).

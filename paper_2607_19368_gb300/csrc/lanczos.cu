@@ -447,21 +447,21 @@ int lanczos_plan(int64_t nmax, int D, int r, int nprob, int* groups, int* ctas_p
   return SLS_OK;
 }
 
-size_t lanczos_scratch_bytes(int64_t nmax, int D, int r, int groups, int g) {
-  return (size_t)groups * lz_layout(nmax, D, r, g).total;
+size_t lanczos_scratch_bytes(int D, int r, int groups, int g) {
+  return (size_t)groups * lz_layout(D, r, g).total;
 }
 
 size_t lanczos_exchange_extra(int64_t N, int D, int r) {
   int groups = 0, g = 0;
   if (lanczos_plan(N, D, r, 1, &groups, &g) != SLS_OK) return 0;
-  const LzLayout L = lz_layout(N, D, r, g);
+  const LzLayout L = lz_layout(D, r, g);
   return L.ones_end - (256 + lz_al((size_t)2 * (r + 4) * 8) + lz_al((size_t)g * D * 8) +
                        lz_al((size_t)D * 8));
 }
 
 int launch_lanczos(const LanczosBatch& bt, void* scratch, size_t scratch_bytes, int* status,
                    int groups, int g, cudaStream_t stream) {
-  const LzLayout L = lz_layout(bt.nmax, bt.D, bt.r, g);
+  const LzLayout L = lz_layout(bt.D, bt.r, g);
   if ((size_t)groups * L.total > scratch_bytes) return SLS_ERR_WORKSPACE;
   // the exchange slots of every group start empty (one strided memset)
   SLS_CUDA_TRY(cudaMemset2DAsync((char*)scratch + L.bar, L.total, 0xff, L.ones_end - L.bar,

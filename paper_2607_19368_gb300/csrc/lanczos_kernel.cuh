@@ -150,8 +150,7 @@ struct LzLayout {
 __host__ __device__ inline size_t lz_al(size_t x) { return (x + 255) & ~(size_t)255; }
 __host__ __device__ inline int lz_exch_len(int D, int r) { return (D + r + 2) & ~1; }
 
-__host__ __device__ inline LzLayout lz_layout(int64_t nmax, int D, int r, int g) {
-  (void)nmax;
+__host__ __device__ inline LzLayout lz_layout(int D, int r, int g) {
   LzLayout L;
   const size_t E = (size_t)lz_exch_len(D, r);
   size_t o = 0;
@@ -879,30 +878,9 @@ SLS_DEV dfloat df_recur(dfloat s, dfloat alpha, dfloat q, dfloat beta, dfloat qp
   return df_norm(t2, lo);
 }
 
-// One step of the sweeps on a pair of columns: (s, lo) += x * (yh + yl).
-// PK: one packed instruction per operation, else two scalar ones.
-template <bool PK>
-SLS_DEV void ofs_step(f32x2_t& s, f32x2_t& lo, f32x2_t x, f32x2_t yh, f32x2_t yl) {
-  if constexpr (PK) {
-    ofs_fma_acc2(s, lo, x, yh, yl);
-  } else {
-    float s0, s1, l0, l1, x0, x1, h0, h1, m0, m1;
-    upk2(s, s0, s1);
-    upk2(lo, l0, l1);
-    upk2(x, x0, x1);
-    upk2(yh, h0, h1);
-    upk2(yl, m0, m1);
-    ofs_fma_acc(s0, l0, x0, h0, m0);
-    ofs_fma_acc(s1, l1, x1, h1, m1);
-    s = pk2(s0, s1);
-    lo = pk2(l0, l1);
-  }
-}
-
-// The sweeps run on packed float32 pairs: against scalar steps the packed form
-// halves the issue slots of the same arithmetic (lanczos 32k 4434 -> 4054 us,
-// windows of 2048 rows 4693 -> 4270 us, 8k 771 -> 733 us).
-constexpr bool LZ_PK = true;
+// The sweeps run on packed float32 pairs, one instruction per operation of two
+// columns: scalar steps take twice the issue slots of the same arithmetic (lanczos
+// 32k 4434 -> 4054 us, windows of 2048 rows 4693 -> 4270 us, 8k 771 -> 733 us).
 
 // One float per row of a batch.
 template <int R>
@@ -963,7 +941,7 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
   if (tid == 0) {
     for (int s = 0; s < TEAMS * ring_stages; ++s) mbar_init(&fullb[s], 1);
     mbar_fence_init();
-    const LzLayout L = lz_layout(bt.nmax, D, r, g);
+    const LzLayout L = lz_layout(D, r, g);
     char* gb = scratch + (size_t)gi * gstride;
     auto offset = [&](const void* p) {
       return (unsigned)(reinterpret_cast<const unsigned char*>(p) - smem_raw);
@@ -1303,8 +1281,8 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
                 dot2_acc2(s0, l0, pk2(f.x, f.y), wh[2 * q], wl[2 * q]);
                 dot2_acc2(s0, l0, pk2(f.z, f.w), wh[2 * q + 1], wl[2 * q + 1]);
               } else {
-                ofs_step<LZ_PK>(s0, l0, pk2(f.x, f.y), wh[2 * q], wl[2 * q]);
-                ofs_step<LZ_PK>(s0, l0, pk2(f.z, f.w), wh[2 * q + 1], wl[2 * q + 1]);
+                ofs_fma_acc2(s0, l0, pk2(f.x, f.y), wh[2 * q], wl[2 * q]);
+                ofs_fma_acc2(s0, l0, pk2(f.z, f.w), wh[2 * q + 1], wl[2 * q + 1]);
               }
             }
           }
@@ -1450,8 +1428,8 @@ lanczos_kernel(LanczosBatch bt, char* scratch, size_t gstride, int g, int ngroup
                 dot2_acc2(ah[2 * q], al[2 * q], pk2(f.x, f.y), uhp[i], ulp[i]);
                 dot2_acc2(ah[2 * q + 1], al[2 * q + 1], pk2(f.z, f.w), uhp[i], ulp[i]);
               } else {
-                ofs_step<LZ_PK>(sa[2 * q], al[2 * q], pk2(f.x, f.y), uhp[i], ulp[i]);
-                ofs_step<LZ_PK>(sa[2 * q + 1], al[2 * q + 1], pk2(f.z, f.w), uhp[i], ulp[i]);
+                ofs_fma_acc2(sa[2 * q], al[2 * q], pk2(f.x, f.y), uhp[i], ulp[i]);
+                ofs_fma_acc2(sa[2 * q + 1], al[2 * q + 1], pk2(f.z, f.w), uhp[i], ulp[i]);
               }
             }
           }
