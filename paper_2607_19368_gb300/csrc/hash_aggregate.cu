@@ -1721,10 +1721,11 @@ agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __rest
 // of x/|x|; window_score_combine_kernel adds a window's parts in order and forms
 // the score.  The parts are a function of the window and the row width alone, so a
 // window's score, and with it its route, has the same bits alone, in any batch and
-// on any number of SMs, and no chain of sums grows with the batch.  About 128 rows
-// each (64 of rows wider than 4096): parts that fill the GPU evenly for the batch at
-// hand are a little faster (16 prompts of 16384 tokens, d = 4096: the pass in 572 us
-// against 599; one prompt 132 against 141), parts of 256 rows slower (607; 189).
+// on any number of SMs, and no chain of sums grows with the batch.  About 80 rows
+// each (64 of rows wider than 4096).  Pass times in us for 16 prompts of 16384 tokens,
+// one of 9000 and two of 12764 (d = 4096, 4096, 3496): parts that fill the GPU evenly for
+// the batch at hand 573, 123, 158; 64 rows 626, 122, 167; 80 rows 611, 129, 149; 128 rows
+// 600, 144, 179; one part per 256 rows 607 and up to half as long again.
 
 // ---------------------------------------------------------------------------
 // The score pass with the chunk path folded in (adaptive backend below rho =
@@ -1747,7 +1748,7 @@ __host__ __device__ inline int chunk_gstart(int n, int m, int g) {
 }
 // parts of a window of n tokens, at most, and groups per part
 __host__ __device__ inline int score_parts(int64_t n, int d) {
-  const int rows = d > 4096 ? 64 : 128;
+  const int rows = d > 4096 ? 64 : 80;
   return n < rows ? 1 : (int)(n / rows);
 }
 __host__ __device__ inline int score_gpp(int n, int m, int d) {
@@ -2315,8 +2316,8 @@ int launch_score_chunk_dtype(const void* X, int d, int64_t ldx, const ProbDesc* 
 }  // namespace
 
 // Part sums go to the aggregation's partial rows, idle at that time; where those are
-// too few (windows of fewer than 64 tokens; some short prompts of wide rows) they
-// have room of their own.
+// too few (windows of fewer than 64 tokens; prompts of hardly more than one window;
+// some of wide rows) they have room of their own.
 size_t score_part_floats(int64_t nprob, int64_t nmax, int64_t Ntot, int d) {
   const int64_t pairs = nprob * score_parts(nmax, d);
   return 2 * pairs > (int64_t)agg_part_capacity(Ntot) ? (size_t)pairs * 2 * (size_t)d : 0;
