@@ -1579,15 +1579,42 @@ SLS_DEV float warp_sums(float (&v)[R]) {
 // macro_embed) or stores them as a partial sum.
 //
 // Bound by reading X: an SM keeps 100 KB of rows in flight, and an item's chain of
-// descriptor, member ids and rows hides behind the other CTAs'.
+// descriptor, member ids and rows hides behind the other CTAs', unless its members are
+// few: then the chain is the time, and the next item's is fetched ahead.  Whole calls,
+// us (a bulk copy per row as below / neither / fetched ahead / ahead on twice the CTAs;
+// groups of m consecutive tokens):
+//   N = 32768, d = 3584 bf16   m = 1  321 / 426 / 370 / 250     m = 2  278 / 266 / 239 / 178
+//                              m = 4  246 / 175 / 166 / 148     m = 8  232 / 124 / 121 / 122
+//   N = 131072, d = 5120 bf16  m = 2  684 / 920 / 815           m = 4  532 / 640 / 579
+// On Zipf-distributed codes fetching ahead costs 2% at rho = 16 (N = 32756, d = 3584:
+// 151 -> 154 us), and twice the CTAs draw out a long item (rho = 4, N = 3000: 98 -> 115):
+// hence the lines at 6 and 3 members.
 // The former pass streamed each row through a shared-memory ring with one bulk
 // copy per row; issuing those took a producer warp about 1000 cycles per row
 // (N = 32756, d = 3584: 90 -> 58 us, against 35 us for the bytes; N = 8180,
 // d = 4096: 43 -> 29).
 // ---------------------------------------------------------------------------
 
-template <typename T, int NV>
-__global__ void __launch_bounds__(AGG_T, NV == 1 ? 4 : 2)
+// Which items the launch expects, by the members per macro-token.
+enum AggItems {
+  AGG_LONG,   // 6 members and more
+  AGG_FEW,    // fewer: an item's chain of ticket, descriptor and ids outlasts its rows, so
+              // the next item's is fetched while this one's rows arrive
+  AGG_BRIEF   // fewer than 3, NV = 2: besides, batches of two rows on twice the CTAs
+};
+
+// Rows per batch and CTAs per SM.
+template <int NV, AggItems K>
+constexpr int agg_rows() {
+  return NV != 2 ? agg_batch<NV>() : K == AGG_BRIEF ? 2 : 8;
+}
+template <int NV, AggItems K>
+constexpr int agg_ctas() {
+  return NV == 1 || K == AGG_BRIEF ? 4 : 2;
+}
+
+template <typename T, int NV, AggItems K>
+__global__ void __launch_bounds__(AGG_T, agg_ctas<NV, K>())
 agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __restrict__ perm,
                   const int* __restrict__ mstart, const int* __restrict__ mlen,
                   const int2* __restrict__ items, int* __restrict__ aux,
@@ -1599,7 +1626,8 @@ agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __rest
   // NV = 2 (d up to 4096 in bf16): twice the rows in flight on half the CTAs, so
   // that a long item ends sooner (N = 8180, d = 4096: 31 -> 26 us); NV = 1 keeps
   // four CTAs (N = 20000, d = 512: 198 us for the call against 227).
-  constexpr int MB = NV == 2 ? 8 : agg_batch<NV>();
+  constexpr int MB = agg_rows<NV, K>();
+  constexpr bool AHEAD = K != AGG_LONG;
   constexpr int NW = AGG_T / 32, LPR = 32 / MB;
   __shared__ float shq[2][AGG_CH][NW];  // row |x|^2 by warp
   __shared__ float shm[2][NW];          // |member sum|^2 by warp
@@ -1609,21 +1637,45 @@ agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __rest
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int* counts = agg_aux(aux).counts;
   const int nitems = counts[0];
-  int buf = 0;
-  for (int it = blockIdx.x; it < nitems; it = s_next[buf], buf ^= 1) {
-    const int2 item = items[it];
-    // the next item, handed out by a ticket (read after the item's barrier)
-    if (tid == 0) s_next[buf] = (int)gridDim.x + atomicAdd(&counts[3], 1);
-    const int m = item.x, c = item.y;
-    const int len = mlen[m], ps = pt_start[m];
-    const int n = min(len - c * AGG_CH, AGG_CH);
-    const int* ids = perm + mstart[m] + c * AGG_CH;
+  // An item: its macro-token m (len members, partial slot ps), chunk c of it, the first
+  // of its n member ids, and with `id` those of its first 32 rows, a lane each.
+  struct Item {
+    int m, c, len, ps, first, id;
+    __device__ int n() const { return min(len - c * AGG_CH, AGG_CH); }
+  };
+  auto open_item = [&](Item& I, int2 mc) {
+    I.m = mc.x;
+    I.c = mc.y;
+    I.len = mlen[mc.x];
+    I.ps = pt_start[mc.x];
+    I.first = mstart[mc.x] + mc.y * AGG_CH;
+  };
+  auto fetch_ids = [&](Item& I) { I.id = lane < I.n() ? perm[I.first + lane] : 0; };
+  Item I{};
+  int buf = 0, it = blockIdx.x;
+  int nx = it + gridDim.x;  // AHEAD: the item after this one
+  if (AHEAD && it < nitems) {
+    open_item(I, items[it]);
+    fetch_ids(I);
+  }
+  while (it < nitems) {
+    if (!AHEAD) {
+      open_item(I, items[it]);
+      fetch_ids(I);
+    }
+    // a later item, handed out by a ticket (read after this one's barrier)
+    if (tid == 0) s_next[buf] = (AHEAD ? 2 : 1) * (int)gridDim.x + atomicAdd(&counts[3], 1);
+    Item X1{};
+    int2 next_mc = make_int2(0, 0);
+    if (AHEAD && nx < nitems) next_mc = items[nx];
+    const int m = I.m, c = I.c, len = I.len, ps = I.ps, n = I.n();
+    const int* ids = perm + I.first;
     f32x2_t acc[PN];
 #pragma unroll
     for (int e = 0; e < PN; ++e) acc[e] = 0ull;
-    int id = 0;
+    int id = I.id;
     for (int s = 0; s < n; s += MB) {
-      if ((s & 31) == 0) id = s + lane < n ? ids[s + lane] : 0;  // MB divides 32
+      if (s != 0 && (s & 31) == 0) id = s + lane < n ? ids[s + lane] : 0;  // MB divides 32
       uint4 raw[MB][NV];
 #pragma unroll
       for (int j = 0; j < MB; ++j) {
@@ -1644,6 +1696,9 @@ agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __rest
           if (s + j < n && c0 < d) raw[j][q] = __ldcs(reinterpret_cast<const uint4*>(x + c0));
         }
       }
+      // the next item's lengths and offsets while this one's rows are on their way, its
+      // ids below
+      if (AHEAD && s == 0 && nx < nitems) open_item(X1, next_mc);
       float sq[MB];
 #pragma unroll
       for (int j = 0; j < MB; ++j) {
@@ -1661,6 +1716,7 @@ agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __rest
       const float t = warp_sums<MB>(sq);
       if (lane % LPR == 0 && s + lane / LPR < n) shq[buf][s + lane / LPR][warp] = t;
     }
+    if (AHEAD && nx < nitems) fetch_ids(X1);
     float v[NV * V];
     float msq = 0.f;
 #pragma unroll
@@ -1706,6 +1762,11 @@ agg_member_kernel(const T* __restrict__ X, int d, int64_t ldx, const int* __rest
       if (tid == 0) part_eta[ps + c] = eta;
     }
     store_row<V, NV>(v, scale, d, dst);
+    const int ticket = s_next[buf];
+    buf ^= 1;
+    it = AHEAD ? nx : ticket;
+    nx = ticket;
+    if (AHEAD) I = X1;
   }
 }
 
@@ -2228,12 +2289,15 @@ int launch_agg_t(const void* X, int d, int64_t ldx, const int* perm, const int* 
   SLS_LAUNCH_CHECK();
   // CTAs that fit the GPU at once; items by ticket
   int occ = 0;
-  SLS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, agg_member_kernel<T, NV>,
-                                                             AGG_T, 0));
+  auto fn = agg_member_kernel<T, NV, AGG_LONG>;
+  if (Ntot < 6 * Mtot) fn = agg_member_kernel<T, NV, AGG_FEW>;
+  if constexpr (NV == 2)
+    if (Ntot < 3 * Mtot) fn = agg_member_kernel<T, NV, AGG_BRIEF>;
+  SLS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, AGG_T, 0));
   int64_t grid = (int64_t)sms * (occ < 1 ? 1 : occ);
   const int64_t most = Mtot + Ntot / AGG_CH;  // items at most
   if (grid > most) grid = most;
-  agg_member_kernel<T, NV><<<(unsigned)grid, AGG_T, 0, stream>>>(
+  fn<<<(unsigned)grid, AGG_T, 0, stream>>>(
       (const T*)X, d, ldx, perm, mstart, mlen, items, aux, pt_start, renorm, Xt, part, part_eta,
       status, Ntot);
   SLS_LAUNCH_CHECK();
