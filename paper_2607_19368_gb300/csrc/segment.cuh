@@ -35,11 +35,14 @@ enum class SegRoute {
 // portable size is 8): cluster_fits says whether this one does.  Its hardware
 // barrier costs 0.2 us, the grid's 2.5 us, and the computation holds about thirty
 // (N = 8180: 82 -> 50 us, N = 32756: 132 -> 70); below 4096 tokens a CTA by itself,
-// its sort in shared memory, is faster (N = 1500: 124 us against 148), above 262144
-// the grid's SMs are worth their barriers.  Without the cluster the grid starts
-// where it beats one CTA.
+// its sort in shared memory, is faster (N = 1500: 124 us against 148), above 81920
+// the grid's SMs are worth their barriers.  Calls on Zipf-distributed codes, us, cluster
+// / grid, 16 bits and rho = 16, 16 and 4, 8 and 8: N = 65536 155 / 191, 363 / 361, 223 /
+// 249; 81920 181 / 202, 430 / 409, 247 / 262; 98304 204 / 213, 530 / 481, 283 / 282;
+// 131060 458 / 378, 623 / 544, 342 / 317; 262144 633 / 467, 1029 / 862, 581 / 480.
+// Without the cluster the grid starts where it beats one CTA.
 constexpr int SEG_CL = 16;
-constexpr int64_t SEG_CLUSTER_MIN_N = 4096, SEG_CLUSTER_MAX_N = 1 << 18, SEG_GRID_MIN_N = 8192;
+constexpr int64_t SEG_CLUSTER_MIN_N = 4096, SEG_CLUSTER_MAX_N = 81920, SEG_GRID_MIN_N = 8192;
 
 inline SegRoute segment_route(int nprob, int64_t nmax, bool has_status, bool cluster_fits) {
   if (nmax <= 32) return SegRoute::warp;

@@ -1,6 +1,6 @@
 """Clusters, exact-length adjustment and macro-tokens (Sec. 3.3-3.4) of one prompt
 at the edges of the cluster launch (from 4096 tokens) and of the cooperative grid
-above 262144, against the oracle: maps bit for bit.  Embeddings within 1e-4: a
+above 81920, against the oracle: maps bit for bit.  Embeddings within 1e-4: a
 member sum adds 64 rows in order and then N / 64 partial sums, so its error per
 member is below (64 + N / 64) 2^-24 max |x| (N = 9001: 205 x 6e-8 x 5 = 6e-5; the
 larger N have at most a few hundred members in a macro-token).  The code distributions cover merging (more
@@ -43,6 +43,7 @@ def _codes(g, N, kind):
     (4096, 264, 17, "many", "max"), (8180, 2056, 511, "many", "max"),
     (9001, 24, 4000, "few", "median"), (9001, 24, 5, "one", "max"),
     (9001, 24, 900, "one", "mean"), (40000, 16, 2500, "wide", "mean"),
+    (81920, 8, 20000, "few", "median"), (81921, 8, 5000, "wide", "mean"),
     (262144, 8, 16384, "many", "max"), (262145, 8, 16384, "few", "max")])
 def test_aggregate_cluster_matches_oracle(sls, N, d, M, kind, scheme):
     g = np.random.default_rng(N + M)

@@ -29,7 +29,7 @@ def route(tmp_path_factory):
 
 
 def test_routes(route):
-    one = [1, 32, 33, 4095, 4096, 8191, 8192, 262144, 262145, 1 << 30]
+    one = [1, 32, 33, 4095, 4096, 8191, 8192, 81920, 81921, 1 << 30]
     assert route(*[(1, n, 1, 1) for n in one]) == [
         WARP, WARP, CTA, CTA, CLUSTER, CLUSTER, CLUSTER, CLUSTER, GRID, GRID]
     # no cluster on this device: one CTA up to 8191 tokens, the grid from there
