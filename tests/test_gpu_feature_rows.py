@@ -52,3 +52,20 @@ def test_a_row_of_huge_arguments_leaves_its_neighbours(sls, dtype, d, D):
     want = (2.0 / D) ** 0.5 * torch.cos(X[70].double() @ W.double().T + b.double())
     # float32 sums of about 1e6 leave 2^-24 of that in the argument, a few times over
     assert (got[70].double() - want).abs().max() <= (2.0 / D) ** 0.5 * 8 * 5e6 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("phi_dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("N,d,D", [(40, 64, 36), (900, 72, 700), (5000, 65, 1060)])
+def test_unaligned_output(sls, N, d, D, phi_dtype):
+    """Phi at an address that forbids wide stores, in each tile size of the float32
+    kernel; the elements around it stay as they are."""
+    g = torch.Generator(device="cuda").manual_seed(N)
+    X = torch.randn(N, d, generator=g, device="cuda") / d ** 0.5
+    W = torch.randn(D, d, generator=g, device="cuda")
+    b = torch.rand(D, generator=g, device="cuda") * 6.28
+    ref = sls.feature_map(X, W, b, phi_dtype=phi_dtype)
+    for off in (1, 2, 3):
+        buf = torch.full((N * D + 8,), 7.0, device="cuda", dtype=phi_dtype)
+        got = sls.feature_map(X, W, b, out=buf[off:off + N * D].view(N, D))
+        assert torch.equal(got, ref)
+        assert torch.all(buf[:off] == 7.0) and torch.all(buf[off + N * D:] == 7.0)
